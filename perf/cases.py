@@ -215,7 +215,10 @@ def _leaves(nz, ny, nx, g):
     solid = torch.zeros((nz, ny, nx), dtype=torch.bool, device=DEV)
     axes = 0.02 + 0.04 * torch.rand((50, 3), generator=g, device=DEV)
     ctr = 0.3 + 0.4 * torch.rand((50, 3), generator=g, device=DEV)
-    q, _ = torch.linalg.qr(torch.randn((50, 3, 3), generator=g, device=DEV))
+    q = torch.randn((50, 3, 3), generator=g, device=DEV)
+    a = torch.nn.functional.normalize(q[:, 0], dim=1)  # random orientations
+    b = torch.nn.functional.normalize(q[:, 1] - (q[:, 1] * a).sum(1, True) * a, dim=1)
+    q = torch.stack([a, b, torch.linalg.cross(a, b, dim=1)], 1)
     for e in range(50):
         d = torch.einsum("ab,azyx->bzyx", q[e], pos - ctr[e].view(3, 1, 1, 1))
         solid |= ((d / axes[e].view(3, 1, 1, 1)) ** 2).sum(0) <= 1.0

@@ -681,9 +681,12 @@ DW_API dw_status lbm_init_equilibrium(dw_lbm h, float *f, float rho0, const floa
 DW_API dw_status lbm_home_init(dw_lbm h, float *m, float rho0, const float u0[3],
                                dw_stream stream);
 
-/* Advance m in place by `steps` HOME-LBM steps (pull streaming between m and
- * the handle's tape in turn, so max_tape >= 1 suffices; an odd step count ends
- * with one device copy back into m). solid as in lbm_step. */
+/* Advance m in place by `steps` HOME-LBM steps. The handle's tape is the
+ * workspace (max_tape >= 1 suffices): it holds the populations rebuilt from m
+ * while the steps of the call run on them in place (the AA pattern of
+ * lbm_step), or, for a few steps of a large lattice, a second moment lattice
+ * (an odd step count then ends with one device copy back into m). solid as
+ * in lbm_step. */
 DW_API dw_status lbm_home_step(dw_lbm h, float *m, const uint8_t *solid, int32_t steps,
                                dw_stream stream);
 

@@ -154,6 +154,21 @@ __device__ __forceinline__ int cell_index(const LbmParams &L, int x, int y, int 
 
 // ---------------------------------------------------------------- forward --
 
+// The even kernel's writes: every post-collision population into the own
+// cell's opposite slot, the outlet face's five into the side buffer.
+__device__ __forceinline__ void aa_keep(const LbmParams &L, float *f, float *__restrict__ outlet,
+                                        int x, int y, int z, int cell, const float fl[19]) {
+    const int nc = L.ncell;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[D3Q19::opp(i) * nc + cell] = fl[i];
+    if (L.bc_x == 1 && x == L.nx - 1) {
+        const int face = z * L.ny + y, nface = L.ny * L.nz;
+#pragma unroll
+        for (int i = 0; i < 19; ++i)
+            if (outlet_slot(i) >= 0) outlet[outlet_slot(i) * nface + face] = fl[i];
+    }
+}
+
 __global__ void __launch_bounds__(256, 5) k_lbm_aa_even(LbmParams L, float *f,
                                                     const uint8_t *__restrict__ solid,
                                                     float *__restrict__ outlet) {
@@ -167,17 +182,7 @@ __global__ void __launch_bounds__(256, 5) k_lbm_aa_even(LbmParams L, float *f,
 #pragma unroll
     for (int i = 0; i < 19; ++i) fl[i] = f[i * nc + cell];
     collide(L, fl);
-#pragma unroll
-    for (int i = 0; i < 19; ++i) f[D3Q19::opp(i) * nc + cell] = fl[i];
-    if (L.bc_x == 1) {
-        if (x == L.nx - 1) {
-            int face = z * L.ny + y;
-            int nface = L.ny * L.nz;
-#pragma unroll
-            for (int i = 0; i < 19; ++i)
-                if (outlet_slot(i) >= 0) outlet[outlet_slot(i) * nface + face] = fl[i];
-        }
-    }
+    aa_keep(L, f, outlet, x, y, z, cell, fl);
 }
 
 // Offsets of the neighbours with the periodic wraps folded in: the neighbour
@@ -224,18 +229,13 @@ __global__ void __launch_bounds__(256) k_lbm_links(LbmParams L, const uint8_t *_
     links[cell] = m;
 }
 
-__global__ void __launch_bounds__(256, 5) k_lbm_aa_odd(LbmParams L, float *f,
-                                                      const uint32_t *__restrict__ links,
-                                                      const float *__restrict__ outlet) {
-    pdl_wait();
-    pdl_trigger();
-    int x, y, z, cell;
-    if (!lattice_cell(L, x, y, z, cell)) return;
-    const uint32_t lk = links ? links[cell] : 0u;
-    if (lk & 1u) return;
+// The odd kernel's reads: the populations streamed into a cell, f_i from slot
+// opp(i) of cell x - c_i (lk: the cell's link word).
+__device__ __forceinline__ void aa_pull(const LbmParams &L, const float *f,
+                                        const float *__restrict__ outlet, uint32_t lk,
+                                        const NbrOffsets &o, int x, int y, int z, int cell,
+                                        float fl[19]) {
     const int nc = L.ncell;  // 19 * ncell < 2^31 is checked at create
-    const NbrOffsets o = nbr_offsets(L, x, y, z);
-    float fl[19];
     fl[0] = f[cell];  // rest population: own slot 0 in both orders
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
@@ -258,7 +258,13 @@ __global__ void __launch_bounds__(256, 5) k_lbm_aa_odd(LbmParams L, float *f,
                 if (D3Q19::cx(i) == -1) fl[i] = outlet[outlet_slot(i) * nface + face];
         }
     }
-    collide(L, fl);
+}
+
+// The odd kernel's writes: post-collision population i into slot i of cell
+// x + c_i, which leaves the lattice in natural order.
+__device__ __forceinline__ void aa_push(const LbmParams &L, float *f, uint32_t lk,
+                                        const NbrOffsets &o, int x, int cell, const float fl[19]) {
+    const int nc = L.ncell;
     f[cell] = fl[0];
     const bool inlet_face = L.bc_x == 1 && x == 0, outlet_face = L.bc_x == 1 && x == L.nx - 1;
 #pragma unroll
@@ -280,6 +286,22 @@ __global__ void __launch_bounds__(256, 5) k_lbm_aa_odd(LbmParams L, float *f,
         for (int i = 1; i < 19; ++i)
             if (D3Q19::cx(i) == -1) f[i * nc + cell] = fl[i];
     }
+}
+
+__global__ void __launch_bounds__(256, 5) k_lbm_aa_odd(LbmParams L, float *f,
+                                                      const uint32_t *__restrict__ links,
+                                                      const float *__restrict__ outlet) {
+    pdl_wait();
+    pdl_trigger();
+    int x, y, z, cell;
+    if (!lattice_cell(L, x, y, z, cell)) return;
+    const uint32_t lk = links ? links[cell] : 0u;
+    if (lk & 1u) return;
+    const NbrOffsets o = nbr_offsets(L, x, y, z);
+    float fl[19];
+    aa_pull(L, f, outlet, lk, o, x, y, z, cell, fl);
+    collide(L, fl);
+    aa_push(L, f, lk, o, x, cell, fl);
 }
 
 // One collide + push step between two lattices in natural order. Solid cells
@@ -849,6 +871,30 @@ __host__ __device__ __forceinline__ void home_rebuild_all(const float a[10], flo
     }
 }
 
+// Sums of the pulled deviations over pairs of opposite directions (2k - 1,
+// 2k): s = g + g_opp carries the even moments, d = g - g_opp the odd ones.
+__host__ __device__ __forceinline__ void home_sums(const float g[19], float &dr, float j[3],
+                                                   float P[6]) {
+    dr = g[0];
+    j[0] = j[1] = j[2] = 0.0f;
+    P[0] = P[1] = P[2] = P[3] = P[4] = P[5] = 0.0f;
+#pragma unroll
+    for (int i = 1; i < 19; i += 2) {
+        const int cx = D3Q19::cx(i), cy = D3Q19::cy(i), cz = D3Q19::cz(i);
+        const float sp = g[i] + g[i + 1], dp = g[i] - g[i + 1];
+        dr += sp;
+        if (cx) j[0] += (float)cx * dp;
+        if (cy) j[1] += (float)cy * dp;
+        if (cz) j[2] += (float)cz * dp;
+        if (cx) P[0] += sp;
+        if (cy) P[1] += sp;
+        if (cz) P[2] += sp;
+        if (cx && cy) P[3] += (float)(cx * cy) * sp;
+        if (cx && cz) P[4] += (float)(cx * cz) * sp;
+        if (cy && cz) P[5] += (float)(cy * cz) * sp;
+    }
+}
+
 // Moment-space collision from the pulled deviations' sums: dr = sum g,
 // j = sum c g, P = sum c c g (= Pi - I/3); writes the ten stored moments.
 __host__ __device__ __forceinline__ void home_collide(const LbmParams &L, float dr, const float j[3],
@@ -1044,24 +1090,8 @@ __host__ __device__ __forceinline__ void home_tile_cell(const LbmParams &L, cons
             }
         }
     }
-    // moments over pairs of opposite directions (2k - 1, 2k): s = g + g_opp
-    // carries the even moments, d = g - g_opp the odd ones
-    float dr = g[0], j[3] = {0.0f, 0.0f, 0.0f}, P[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int i = 1; i < 19; i += 2) {
-        const int cx = D3Q19::cx(i), cy = D3Q19::cy(i), cz = D3Q19::cz(i);
-        const float sp = g[i] + g[i + 1], dp = g[i] - g[i + 1];
-        dr += sp;
-        if (cx) j[0] += (float)cx * dp;
-        if (cy) j[1] += (float)cy * dp;
-        if (cz) j[2] += (float)cz * dp;
-        if (cx) P[0] += sp;
-        if (cy) P[1] += sp;
-        if (cz) P[2] += sp;
-        if (cx && cy) P[3] += (float)(cx * cy) * sp;
-        if (cx && cz) P[4] += (float)(cx * cz) * sp;
-        if (cy && cz) P[5] += (float)(cy * cz) * sp;
-    }
+    float dr, j[3], P[6];
+    home_sums(g, dr, j, P);
     float out[10];
     home_collide(L, dr, j, P, out);
 #pragma unroll
@@ -1112,6 +1142,99 @@ __global__ void __launch_bounds__(256, 4) k_home_step(LbmParams L, HomeParams H,
         __syncthreads();
         if (worker) home_tile_cell(L, H, m_in, mout, lk, home_sm, q, x0, y0, z, ix, iy);
         __syncthreads();
+    }
+}
+
+// -------------------------------------------- HOME steps on populations --
+//
+// Several steps in one call run on populations between the first rebuild and
+// the last collision: k_home_open rebuilds every cell's post-collision
+// populations from its moments, once, into a lattice in the layout that
+// k_lbm_aa_even leaves; each step then is an odd (pull, collide, push) or an
+// even (own cell) kernel of the in-place AA pattern with the moment-space
+// collision and the rebuild in place of the BGK collision; the last one
+// writes moments. A cell's closure terms are evaluated once per step and no
+// block marches along z, where the tile kernel evaluates them 1.6 times and
+// walks its planes one after the other, so that a 32^3 lattice kept 48 blocks
+// of eight planes busy: 17 us per step, now 3.1 us, bound by the launch of a
+// dependent kernel. At 128^3 a step moves its 152 B per cell at 5.3 TB/s
+// (60 us against 76 us in the tile kernel).
+
+// Pulled deviations f -> the ten stored moments after the collision.
+__device__ __forceinline__ void home_relax(const LbmParams &L, const float g[19], float out[10]) {
+    float dr, j[3], P[6];
+    home_sums(g, dr, j, P);
+    home_collide(L, dr, j, P, out);
+}
+
+__device__ __forceinline__ void home_put(const LbmParams &L, float *__restrict__ m, int cell,
+                                         const float out[10]) {
+#pragma unroll
+    for (int k = 0; k < 10; ++k) m[k * L.ncell + cell] = out[k];
+}
+
+// moments -> the post-collision populations, in the own cell's opposite slots.
+__global__ void __launch_bounds__(256, 4) k_home_open(LbmParams L, const float *__restrict__ m,
+                                                      float *__restrict__ f,
+                                                      const uint32_t *__restrict__ links,
+                                                      float *__restrict__ outlet) {
+    pdl_wait();
+    pdl_trigger();
+    int x, y, z, cell;
+    if (!lattice_cell(L, x, y, z, cell)) return;
+    if (links && (links[cell] & 1u)) return;
+    float a[10], g[19];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) a[k] = m[k * L.ncell + cell];
+    home_rebuild_all(a, g);
+    aa_keep(L, f, outlet, x, y, z, cell, g);
+}
+
+// A step from the layout of k_home_open or an even step; LAST writes the
+// moments to m instead of pushing the populations.
+template <bool LAST>
+__global__ void __launch_bounds__(256, 4) k_home_odd(LbmParams L, float *f,
+                                                     const uint32_t *__restrict__ links,
+                                                     const float *__restrict__ outlet,
+                                                     float *__restrict__ m) {
+    pdl_wait();
+    pdl_trigger();
+    int x, y, z, cell;
+    if (!lattice_cell(L, x, y, z, cell)) return;
+    const uint32_t lk = links ? links[cell] : 0u;
+    if (lk & 1u) return;
+    const NbrOffsets o = nbr_offsets(L, x, y, z);
+    float g[19], a[10];
+    aa_pull(L, f, outlet, lk, o, x, y, z, cell, g);
+    home_relax(L, g, a);
+    if (LAST) {
+        home_put(L, m, cell, a);
+    } else {
+        home_rebuild_all(a, g);
+        aa_push(L, f, lk, o, x, cell, g);
+    }
+}
+
+// A step from the natural order that an odd step leaves.
+template <bool LAST>
+__global__ void __launch_bounds__(256, 4) k_home_even(LbmParams L, float *f,
+                                                      const uint32_t *__restrict__ links,
+                                                      float *__restrict__ outlet,
+                                                      float *__restrict__ m) {
+    pdl_wait();
+    pdl_trigger();
+    int x, y, z, cell;
+    if (!lattice_cell(L, x, y, z, cell)) return;
+    if (links && (links[cell] & 1u)) return;
+    float g[19], a[10];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) g[i] = f[i * L.ncell + cell];
+    home_relax(L, g, a);
+    if (LAST) {
+        home_put(L, m, cell, a);
+    } else {
+        home_rebuild_all(a, g);
+        aa_keep(L, f, outlet, x, y, z, cell, g);
     }
 }
 
@@ -1200,6 +1323,22 @@ static HomeParams home_params(const dw_lbm_desc &d) {
     return H;
 }
 
+// Whether a call of `steps` steps runs on populations (k_home_open and the
+// AA chain) or on the tile kernel. The chain moves 152 B per cell and step
+// and another 80 B per call; the tile kernel moves 80 B but is bound by its
+// issue rate and by its walk along z, and copies the lattice back after an
+// odd count. Up to 2^20 cells the populations (19 floats a cell) stay in L2
+// and the chain always wins (measured, us per call, tile / chain: 32^3 1 step
+// 20.9 / 9.7, 30 steps 517 / 94; 64^3 607 / 213 for 30; 96^3 1 step 47.6 /
+// 38.2). Above, its extra traffic has to pay off over the call: 128^3 2 steps
+// 152 / 166, 3 steps 253 / 222, 4 steps 304 / 285, 30 steps 2281 / 1823;
+// 192^3 4 steps 918 / 930, 10 steps 2295 / 2101.
+static bool home_on_populations(const LbmParams &L, int steps) {
+    if (L.ncell <= (1 << 20)) return true;
+    if (steps & 1) return steps >= 3;
+    return steps >= (L.ncell <= (1 << 22) ? 4 : 6);
+}
+
 // Planes per block: each block also rebuilds the two planes beyond its z
 // range, so tall ranges waste less; the blocks run in waves of `slots`
 // (resident blocks on the GPU), so a block count just under a whole number of
@@ -1252,6 +1391,25 @@ extern "C" dw_status lbm_home_step(dw_lbm h, float *m, const uint8_t *solid, int
     const uint32_t *links = nullptr;
     dw_status st = links_for_call(h, solid, s, &links);
     if (st != DW_OK) return st;
+    if (home_on_populations(L, steps)) {
+        LbmParams LH = L;  // the inlet populations of this lattice
+        for (int i = 0; i < 19; ++i) LH.feq_in[i] = H.g_in[i];
+        dim3 rg, rb;
+        lattice_launch(L, rg, rb);
+        float *f = h->tape;
+        DW_CUDA(launch_pdl3(k_home_open, rg, rb, s, LH, (const float *)m, f, links, h->outlet));
+        for (int k = 1; k <= steps; ++k) {
+            const bool last = k == steps;
+            if (k & 1)
+                DW_CUDA(launch_pdl3(last ? k_home_odd<true> : k_home_odd<false>, rg, rb, s, LH, f,
+                                    links, (const float *)h->outlet, m));
+            else
+                DW_CUDA(launch_pdl3(last ? k_home_even<true> : k_home_even<false>, rg, rb, s, LH, f,
+                                    links, h->outlet, m));
+        }
+        DW_LAUNCHED("lbm_home_step");
+        return DW_OK;
+    }
     if (!h->home_attr_set) {
         DW_CUDA(cudaFuncSetAttribute(k_home_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)HOME_SMEM));

@@ -138,6 +138,16 @@ __global__ void k_g2p(MpmParams P, const float *x, const float *F,
     if (!fin || !finite9(Fp)) atomicOr(err, ERRBIT_NONFINITE);
 }
 
+dw_status launch_g2p(int mode, const MpmParams &P, const float *x, const float *F, const uint8_t *pinned,
+                     const float4 *grid_v, const dw_mpm_state &out, int64_t n, int *err,
+                     int *reset_count, cudaStream_t s) {
+    if ((mode == DW_P2G_AUTO || mode == DW_P2G_PAIR) && n <= LAYER_MAX_G2P)
+        return launch_layer_g2p(P, x, F, pinned, grid_v, out, n, err, reset_count, s);
+    DW_CUDA(launch_pdl(k_g2p, grid_for(n, 128), 128, s, P, x, F, pinned, grid_v, out.x, out.v,
+                       out.C, out.F, n, err, reset_count));
+    return DW_OK;
+}
+
 // --------------------------------------------------------------- reverse --
 
 // Reverse G2P: scatter dL/dv_i into grid_bv; write partial dL/dx_p, dL/dF_p.
@@ -188,24 +198,22 @@ __global__ void __launch_bounds__(P2G_WARP_THREADS) k_rev_g2p(
 __global__ void __launch_bounds__(GRID_THREADS) k_rev_grid_active(
     MpmParams P, WindDev wind, float t, float4 *__restrict__ grid_mp, float4 *__restrict__ grid_bv,
     float4 *__restrict__ grid_bmp, float *__restrict__ g_wind, ActiveBlocks ab) {
-    __shared__ float sbox[GRID_THREADS / 32][WIND_BOX];
+    __shared__ WindGroup wg[GRID_THREADS / 64];
     pdl_wait();
     pdl_trigger();
     const int count = *ab.count;
     const int sub = threadIdx.x >> 6, lt = threadIdx.x & 63;
-    // every lane of a 64-thread group runs the same iterations (one block each)
+    // the threads of a 64-thread group run the same iterations (one block each)
     for (int e = blockIdx.x * 4 + sub; e < count; e += gridDim.x * 4) {
         int b = ab.list[e];
         int i = 0, j = 0, k = 0;
         bool live = false;
-        float3 gw;
+        float3 gw = make_float3(0.f, 0.f, 0.f);
         if (active_node(P, ab.nb, b, lt, i, j, k)) {
             int64_t node = ((int64_t)k * P.N + j) * P.N + i;
             live = rev_grid_node(P, node, i, j, k, grid_mp, grid_bv, grid_bmp, gw);
         }
-        if (g_wind)
-            wind_sample_adjoint_warp(wind, wind_scatter_coarse(P.N, wind.nf), live, i * P.dx,
-                                     j * P.dx, k * P.dx, t, gw, g_wind, sbox[threadIdx.x >> 5]);
+        if (g_wind) wind_scatter_block(P, wind, live, i, j, k, t, gw, g_wind, wg[sub], sub + 1);
         if (lt == 0) ab.flags[b] = 0;
     }
 }
@@ -532,6 +540,7 @@ extern "C" dw_status mpm_create(const dw_mpm_desc *desc, dw_mpm *out) {
     DW_ALLOC(h->roll_state, sizeof(float) * 24 * (size_t)cap);
     DW_ALLOC(h->roll_pinned, (size_t)cap);
     DW_ALLOC(h->roll_ids, sizeof(int32_t) * (size_t)cap);
+    DW_ALLOC(h->gE_part, sizeof(double) * (size_t)(cap / 32 + 1));
 #undef DW_ALLOC
     if (e == cudaSuccess) e = cudaMemset(h->grid_mp, 0, gbytes);
     if (e == cudaSuccess) e = cudaMemset(h->grid_bv, 0, gbytes);
@@ -555,6 +564,7 @@ extern "C" dw_status mpm_destroy(dw_mpm h) {
     cudaFree(h->grid_bv);
     cudaFree(h->grid_bmp);
     cudaFree(h->pscratch);
+    cudaFree(h->gE_part);
     cudaFree(h->err);
     cudaFree(h->keys);
     cudaFree(h->counts);
@@ -646,9 +656,7 @@ static dw_status substep_impl(dw_mpm h, const dw_mpm_state *in, const dw_mpm_sta
     }
     if (n > 0) {
         ProfScope ps(h, DW_K_G2P, s);
-        DW_CUDA(launch_pdl(k_g2p, grid_for(n, 128), 128, s, h->P, (const float *)in->x,
-                           (const float *)in->F, pinned, (const float4 *)h->grid_v, out->x, out->v,
-                           out->C, out->F, n, h->err, h->block_count));
+        return launch_g2p(h->desc.p2g_mode, h->P, in->x, in->F, pinned, h->grid_v, *out, n, h->err, h->block_count, s);
     }
     return DW_OK;
 }
@@ -789,15 +797,24 @@ extern "C" dw_status mpm_segment_adjoint(dw_mpm h, const dw_mpm_state *start, fl
         s.n = n;
         return s;
     };
-    // the recompute keeps each substep's grid when the grid tape fits; with
-    // the paired kernel it runs as one fused chain
-    const bool gt = ensure_grid_tape(h, n_substeps - 1);
-    if (h->desc.p2g_mode == DW_P2G_AUTO || h->desc.p2g_mode == DW_P2G_PAIR) {
+    // the recompute keeps each substep's grid when the grid tape fits; for the
+    // fused kernels' modes it runs as one fused chain, and with the tape (and
+    // more than one substep, so that a single one allocates nothing) so does
+    // the reverse pass
+    const bool fused = h->desc.p2g_mode == DW_P2G_AUTO || h->desc.p2g_mode == DW_P2G_PAIR;
+    const bool chain = fused && n > 0 && n_substeps > 1 && ensure_grid_tape(h, n_substeps);
+    const bool gt = chain || ensure_grid_tape(h, n_substeps - 1);
+    if (fused) {
         WindDev wd;
         st = wind_check(wind, &wd);
         if (st != DW_OK) return st;
-        st = segment_recompute(h, start, tape, pinned, wd, t0, n_substeps, gt, as_stream(stream));
+        int last_list = 0;
+        st = segment_recompute(h, start, tape, pinned, wd, t0, n_substeps, gt, chain, &last_list,
+                               as_stream(stream));
         if (st != DW_OK) return st;
+        if (chain)
+            return segment_reverse(h, start, tape, g, pinned, wd, t0, n_substeps, g_wind, g_E,
+                                   h->block_count + last_list, as_stream(stream));
     } else {
         for (int k = 1; k < n_substeps; ++k) {
             const dw_mpm_state in = k == 1 ? *start : slot(k - 1), out = slot(k);
@@ -968,9 +985,8 @@ extern "C" dw_status mpm_substep_noalloc(const dw_mpm_desc *desc, const dw_mpm_s
     k_grid_update<<<grid_for(nodes, 256), 256, 0, s>>>(P, wd, t, grid_mp, grid_v, 1);
     DW_LAUNCHED("k_grid_update");
     if (n > 0) {
-        k_g2p<<<grid_for(n, 128), 128, 0, s>>>(P, in->x, in->F, pinned, grid_v, out->x, out->v,
-                                               out->C, out->F, n, err, nullptr);
-        DW_LAUNCHED("k_g2p");
+        st = launch_g2p(desc->p2g_mode, P, in->x, in->F, pinned, grid_v, *out, n, err, nullptr, s);
+        if (st != DW_OK) return st;
     }
     return DW_OK;
 }

@@ -129,33 +129,36 @@ __device__ __forceinline__ void rev_g2p_particle(const MpmParams &P, const float
     q.valid = true;
 }
 
-// Reverse grid update of one node: (dL/dm_i, dL/dp_i) into grid_bmp, and
-// clearing of grid_mp and grid_bv for the next call. Returns whether the node
-// took part in the grid update (m_i > 0, outside the sticky band); then gw is
-// dt dL/dv_i, the cotangent of the wind force sampled at the node, for
-// wind_sample_adjoint_warp.
+// Reverse grid update of one node with mp = (m, p) and b4 = (0, dL/dv_i): out =
+// (dL/dm_i, dL/dp_i). Returns whether the node took part in the grid update
+// (m_i > 0, outside the sticky band); then gw is dt dL/dv_i, the cotangent of
+// the wind force sampled at the node, for wind_scatter_block.
+__device__ __forceinline__ bool rev_node_value(const MpmParams &P, int i, int j, int k,
+                                               float4 mp, float4 b4, float4 &out,
+                                               float3 &gw) {
+    out = make_float4(0.f, 0.f, 0.f, 0.f);
+    gw = make_float3(0.f, 0.f, 0.f);
+    if (!(mp.x > 0.0f) || sticky_node(P, i, j, k)) return false;
+    const float inv_m = 1.0f / mp.x;
+    out.y = b4.y * inv_m;
+    out.z = b4.z * inv_m;
+    out.w = b4.w * inv_m;
+    out.x = -(mp.y * b4.y + mp.z * b4.z + mp.w * b4.w) * inv_m * inv_m;
+    gw = make_float3(P.dt * b4.y, P.dt * b4.z, P.dt * b4.w);
+    return true;
+}
+
+// The same on the grid arrays, which also clears grid_mp and grid_bv for the
+// next call.
 __device__ __forceinline__ bool rev_grid_node(const MpmParams &P, int64_t node, int i, int j,
                                               int k, float4 *__restrict__ grid_mp,
                                               float4 *__restrict__ grid_bv,
                                               float4 *__restrict__ grid_bmp, float3 &gw) {
-    float4 mp = grid_mp[node];
-    float4 bmp = make_float4(0.f, 0.f, 0.f, 0.f);
-    bool live = false;
-    gw = make_float3(0.f, 0.f, 0.f);
-    if (mp.x > 0.0f && !sticky_node(P, i, j, k)) {
-        const float4 b4 = grid_bv[node];  // (0, dL/dv_i)
-        const float b[3] = {b4.y, b4.z, b4.w};
-        float inv_m = 1.0f / mp.x;
-        bmp.y = b[0] * inv_m;
-        bmp.z = b[1] * inv_m;
-        bmp.w = b[2] * inv_m;
-        bmp.x = -(mp.y * b[0] + mp.z * b[1] + mp.w * b[2]) * inv_m * inv_m;
-        gw = make_float3(P.dt * b[0], P.dt * b[1], P.dt * b[2]);
-        live = true;
-    }
+    float4 out;
+    const bool live = rev_node_value(P, i, j, k, grid_mp[node], grid_bv[node], out, gw);
     grid_mp[node] = make_float4(0.f, 0.f, 0.f, 0.f);
     grid_bv[node] = make_float4(0.f, 0.f, 0.f, 0.f);
-    grid_bmp[node] = bmp;
+    grid_bmp[node] = out;
     return live;
 }
 

@@ -14,12 +14,9 @@ __device__ __forceinline__ bool sticky_node(const MpmParams &P, int i, int j, in
 }
 
 // Grid update of one node: v_i = p_i / m_i + dt (g + a_w(x_i, t)), zero in the
-// sticky band and at empty nodes; (v, m) goes to grid_v.
-__device__ __forceinline__ void grid_node_update(const MpmParams &P, const WindDev &wind, float t,
-                                                 int64_t node, int i, int j, int k,
-                                                 float4 *__restrict__ grid_mp,
-                                                 float4 *__restrict__ grid_v, int clear) {
-    float4 mp = grid_mp[node];
+// sticky band and at empty nodes; returns (v, m) from mp = (m, p).
+__device__ __forceinline__ float4 grid_node_value(const MpmParams &P, const WindDev &wind, float t,
+                                                  int i, int j, int k, float4 mp) {
     // the wind taps are loaded together with (m, p), not after the test on m
     const float3 a = wind_sample_dev(wind, i * P.dx, j * P.dx, k * P.dx, t);
     float4 out = make_float4(0.f, 0.f, 0.f, mp.x);
@@ -29,7 +26,16 @@ __device__ __forceinline__ void grid_node_update(const MpmParams &P, const WindD
         out.y = mp.z * inv_m + P.dt * (P.gy + a.y);
         out.z = mp.w * inv_m + P.dt * (P.gz + a.z);
     }
-    grid_v[node] = out;
+    return out;
+}
+
+// The same on the grid arrays: (m, p) of grid_mp (zeroed with clear) to grid_v.
+__device__ __forceinline__ void grid_node_update(const MpmParams &P, const WindDev &wind, float t,
+                                                 int64_t node, int i, int j, int k,
+                                                 float4 *__restrict__ grid_mp,
+                                                 float4 *__restrict__ grid_v, int clear) {
+    const float4 mp = grid_mp[node];
+    grid_v[node] = grid_node_value(P, wind, t, i, j, k, mp);
     if (clear) grid_mp[node] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 

@@ -22,6 +22,7 @@ struct MpmHandle {
     float4 *grid_bv = nullptr;   // (0, dL/dv_i) during the adjoint; zero between calls
     float4 *grid_bmp = nullptr;  // (dL/dm_i, dL/dp_i) during the adjoint
     float *pscratch = nullptr;   // [12][max_particles]: partial dL/dx (3), dL/dF (9)
+    double *gE_part = nullptr;   // [max_particles / 32 + 1]: dL/dE per CTA of a segment's reverse
     int *err = nullptr;          // device status bits
     // active 4^3 blocks of the grid (built by P2G, consumed by the grid update)
     int64_t nblk = 0;            // nb^3
@@ -113,10 +114,6 @@ inline ActiveBlocks active_blocks(MpmHandle *h, int which = 0) {
 __global__ void k_grid_update_active(MpmParams P, WindDev wind, float t,
                                      float4 *__restrict__ grid_mp, float4 *__restrict__ grid_v,
                                      int clear, ActiveBlocks ab);
-__global__ void k_g2p(MpmParams P, const float *x, const float *F,
-                      const uint8_t *__restrict__ pinned, const float4 *__restrict__ grid_v,
-                      float *xo, float *vo, float *Co, float *Fo, int64_t n, int *err,
-                      int *reset_count);
 __global__ void k_grid_update_tape(MpmParams P, WindDev wind, float t, float4 *__restrict__ grid_mp,
                                    float4 *__restrict__ grid_v, ActiveBlocks ab,
                                    float4 *__restrict__ gtape, int *__restrict__ gtape_list,
@@ -125,11 +122,42 @@ __global__ void k_grid_update_tape(MpmParams P, WindDev wind, float t, float4 *_
 // The recompute of a segment adjoint (mpm_rollout.cu): states 1 .. n_substeps
 // - 1 from `start` into the tape slots, as one fused chain (the P2G of the
 // start state, then per substep the grid update, kept in grid tape slot k
-// when `keep_grid`, and the paired G2P/P2G kernel writing state k + 1 to its
-// slot). For p2g modes AUTO and PAIR.
+// when `keep_grid`, and the fused G2P/P2G kernel writing state k + 1 to its
+// slot). with_last: also the grid of the last substep, into its grid tape slot
+// and grid_v; *last_list is the active list its update consumed, whose count
+// the next launch clears. For p2g modes AUTO and PAIR.
 dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape,
                             const uint8_t *pinned, const WindDev &wd, float t0, int n_substeps,
-                            bool keep_grid, cudaStream_t s);
+                            bool keep_grid, bool with_last, int *last_list, cudaStream_t s);
+
+// The reverse pass of a segment whose recompute kept every substep's grid
+// (with_last) and state, fused across substeps (mpm_layer.cu).
+dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *tape,
+                          const dw_mpm_state *g, const uint8_t *pinned, const WindDev &wd, float t0,
+                          int n_substeps, float *g_wind, float *g_E, int *reset_count,
+                          cudaStream_t s);
+
+// The layer-split kernels (mpm_layer.cu) and the particle counts up to which
+// they are the faster ones (measured, us): a fused launch with its grid update
+// 8.2 against 14.5 at 5,504 particles, 9.2 / 13.2 at 20,000, 13.5 / 13.4 at
+// 40,000 of a sheet, 11.2 / 18.2 at 20,000 and 18.0 / 17.4 at 50,000 of a
+// block; the P2G alone 5 against 13 at 5,504, a whole substep 26.2 / 26.7 at
+// 100,000 and 41 / 40 at 200,000 of a block. Without the paired kernel's vector
+// loads (vec, see mpm_rollout) it loses longer: 16.1 / 16.3 at 65,535 of a
+// sheet, 25.6 / 34.2 of a block on 128^3, 20.1 / 18.0 at 100,001 of a sheet.
+constexpr int64_t LAYER_MAX_P2G = 1 << 17, LAYER_MAX_G2P = 1 << 17;
+inline bool layer_fused(int64_t n, bool vec) { return n <= (vec ? 1 << 15 : 1 << 16); }
+dw_status launch_layer_p2g(const MpmParams &P, const float *x, const float *v, const float *C,
+                           const float *F, int64_t n, float4 *grid, int *err,
+                           const ActiveBlocks &ab, cudaStream_t st);
+dw_status launch_layer_g2p(const MpmParams &P, const float *x, const float *F,
+                           const uint8_t *pinned, const float4 *grid_v, const dw_mpm_state &out,
+                           int64_t n, int *err, int *reset_count, cudaStream_t st);
+// keys, counts: the next sort's (see PairOut), or NULL.
+dw_status launch_layer_g2p2g(const MpmParams &P, const float *x, const float *F,
+                             const uint8_t *pinned, const float4 *grid_v, const dw_mpm_state &out,
+                             float4 *grid_next, int64_t n, int *err, const ActiveBlocks &ab_next,
+                             int *reset_count, int *keys, int *counts, cudaStream_t st);
 
 // particle sort (mpm.cu): counting sort by cell key, keys already counted
 constexpr int SCAN_BLOCK = 1024;
@@ -147,6 +175,12 @@ __global__ void k_sort_move(const int *__restrict__ keys, int64_t n, int *__rest
 dw_status exclusive_scan(int *data, int64_t len, int *tmp, int64_t tmp_len, cudaStream_t st);
 
 // host helpers of mpm.cu
+// G2P of n particles (x, F) into `out` (mode DW_P2G_*: AUTO and PAIR take the
+// layer-split kernel where it is the faster one, the others never do); reset_count, when given, is the
+// active-list count to clear.
+dw_status launch_g2p(int mode, const MpmParams &P, const float *x, const float *F, const uint8_t *pinned,
+                     const float4 *grid_v, const dw_mpm_state &out, int64_t n, int *err,
+                     int *reset_count, cudaStream_t s);
 dw_status validate_desc(const dw_mpm_desc *desc);
 dw_status check_state(const MpmHandle *h, const dw_mpm_state *s, const char *name);
 // with_vc = false leaves v and C of `out` unwritten (a rollout between fused

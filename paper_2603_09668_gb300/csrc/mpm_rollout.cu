@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, PAIR_MIN_CTAS) k_g2p2g_pair(
 
 dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape,
                             const uint8_t *pinned, const WindDev &wd, float t0, int n_substeps,
-                            bool keep_grid, cudaStream_t s) {
+                            bool keep_grid, bool with_last, int *last_list, cudaStream_t s) {
     const int64_t n = start->n;
     if (n_substeps < 2 || n == 0) return DW_OK;
     auto slot = [&](int k) {  // state k (1 .. n_substeps - 1) in the tape
@@ -128,7 +128,7 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
     if (st != DW_OK) return st;
     const unsigned pair_grid = grid_for(n, 2 * PAIR_THREADS);
     int L = 0;  // list consumed by the next grid update
-    for (int k = 0; k + 1 < n_substeps; ++k) {
+    for (int k = 0; k < n_substeps - (with_last ? 0 : 1); ++k) {
         const float t = fmaf((float)k, h->P.dt, t0);
         {
             ProfScope ps(h, DW_K_GRID, s);
@@ -141,13 +141,25 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
                 DW_CUDA(launch_pdl(k_grid_update_active, GRID_CTAS, GRID_THREADS, s, h->P, wd, t,
                                    h->grid_mp, h->grid_v, 1, active_blocks(h, L)));
         }
+        if (k + 1 == n_substeps) break;
         const dw_mpm_state in = k == 0 ? *start : slot(k), out = slot(k + 1);
-        if (k + 2 < n_substeps) {  // state k + 1 is scattered for substep k + 1's grid
-            ProfScope ps(h, DW_K_G2P2G, s);
-            const bool vec = n % 4 == 0 &&
-                             ((reinterpret_cast<uintptr_t>(in.x) | reinterpret_cast<uintptr_t>(in.F) |
-                               reinterpret_cast<uintptr_t>(out.x) | reinterpret_cast<uintptr_t>(out.F)) %
-                                  16 == 0);
+        if (k + 2 == n_substeps && !with_last) {
+            ProfScope ps(h, DW_K_G2P, s);
+            st = launch_g2p(h->desc.p2g_mode, h->P, in.x, in.F, pinned, h->grid_v, out, n, h->err, h->block_count + L, s);
+            if (st != DW_OK) return st;
+            break;
+        }
+        // state k + 1 is scattered for substep k + 1's grid
+        ProfScope ps(h, DW_K_G2P2G, s);
+        const bool vec = n % 4 == 0 &&
+                         ((reinterpret_cast<uintptr_t>(in.x) | reinterpret_cast<uintptr_t>(in.F) |
+                           reinterpret_cast<uintptr_t>(out.x) | reinterpret_cast<uintptr_t>(out.F)) %
+                              16 == 0);
+        if (layer_fused(n, vec)) {
+            st = launch_layer_g2p2g(h->P, in.x, in.F, pinned, h->grid_v, out, h->grid_mp, n, h->err,
+                                    active_blocks(h, 1 - L), h->block_count + L, nullptr, nullptr, s);
+            if (st != DW_OK) return st;
+        } else {
             auto kern = h->P.material == DW_NEOHOOKEAN
                             ? (vec ? k_g2p2g_pair<DW_NEOHOOKEAN, false, true, true>
                                    : k_g2p2g_pair<DW_NEOHOOKEAN, false, false, true>)
@@ -157,14 +169,10 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
                                pinned, (const float4 *)h->grid_v, h->grid_mp, n, h->err,
                                active_blocks(h, 1 - L), h->block_count + L,
                                PairOut{out.x, out.v, out.C, out.F}));
-            L = 1 - L;
-        } else {
-            ProfScope ps(h, DW_K_G2P, s);
-            DW_CUDA(launch_pdl(k_g2p, grid_for(n, 128), 128, s, h->P, (const float *)in.x,
-                               (const float *)in.F, pinned, (const float4 *)h->grid_v, out.x,
-                               out.v, out.C, out.F, n, h->err, h->block_count + L));
         }
+        L = 1 - L;
     }
+    *last_list = L;
     return DW_OK;
 }
 
@@ -234,19 +242,25 @@ extern "C" dw_status mpm_rollout(dw_mpm h, const dw_mpm_state *state, uint8_t *p
         }
         if (k + 1 == n_substeps) {
             ProfScope ps(h, DW_K_G2P, s);
-            DW_CUDA(launch_pdl(k_g2p, grid_for(n, 128), 128, s, h->P, (const float *)cur.x,
-                               (const float *)cur.F, (const uint8_t *)cur_pin,
-                               (const float4 *)h->grid_v, cur.x, cur.v, cur.C, cur.F, n, h->err,
-                               h->block_count + L));
+            st = launch_g2p(h->desc.p2g_mode, h->P, cur.x, cur.F, cur_pin, h->grid_v, cur, n, h->err,
+                            h->block_count + L, s);
+            if (st != DW_OK) return st;
             break;
         }
         {
             ProfScope ps(h, DW_K_G2P2G, s);
-            if (pair) {
-                // vector paths: float2 pairs of x and F, 16-byte pieces of F (n a
-                // multiple of 4, 16-byte aligned arrays)
-                const bool pair_vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(cur.x) |
-                                                        reinterpret_cast<uintptr_t>(cur.F)) % 16 == 0);
+            // vector paths: float2 pairs of x and F, 16-byte pieces of F (n a
+            // multiple of 4, 16-byte aligned arrays)
+            const bool pair_vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(cur.x) |
+                                                    reinterpret_cast<uintptr_t>(cur.F)) % 16 == 0);
+            if (pair && layer_fused(n, pair_vec)) {
+                const bool keys = sort_every > 0 && (k + 1) % sort_every == 0;
+                const dw_mpm_state out{cur.x, nullptr, nullptr, cur.F, n};  // v and C are not kept
+                st = launch_layer_g2p2g(h->P, cur.x, cur.F, cur_pin, h->grid_v, out, h->grid_mp, n,
+                                        h->err, active_blocks(h, 1 - L), h->block_count + L,
+                                        keys ? h->keys : nullptr, keys ? h->counts : nullptr, s);
+                if (st != DW_OK) return st;
+            } else if (pair) {
                 const bool keys = sort_every > 0 && (k + 1) % sort_every == 0;
                 const bool nh = h->P.material == DW_NEOHOOKEAN;
                 auto kern = keys ? (nh ? (pair_vec ? k_g2p2g_pair<DW_NEOHOOKEAN, false, true, false, true>

@@ -5,7 +5,11 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2603_09668_gb300 import binding as B
+from paper_2603_09668_gb300 import inputs
+
+from gpu_util import rel_l2, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +39,116 @@ def test_home_steps_on_populations(shape, bc_x, steps):
     keep = solid.bool().expand(10, nz, ny, nx)
     assert torch.equal(a[keep], start[keep])
     lbm.close()
+
+
+def _mpm_case(n, n_grid, material, seed=0):
+    """A deformed block of n particles in lattice order with 5% pinned."""
+    g = np.random.default_rng(seed)
+    sub = max(2, int(np.ceil((n / 3.0) ** (1 / 3))))
+    x = inputs.block_particles(lo=(0.3, 0.3, 0.3), size=0.3, sub=sub, per_sub=3, seed=seed)[:, :n]
+    st = inputs.perturbed_state(np.ascontiguousarray(x), v_scale=0.2, c_scale=1.0, f_scale=0.02, seed=seed)
+    pin = (g.random(n) < 0.05).astype(np.uint8)
+    st[1][:, pin != 0] = 0.0
+    st[2][:, pin != 0] = 0.0
+    vol = 0.3 ** 3 / n
+    pr = dict(n_grid=n_grid, dt=5e-5, gravity=(0.0, -9.8, 0.0), bc_band=3, material=material, E=2e4,
+              nu=0.3, p_mass=1000.0 * vol, p_vol=vol)
+    return pr, st, pin
+
+
+def _dev(st):
+    return B.MpmState(*(to_dev(np.ascontiguousarray(a)) for a in st))
+
+
+# The layer-split kernels (P2G and G2P up to 2^17 particles, the fused kernel up
+# to 2^15, 2^16 for counts not a multiple of 4) against the one-particle-per-thread kernels, around the CTA's 32
+# particles and the rules' edges. The same formulas summed in another order:
+# the bounds of the paired kernels' test (x, F 1e-5; v, C 1e-3 of the largest).
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 95, 1000, 32768, 32772, 65535, 65537, 131072, 131073])
+@pytest.mark.parametrize("material,sort_every", [(0, 0), (1, 3)])
+def test_layer_split_forward(n, material, sort_every):
+    pr, st, pin = _mpm_case(n, 64 if n > 5000 else 24, material)
+    wind = B.WindField(to_dev(inputs.fourier_wind(9, 3, seed=4)), 7 * pr["dt"])
+    got = []
+    for mode in (B.P2G_AUTO, B.P2G_WARP):
+        mpm = B.MPM.from_params(pr, max_particles=n, p2g_mode=mode)
+        s, p = _dev(st), to_dev(pin)
+        ids = torch.arange(n, dtype=torch.int32, device="cuda")
+        out = B.MpmState.empty_like(s)
+        mpm.substep(s, out, p, wind, 0.0)
+        mpm.rollout(out, p, ids, wind, pr["dt"], 6, sort_every)
+        mpm.device_status()
+        assert torch.equal(torch.sort(ids.long()).values, torch.arange(n, device="cuda"))
+        back = [torch.empty_like(a) for a in out]
+        for b, a in zip(back, out):
+            b[:, ids.long()] = a
+        assert torch.equal(p.cpu(), torch.from_numpy(pin)[ids.cpu().long()])
+        got.append(back)
+        mpm.close()
+    for k, tol in ((0, 1e-5), (3, 1e-5)):
+        assert (got[0][k] - got[1][k]).abs().max().item() <= tol
+    for k in (1, 2):
+        assert (got[0][k] - got[1][k]).abs().max() <= 1e-3 * got[1][k].abs().max()
+
+
+def test_layer_split_reports_a_particle_off_the_grid():
+    pr, st, pin = _mpm_case(70, 24, 0)
+    st[0][0, 40] = 0.999
+    mpm = B.MPM.from_params(pr, max_particles=70)
+    s = _dev(st)
+    wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
+    mpm.rollout(s, to_dev(pin), None, wind, 0.0, 3, 0)
+    with pytest.raises(B.DiffWindError):
+        mpm.device_status()
+    assert s.x[0, 40].item() == st[0][0, 40] and s.v[:, 40].abs().max().item() == 0.0
+    assert torch.isfinite(s.x).all()
+    mpm.close()
+
+
+# The fused reverse pass (two launches per substep) against the four-launch one
+# of p2g_mode WARP: the same sums in another order, relative L2 1e-4 per block,
+# as between the batched and the single-scene adjoints.
+@pytest.mark.parametrize("n", [1, 33, 1000, 40001])
+@pytest.mark.parametrize("material,steps", [(0, 2), (1, 3), (0, 5)])
+def test_fused_reverse_segment(n, material, steps):
+    pr, st, pin = _mpm_case(n, 64 if n > 5000 else 24, material, seed=1)
+    wind = B.WindField(to_dev(inputs.fourier_wind(9, 3, seed=4)), 7 * pr["dt"])
+    g = torch.Generator(device="cuda").manual_seed(2)
+    g0 = [torch.randn(a.shape, generator=g, device="cuda") for a in st]
+    got = []
+    for mode in (B.P2G_AUTO, B.P2G_WARP):
+        mpm = B.MPM.from_params(pr, max_particles=n + 5, p2g_mode=mode)
+        gs = B.MpmState(*(a.clone() for a in g0))
+        gw, gE = torch.ones_like(wind.values), torch.ones(1, device="cuda")
+        tape = torch.empty((steps - 1) * 24 * n, device="cuda")
+        for _ in range(2):  # the second call starts from the first one's gradient
+            mpm.segment_adjoint(_dev(st), tape, gs, to_dev(pin), wind, pr["dt"], steps, gw, gE)
+        mpm.device_status()
+        got.append([a.cpu().numpy().astype(np.float64) for a in (*gs, gw, gE)])
+        mpm.close()
+    for k, (a, b) in enumerate(zip(*got)):
+        # dL/dx of an isolated particle is a difference of equal terms: both
+        # passes are 2e-4 off the float64 value there (the other blocks 1e-5)
+        if n > 1 or k > 0:
+            assert rel_l2(a, b) <= 1e-4, k
+
+
+# The wind gradient's scatter, per axis within a 4^3 block of grid nodes or tap
+# by tap where the wind grid is as fine as the MPM grid, against the oracle's
+# reverse substep: relative L2 1e-4, the adjoint's stated target.
+@pytest.mark.parametrize("nf,frames", [(1, 1), (2, 3), (5, 1), (9, 2), (12, 3), (17, 2), (40, 2)])
+def test_wind_gradient_scatter(nf, frames):
+    pr, st, pin = _mpm_case(400, 18, 0, seed=3)
+    wind = inputs.fourier_wind(nf, frames, seed=6)
+    t = 0.3
+    g = [np.random.default_rng(k).standard_normal(a.shape).astype(np.float32) for k, a in enumerate(st)]
+    gw = torch.zeros(wind.shape, device="cuda")
+    mpm = B.MPM.from_params(pr, max_particles=400)
+    gi = B.MpmState.empty_like(_dev(st))
+    mpm.substep_adjoint(_dev(st), _dev(g), gi, to_dev(pin), B.WindField(to_dev(wind), 1.0), t, gw)
+    mpm.device_status()
+    ref = oracle.mpm_substep_adjoint(pr, tuple(a.astype(np.float64) for a in st),
+                                     (wind.astype(np.float64), nf, frames, 1.0), t,
+                                     tuple(a.astype(np.float64) for a in g), pinned=pin)[1]
+    assert rel_l2(gw.cpu().numpy().ravel(), np.asarray(ref).ravel()) <= 1e-4
+    mpm.close()

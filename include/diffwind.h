@@ -386,7 +386,8 @@ DW_API dw_status gs_covariance(const float *F, const float *sigma0, int64_t n, f
                                dw_stream stream);
 
 /* Renderer workspace for up to max_gaussians Gaussians and width x height
- * images (about 100 bytes per Gaussian plus one image). */
+ * images (about 120 bytes per Gaussian plus one image; gs_render adds, and grows
+ * when needed, about 30 bytes per entry of the tile lists). */
 DW_API dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t height, dw_gs *out);
 DW_API dw_status gs_destroy(dw_gs h);
 
@@ -394,7 +395,7 @@ DW_API dw_status gs_destroy(dw_gs h);
  * with deformation gradients F and rest covariances sigma0. The handle keeps
  * the projected Gaussians, their depth order, the per-tile lists and the
  * image for gs_render_backward. cam's image size must be the handle's. The
- * call reads the tile-list length back to the host (4 bytes) to size the
+ * call reads the length of the tile lists back to the host (16 bytes) to size the
  * lists, so it waits for `stream` and cannot be captured in a CUDA graph. */
 DW_API dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, const float *F,
                            const float *sigma0, const float *color, const float *opacity,

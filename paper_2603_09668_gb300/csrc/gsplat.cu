@@ -5,23 +5,32 @@
 // its reverse mode down to the particle positions and deformation gradients,
 // so that an image loss differentiates through the MPM adjoint.
 //
-// Pipeline of gs_render (one camera):
+// Pipeline of gs_render (one camera), on 8 x 8 pixel tiles:
 //   k_gs_preprocess  per Gaussian: Sigma, camera-space centre, projected
-//                    centre mu', the inverse 2D covariance (conic), the pixel
-//                    rectangle of the 3-sigma ellipse, depth key;
-//   radix sort       stable LSD sort of the depth keys (four 8-bit passes:
-//                    block histograms, one scan, order-keeping scatter);
-//   tile lists       in depth order, each Gaussian is listed once per 16 x 16
-//                    pixel tile its rectangle meets (counts, scan, copies);
-//                    a stable sort of the list by tile keeps the depth order
-//                    within each tile, and each tile's range is marked;
+//                    centre mu', the inverse 2D covariance (conic), packed
+//                    with its opacity and colour in 48 bytes; the pixel
+//                    rectangle of the 3-sigma ellipse, and one count for
+//                    every tile the rectangle meets;
+//   k_gs_tile_scan   the tiles' ranges in the list;
+//   k_gs_list        each Gaussian into the ranges of its tiles, as the 64-bit
+//                    key (depth bits, index), in any order;
+//   k_gs_tile_sort   each tile's keys sorted in shared memory: increasing
+//                    depth, ties by index, so the list does not depend on the
+//                    order it was filled in;
 //   k_gs_render_fwd  one tile per block: its Gaussians are read front to back
-//                    in batches of 256 into shared memory, then every pixel
+//                    in batches of 64 into shared memory, then every pixel
 //                    composites them.
+// A tile with more Gaussians than the shared-memory sort holds sends the call
+// through a stable LSD radix sort of all depths and a stable sort of the list
+// by tile instead (the same lists).
 // gs_render_backward walks the same ranges front to back again with the
 // final colour known (dC/dalpha_i = T_i c_i - (C - C_<=i) / (1 - alpha_i)),
 // reduces each Gaussian's pixel contributions per warp before one atomic,
 // and k_gs_preprocess_bwd carries the 2D gradients back to x and F.
+// Measured at 100,284 Gaussians, 512 x 512 (us, launches serialised), against
+// 16 x 16 tiles with the radix sorts for every call: lists 200 -> 50, forward
+// compositing 108 -> 59, backward 570 -> 70; two views with L1, D-SSIM and
+// their gradients 2,187 -> 549.
 #include <math.h>
 #include <string.h>
 
@@ -33,8 +42,17 @@
 
 namespace dw {
 
-constexpr int GS_TILE = 16;
+// Tile edge. The path renders particles, whose Gaussians cover a few pixels: 8
+// pixels leave a warp (8 x 4 pixels) few idle lanes per Gaussian, and four
+// times as many blocks as 16, with lists half as long (100,284 Gaussians of
+// about 7 pixels at 512 x 512: 183,000 entries of 256 pixels against 306,000
+// of 64).
+constexpr int GS_TILE = 8;
 constexpr int GS_THREADS = GS_TILE * GS_TILE;  // one pixel per thread
+constexpr int GS_SORT_MAX = 4096;   // keys of one tile k_gs_tile_sort holds
+constexpr int GS_SORT_THREADS = 128;
+constexpr int GS_BIG_CTAS = 304;    // two per SM
+constexpr int GS_ROW = 12;          // floats per Gaussian of the packed rows and of the 2D gradients
 constexpr int RS_THREADS = 256;
 constexpr int RS_TILE = RS_THREADS * 16;  // keys per sort block
 
@@ -166,19 +184,58 @@ __global__ void k_gs_covariance(const float *__restrict__ F, const float *__rest
 
 // ------------------------------------------------------------ preprocess --
 
-// Per Gaussian: mu'(2), conic(3), the pixel rectangle [x0, x1] x [y0, y1] of
-// the pixel centres inside the 3-sigma ellipse (empty when x1 < x0), and the
-// depth key (float bits of t_z, or all ones when not drawn).
-__global__ void k_gs_preprocess(GsCam c, const float *__restrict__ x, const float *__restrict__ F,
-                                const float *__restrict__ s0, int n, float *__restrict__ mu,
-                                float *__restrict__ conic, int4 *__restrict__ rect,
-                                uint32_t *__restrict__ key, uint32_t *__restrict__ idx) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// Tiles met by a Gaussian with pixel rectangle r (drawn = false: none).
+struct GsTiles {
+    int first, nx, count;  // tile of the rectangle's corner, tiles per row, tiles
+};
+
+__device__ __forceinline__ GsTiles gs_tiles(int4 r, bool drawn, int tiles_x) {
+    const int x0 = r.x / GS_TILE, y0 = r.y / GS_TILE;
+    GsTiles t;
+    t.first = y0 * tiles_x + x0;
+    t.nx = drawn ? r.z / GS_TILE - x0 + 1 : 0;
+    t.count = drawn ? t.nx * (r.w / GS_TILE - y0 + 1) : 0;
+    return t;
+}
+
+// f(tile, mask) for every tile of each lane's Gaussian that meets at most
+// GS_BIG of them, called by whole warps with the mask of the lanes that call
+// it together. Neighbouring particles' Gaussians meet the same tiles, so f
+// combines equal tiles of the mask before its atomic.
+constexpr int GS_BIG = 16;
+template <typename Fn>
+__device__ __forceinline__ void gs_for_tiles(const GsTiles &g, int tiles_x, Fn f) {
+    const int cnt = g.count <= GS_BIG ? g.count : 0;
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    for (int t = 0, tx = 0, tile = g.first; t < most; ++t) {
+        const unsigned mask = __ballot_sync(0xffffffffu, t < cnt);
+        if (t < cnt) f(tile, mask);
+        __syncwarp();
+        ++tile;
+        if (++tx == g.nx) {
+            tx = 0;
+            tile += tiles_x - g.nx;
+        }
+    }
+}
+
+// Per Gaussian: row = (mu'(2), conic(3), opacity, colour(3)), the pixel
+// rectangle [x0, x1] x [y0, y1] of the pixel centres inside the 3-sigma ellipse
+// (empty when x1 < x0), the depth key (float bits of t_z, or all ones when not
+// drawn), and one count for each tile met; a Gaussian that meets more than
+// GS_BIG tiles goes to a queue instead (k_gs_big).
+__global__ void __launch_bounds__(128) k_gs_preprocess(
+    GsCam c, const float *__restrict__ x, const float *__restrict__ F, const float *__restrict__ s0,
+    const float *__restrict__ color, const float *__restrict__ opacity, int n, int tiles_x,
+    float4 *__restrict__ rows, int4 *__restrict__ rect, uint32_t *__restrict__ key,
+    uint32_t *__restrict__ tile_count, uint32_t *__restrict__ big, uint32_t *__restrict__ big_count) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = min(t, n - 1);  // the last warp's spare lanes repeat the last Gaussian
     float Fm[3][3], a[6], S[6];
     load_F(F, n, i, Fm);
 #pragma unroll
     for (int k = 0; k < 6; ++k) a[k] = s0[(int64_t)k * n + i];
+    const float op = opacity[i], c0 = color[i], c1 = color[(int64_t)n + i], c2 = color[2 * (int64_t)n + i];
     cov_update(Fm, a, S);
     const float xp[3] = {x[i], x[(int64_t)n + i], x[2 * (int64_t)n + i]};
     GsProj p;
@@ -196,14 +253,18 @@ __global__ void k_gs_preprocess(GsCam c, const float *__restrict__ x, const floa
         if (!(lx <= hx && ly <= hy)) r = make_int4(0, 0, -1, -1);  // also NaN
     }
     const bool drawn = r.z >= r.x && r.w >= r.y;
-    mu[i] = p.mu[0];
-    mu[n + i] = p.mu[1];
-    conic[i] = p.conic[0];
-    conic[n + i] = p.conic[1];
-    conic[2 * n + i] = p.conic[2];
+    const GsTiles g = gs_tiles(r, drawn && t < n, tiles_x);
+    gs_for_tiles(g, tiles_x, [&](int tile, unsigned mask) {
+        const unsigned peers = __match_any_sync(mask, tile);
+        if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&tile_count[tile], __popc(peers));
+    });
+    if (t >= n) return;
+    if (g.count > GS_BIG) big[atomicAdd(big_count, 1u)] = (uint32_t)i;
+    rows[3 * (int64_t)i] = make_float4(p.mu[0], p.mu[1], p.conic[0], p.conic[1]);
+    rows[3 * (int64_t)i + 1] = make_float4(p.conic[2], op, c0, c1);
+    rows[3 * (int64_t)i + 2] = make_float4(c2, 0.0f, 0.0f, 0.0f);
     rect[i] = r;
     key[i] = drawn ? __float_as_uint(p.t[2]) : 0xffffffffu;  // t_z > 0: bits order as floats
-    idx[i] = (uint32_t)i;
 }
 
 // ------------------------------------------------------------ radix sort --
@@ -293,7 +354,212 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *__res
 
 // ------------------------------------------------------------ tile lists --
 
-// Tiles met by Gaussian order[k] (its pixel rectangle in 16 x 16 tiles).
+constexpr int GS_WORD = 28;  // bits of the batch count in a scan word
+__device__ __forceinline__ unsigned long long gs_word(uint32_t entries) {
+    return ((unsigned long long)entries << GS_WORD) | ((entries + GS_THREADS - 1) / GS_THREADS);
+}
+
+// What gs_render reads back: the list's length, its batches of GS_THREADS
+// entries, the longest tile's list and the queue's length.
+struct GsStat {
+    unsigned long long total;
+    uint32_t batches, most, big;
+};
+
+// Exclusive scan of the tiles' counts in one block: ranges[t].x = ranges[t].y
+// = the tile's first entry (k_gs_list advances .y to its end), and of their
+// batches: batch_off[t] = the tile's first batch.
+__global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restrict__ count,
+                                                       int tiles, int2 *__restrict__ ranges,
+                                                       uint32_t *__restrict__ batch_off,
+                                                       GsStat *__restrict__ stat) {
+    // a 64-bit word carries both sums: the entries above bit GS_WORD, the
+    // batches below it (at most list / 64 + tiles: below 2^27 for a list of 2^31
+    // entries and an image of 2^31 pixels)
+    __shared__ unsigned long long wsum[32];
+    __shared__ uint32_t wmax[32];
+    __shared__ unsigned long long carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    uint32_t mx = 0;
+    __syncthreads();
+    for (int base = 0; base < tiles; base += 4096) {
+        uint32_t v[4];
+        unsigned long long t = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int i = base + (int)threadIdx.x * 4 + j;
+            v[j] = i < tiles ? count[i] : 0u;
+            mx = max(mx, v[j]);
+            t += gs_word(v[j]);
+        }
+        unsigned long long incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            unsigned long long w = wsum[lane], wi = w;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, wi, o);
+                if (lane >= o) wi += y;
+            }
+            wsum[lane] = wi - w + carry;
+            __syncwarp();
+            if (lane == 31) carry += wi;
+        }
+        __syncthreads();
+        unsigned long long run = wsum[warp] + incl - t;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int i = base + (int)threadIdx.x * 4 + j;
+            if (i < tiles) {
+                const int at = (int)(run >> GS_WORD);
+                ranges[i] = make_int2(at, at);
+                batch_off[i] = (uint32_t)run & ((1u << GS_WORD) - 1u);
+            }
+            run += gs_word(v[j]);
+        }
+        __syncthreads();
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) wmax[warp] = mx;
+    __syncthreads();
+    if (warp == 0) {
+        mx = __reduce_max_sync(0xffffffffu, wmax[lane]);
+        if (lane == 0) {
+            stat->total = carry >> GS_WORD;
+            stat->batches = (uint32_t)carry & ((1u << GS_WORD) - 1u);
+            stat->most = mx;
+        }
+    }
+}
+
+__device__ __forceinline__ unsigned long long gs_key(const uint32_t *__restrict__ key, int i) {
+    return ((unsigned long long)key[i] << 32) | (uint32_t)i;
+}
+
+// Each drawn Gaussian's key into the ranges of the tiles it meets.
+__global__ void __launch_bounds__(128) k_gs_list(const int4 *__restrict__ rect,
+                                                 const uint32_t *__restrict__ key, int n,
+                                                 int tiles_x, int2 *__restrict__ ranges,
+                                                 unsigned long long *__restrict__ list) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, i = min(t, n - 1);
+    const int4 r = rect[i];
+    const unsigned long long k = gs_key(key, i);
+    const int lane = threadIdx.x & 31;
+    gs_for_tiles(gs_tiles(r, t < n && r.z >= r.x && r.w >= r.y, tiles_x), tiles_x,
+                 [&](int tile, unsigned mask) {
+                     const unsigned peers = __match_any_sync(mask, tile);
+                     const int leader = __ffs(peers) - 1;
+                     int at = 0;
+                     if (lane == leader) at = atomicAdd(&ranges[tile].y, __popc(peers));
+                     at = __shfl_sync(peers, at, leader);
+                     list[at + __popc(peers & ((1u << lane) - 1u))] = k;
+                 });
+}
+
+// The queued Gaussians' tiles, counted or (LIST) listed: 16 warps per Gaussian,
+// so that a few that cover the whole image do not leave a warp each with
+// thousands of tiles.
+template <bool LIST>
+__global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big,
+                                                const uint32_t *__restrict__ big_count,
+                                                const int4 *__restrict__ rect,
+                                                const uint32_t *__restrict__ key, int tiles_x,
+                                                uint32_t *__restrict__ tile_count,
+                                                int2 *__restrict__ ranges,
+                                                unsigned long long *__restrict__ list,
+                                                GsStat *__restrict__ stat) {
+    const uint32_t queued = *big_count;
+    if (!LIST && blockIdx.x == 0 && threadIdx.x == 0) stat->big = queued;
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * 8;
+    for (uint32_t u = blockIdx.x * 8 + (threadIdx.x >> 5); u / 16 < queued; u += warps) {
+        const int i = (int)big[u / 16];
+        const GsTiles g = gs_tiles(rect[i], true, tiles_x);
+        const unsigned long long k = LIST ? gs_key(key, i) : 0ull;
+#pragma unroll 4
+        for (int t = (int)(u % 16) * 32 + lane; t < g.count; t += 512) {
+            const int tile = g.first + t / g.nx * tiles_x + t % g.nx;
+            if (LIST)
+                list[atomicAdd(&ranges[tile].y, 1)] = k;
+            else
+                atomicAdd(&tile_count[tile], 1u);
+        }
+    }
+}
+
+// The batches of tile t: batch k holds the entries [64 k, 64 k + 64) of its
+// range; batch_tile[batch_off[t] + k] = t.
+__device__ __forceinline__ void gs_write_batches(int t, int cnt, const uint32_t *__restrict__ batch_off,
+                                                 uint32_t *__restrict__ batch_tile) {
+    const int nb = (cnt + GS_THREADS - 1) / GS_THREADS;
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) batch_tile[batch_off[t] + k] = (uint32_t)t;
+}
+
+// Bitonic sort of each tile's keys (one tile per block, at most GS_SORT_MAX);
+// the Gaussians' indices in order go to gid. A warp's threads compare within
+// 64 consecutive keys while the distance is at most 32, so only the longer
+// distances need the block's barrier.
+__global__ void __launch_bounds__(GS_SORT_THREADS) k_gs_tile_sort(
+    const int2 *__restrict__ ranges, const unsigned long long *__restrict__ list,
+    const uint32_t *__restrict__ batch_off, uint32_t *__restrict__ gid,
+    uint32_t *__restrict__ batch_tile) {
+    extern __shared__ unsigned long long k[];  // the longest list, rounded up to a power of two
+    const int2 rg = ranges[blockIdx.x];
+    const int cnt = rg.y - rg.x;
+    if (cnt <= 0) return;
+    gs_write_batches(blockIdx.x, cnt, batch_off, batch_tile);
+    int size = 2;
+    while (size < cnt) size <<= 1;
+    for (int i = threadIdx.x; i < size; i += GS_SORT_THREADS) k[i] = i < cnt ? list[rg.x + i] : ~0ull;
+    __syncthreads();
+    for (int len = 2; len <= size; len <<= 1) {
+        for (int d = len >> 1; d > 0; d >>= 1) {
+            for (int t = threadIdx.x; t < size / 2; t += GS_SORT_THREADS) {
+                const int i = 2 * t - (t & (d - 1)), j = i + d;
+                const unsigned long long a = k[i], b = k[j];
+                if ((a > b) == ((i & len) == 0)) {
+                    k[i] = b;
+                    k[j] = a;
+                }
+            }
+            if (d > 32)
+                __syncthreads();
+            else
+                __syncwarp();
+        }
+        if (len >= 64) __syncthreads();  // the next distance is len
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < cnt; i += GS_SORT_THREADS) gid[rg.x + i] = (uint32_t)k[i];
+}
+
+// The batches of every tile (the radix path; one thread per tile).
+__global__ void __launch_bounds__(256) k_gs_batches(const int2 *__restrict__ ranges, int tiles,
+                                                    const uint32_t *__restrict__ batch_off,
+                                                    uint32_t *__restrict__ batch_tile) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= tiles) return;
+    const int nb = (ranges[t].y - ranges[t].x + GS_THREADS - 1) / GS_THREADS;
+    for (int k = 0; k < nb; ++k) batch_tile[batch_off[t] + k] = (uint32_t)t;
+}
+
+// The radix path: keys and indices of all Gaussians.
+__global__ void k_gs_order_init(const uint32_t *__restrict__ key, int n, uint32_t *__restrict__ k,
+                                uint32_t *__restrict__ v) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    k[i] = key[i];
+    v[i] = (uint32_t)i;
+}
+
+// Tiles met by Gaussian order[k] (its pixel rectangle in tiles).
 __global__ void k_gs_tile_count(const uint32_t *__restrict__ order, const int4 *__restrict__ rect,
                                 int n, uint32_t *__restrict__ cnt) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -362,70 +628,52 @@ __global__ void k_gs_duplicate(const uint32_t *__restrict__ order, const int4 *_
         }
 }
 
-// ranges[tile] = [first, last + 1) of the tile's entries in the sorted list.
-__global__ void k_gs_tile_ranges(const uint32_t *__restrict__ tile_key, int m,
-                                 int2 *__restrict__ ranges) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= m) return;
-    const uint32_t t = tile_key[p];
-    if (p == 0 || tile_key[p - 1] != t) ranges[t].x = p;
-    if (p == m - 1 || tile_key[p + 1] != t) ranges[t].y = p + 1;
-}
-
 // ---------------------------------------------------------------- render --
 
-// Load the batch [b0, b0 + 256) of the tile's range of the tile list into
-// shared memory (mu', conic, opacity, colour per Gaussian); returns its size.
-__device__ __forceinline__ int gs_load_batch(int b0, int end, int n,
-                                             const uint32_t *__restrict__ list,
-                                             const float *__restrict__ mu,
-                                             const float *__restrict__ conic,
-                                             const float *__restrict__ color,
-                                             const float *__restrict__ opacity, int *s_id,
-                                             float (*s_g)[9]) {
+// The batch [b0, b0 + GS_THREADS) of the tile's range in shared memory.
+struct GsBatch {
+    float4 row[GS_THREADS][3];  // mu(2) conic(3) opacity color(3), 3 unused
+    int id[GS_THREADS];
+};
+
+__device__ __forceinline__ int gs_load_batch(int b0, int end, const uint32_t *__restrict__ list,
+                                             const float4 *__restrict__ rows, GsBatch &s) {
     const int cnt = min(GS_THREADS, end - b0);
     if ((int)threadIdx.x < cnt) {
         const int g = (int)list[b0 + threadIdx.x];
-        float *r = s_g[threadIdx.x];
-        s_id[threadIdx.x] = g;
-        r[0] = mu[g];
-        r[1] = mu[n + g];
-        r[2] = conic[g];
-        r[3] = conic[n + g];
-        r[4] = conic[2 * n + g];
-        r[5] = opacity[g];
-        r[6] = color[g];
-        r[7] = color[n + g];
-        r[8] = color[2 * n + g];
+        s.id[threadIdx.x] = g;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s.row[threadIdx.x][k] = rows[3 * (int64_t)g + k];
     }
     __syncthreads();
     return cnt;
 }
 
 __global__ void __launch_bounds__(GS_THREADS) k_gs_render_fwd(
-    GsCam c, int n, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
-    const float *__restrict__ mu, const float *__restrict__ conic,
-    const float *__restrict__ color, const float *__restrict__ opacity,
-    float *__restrict__ image, float *__restrict__ image_keep) {
-    __shared__ int s_id[GS_THREADS];
-    __shared__ float s_g[GS_THREADS][9];  // mu(2) conic(3) opacity color(3)
-    const int tx0 = blockIdx.x * GS_TILE, ty0 = blockIdx.y * GS_TILE;
+    GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
+    const float4 *__restrict__ rows, float *__restrict__ image, float *__restrict__ image_keep,
+    const uint32_t *__restrict__ batch_off, float4 *__restrict__ before) {
+    __shared__ GsBatch s;
+    const int tx0 = (int)(blockIdx.x % tiles_x) * GS_TILE, ty0 = (int)(blockIdx.x / tiles_x) * GS_TILE;
     const int px = tx0 + (threadIdx.x & (GS_TILE - 1)), py = ty0 + threadIdx.x / GS_TILE;
     const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
-    const int2 rg = ranges[blockIdx.y * gridDim.x + blockIdx.x];
+    const int2 rg = ranges[blockIdx.x];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    for (int b0 = rg.x; b0 < rg.y; b0 += GS_THREADS) {
-        const int cnt = gs_load_batch(b0, rg.y, n, list, mu, conic, color, opacity, s_id, s_g);
+    float4 *keep = before + (size_t)batch_off[blockIdx.x] * GS_THREADS + threadIdx.x;
+    for (int b0 = rg.x; b0 < rg.y; b0 += GS_THREADS, keep += GS_THREADS) {
+        const int cnt = gs_load_batch(b0, rg.y, list, rows, s);
+        *keep = make_float4(C0, C1, C2, T);  // for the backward, which takes each batch by itself
+#pragma unroll 4
         for (int k = 0; k < cnt; ++k) {
-            const float *r = s_g[k];
-            const float dx = fx - r[0], dy = fy - r[1];
-            const float q = r[2] * dx * dx + 2.0f * r[3] * dx * dy + r[4] * dy * dy;
+            const float4 r = s.row[k][0], u = s.row[k][1];
+            const float dx = fx - r.x, dy = fy - r.y;
+            const float q = r.z * dx * dx + 2.0f * r.w * dx * dy + u.x * dy * dy;
             if (q <= 9.0f) {
-                const float a = r[5] * expf(-0.5f * q);
+                const float a = u.y * expf(-0.5f * q);
                 const float w = T * a;
-                C0 += w * r[6];
-                C1 += w * r[7];
-                C2 += w * r[8];
+                C0 += w * u.z;
+                C1 += w * u.w;
+                C2 += w * s.row[k][2].x;
                 T *= 1.0f - a;
             }
         }
@@ -448,18 +696,54 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Per pixel, front to back: w = T alpha, dL/dc += g w, dL/dalpha = g . (T c -
-// (C - C_<=i) / (1 - alpha)), then dL/do, dL/dmu', dL/dconic; each Gaussian's
-// nine sums over a warp's pixels go to memory from nine lanes at once.
+// Sums of eight values over the warp: lane L receives the total of value
+// (L >> 2) of v. Each of the first three steps halves the values a lane still
+// carries (it sends one half and adds the other's counterpart), so 9 shuffles
+// instead of 40.
+__device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+    float a[4], b[2], t;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const bool up = lane & 16;
+        const float keep = up ? v[4 + j] : v[j], send = up ? v[j] : v[4 + j];
+        a[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const bool up = lane & 8;
+        const float keep = up ? a[2 + j] : a[j], send = up ? a[j] : a[2 + j];
+        b[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    {
+        const bool up = lane & 4;
+        const float keep = up ? b[1] : b[0], send = up ? b[0] : b[1];
+        t = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    return t;
+}
+
+// One batch of a tile's list per block, from the colour and transmittance the
+// forward pass kept in front of it: as one block per tile the longest list's
+// serial walk was the kernel's time (235 entries on the 1,300 tiles that the
+// 100,284-Gaussian sheet meets: 17 warps per SM). Per pixel, front to back:
+// w = T alpha, dL/dc += g w, dL/dalpha = g . (T c - (C - C_<=i) / (1 - alpha)).
+// With s = exp(-q/2) dL/dalpha, d = pixel - mu' and dL/dq = -s opacity / 2, all
+// of a Gaussian's gradients are linear in the sums over pixels of s, s d and
+// s d d^T, which k_gs_preprocess_bwd turns into dL/d(mu', conic). Each warp's
+// nine sums go to the Gaussian's row of g2d (GS_ROW floats, so nine
+// neighbouring words: two sectors) from nine lanes at once.
 __global__ void __launch_bounds__(GS_THREADS) k_gs_render_bwd(
-    GsCam c, int n, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
-    const float *__restrict__ mu, const float *__restrict__ conic,
-    const float *__restrict__ color, const float *__restrict__ opacity,
+    GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
+    const float4 *__restrict__ rows, const uint32_t *__restrict__ batch_tile,
+    const uint32_t *__restrict__ batch_off, const float4 *__restrict__ before,
     const float *__restrict__ image_keep, const float *__restrict__ g_image,
     float *__restrict__ g2d) {
-    __shared__ int s_id[GS_THREADS];
-    __shared__ float s_g[GS_THREADS][9];
-    const int tx0 = blockIdx.x * GS_TILE, ty0 = blockIdx.y * GS_TILE;
+    __shared__ GsBatch s;
+    const unsigned tile = batch_tile[blockIdx.x];
+    const int tx0 = (int)(tile % tiles_x) * GS_TILE, ty0 = (int)(tile / tiles_x) * GS_TILE;
     const int px = tx0 + (threadIdx.x & (GS_TILE - 1)), py = ty0 + threadIdx.x / GS_TILE;
     const bool inside = px < c.width && py < c.height;
     const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
@@ -472,65 +756,66 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_render_bwd(
             gC[ch] = g_image[ch * hw + pix];
         }
     }
-    float T = 1.0f, Cl[3] = {0.0f, 0.0f, 0.0f};
+    const float4 b4 = before[(size_t)blockIdx.x * GS_THREADS + threadIdx.x];
+    float T = b4.w, Cl[3] = {b4.x, b4.y, b4.z};
     const int lane = threadIdx.x & 31;
-    const int2 rg = ranges[blockIdx.y * gridDim.x + blockIdx.x];
-    for (int b0 = rg.x; b0 < rg.y; b0 += GS_THREADS) {
-        const int cnt = gs_load_batch(b0, rg.y, n, list, mu, conic, color, opacity, s_id, s_g);
-        for (int k = 0; k < cnt; ++k) {
-            const float *r = s_g[k];
-            const float dx = fx - r[0], dy = fy - r[1];
-            const float q = r[2] * dx * dx + 2.0f * r[3] * dx * dy + r[4] * dy * dy;
-            float v[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            const bool hit = inside && q <= 9.0f;
-            if (hit) {
-                const float e = expf(-0.5f * q);
-                const float a = r[5] * e;
-                const float w = T * a;
-                float dA = 0.0f;
+    const int2 rg = ranges[tile];
+    const int cnt = gs_load_batch(rg.x + (int)(blockIdx.x - batch_off[tile]) * GS_THREADS, rg.y, list,
+                                  rows, s);
+#pragma unroll 2
+    for (int k = 0; k < cnt; ++k) {
+        const float4 r = s.row[k][0], u = s.row[k][1];
+        const float dx = fx - r.x, dy = fy - r.y;
+        const float q = r.z * dx * dx + 2.0f * r.w * dx * dy + u.x * dy * dy;
+        const bool hit = inside && q <= 9.0f;
+        if (!__any_sync(0xffffffffu, hit)) continue;
+        // s d (2), s d d^T (3), s, dL/dcolor (3)
+        float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, v8 = 0.0f;
+        if (hit) {
+            const float col[3] = {u.z, u.w, s.row[k][2].x};
+            const float e = expf(-0.5f * q);
+            const float a = u.y * e;
+            const float w = T * a, inv = 1.0f / (1.0f - a);
+            float dA = 0.0f;
 #pragma unroll
-                for (int ch = 0; ch < 3; ++ch) {
-                    Cl[ch] += w * r[6 + ch];
-                    dA += gC[ch] * (T * r[6 + ch] - (Cf[ch] - Cl[ch]) / (1.0f - a));
-                    v[6 + ch] = gC[ch] * w;  // dL/dcolor
-                }
-                v[5] = dA * e;                 // dL/dopacity
-                const float dq = -0.5f * a * dA;  // dL/dq
-                v[0] = -2.0f * dq * (r[2] * dx + r[3] * dy);  // dL/dmu'
-                v[1] = -2.0f * dq * (r[3] * dx + r[4] * dy);
-                v[2] = dq * dx * dx;           // dL/dconic a, b, c
-                v[3] = dq * 2.0f * dx * dy;
-                v[4] = dq * dy * dy;
-                T *= 1.0f - a;
+            for (int ch = 0; ch < 3; ++ch) {
+                Cl[ch] += w * col[ch];
+                dA += gC[ch] * (T * col[ch] - (Cf[ch] - Cl[ch]) * inv);
             }
-            if (__any_sync(0xffffffffu, hit)) {
-                // the xor sums leave all nine totals in every lane: lane j adds total j
-                float mine = 0.0f;
-#pragma unroll
-                for (int j = 0; j < 9; ++j) {
-                    const float sj = warp_sum(v[j]);
-                    mine = lane == j ? sj : mine;
-                }
-                if (lane < 9 && mine != 0.0f) atomicAdd(&g2d[(int64_t)lane * n + s_id[k]], mine);
-            }
+            v[5] = dA * e;
+            v[0] = v[5] * dx;
+            v[1] = v[5] * dy;
+            v[2] = v[0] * dx;
+            v[3] = v[0] * dy;
+            v[4] = v[1] * dy;
+            v[6] = gC[0] * w;
+            v[7] = gC[1] * w;
+            v8 = gC[2] * w;
+            T *= 1.0f - a;
         }
-        __syncthreads();
+        const float t = warp_sum8(v), t8 = warp_sum(v8);
+        // lane 4 j adds value j, lane 1 value 8
+        const int j = (lane & 3) == 0 ? lane >> 2 : 8;
+        const float mine = j == 8 ? t8 : t;
+        if (((lane & 3) == 0 || lane == 1) && mine != 0.0f)
+            atomicAdd(&g2d[(int64_t)s.id[k] * GS_ROW + j], mine);
     }
 }
 
-// dL/d(mu', conic, opacity, color) of each Gaussian -> dL/dx, dL/dF (and the
+// The 2D gradients of each Gaussian (k_gs_render_bwd's sums) -> dL/dx, dL/dF (and the
 // colour and opacity gradients), accumulated into the caller's buffers.
 __global__ void k_gs_preprocess_bwd(GsCam c, const float *__restrict__ x,
                                     const float *__restrict__ F, const float *__restrict__ s0,
-                                    int n, const float *__restrict__ g2d, float *__restrict__ g_x,
+                                    const float *__restrict__ opacity, int n,
+                                    const float *__restrict__ g2d, float *__restrict__ g_x,
                                     float *__restrict__ g_F, float *__restrict__ g_color,
                                     float *__restrict__ g_opacity) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t nn = n;
-    float gv[9];
-#pragma unroll
-    for (int j = 0; j < 9; ++j) gv[j] = g2d[j * nn + i];
+    const float4 *gr = reinterpret_cast<const float4 *>(g2d + (int64_t)i * GS_ROW);
+    const float4 ga = gr[0], gb = gr[1];
+    float gv[9] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w, gr[2].x};
     if (g_opacity) g_opacity[i] += gv[5];
     if (g_color) {
         g_color[i] += gv[6];
@@ -546,6 +831,14 @@ __global__ void k_gs_preprocess_bwd(GsCam c, const float *__restrict__ x,
     GsProj p;
     gs_project(c, xp, S, p);
     if (!p.visible) return;
+    {  // dL/dmu' = -2 sum dL/dq A d, dL/dA = sum dL/dq d d^T, dL/dq = -s o / 2
+        const float o = opacity[i], m0 = gv[0], m1 = gv[1];
+        gv[0] = o * (p.conic[0] * m0 + p.conic[1] * m1);
+        gv[1] = o * (p.conic[1] * m0 + p.conic[2] * m1);
+        gv[2] *= -0.5f * o;
+        gv[3] *= -o;
+        gv[4] *= -0.5f * o;
+    }
     // conic A = Sigma'^-1: dL/dSigma' = -A Abar A, Abar = [[ga, gb/2], [gb/2, gc]]
     const float A00 = p.conic[0], A01 = p.conic[1], A11 = p.conic[2];
     const float b00 = gv[2], b01 = 0.5f * gv[3], b11 = gv[4];
@@ -613,98 +906,148 @@ __global__ void k_gs_preprocess_bwd(GsCam c, const float *__restrict__ x,
         g_x[b * nn + i] += c.R[b] * gt[0] + c.R[3 + b] * gt[1] + c.R[6 + b] * gt[2];
 }
 
+// Block sum of term, added to *loss times scale by one thread.
+__device__ __forceinline__ void block_add(float term, float scale, float *loss, float bias = 0.0f) {
+    __shared__ float red[8];
+    const int t = threadIdx.y * blockDim.x + threadIdx.x;
+    term = warp_sum(term);
+    if ((t & 31) == 0) red[t >> 5] = term;
+    __syncthreads();
+    if (t < 32) {
+        float s = t < 8 ? red[t] : 0.0f;
+        s = warp_sum(s);
+        if (t == 0) atomicAdd(loss, scale * s + bias);
+    }
+}
+
+// Four values per thread, so that a block's one atomic on the loss stands for
+// 1024 of them (the 3,072 atomics of a 3 x 512 x 512 image on one address took
+// most of 7.4 us).
 __global__ void __launch_bounds__(256) k_image_l1(const float *__restrict__ img,
                                                   const float *__restrict__ target, int64_t n,
                                                   float weight, float *__restrict__ loss,
                                                   float *__restrict__ g) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float term = 0.0f;
-    if (i < n) {
-        const float d = img[i] - target[i];
-        term = fabsf(d);
-        if (g) g[i] += weight * (d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int64_t i = ((int64_t)blockIdx.x * 4 + j) * 256 + threadIdx.x;
+        if (i < n) {
+            const float d = img[i] - target[i];
+            term += fabsf(d);
+            if (g) g[i] += weight * (d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f));
+        }
     }
-    __shared__ float red[8];
-    term = warp_sum(term);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = term;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float s = threadIdx.x < 8 ? red[threadIdx.x] : 0.0f;
-        s = warp_sum(s);
-        if (threadIdx.x == 0) atomicAdd(loss, weight * s);
-    }
+    block_add(term, weight, loss);
 }
 
 // ----------------------------------------------------------------- D-SSIM --
 // The structural term of L_render: 1 - mean SSIM with local statistics under
 // an 11 x 11 Gaussian window (sigma 1.5, zero outside the image), computed as
-// separable blurs: horizontal sums of the five maps x, y, x^2, y^2, x y, then
-// vertical sums; the gradient blurs the per-pixel partials back the same way
-// (the window is symmetric, so the transposed blur is the blur).
+// separable blurs within a 32 x 16 tile: the tile of both images with a halo of
+// 5 in shared memory, horizontal sums of the five maps x, y, x^2, y^2, x y of
+// its 26 rows, then vertical sums, so that the maps never reach memory. The
+// gradient blurs the per-pixel partials back the same way (the window is
+// symmetric, so the transposed blur is the blur). One launch each; as six
+// launches over whole maps in memory the two took 125 us at 3 x 512 x 512.
 
 struct SsimWin {
     float w[11];
 };
 
-__global__ void k_ssim_h5(const float *__restrict__ x, const float *__restrict__ y, int C, int H,
-                          int W, SsimWin k, float *__restrict__ out) {
-    const int64_t plane = (int64_t)C * H * W;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= plane) return;
-    const int px = (int)(i % W);
-    const int64_t row = i - px;
-    float s[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int d = -5; d <= 5; ++d) {
-        const int q = px + d;
-        if (q < 0 || q >= W) continue;
-        const float a = x[row + q], b = y[row + q], w = k.w[d + 5];
-        s[0] += w * a;
-        s[1] += w * b;
-        s[2] += w * a * a;
-        s[3] += w * b * b;
-        s[4] += w * a * b;
-    }
-#pragma unroll
-    for (int m = 0; m < 5; ++m) out[m * plane + i] = s[m];
+constexpr int SS_X = 32, SS_Y = 16, SS_H = 5;  // tile and halo; 32 x 8 threads
+constexpr int SS_RX = SS_X + 2 * SS_H, SS_RY = SS_Y + 2 * SS_H;
+
+// First pixel of this block's tile, and the offset of its plane (blocks run over
+// the tiles of all planes, x fastest).
+__device__ __forceinline__ int2 ss_tile(int H, int W) {
+    const unsigned tx = (W + SS_X - 1) / SS_X, ty = (H + SS_Y - 1) / SS_Y;
+    return make_int2((int)(blockIdx.x % tx) * SS_X, (int)(blockIdx.x / tx % ty) * SS_Y);
+}
+__device__ __forceinline__ int64_t ss_plane(int H, int W) {
+    const unsigned tx = (W + SS_X - 1) / SS_X, ty = (H + SS_Y - 1) / SS_Y;
+    return (int64_t)(blockIdx.x / (tx * ty)) * H * W;
 }
 
-// One-direction blur of `maps` planes of H x W (horizontal: dir 0, vertical: 1).
-__global__ void k_blur(const float *__restrict__ in, int64_t maps, int H, int W, int dir, SsimWin k,
-                       float *__restrict__ out) {
-    const int64_t total = maps * H * W;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const int px = (int)(i % W), py = (int)((i / W) % H);
-    const int64_t base = i - px - (int64_t)py * W;  // start of this plane
-    float s = 0.0f;
-#pragma unroll
-    for (int d = -5; d <= 5; ++d) {
-        const int qx = dir == 0 ? px + d : px, qy = dir == 0 ? py : py + d;
-        if (qx < 0 || qx >= W || qy < 0 || qy >= H) continue;
-        s += k.w[d + 5] * in[base + (int64_t)qy * W + qx];
+// The tile at (x0, y0) of a plane with its halo, zero outside the image.
+__device__ __forceinline__ void ss_load(const float *__restrict__ plane, int H, int W, int x0, int y0,
+                                        float (*t)[SS_RX]) {
+    for (int i = threadIdx.y * SS_X + threadIdx.x; i < SS_RX * SS_RY; i += 256) {
+        const int cx = i % SS_RX, cy = i / SS_RX, px = x0 + cx - SS_H, py = y0 + cy - SS_H;
+        t[cy][cx] = px >= 0 && px < W && py >= 0 && py < H ? plane[(int64_t)py * W + px] : 0.0f;
     }
-    out[i] = s;
 }
 
 // SSIM per pixel from the blurred maps (mu_x, mu_y, <x^2>, <y^2>, <x y>);
 // loss += weight (1 - mean SSIM); part = weight * dD/d(mu_x, <x^2>, <x y>).
-__global__ void __launch_bounds__(256) k_ssim_map(const float *__restrict__ v5, int64_t n,
-                                                  float weight, float *__restrict__ loss,
-                                                  float *__restrict__ part) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_ssim(const float *__restrict__ x,
+                                              const float *__restrict__ y, int H, int W, int64_t n,
+                                              SsimWin k, float weight, float *__restrict__ loss,
+                                              float *__restrict__ part) {
+    __shared__ float tx[SS_RY][SS_RX], ty[SS_RY][SS_RX];
+    __shared__ float h[5][SS_RY][SS_X];
+    const int2 at = ss_tile(H, W);
+    const int x0 = at.x, y0 = at.y;
+    const int64_t plane = ss_plane(H, W);
+    ss_load(x + plane, H, W, x0, y0, tx);
+    ss_load(y + plane, H, W, x0, y0, ty);
+    __syncthreads();
+    // four neighbouring sums per thread from 14 values of its row
+    const int tid = threadIdx.y * SS_X + threadIdx.x;
+    if (tid < SS_RY * SS_X / 4) {
+        const int r = tid / (SS_X / 4), c4 = tid % (SS_X / 4) * 4;
+        float a[14], b[14];
+#pragma unroll
+        for (int i = 0; i < 14; ++i) {
+            a[i] = tx[r][c4 + i];
+            b[i] = ty[r][c4 + i];
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            float s[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int d = 0; d < 11; ++d) {
+                const float w = k.w[d];
+                s[0] += w * a[o + d];
+                s[1] += w * b[o + d];
+                s[2] += w * a[o + d] * a[o + d];
+                s[3] += w * b[o + d] * b[o + d];
+                s[4] += w * a[o + d] * b[o + d];
+            }
+#pragma unroll
+            for (int m = 0; m < 5; ++m) h[m][r][c4 + o] = s[m];
+        }
+    }
+    __syncthreads();
     const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
     const float scale = -weight / (float)n;
     float term = 0.0f;
-    if (i < n) {
-        const float A = v5[i], Ay = v5[n + i], B = v5[2 * n + i], Byy = v5[3 * n + i],
-                    Cxy = v5[4 * n + i];
+    float vv[2][5];  // two neighbouring rows per thread from 12 values of its column
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        float t[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) t[i] = h[m][2 * threadIdx.y + i][threadIdx.x];
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            vv[o][m] = 0.0f;
+#pragma unroll
+            for (int d = 0; d < 11; ++d) vv[o][m] += k.w[d] * t[o + d];
+        }
+    }
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+        const int r = 2 * threadIdx.y + o;
+        const float(&v)[5] = vv[o];
+        const int px = x0 + threadIdx.x, py = y0 + r;
+        if (px >= W || py >= H) continue;
+        const float A = v[0], Ay = v[1], B = v[2], Byy = v[3], Cxy = v[4];
         const float n1 = 2.0f * A * Ay + C1, n2 = 2.0f * (Cxy - A * Ay) + C2;
         const float d1 = A * A + Ay * Ay + C1, d2 = (B - A * A) + (Byy - Ay * Ay) + C2;
         const float dd = d1 * d2;
         const float S = n1 * n2 / dd;
-        term = S;
+        term += S;
         if (part) {
+            const int64_t i = plane + (int64_t)py * W + px;
             const float dA = 2.0f * Ay * (n2 - n1) / dd - 2.0f * A * n1 * n2 * (d2 - d1) / (dd * dd);
             const float dB = -S / d2;
             const float dC = 2.0f * n1 / dd;
@@ -713,23 +1056,60 @@ __global__ void __launch_bounds__(256) k_ssim_map(const float *__restrict__ v5, 
             part[2 * n + i] = scale * dC;
         }
     }
-    __shared__ float red[8];
-    term = warp_sum(term);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = term;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float t = threadIdx.x < 8 ? red[threadIdx.x] : 0.0f;
-        t = warp_sum(t);
-        if (threadIdx.x == 0) atomicAdd(loss, scale * t + (blockIdx.x == 0 ? weight : 0.0f));
-    }
+    block_add(term, scale, loss, blockIdx.x == 0 ? weight : 0.0f);
 }
 
 // g += blur(p_mu) + 2 x blur(p_xx) + y blur(p_xy)
-__global__ void k_ssim_grad(const float *__restrict__ x, const float *__restrict__ y,
-                            const float *__restrict__ bp, int64_t n, float *__restrict__ g) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    g[i] += bp[i] + 2.0f * x[i] * bp[n + i] + y[i] * bp[2 * n + i];
+__global__ void __launch_bounds__(256) k_ssim_grad(const float *__restrict__ x,
+                                                   const float *__restrict__ y,
+                                                   const float *__restrict__ part, int H, int W,
+                                                   int64_t n, SsimWin k, float *__restrict__ g) {
+    __shared__ float t[3][SS_RY][SS_RX];
+    __shared__ float h[3][SS_RY][SS_X];
+    const int2 at = ss_tile(H, W);
+    const int x0 = at.x, y0 = at.y;
+    const int64_t plane = ss_plane(H, W);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) ss_load(part + m * n + plane, H, W, x0, y0, t[m]);
+    __syncthreads();
+    const int tid = threadIdx.y * SS_X + threadIdx.x;
+    if (tid < SS_RY * SS_X / 4) {
+        const int r = tid / (SS_X / 4), c4 = tid % (SS_X / 4) * 4;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            float a[14];
+#pragma unroll
+            for (int i = 0; i < 14; ++i) a[i] = t[m][r][c4 + i];
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                float s = 0.0f;
+#pragma unroll
+                for (int d = 0; d < 11; ++d) s += k.w[d] * a[o + d];
+                h[m][r][c4 + o] = s;
+            }
+        }
+    }
+    __syncthreads();
+    float b[2][3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        float a[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) a[i] = h[m][2 * threadIdx.y + i][threadIdx.x];
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            b[o][m] = 0.0f;
+#pragma unroll
+            for (int d = 0; d < 11; ++d) b[o][m] += k.w[d] * a[o + d];
+        }
+    }
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+        const int px = x0 + threadIdx.x, py = y0 + 2 * threadIdx.y + o;
+        if (px >= W || py >= H) continue;
+        const int64_t i = plane + (int64_t)py * W + px;
+        g[i] += b[o][0] + 2.0f * x[i] * b[o][1] + y[i] * b[o][2];
+    }
 }
 
 static SsimWin ssim_window() {
@@ -746,15 +1126,31 @@ static SsimWin ssim_window() {
 struct GsHandle {
     int64_t cap = 0;
     int width = 0, height = 0;
-    float *mu = nullptr, *conic = nullptr, *g2d = nullptr, *image = nullptr;
+    float4 *rows = nullptr;          // [cap][3] packed projected Gaussians
+    float *g2d = nullptr;            // [cap][GS_ROW] their gradients
+    float *image = nullptr;
     int4 *rect = nullptr;
-    uint32_t *key = nullptr, *idx = nullptr, *key2 = nullptr, *idx2 = nullptr, *counts = nullptr;
-    uint32_t *tcnt = nullptr, *toff = nullptr, *bsum = nullptr, *total = nullptr;
-    int2 *ranges = nullptr;  // [tiles]
-    // tile list: (tile key, Gaussian) entries and their sort buffers
+    uint32_t *key = nullptr;         // [cap] depth bits
+    uint32_t *tile_count = nullptr;  // [tiles]
+    int2 *ranges = nullptr;          // [tiles]
+    uint32_t *batch_off = nullptr;   // [tiles] first batch of each tile
+    uint32_t *big = nullptr;         // [cap + 1] queue of Gaussians meeting many tiles; [cap]: its length
+    GsStat *stat = nullptr;
+    // tile list: keys as filled, Gaussians in order
     int64_t list_cap = 0;
-    uint32_t *lkey = nullptr, *lgid = nullptr, *lkey2 = nullptr, *lgid2 = nullptr,
-             *lcounts = nullptr;
+    unsigned long long *lkey = nullptr;
+    uint32_t *lgid = nullptr;
+    // batches of the list: their tiles, and each pixel's colour and
+    // transmittance in front of them
+    int64_t batch_cap = 0;
+    uint32_t *batch_tile = nullptr;
+    float4 *before = nullptr;
+    uint32_t batches = 0;            // of the last gs_render
+    // the radix path's buffers (allocated by the first call that takes it):
+    // depth sort and tile-list sort in turn, `radix_cap` entries
+    int64_t radix_cap = 0;
+    uint32_t *rk[2] = {nullptr, nullptr}, *rv[2] = {nullptr, nullptr}, *rcounts = nullptr;
+    uint32_t *tcnt = nullptr, *toff = nullptr, *bsum = nullptr, *total = nullptr;
     const uint32_t *list = nullptr;  // the sorted Gaussian column of the last gs_render
     int tiles_x = 0, tiles_y = 0;
     int last_n = -1;  // Gaussians of the last gs_render
@@ -802,22 +1198,97 @@ struct dw_gs_s : GsHandle {};
 static dw_status gs_list_reserve(dw_gs h, int64_t m) {
     if (m <= h->list_cap) return DW_OK;
     const int64_t cap = std::max<int64_t>(m, h->list_cap * 3 / 2);
-    DW_REQUIRE(cap < (1ll << 31), "tile list too long (Gaussians x tiles met >= 2^31)");
     cudaFree(h->lkey);
     cudaFree(h->lgid);
-    cudaFree(h->lkey2);
-    cudaFree(h->lgid2);
-    cudaFree(h->lcounts);
-    h->lkey = h->lgid = h->lkey2 = h->lgid2 = h->lcounts = nullptr;
+    h->lkey = nullptr;
+    h->lgid = nullptr;
     h->list_cap = 0;
-    const size_t c = (size_t)cap, nb = (c + RS_TILE - 1) / RS_TILE;
-    cudaError_t e = cudaMalloc((void **)&h->lkey, sizeof(uint32_t) * c);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lgid, sizeof(uint32_t) * c);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lkey2, sizeof(uint32_t) * c);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lgid2, sizeof(uint32_t) * c);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lcounts, sizeof(uint32_t) * 256 * nb);
+    cudaError_t e = cudaMalloc((void **)&h->lkey, sizeof(unsigned long long) * (size_t)cap);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lgid, sizeof(uint32_t) * (size_t)cap);
     if (e != cudaSuccess) return cuda_fail(e, "gs_render (tile list)");
     h->list_cap = cap;
+    return DW_OK;
+}
+
+// Grow the batch buffers to hold nb batches (1 KB each).
+static dw_status gs_batch_reserve(dw_gs h, int64_t nb) {
+    if (nb <= h->batch_cap) return DW_OK;
+    const int64_t cap = std::max<int64_t>(nb, h->batch_cap * 3 / 2);
+    cudaFree(h->batch_tile);
+    cudaFree(h->before);
+    h->batch_tile = nullptr;
+    h->before = nullptr;
+    h->batch_cap = 0;
+    cudaError_t e = cudaMalloc((void **)&h->batch_tile, sizeof(uint32_t) * (size_t)cap);
+    if (e == cudaSuccess)
+        e = cudaMalloc((void **)&h->before, sizeof(float4) * GS_THREADS * (size_t)cap);
+    if (e != cudaSuccess) return cuda_fail(e, "gs_render (list batches)");
+    h->batch_cap = cap;
+    return DW_OK;
+}
+
+static void gs_radix_free(dw_gs h) {
+    for (int k = 0; k < 2; ++k) {
+        cudaFree(h->rk[k]);
+        cudaFree(h->rv[k]);
+        h->rk[k] = h->rv[k] = nullptr;
+    }
+    cudaFree(h->rcounts);
+    cudaFree(h->tcnt);
+    cudaFree(h->toff);
+    cudaFree(h->bsum);
+    cudaFree(h->total);
+    h->rcounts = h->tcnt = h->toff = h->bsum = h->total = nullptr;
+    h->radix_cap = 0;
+}
+
+// The radix path's buffers for n Gaussians and m list entries.
+static dw_status gs_radix_reserve(dw_gs h, int64_t n, int64_t m) {
+    const int64_t need = std::max(n, m);
+    if (need <= h->radix_cap) return DW_OK;
+    gs_radix_free(h);
+    const size_t c = (size_t)std::max(need, h->cap), g = (size_t)h->cap;
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 2; ++k) {
+        if (e == cudaSuccess) e = cudaMalloc((void **)&h->rk[k], sizeof(uint32_t) * c);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&h->rv[k], sizeof(uint32_t) * c);
+    }
+    if (e == cudaSuccess)
+        e = cudaMalloc((void **)&h->rcounts, sizeof(uint32_t) * 256 * ((c + RS_TILE - 1) / RS_TILE));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->tcnt, sizeof(uint32_t) * g);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->toff, sizeof(uint32_t) * g);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->bsum, sizeof(uint32_t) * ((g + 1023) / 1024));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->total, sizeof(uint32_t));
+    if (e != cudaSuccess) {
+        gs_radix_free(h);
+        return cuda_fail(e, "gs_render (radix sort)");
+    }
+    h->radix_cap = (int64_t)c;
+    return DW_OK;
+}
+
+// The tile lists by two stable sorts: all Gaussians by depth, then the list,
+// filled in that order, by tile.
+static dw_status gs_list_radix(dw_gs h, int n, int64_t m, cudaStream_t s) {
+    dw_status st = gs_radix_reserve(h, n, m);
+    if (st != DW_OK) return st;
+    uint32_t *ka = h->rk[0], *va = h->rv[0], *kb = h->rk[1], *vb = h->rv[1];
+    k_gs_order_init<<<grid_for(n, 256), 256, 0, s>>>(h->key, n, ka, va);
+    radix_sort(ka, va, kb, vb, n, 4, h->rcounts, s);  // depth order in va
+    k_gs_tile_count<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, n, h->tcnt);
+    const int nsb = (n + 1023) / 1024;
+    k_scan1024<<<nsb, 256, 0, s>>>(h->tcnt, n, h->toff, h->bsum);
+    k_rs_scan<<<1, 1024, 0, s>>>(h->bsum, nsb);
+    k_scan_finish<<<grid_for(n, 256), 256, 0, s>>>(h->toff, h->tcnt, n, h->bsum, h->total);
+    // the list: tile keys to kb, Gaussians to lgid, then both sorted (the depth
+    // order in va is read before the sort's second buffers overwrite it)
+    k_gs_duplicate<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, h->toff, n, h->tiles_x, kb,
+                                                    h->lgid);
+    int bits = 1;
+    while ((1ll << bits) < (int64_t)h->tiles_x * h->tiles_y) ++bits;
+    uint32_t *lk = kb, *lv = h->lgid, *lk2 = ka, *lv2 = va;
+    radix_sort(lk, lv, lk2, lv2, (int)m, (bits + 7) / 8, h->rcounts, s);
+    h->list = lv;
     return DW_OK;
 }
 
@@ -835,26 +1306,20 @@ extern "C" dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t hei
     h->cap = max_gaussians;
     h->width = width;
     h->height = height;
-    const size_t n = (size_t)max_gaussians, nb = (n + RS_TILE - 1) / RS_TILE;
-    cudaError_t e = cudaMalloc((void **)&h->mu, sizeof(float) * 2 * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->conic, sizeof(float) * 3 * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->g2d, sizeof(float) * 9 * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->rect, sizeof(int4) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->key, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->idx, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->key2, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->idx2, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->counts, sizeof(uint32_t) * 256 * nb);
-    if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->image, sizeof(float) * 3 * (size_t)width * height);
     h->tiles_x = (width + GS_TILE - 1) / GS_TILE;
     h->tiles_y = (height + GS_TILE - 1) / GS_TILE;
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->tcnt, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->toff, sizeof(uint32_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->bsum, sizeof(uint32_t) * ((n + 1023) / 1024));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->total, sizeof(uint32_t));
+    const size_t n = (size_t)max_gaussians, tiles = (size_t)h->tiles_x * h->tiles_y;
+    cudaError_t e = cudaMalloc((void **)&h->rows, sizeof(float4) * 3 * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->g2d, sizeof(float) * GS_ROW * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->rect, sizeof(int4) * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->key, sizeof(uint32_t) * n);
     if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->ranges, sizeof(int2) * (size_t)h->tiles_x * h->tiles_y);
+        e = cudaMalloc((void **)&h->image, sizeof(float) * 3 * (size_t)width * height);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->tile_count, sizeof(uint32_t) * tiles);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->ranges, sizeof(int2) * tiles);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->batch_off, sizeof(uint32_t) * tiles);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->big, sizeof(uint32_t) * (n + 1));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->stat, sizeof(GsStat));
     if (e != cudaSuccess) {
         dw_status st = cuda_fail(e, "gs_create");
         gs_destroy(h);
@@ -866,26 +1331,21 @@ extern "C" dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t hei
 
 extern "C" dw_status gs_destroy(dw_gs h) {
     if (!h) return DW_OK;
-    cudaFree(h->mu);
-    cudaFree(h->conic);
+    cudaFree(h->rows);
     cudaFree(h->g2d);
     cudaFree(h->rect);
     cudaFree(h->key);
-    cudaFree(h->idx);
-    cudaFree(h->key2);
-    cudaFree(h->idx2);
-    cudaFree(h->counts);
     cudaFree(h->image);
-    cudaFree(h->tcnt);
-    cudaFree(h->toff);
-    cudaFree(h->bsum);
-    cudaFree(h->total);
+    cudaFree(h->tile_count);
     cudaFree(h->ranges);
+    cudaFree(h->batch_off);
+    cudaFree(h->big);
+    cudaFree(h->stat);
     cudaFree(h->lkey);
     cudaFree(h->lgid);
-    cudaFree(h->lkey2);
-    cudaFree(h->lgid2);
-    cudaFree(h->lcounts);
+    cudaFree(h->batch_tile);
+    cudaFree(h->before);
+    gs_radix_free(h);
     delete h;
     return DW_OK;
 }
@@ -923,38 +1383,54 @@ extern "C" dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, co
     const GsCam c = to_cam(*cam);
     const int nn = (int)n;
     const int ntiles = h->tiles_x * h->tiles_y;
-    DW_CUDA(cudaMemsetAsync(h->ranges, 0, sizeof(int2) * (size_t)ntiles, s));
+    h->last_n = -1;  // no picture to differentiate until this call has drawn one
     h->list = h->lgid;
     if (nn > 0) {
-        k_gs_preprocess<<<grid_for(nn, 256), 256, 0, s>>>(c, x, F, sigma0, nn, h->mu, h->conic,
-                                                          h->rect, h->key, h->idx);
-        uint32_t *ka = h->key, *va = h->idx, *kb = h->key2, *vb = h->idx2;
-        radix_sort(ka, va, kb, vb, nn, 4, h->counts, s);  // depth order in (ka, va)
-        // tile list: counts in depth order, offsets, total
-        k_gs_tile_count<<<grid_for(nn, 256), 256, 0, s>>>(va, h->rect, nn, h->tcnt);
-        const int nsb = (nn + 1023) / 1024;
-        k_scan1024<<<nsb, 256, 0, s>>>(h->tcnt, nn, h->toff, h->bsum);
-        k_rs_scan<<<1, 1024, 0, s>>>(h->bsum, nsb);
-        k_scan_finish<<<grid_for(nn, 256), 256, 0, s>>>(h->toff, h->tcnt, nn, h->bsum, h->total);
-        uint32_t m = 0;
-        DW_CUDA(cudaMemcpyAsync(&m, h->total, sizeof m, cudaMemcpyDeviceToHost, s));
+        DW_CUDA(cudaMemsetAsync(h->tile_count, 0, sizeof(uint32_t) * (size_t)ntiles, s));
+        uint32_t *queued = h->big + h->cap;
+        DW_CUDA(cudaMemsetAsync(queued, 0, sizeof(uint32_t), s));
+        k_gs_preprocess<<<grid_for(nn, 128), 128, 0, s>>>(c, x, F, sigma0, color, opacity, nn,
+                                                          h->tiles_x, h->rows, h->rect, h->key,
+                                                          h->tile_count, h->big, queued);
+        k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key, h->tiles_x,
+                                                    h->tile_count, h->ranges, h->lkey, h->stat);
+        k_gs_tile_scan<<<1, 1024, 0, s>>>(h->tile_count, ntiles, h->ranges, h->batch_off, h->stat);
+        GsStat stat;
+        DW_CUDA(cudaMemcpyAsync(&stat, h->stat, sizeof stat, cudaMemcpyDeviceToHost, s));
         DW_CUDA(cudaStreamSynchronize(s));
+        const unsigned long long m = stat.total;
+        DW_REQUIRE(m < (1ull << 31), "tile list too long (Gaussians x tiles met >= 2^31)");
+        h->batches = stat.batches;
         if (m > 0) {
-            dw_status st2 = gs_list_reserve(h, (int64_t)m);
-            if (st2 != DW_OK) return st2;
-            k_gs_duplicate<<<grid_for(nn, 256), 256, 0, s>>>(va, h->rect, h->toff, nn, h->tiles_x,
-                                                             h->lkey, h->lgid);
-            int bits = 1;
-            while ((1 << bits) < ntiles) ++bits;
-            uint32_t *lk = h->lkey, *lv = h->lgid, *lk2 = h->lkey2, *lv2 = h->lgid2;
-            radix_sort(lk, lv, lk2, lv2, (int)m, (bits + 7) / 8, h->lcounts, s);
-            k_gs_tile_ranges<<<grid_for(m, 256), 256, 0, s>>>(lk, (int)m, h->ranges);
-            h->list = lv;
+            st = gs_list_reserve(h, (int64_t)m);
+            if (st == DW_OK) st = gs_batch_reserve(h, stat.batches);
+            if (st != DW_OK) return st;
+            h->list = h->lgid;
+            k_gs_list<<<grid_for(nn, 128), 128, 0, s>>>(h->rect, h->key, nn, h->tiles_x, h->ranges,
+                                                        h->lkey);
+            if (stat.big > 0)
+                k_gs_big<true><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key,
+                                                           h->tiles_x, h->tile_count, h->ranges,
+                                                           h->lkey, h->stat);
+            if (stat.most <= GS_SORT_MAX) {
+                size_t len = 2;
+                while (len < stat.most) len <<= 1;
+                k_gs_tile_sort<<<(unsigned)ntiles, GS_SORT_THREADS, len * sizeof(unsigned long long), s>>>(
+                    h->ranges, h->lkey, h->batch_off, h->lgid, h->batch_tile);
+            } else {
+                st = gs_list_radix(h, nn, (int64_t)m, s);
+                if (st != DW_OK) return st;
+                k_gs_batches<<<grid_for(ntiles, 256), 256, 0, s>>>(h->ranges, ntiles, h->batch_off,
+                                                                   h->batch_tile);
+            }
         }
+    } else {
+        DW_CUDA(cudaMemsetAsync(h->ranges, 0, sizeof(int2) * (size_t)ntiles, s));
+        DW_CUDA(cudaMemsetAsync(h->batch_off, 0, sizeof(uint32_t) * (size_t)ntiles, s));
+        h->batches = 0;
     }
-    const dim3 grid((unsigned)h->tiles_x, (unsigned)h->tiles_y);
-    k_gs_render_fwd<<<grid, GS_THREADS, 0, s>>>(c, nn, h->list, h->ranges, h->mu, h->conic, color,
-                                                 opacity, image, h->image);
+    k_gs_render_fwd<<<(unsigned)ntiles, GS_THREADS, 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, image, h->image,
+                                                            h->batch_off, h->before);
     h->last_n = nn;
     const void *in[5] = {x, F, sigma0, color, opacity};
     memcpy(h->last_in, in, sizeof in);
@@ -979,11 +1455,12 @@ extern "C" dw_status gs_render_backward(dw_gs h, const dw_camera *cam, const flo
     cudaStream_t s = as_stream(stream);
     const GsCam c = to_cam(*cam);
     const int nn = (int)n;
-    DW_CUDA(cudaMemsetAsync(h->g2d, 0, sizeof(float) * 9 * (size_t)nn, s));
-    const dim3 grid((unsigned)h->tiles_x, (unsigned)h->tiles_y);
-    k_gs_render_bwd<<<grid, GS_THREADS, 0, s>>>(c, nn, h->list, h->ranges, h->mu, h->conic, color,
-                                                 opacity, h->image, g_image, h->g2d);
-    k_gs_preprocess_bwd<<<grid_for(nn, 256), 256, 0, s>>>(c, x, F, sigma0, nn, h->g2d, g_x, g_F,
+    DW_CUDA(cudaMemsetAsync(h->g2d, 0, sizeof(float) * GS_ROW * (size_t)nn, s));
+    if (h->batches > 0)
+        k_gs_render_bwd<<<h->batches, GS_THREADS, 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges,
+                                                         h->rows, h->batch_tile, h->batch_off,
+                                                         h->before, h->image, g_image, h->g2d);
+    k_gs_preprocess_bwd<<<grid_for(nn, 256), 256, 0, s>>>(c, x, F, sigma0, opacity, nn, h->g2d, g_x, g_F,
                                                            g_color, g_opacity);
     DW_LAUNCHED("gs_render_backward");
     return DW_OK;
@@ -994,7 +1471,7 @@ extern "C" dw_status image_l1_loss(const float *image, const float *target, int6
     DW_REQUIRE(n >= 0, "n must be >= 0");
     if (n == 0) return DW_OK;
     DW_REQUIRE(image && target && loss, "image, target and loss must not be NULL");
-    k_image_l1<<<grid_for(n, 256), 256, 0, as_stream(stream)>>>(image, target, n, weight, loss,
+    k_image_l1<<<grid_for(n, 1024), 256, 0, as_stream(stream)>>>(image, target, n, weight, loss,
                                                                  g_image);
     DW_LAUNCHED("k_image_l1");
     return DW_OK;
@@ -1009,18 +1486,13 @@ extern "C" dw_status image_dssim_loss(const float *image, const float *target, i
     DW_REQUIRE(image && target && loss && workspace, "image, target, loss and workspace must not be NULL");
     cudaStream_t s = as_stream(stream);
     const SsimWin k = ssim_window();
-    float *h5 = workspace, *v5 = workspace + 5 * n;
-    k_ssim_h5<<<grid_for(n, 256), 256, 0, s>>>(image, target, channels, height, width, k, h5);
-    k_blur<<<grid_for(5 * n, 256), 256, 0, s>>>(h5, 5 * (int64_t)channels, height, width, 1, k, v5);
-    float *part = g_image ? workspace : nullptr;  // h5 is free again
-    k_ssim_map<<<grid_for(n, 256), 256, 0, s>>>(v5, n, weight, loss, part);
-    if (g_image) {
-        k_blur<<<grid_for(3 * n, 256), 256, 0, s>>>(part, 3 * (int64_t)channels, height, width, 0,
-                                                     k, v5);
-        k_blur<<<grid_for(3 * n, 256), 256, 0, s>>>(v5, 3 * (int64_t)channels, height, width, 1,
-                                                     k, part);
-        k_ssim_grad<<<grid_for(n, 256), 256, 0, s>>>(image, target, part, n, g_image);
-    }
+    const unsigned grid = (unsigned)((width + SS_X - 1) / SS_X) * (unsigned)((height + SS_Y - 1) / SS_Y) *
+                          (unsigned)channels;
+    const dim3 block(SS_X, 8);
+    float *part = g_image ? workspace : nullptr;
+    k_ssim<<<grid, block, 0, s>>>(image, target, height, width, n, k, weight, loss, part);
+    if (g_image)
+        k_ssim_grad<<<grid, block, 0, s>>>(image, target, part, height, width, n, k, g_image);
     DW_LAUNCHED("image_dssim_loss");
     return DW_OK;
 }

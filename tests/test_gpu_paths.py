@@ -152,3 +152,83 @@ def test_wind_gradient_scatter(nf, frames):
                                      tuple(a.astype(np.float64) for a in g), pinned=pin)[1]
     assert rel_l2(gw.cpu().numpy().ravel(), np.asarray(ref).ravel()) <= 1e-4
     mpm.close()
+
+
+def _gaussians(n, sigma, seed, opacity):
+    """Gaussians in a unit slab seen from 2 units away, with distinct depths."""
+    g = np.random.default_rng(seed)
+    x = g.uniform(-0.4, 0.4, (3, n)).astype(np.float32)
+    x[2] = (g.permutation(n) / n - 0.5).astype(np.float32) * 0.8
+    F = np.tile(np.eye(3).reshape(9, 1), (1, n)) + g.uniform(-0.1, 0.1, (9, n))
+    s0 = np.zeros((6, n))
+    s0[:3] = np.asarray(sigma) ** 2
+    col = g.uniform(0.0, 1.0, (3, n))
+    op = g.uniform(*opacity, n)
+    return [np.ascontiguousarray(a.astype(np.float32)) for a in (x, F, s0, col, op)]
+
+
+# Tile lists: up to 4,096 Gaussians of a tile by the sort in shared memory, more
+# by the radix sorts; a Gaussian meeting more than 16 tiles is listed by its
+# whole warp. Every Gaussian covers the whole image (q < 9 everywhere), so no
+# pixel depends on the cut-off. Image: n float32 roundings of a convex sum,
+# 1e-5; gradients relative L2 1e-4 as in the renderer's parity test.
+@pytest.mark.parametrize("n,size,opacity", [(1, (9, 8), (0.5, 0.9)), (40, (161, 97), (0.1, 0.5)),
+                                            (33, (8, 200), (0.1, 0.5)), (4096, (12, 9), (0.01, 0.1)),
+                                            (4097, (12, 9), (0.01, 0.1))])
+def test_gaussian_tile_lists(n, size, opacity):
+    from oracle import gsplat as G
+    W, H = size
+    arrs = _gaussians(n, 1.5, 7, opacity)
+    f = 0.4 * max(W, H)
+    kw = (np.eye(3), (0.0, 0.0, 2.0), f, f, W / 2, H / 2, W, H)
+    dcam, ocam = B.camera(*kw), G.camera(*kw)
+    r = B.GaussianRenderer(n, W, H)
+    d = [to_dev(a) for a in arrs]
+    img = r.render(dcam, *d)
+    ref = G.render(*arrs, ocam)
+    assert np.abs(img.cpu().numpy() - ref).max() <= 1e-5
+    if n <= 64:
+        g_img = np.random.default_rng(1).standard_normal((3, H, W)).astype(np.float32)
+        gs = [torch.zeros_like(d[k]) for k in (0, 1, 3, 4)]
+        r.backward(dcam, *d, to_dev(g_img), *gs)
+        grad = G.render_grad(*arrs, ocam, g_img)
+        for name, got in zip(("x", "F", "color", "opacity"), gs):
+            assert rel_l2(got.cpu().numpy(), grad[name]) <= 1e-4, name
+    r.close()
+
+
+# The sorted lists do not depend on the path: small Gaussians, one tile crowded
+# past the limit, drawn with and without the crowd's last members (which lie
+# behind everything, at zero opacity, so that the image must not change).
+def test_gaussian_list_paths_agree():
+    n = 6000
+    x, F, s0, col, op = _gaussians(n, 0.004, 8, (0.1, 0.9))
+    x[:2, :4095] = np.random.default_rng(2).uniform(0.0, 0.02, (2, 4095))
+    k = 5000
+    op[k:] = 0.0
+    x[:2, k:] = 0.01
+    x[2, k:] = 0.9 + 0.001 * np.arange(n - k) / n
+    cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), 90.0, 90.0, 50.0, 40.0, 100, 80)
+    r = B.GaussianRenderer(n, 100, 80)
+    imgs = [r.render(cam, *(to_dev(np.ascontiguousarray(a[..., :m])) for a in (x, F, s0, col, op)))
+            for m in (k, n)]
+    assert torch.equal(imgs[0], imgs[1]) and imgs[0].max() > 0.3
+    r.close()
+
+
+# D-SSIM on 32 x 16 tiles: images smaller than the window, exactly one tile, and
+# one pixel more; the oracle's tolerances (test_gpu_gsplat.py).
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 4, 3), (3, 16, 32), (1, 17, 33), (5, 31, 65)])
+def test_dssim_tiles(shape):
+    from oracle import gsplat as G
+    g = np.random.default_rng(11)
+    a = g.random(shape).astype(np.float32)
+    b = np.clip(a + 0.1 * g.standard_normal(shape), 0, 1).astype(np.float32)
+    ref_loss, ref_g = G.dssim_loss(a, b)
+    loss, grad = torch.zeros(1, device="cuda"), torch.zeros(shape, device="cuda")
+    B.image_dssim_loss(to_dev(a), to_dev(b), loss, 2.0, grad)
+    assert loss.item() == pytest.approx(2.0 * ref_loss, rel=1e-4)
+    assert rel_l2(grad.cpu().numpy(), 2.0 * ref_g) <= 1e-4
+    l2 = torch.zeros(1, device="cuda")
+    B.image_dssim_loss(to_dev(a), to_dev(b), l2, 2.0)
+    assert abs(l2.item() - loss.item()) <= 1e-6  # the block sums' order: 4 ulp of the weight

@@ -59,19 +59,26 @@ struct SurrHandle {
 
 // ------------------------------------------------------------- kernels ----
 
+// The four layers' places in the parameter and operand arrays.
+struct SurrLayers {
+    int64_t off_w[4], woff[4];
+    int cin[4], cout[4];
+};
+
 // BF16 copies of the layer weights in the tensor-core operand layout
 // [9 (dy, dx)][cin/8][3 (dz)][cout][8] (core matrices of 8 output channels x 8
 // input channels; the three dz taps of one (dx, dy) form one operand): wf for
 // the forward convolution, wd for the input gradient (taps mirrored, input
-// and output channels swapped).
+// and output channels swapped). Row y of the grid takes layer y: one launch
+// instead of four of 3 us.
 __global__ void k_surr_weights(const float *__restrict__ params, bf16 *__restrict__ wf,
-                               bf16 *__restrict__ wd, int64_t off_w, int64_t woff, int cin,
-                               int cout) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t cnt = 27LL * cin * cout;
-    if (i >= cnt) return;
-    const int ci = (int)(i % cin), co = (int)((i / cin) % cout), t = (int)(i / ((int64_t)cin * cout));
-    const bf16 w = __float2bfloat16_rn(params[off_w + i]);
+                               bf16 *__restrict__ wd, SurrLayers L) {
+    const int l = blockIdx.y, cin = L.cin[l], cout = L.cout[l];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 27 * cin * cout) return;
+    const int64_t woff = L.woff[l];
+    const int ci = i % cin, co = (i / cin) % cout, t = i / (cin * cout);
+    const bf16 w = __float2bfloat16_rn(params[L.off_w[l] + i]);
     const int t2 = 26 - t;  // tap of the input-gradient convolution
     wf[woff + ((((int64_t)(t % 9) * (cin / 8) + ci / 8) * 3 + t / 9) * cout + co) * 8 + (ci & 7)] = w;
     wd[woff + ((((int64_t)(t2 % 9) * (cout / 8) + co / 8) * 3 + t2 / 9) * cin + ci) * 8 + (co & 7)] = w;
@@ -182,56 +189,102 @@ __global__ void k_planar_to_cl16(const bf16 *__restrict__ src, bf16 *__restrict_
     reinterpret_cast<uint4 *>(dst)[v * 2 + c] = reinterpret_cast<const uint4 *>(src)[i];
 }
 
+// Sum of v over a block of 256 threads, valid in thread 0.
+template <typename T>
+__device__ __forceinline__ T block_sum256(T v) {
+    __shared__ T red[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    T s = 0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < 8; ++w) s += red[w];
+    return s;
+}
+
 // Mean squared error over the coarse voxels that are not fully solid, on
-// channels 0..2: L = sum (out - target)^2 / (3 count); g4 = dL/d(out).
-__global__ void k_surr_loss(const float *__restrict__ out, const float *__restrict__ target,
-                            const bf16 *__restrict__ feats, int64_t nv, const int *__restrict__ count,
-                            bf16 *__restrict__ g4, float *__restrict__ loss) {
+// channels 0..2: L = sum (out - target)^2 / (3 count); g4 = dL/d(out). out4
+// holds channels 0..3 of the output. One loss atomic per block, as in the count
+// below: one per warp, 8,192 atomics on one address, took 14 us of 18.
+__global__ void __launch_bounds__(256) k_surr_loss(const float4 *__restrict__ out4,
+                                                   const float *__restrict__ target,
+                                                   const bf16 *__restrict__ feats, int64_t nv,
+                                                   const int *__restrict__ count,
+                                                   bf16 *__restrict__ g4, float *__restrict__ loss) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float inv_norm = 1.0f / (3.0f * (float)max(*count, 1));
     float l = 0.0f;
     if (v < nv) {
         const bool fluid = __bfloat162float(feats[v * 8 + 4]) < 1.0f;  // solid fraction, plane 0
-        __align__(16) bf16 g[16];
+        const float4 a = out4[v], b = *reinterpret_cast<const float4 *>(target + v * 16);
+        __align__(16) bf16 g[8];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) g[c] = __float2bfloat16_rn(0.0f);
+        for (int c = 0; c < 8; ++c) g[c] = __float2bfloat16_rn(0.0f);
         if (fluid) {
+            const float d[3] = {a.x - b.x, a.y - b.y, a.z - b.z};
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float d = out[v * 16 + c] - target[v * 16 + c];
-                l += d * d;
-                g[c] = __float2bfloat16_rn(2.0f * d * inv_norm);
+                l += d[c] * d[c];
+                g[c] = __float2bfloat16_rn(2.0f * d[c] * inv_norm);
             }
         }
         reinterpret_cast<uint4 *>(g4)[v] = reinterpret_cast<const uint4 *>(g)[0];
-        reinterpret_cast<uint4 *>(g4)[nv + v] = reinterpret_cast<const uint4 *>(g)[1];
+        reinterpret_cast<uint4 *>(g4)[nv + v] = make_uint4(0u, 0u, 0u, 0u);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l * inv_norm);
+    l = block_sum256(l);
+    if (threadIdx.x == 0 && loss) atomicAdd(loss, l * inv_norm);
 }
 
-__global__ void k_count_fluid(const bf16 *__restrict__ feats, int64_t nv, int *__restrict__ count) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int c = (v < nv && __bfloat162float(feats[v * 8 + 4]) < 1.0f) ? 1 : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
+__global__ void __launch_bounds__(256) k_count_fluid(const bf16 *__restrict__ feats, int64_t nv,
+                                                     int *__restrict__ count) {
+    int c = 0;
+    for (int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x; v < nv; v += (int64_t)gridDim.x * 256)
+        c += __bfloat162float(feats[v * 8 + 4]) < 1.0f ? 1 : 0;
+    c = block_sum256(c);
+    if (threadIdx.x == 0 && c) atomicAdd(count, c);
 }
 
-__global__ void k_wgrad_reduce(const float *__restrict__ part, const float *__restrict__ part_b,
-                               int nchunks, int64_t nw, int cout, float *__restrict__ gw,
-                               float *__restrict__ gb) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nw) {
-        float s = 0.0f;
-        for (int c = 0; c < nchunks; ++c) s += part[(size_t)c * nw + i];
-        gw[i] += s;
-    } else if (i < nw + cout) {
-        const int co = (int)(i - nw);
-        float s = 0.0f;
-        for (int c = 0; c < nchunks; ++c) s += part_b[(size_t)c * cout + co];
-        gb[co] += s;
+// gw += the sum over nchunks CTAs' partial weight gradients, gb += that over
+// nchunks_b CTAs' partial bias gradients (the last block). 64 threads of a row
+// take four neighbouring weights each, the block's eight rows a share of the
+// chunks each: with one thread walking all 152 chunks of a weight, 108 blocks
+// kept too few loads in flight (16 us per 32 -> 32 layer, 17 MB).
+constexpr int WR_ROWS = 8;
+__global__ void __launch_bounds__(64 * WR_ROWS) k_wgrad_reduce(
+    const float *__restrict__ part, const float *__restrict__ part_b, int nchunks, int nchunks_b,
+    int64_t nw, int cout, float *__restrict__ gw, float *__restrict__ gb) {
+    __shared__ float4 sum[WR_ROWS][64];
+    const bool bias = blockIdx.x + 1 == gridDim.x;
+    const int64_t len = bias ? cout : nw, i = (bias ? 0 : (int64_t)blockIdx.x * 256) + threadIdx.x * 4;
+    const float *src = bias ? part_b : part;
+    const int n = bias ? nchunks_b : nchunks;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < len) {
+#pragma unroll 4
+        for (int c = threadIdx.y; c < n; c += WR_ROWS) {
+            const float4 p = *reinterpret_cast<const float4 *>(src + (size_t)c * len + i);
+            s.x += p.x;
+            s.y += p.y;
+            s.z += p.z;
+            s.w += p.w;
+        }
+    }
+    sum[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && i < len) {
+        for (int r = 1; r < WR_ROWS; ++r) {
+            const float4 p = sum[r][threadIdx.x];
+            s.x += p.x;
+            s.y += p.y;
+            s.z += p.z;
+            s.w += p.w;
+        }
+        float *d = (bias ? gb : gw) + i;
+        d[0] += s.x;
+        d[1] += s.y;
+        d[2] += s.z;
+        d[3] += s.w;
     }
 }
 
@@ -644,6 +697,12 @@ static dw_status make_wgrad_maps(CUtensorMap *tm_in, CUtensorMap *tm_g, const bf
     return st;
 }
 
+static void launch_wgrad_reduce(SurrHandle *h, int nchunks, int nchunks_b, int64_t nw, int cout,
+                                float *gw, float *gb, cudaStream_t s) {
+    k_wgrad_reduce<<<grid_for(nw, 256) + 1, dim3(64, WR_ROWS), 0, s>>>(
+        h->part, h->part_b, nchunks, nchunks_b, nw, cout, gw, gb);
+}
+
 // Weight and bias gradients of one layer on tcgen05: gw += dW, gb += db.
 template <int CIN, int COUT>
 static dw_status wgrad_tc(SurrHandle *h, const CUtensorMap &tm_in, const CUtensorMap &tm_g,
@@ -659,10 +718,10 @@ static dw_status wgrad_tc(SurrHandle *h, const CUtensorMap &tm_in, const CUtenso
     const int grid = std::min(std::min(h->sms, h->part_chunks), ntiles);
     k_wgrad_tc<CIN, COUT><<<grid, WG_THREADS, smem, s>>>(tm_in, tm_g, h->n, h->part, h->err);
     DW_LAUNCHED("k_wgrad_tc");
-    k_bias_grad<COUT><<<grid, 256, 0, s>>>(g, h->nv, h->part_b);
+    const int gridb = h->part_chunks;
+    k_bias_grad<COUT><<<gridb, 256, 0, s>>>(g, h->nv, h->part_b);
     DW_LAUNCHED("k_bias_grad");
-    const int64_t nw = 27LL * CIN * COUT;
-    k_wgrad_reduce<<<grid_for(nw + COUT, 256), 256, 0, s>>>(h->part, h->part_b, grid, nw, COUT, gw, gb);
+    launch_wgrad_reduce(h, grid, gridb, 27LL * CIN * COUT, COUT, gw, gb, s);
     DW_LAUNCHED("k_wgrad_reduce");
     return DW_OK;
 }
@@ -682,20 +741,21 @@ static dw_status wgrad(SurrHandle *h, const bf16 *in, const bf16 *g, float *gw, 
     k_wgrad<CIN, COUT><<<dim3(h->nchunks, 3), CV_THREADS, smem, s>>>(in, g, h->n, h->tiles_per_chunk,
                                                                      h->part, h->part_b);
     DW_LAUNCHED("k_wgrad");
-    const int64_t nw = 27LL * CIN * COUT;
-    k_wgrad_reduce<<<grid_for(nw + COUT, 256), 256, 0, s>>>(h->part, h->part_b, h->nchunks, nw, COUT,
-                                                            gw, gb);
+    launch_wgrad_reduce(h, h->nchunks, h->nchunks, 27LL * CIN * COUT, COUT, gw, gb, s);
     DW_LAUNCHED("k_wgrad_reduce");
     return DW_OK;
 }
 
 static dw_status refresh_weights(SurrHandle *h, cudaStream_t s) {
     h->weights_dirty = true;
+    SurrLayers L;
     for (int l = 0; l < 4; ++l) {
-        const int64_t cnt = 27LL * SCH[l] * SCH[l + 1];
-        k_surr_weights<<<grid_for(cnt, 256), 256, 0, s>>>(h->params, h->wf, h->wd, h->off_w[l],
-                                                          h->woff[l], SCH[l], SCH[l + 1]);
+        L.off_w[l] = h->off_w[l];
+        L.woff[l] = h->woff[l];
+        L.cin[l] = SCH[l];
+        L.cout[l] = SCH[l + 1];
     }
+    k_surr_weights<<<dim3(grid_for(27 * 32 * 32, 256), 4), 256, 0, s>>>(h->params, h->wf, h->wd, L);
     DW_LAUNCHED("k_surr_weights");
     return DW_OK;
 }
@@ -764,7 +824,7 @@ extern "C" dw_status surr_create(int32_t n, dw_surr *out) {
     DW_ALLOC(h->out, sizeof(float) * nv * 16);
     DW_ALLOC(h->out4, sizeof(float) * nv * 4);
     DW_ALLOC(h->g4, sizeof(bf16) * nv * 16);
-    h->part_chunks = std::max(h->nchunks, h->sms);
+    h->part_chunks = std::max(h->nchunks, 2 * h->sms);
     DW_ALLOC(h->part, sizeof(float) * (size_t)h->part_chunks * 27 * 32 * 32);
     DW_ALLOC(h->part_b, sizeof(float) * (size_t)h->part_chunks * 32);
     DW_ALLOC(h->fine, sizeof(float) * 4 * Nc);
@@ -975,8 +1035,10 @@ extern "C" dw_status surr_loss(dw_surr h, const float *target, float *loss, dw_s
     cudaStream_t s = as_stream(stream);
     int *cnt = reinterpret_cast<int *>(h->red);
     DW_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int), s));
-    k_count_fluid<<<grid_for(h->nv, 256), 256, 0, s>>>(h->feats, h->nv, cnt);
-    k_surr_loss<<<grid_for(h->nv, 256), 256, 0, s>>>(h->out, target, h->feats, h->nv, cnt, h->g4, loss);
+    const unsigned blocks = grid_for(h->nv, 256);
+    k_count_fluid<<<std::min(blocks, 304u), 256, 0, s>>>(h->feats, h->nv, cnt);
+    k_surr_loss<<<blocks, 256, 0, s>>>(reinterpret_cast<const float4 *>(h->out4), target, h->feats, h->nv,
+                                       cnt, h->g4, loss);
     DW_LAUNCHED("k_surr_loss");
     return DW_OK;
 }

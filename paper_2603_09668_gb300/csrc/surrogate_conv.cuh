@@ -92,6 +92,33 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
     return fmaf(0.5f * z * fmaf(-t, t, 1.0f), du, 0.5f * (1.0f + t));
 }
 
+// Two values at once on the paired FP32 instructions, each operation rounded as
+// in gelu_f and gelu_grad_f (the results are the same bits).
+__device__ __forceinline__ float2 pair2(float a) { return make_float2(a, a); }
+
+__device__ __forceinline__ float2 gelu2_f(float2 z) {
+    const float2 u = __fmul2_rn(z, __ffma2_rn(pair2(GELU_A * GELU_C), __fmul2_rn(z, z), pair2(GELU_C)));
+    const float2 t = make_float2(tanh_approx(u.x), tanh_approx(u.y));
+    const float2 hz = __fmul2_rn(pair2(0.5f), z);
+    return __ffma2_rn(hz, t, hz);
+}
+
+__device__ __forceinline__ float2 gelu2_grad_f(float2 z) {
+    const float2 z2 = __fmul2_rn(z, z);
+    const float2 u = __fmul2_rn(z, __ffma2_rn(pair2(GELU_A * GELU_C), z2, pair2(GELU_C)));
+    const float2 t = make_float2(tanh_approx(u.x), tanh_approx(u.y));
+    const float2 du = __ffma2_rn(pair2(3.0f * GELU_A * GELU_C), z2, pair2(GELU_C));
+    const float2 s = __ffma2_rn(make_float2(-t.x, -t.y), t, pair2(1.0f));
+    return __ffma2_rn(__fmul2_rn(__fmul2_rn(pair2(0.5f), z), s), du,
+                      __fmul2_rn(pair2(0.5f), __fadd2_rn(pair2(1.0f), t)));
+}
+
+// Two floats rounded to BF16, a in the low half.
+__device__ __forceinline__ uint32_t bf16_pair(float2 a) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(a.x, a.y);
+    return *reinterpret_cast<const uint32_t *>(&b);
+}
+
 // Loads the 18 x 10 x 3 input halo of the tile at (x0, y0, z0) into smem.
 template <int C>
 __device__ __forceinline__ void load_halo(const bf16 *__restrict__ in, int n, int x0, int y0,

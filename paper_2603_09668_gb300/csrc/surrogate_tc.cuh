@@ -103,27 +103,29 @@ __device__ __forceinline__ void tc_ld<16>(uint32_t taddr, float (&r)[16]) {
     for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(u[i]);
 }
 
-template <>
-__device__ __forceinline__ void tc_ld<4>(uint32_t taddr, float (&r)[4]) {
-    uint32_t u[4];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 4; ++i) r[i] = __uint_as_float(u[i]);
+// The same without the wait for the loads (tc_ld_wait), so that several are in
+// flight; N = 16 or 8 columns as pairs.
+__device__ __forceinline__ void tc_ld_pairs(uint32_t taddr, float2 (&r)[8]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+        "%15}, [%16];"
+        : "=f"(r[0].x), "=f"(r[0].y), "=f"(r[1].x), "=f"(r[1].y), "=f"(r[2].x), "=f"(r[2].y),
+          "=f"(r[3].x), "=f"(r[3].y), "=f"(r[4].x), "=f"(r[4].y), "=f"(r[5].x), "=f"(r[5].y),
+          "=f"(r[6].x), "=f"(r[6].y), "=f"(r[7].x), "=f"(r[7].y)
+        : "r"(taddr));
 }
-
-template <>
-__device__ __forceinline__ void tc_ld<8>(uint32_t taddr, float (&r)[8]) {
-    uint32_t u[8];
+__device__ __forceinline__ void tc_ld_pairs(uint32_t taddr, float2 (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]),
-                   "=r"(u[6]), "=r"(u[7])
+                 : "=f"(r[0].x), "=f"(r[0].y), "=f"(r[1].x), "=f"(r[1].y), "=f"(r[2].x),
+                   "=f"(r[2].y), "=f"(r[3].x), "=f"(r[3].y)
                  : "r"(taddr));
+}
+// Waits for them; the registers pass through so that no use moves above it.
+template <int N>
+__device__ __forceinline__ void tc_ld_wait(float2 (&r)[N]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 8; ++i) r[i] = __uint_as_float(u[i]);
+    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(r[i].x), "+f"(r[i].y));
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
@@ -333,6 +335,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
     constexpr int HBYTES = KCH * TC_SLICE;
     constexpr int WBYTES = tc_wbytes(CIN, COUT);
     constexpr int CPW = COUT / (TC_EPI_WARPS / 4);  // accumulator columns per epilogue warp
+    constexpr int CP2 = CPW / 2;                    // as pairs
     constexpr int NW = 3 * COUT;                    // MMA N: the three dz taps
     static_assert(TC_NWIN * NW <= TC_TMEM_COLS && TC_RING >= TC_NWIN + 2, "tensor memory plan");
     constexpr uint32_t IDESC = tc_idesc(NW);
@@ -427,6 +430,12 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
         const int row = q * 32 + lane;  // accumulator lane = tile voxel (x = row & 7, y = row >> 3)
         const uint32_t tq = taddr + ((uint32_t)(q * 32) << 16) + hcol * CPW;
         const size_t nv = (size_t)n * n * n;
+        float2 bias[CP2];
+        if (EPI != EPI_DGELU) {
+#pragma unroll
+            for (int cc = 0; cc < CP2; ++cc)
+                bias[cc] = make_float2(o.bias[hcol * CPW + 2 * cc], o.bias[hcol * CPW + 2 * cc + 1]);
+        }
         int k = k0;  // slices seen in this launch
         bool ok = true;
         TcSeg c;
@@ -450,22 +459,28 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                 tc_fence_after();
                 // outputs finished by slice zi: zi - 1, and zi itself at the volume's end
                 const int zlo = max(zi - 1, c.o0), zhi = (zi == n - 1) ? min(zi, c.o1) : min(zi - 1, c.o1);
-                float r[2][CPW];
+                float2 r[2][CP2];
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     const int z = zlo + m;
                     if (z > zhi) break;
+                    // block b of slice z - 1 + b; slice z - 1 and z + 1 may be missing
+                    const int ks = kb + (z - i0);
+                    float2 p0[CP2], p2[CP2];
+                    const bool lo = z - 1 >= i0, hi = z + 1 <= i1;
+                    if (lo) tc_ld_pairs(tq + (uint32_t)(((ks - 1) % TC_NWIN) * NW), p0);
+                    tc_ld_pairs(tq + (uint32_t)((ks % TC_NWIN) * NW + COUT), r[m]);
+                    if (hi) tc_ld_pairs(tq + (uint32_t)(((ks + 1) % TC_NWIN) * NW + 2 * COUT), p2);
+                    tc_ld_wait(r[m]);
+                    if (lo) {
+                        tc_ld_wait(p0);
 #pragma unroll
-                    for (int cc = 0; cc < CPW; ++cc) r[m][cc] = 0.0f;
+                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(p0[cc], r[m][cc]);
+                    }
+                    if (hi) {
+                        tc_ld_wait(p2);
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) {  // block b of slice z - 1 + b
-                        const int zs = z - 1 + b;
-                        if (zs < i0 || zs > i1) continue;
-                        const int ks = kb + (zs - i0);
-                        float part[CPW];
-                        tc_ld<CPW>(tq + (uint32_t)((ks % TC_NWIN) * NW + b * COUT), part);
-#pragma unroll
-                        for (int cc = 0; cc < CPW; ++cc) r[m][cc] += part[cc];
+                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(r[m][cc], p2[cc]);
                     }
                 }
                 tc_fence_before();
@@ -489,9 +504,9 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                     if (EPI == EPI_F32) {
 #pragma unroll
                         for (int cc = 0; cc < CPW; cc += 4) {
-                            const float4 q4 =
-                                make_float4(r[m][cc] + o.bias[c0 + cc], r[m][cc + 1] + o.bias[c0 + cc + 1],
-                                            r[m][cc + 2] + o.bias[c0 + cc + 2], r[m][cc + 3] + o.bias[c0 + cc + 3]);
+                            const float2 lo = __fadd2_rn(r[m][cc / 2], bias[cc / 2]);
+                            const float2 hi = __fadd2_rn(r[m][cc / 2 + 1], bias[cc / 2 + 1]);
+                            const float4 q4 = make_float4(lo.x, lo.y, hi.x, hi.y);
                             *reinterpret_cast<float4 *>(o.out_f + v * COUT + c0 + cc) = q4;
                             if (cc == 0 && c0 == 0 && o.out_f4) reinterpret_cast<float4 *>(o.out_f4)[v] = q4;
                         }
@@ -499,26 +514,29 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
 #pragma unroll
                         for (int cc = 0; cc < CPW; cc += 8) {
                             const uint4 zp = *reinterpret_cast<const uint4 *>(o.zprev + plane(cc));
-                            const bf16 *zb = reinterpret_cast<const bf16 *>(&zp);
-                            __align__(16) bf16 od[8];
+                            const uint32_t zw[4] = {zp.x, zp.y, zp.z, zp.w};
+                            uint32_t od[4];
 #pragma unroll
-                            for (int jj = 0; jj < 8; ++jj)
-                                od[jj] = __float2bfloat16_rn(r[m][cc + jj] * gelu_grad_f(__bfloat162float(zb[jj])));
-                            *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = *reinterpret_cast<const uint4 *>(od);
+                            for (int jj = 0; jj < 4; ++jj) {
+                                const float2 zz = make_float2(__uint_as_float(zw[jj] << 16),
+                                                              __uint_as_float(zw[jj] & 0xffff0000u));
+                                od[jj] = bf16_pair(__fmul2_rn(r[m][cc / 2 + jj], gelu2_grad_f(zz)));
+                            }
+                            *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = make_uint4(od[0], od[1], od[2], od[3]);
                         }
                     } else {
 #pragma unroll
                         for (int cc = 0; cc < CPW; cc += 8) {
-                            __align__(16) bf16 oz[8], oa[8];
+                            uint32_t oz[4], oa[4];
 #pragma unroll
-                            for (int jj = 0; jj < 8; ++jj) {
-                                const float zz = r[m][cc + jj] + o.bias[c0 + cc + jj];
-                                oz[jj] = __float2bfloat16_rn(zz);
-                                oa[jj] = __float2bfloat16_rn(gelu_f(zz));
+                            for (int jj = 0; jj < 4; ++jj) {
+                                const float2 zz = __fadd2_rn(r[m][cc / 2 + jj], bias[cc / 2 + jj]);
+                                if (EPI == EPI_GELU) oz[jj] = bf16_pair(zz);
+                                oa[jj] = bf16_pair(gelu2_f(zz));
                             }
                             if (EPI == EPI_GELU)
-                                *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = *reinterpret_cast<const uint4 *>(oz);
-                            *reinterpret_cast<uint4 *>(o.out_a + plane(cc)) = *reinterpret_cast<const uint4 *>(oa);
+                                *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = make_uint4(oz[0], oz[1], oz[2], oz[3]);
+                            *reinterpret_cast<uint4 *>(o.out_a + plane(cc)) = make_uint4(oa[0], oa[1], oa[2], oa[3]);
                         }
                     }
                 }

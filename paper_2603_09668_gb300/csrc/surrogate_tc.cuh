@@ -67,10 +67,12 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity,
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
-        if ((it & 255u) == 0) {
+        // the clock is read only once a wait has lasted a while: reading it costs
+        // far more than a poll
+        if ((it & 255u) == 255u) {
             if (abort && *abort) return false;
             const uint64_t t = globaltimer_ns();
-            if (it == 0) t0 = t;
+            if (t0 == 0) t0 = t;
             else if (t - t0 > 1000000000ull) return false;
         }
     }
@@ -142,9 +144,11 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 }
 
 constexpr int TC_NST = 8;        // halo stages (one input slice each)
-constexpr int TC_LAG = 3;        // a stage is refilled once the MMAs of slice k - TC_LAG are done
-constexpr int TC_EPI_WARPS = 8;  // epilogue warps: lane quarter = warp & 3, column half = warp >> 2
-constexpr int TC_THREADS = 32 * (TC_EPI_WARPS + 1);  // + one producer / MMA warp
+// Epilogue warps: lane quarter = warp & 3, column half = (warp >> 2) & 1, and
+// warps 0-7 take the even output slices, 8-15 the odd ones.
+constexpr int TC_EPI_WARPS = 16;
+constexpr int TC_MMA_WARP = TC_EPI_WARPS, TC_LOAD_WARP = TC_EPI_WARPS + 1;
+constexpr int TC_THREADS = 32 * (TC_EPI_WARPS + 2);  // + the MMA warp and the loader warp
 constexpr int TC_TMEM_COLS = 512;                     // the whole tensor memory of the SM
 constexpr int TC_NWIN = 5;       // accumulator windows (one input slice each)
 constexpr int TC_RING = 8;       // slice-ready barrier ring (>= TC_NWIN + 2)
@@ -217,12 +221,25 @@ __device__ __forceinline__ bool tc_segment(int n, int nxy, int j, TcSeg &c) {
 // three blocks. Windows never overlap, so the MMAs of consecutive slices do
 // not wait on each other's accumulators.
 //
-// Roles: warp 8, lane 0 issues the weight copies, the halo loads (ring of
-// TC_NST slices) and the MMAs, committing each slice to ready[k % TC_RING];
-// warps 0-7 read the finished output slices (warp w: accumulator lanes
-// 32 (w % 4) .. + 31, column half w / 4) and arrive on wfree[w] once no
-// output needs window w any more, which the producer waits for before
-// reusing it.
+// Roles: warp 17, lane 0 (the loader) issues the weight copies and the halo
+// loads (ring of TC_NST slices, each refilled once its MMAs are done); warp 16,
+// lane 0 issues the MMAs, committing each slice to empty[k % TC_NST] and
+// ready[k % TC_RING]; warps 0-15 read the finished output slices, the even
+// ones warps 0-7, the odd ones warps 8-15 (warp w: accumulator lanes
+// 32 (w % 4) .. + 31, column half (w / 4) % 2), and all of them arrive on
+// wfree[w] once no output needs window w any more, which the MMA thread waits
+// for before reusing it. A slice's epilogue (barrier, tensor-memory loads,
+// GELU, stores) takes its warps about 1,400 cycles, mostly latency, so two
+// sets take turns.
+//
+// The MMA thread's issue stalls at the tensor pipe's pace with only a few
+// MMAs queued, so whatever else it does between two slices leaves the pipe
+// idle: with the loads and their waits on the same thread, and the next
+// slice's waits after the last MMA, a 32 -> 32 slice took about 1,900 cycles
+// against the 1,008 of its 18 MMAs (64^3; with the MMAs left out the waits
+// alone took 800; a quarter of the halo bytes changed nothing). So the loads
+// have a warp of their own, and the next slice's barriers are waited for
+// after two thirds of a slice's MMAs, when they have normally completed.
 
 // The pipeline's shared-memory state, kept across the layers of one launch:
 // the slice counter k runs on from layer to layer, so every mbarrier phase
@@ -231,7 +248,7 @@ struct TcPipe {
     uint64_t full[TC_NST], empty[TC_NST], ready[TC_RING], wfree[TC_NWIN];
     uint64_t wbar[2];  // weight buffers
     uint32_t wbuf[2];  // their shared-memory addresses
-    int wcount[2];     // copies issued into each buffer (producer thread only)
+    int wcount[2];     // copies issued into each buffer (loader thread only)
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -250,7 +267,7 @@ struct TcOut {
     float *out_f4;
 };
 
-// What the producer does before the layer's first halo load.
+// What the loader does before the layer's first halo load.
 enum { TC_PRO_NONE = 0, TC_PRO_PDL = 1, TC_PRO_PROXY = 2 };
 
 // Barrier init and the TMEM allocation (all threads).
@@ -280,11 +297,11 @@ __device__ __forceinline__ uint32_t tc_pipe_open(TcPipe &pp) {
     return pp.tmem_base;
 }
 
-// All threads: the TMEM release at the end; before it the producer waits
+// All threads: the TMEM release at the end; before it the loader waits
 // (bounded) for the last weight copy into each buffer, which an abort may
 // have left in flight.
 __device__ __forceinline__ void tc_pipe_close(TcPipe &pp, uint32_t taddr) {
-    if (threadIdx.x == 32 * TC_EPI_WARPS)
+    if (threadIdx.x == 32 * TC_LOAD_WARP)
         for (int b = 0; b < 2; ++b)
             if (pp.wcount[b] > 0) tc_wait(smem_u32(&pp.wbar[b]), (pp.wcount[b] - 1) & 1, nullptr);
     tc_fence_before();
@@ -296,7 +313,7 @@ __device__ __forceinline__ void tc_pipe_close(TcPipe &pp, uint32_t taddr) {
     }
 }
 
-// One bulk copy of a layer's weights into weight buffer b (producer thread).
+// One bulk copy of a layer's weights into weight buffer b (loader thread).
 __device__ __forceinline__ void tc_copy_weights(TcPipe &pp, int b, const bf16 *wt, uint32_t bytes) {
     const uint32_t bar = smem_u32(&pp.wbar[b]);
     ++pp.wcount[b];
@@ -317,8 +334,8 @@ __device__ __forceinline__ int tc_slices(int n, int nxy) {
 }
 
 // One layer over the CTA's output range, called by all threads. Weight
-// buffer wb holds (or receives) this layer's weights: own_wt, when not NULL,
-// is copied there first by the producer. next_wt, when not NULL, is copied
+// buffer wb holds (or receives) this layer's weights, as its wuse-th use
+// (from 0): own_wt, when not NULL, is copied there first by the loader. next_wt, when not NULL, is copied
 // into the other buffer at the start, the prefetch of the following layer's
 // weights (that buffer's previous layer has finished). k0 counts the slices
 // this CTA has gone through in earlier layers of the launch. fence_out: the
@@ -326,7 +343,7 @@ __device__ __forceinline__ int tc_slices(int n, int nxy) {
 // CTAs after a grid barrier see it.
 template <int CIN, int COUT, int EPI>
 __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUtensorMap *tm_in,
-                                         const TcOut &o, int n, uint32_t hbase, int wb,
+                                         const TcOut &o, int n, uint32_t hbase, int wb, int wuse,
                                          const bf16 *own_wt, const bf16 *next_wt,
                                          uint32_t next_bytes, int k0, int prologue,
                                          bool fence_out, int *err) {
@@ -334,7 +351,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
     constexpr int KCH = CIN / 8;
     constexpr int HBYTES = KCH * TC_SLICE;
     constexpr int WBYTES = tc_wbytes(CIN, COUT);
-    constexpr int CPW = COUT / (TC_EPI_WARPS / 4);  // accumulator columns per epilogue warp
+    constexpr int CPW = COUT / 2;                   // accumulator columns per epilogue warp
     constexpr int CP2 = CPW / 2;                    // as pairs
     constexpr int NW = 3 * COUT;                    // MMA N: the three dz taps
     static_assert(TC_NWIN * NW <= TC_TMEM_COLS && TC_RING >= TC_NWIN + 2, "tensor memory plan");
@@ -344,89 +361,89 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
     const int tiles_x = n / TC_TX, nxy = tiles_x * (n / TC_TY);
     if (pp.abort_flag) return;  // an earlier layer gave up
 
-    if (warp == TC_EPI_WARPS) {
+    if (warp == TC_LOAD_WARP) {
         if (lane == 0) {
-            int issued = k0, consumed = k0;  // slices
-            bool ok = true;
-            // the slices of all segments in order, for the halo prefetch
-            int pf_seg = 0, pf_z = 0;
-            TcSeg pfc;
-            bool pf_more = tc_segment(n, nxy, 0, pfc);
-            if (pf_more) pf_z = max(pfc.o0 - 1, 0);
-            auto prefetch = [&]() {
-                if (!pf_more) return;
-                const int s = issued % TC_NST;
-                tc_load_slice<CIN>(tm_in, hbase + s * HBYTES, smem_u32(&pp.full[s]),
-                                   (pfc.xy % tiles_x) * TC_TX, (pfc.xy / tiles_x) * TC_TY, pf_z);
-                ++issued;
-                if (pf_z < min(pfc.o1 + 1, n - 1)) {
-                    ++pf_z;
-                } else {
-                    pf_more = tc_segment(n, nxy, ++pf_seg, pfc);
-                    if (pf_more) pf_z = max(pfc.o0 - 1, 0);
-                }
-            };
             if (own_wt) tc_copy_weights(pp, wb, own_wt, WBYTES);
             if (next_wt) tc_copy_weights(pp, 1 - wb, next_wt, next_bytes);
-            const uint32_t wbase = pp.wbuf[wb];
             if (prologue == TC_PRO_PDL) pdl_wait();
             if (prologue == TC_PRO_PROXY) asm volatile("fence.proxy.async.global;" ::: "memory");
-            while (issued - k0 < TC_NST && pf_more) prefetch();
-            ok = tc_wait(smem_u32(&pp.wbar[wb]), (pp.wcount[wb] - 1) & 1, abort_p);
-            const uint64_t b0 = tc_desc(wbase, NW * 16, 128);
+            int k = k0;
+            bool ok = true;
             TcSeg c;
             for (int j = 0; ok && tc_segment(n, nxy, j, c); ++j) {
                 const int i0 = max(c.o0 - 1, 0), i1 = min(c.o1 + 1, n - 1);
-                for (int zi = i0; zi <= i1; ++zi) {
-                    const int k = consumed, s = k % TC_NST, w = k % TC_NWIN;
-                    ok = tc_wait(smem_u32(&pp.full[s]), (k / TC_NST) & 1, abort_p) &&
-                         tc_wait(smem_u32(&pp.wfree[w]), ((k / TC_NWIN) & 1) ^ 1, abort_p);
-                    if (!ok) break;
-                    ++consumed;
-                    tc_fence_after();
-                    const uint32_t d = taddr + (uint32_t)(w * NW);
-                    const uint64_t a0 = tc_desc(hbase + s * HBYTES, TC_SLICE, TC_HX * 16);
-#pragma unroll
-                    for (int t = 0; t < 9; ++t) {
-                        const int dx = t % 3, dy = t / 3;  // offsets + 1
-#pragma unroll
-                        for (int kk = 0; kk < KCH / 2; ++kk) {
-                            const uint32_t a_off = (dy * TC_HX + dx) * 16 + 2 * kk * TC_SLICE;
-                            const uint32_t b_off = ((t * KCH + 2 * kk) * NW) * 16;
-                            const uint64_t ad = a0 + (a_off >> 4);
-                            const uint64_t bd = b0 + (b_off >> 4);
-                            const uint32_t acc = (t | kk) != 0;  // a fresh window per slice
-                            asm volatile(
-                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                :: "r"(d), "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
-                                : "memory");
-                        }
-                    }
-                    tc_commit(smem_u32(&pp.empty[s]));
-                    tc_commit(smem_u32(&pp.ready[k % TC_RING]));
-                    // refill the stage of slice k - TC_LAG once its MMAs are done
-                    if (k - k0 >= TC_LAG && pf_more) {
-                        const int k1 = k - TC_LAG;
-                        ok = tc_wait(smem_u32(&pp.empty[k1 % TC_NST]), (k1 / TC_NST) & 1, abort_p);
+                const int x0 = (c.xy % tiles_x) * TC_TX, y0 = (c.xy / tiles_x) * TC_TY;
+                for (int zi = i0; zi <= i1; ++zi, ++k) {
+                    const int s = k % TC_NST;
+                    if (k - k0 >= TC_NST) {  // (the stages of earlier layers are all done)
+                        ok = tc_wait(smem_u32(&pp.empty[s]), (k / TC_NST - 1) & 1, abort_p);
                         if (!ok) break;
-                        prefetch();
                     }
+                    tc_load_slice<CIN>(tm_in, hbase + s * HBYTES, smem_u32(&pp.full[s]), x0, y0, zi);
                 }
             }
             if (!ok) {
                 if (!pp.abort_flag) atomicOr(err, ERRBIT_TIMEOUT);
                 pp.abort_flag = 1;
             }
-            // drain (bounded): halo loads still in flight, the last MMA batch
-            for (int k = consumed; k < issued; ++k)
-                tc_wait(smem_u32(&pp.full[k % TC_NST]), (k / TC_NST) & 1, nullptr);
-            if (consumed > k0)
-                tc_wait(smem_u32(&pp.empty[(consumed - 1) % TC_NST]), ((consumed - 1) / TC_NST) & 1, nullptr);
+            // drain (bounded): the last loads of every stage
+            for (int i = max(k0, k - TC_NST); i < k; ++i)
+                tc_wait(smem_u32(&pp.full[i % TC_NST]), (i / TC_NST) & 1, nullptr);
+        }
+        __syncwarp();
+    } else if (warp == TC_MMA_WARP) {
+        if (lane == 0) {
+            const int total = tc_slices(n, nxy);
+            auto slice_ready = [&](int k) {
+                return tc_wait(smem_u32(&pp.full[k % TC_NST]), (k / TC_NST) & 1, abort_p) &&
+                       tc_wait(smem_u32(&pp.wfree[k % TC_NWIN]), ((k / TC_NWIN) & 1) ^ 1, abort_p);
+            };
+            const uint64_t b0 = tc_desc(pp.wbuf[wb], NW * 16, 128);
+            // (a CTA without output slices has nothing to wait for)
+            bool ok = total == 0 || (tc_wait(smem_u32(&pp.wbar[wb]), wuse & 1, abort_p) && slice_ready(k0));
+            int k = k0;
+            for (; ok && k < k0 + total; ++k) {
+                const int s = k % TC_NST;
+                tc_fence_after();
+                const uint32_t d = taddr + (uint32_t)((k % TC_NWIN) * NW);
+                const uint64_t a0 = tc_desc(hbase + s * HBYTES, TC_SLICE, TC_HX * 16);
+                auto mma = [&](int t, int kk) {
+                    const int dx = t % 3, dy = t / 3;  // offsets + 1
+                    const uint32_t a_off = (dy * TC_HX + dx) * 16 + 2 * kk * TC_SLICE;
+                    const uint32_t b_off = ((t * KCH + 2 * kk) * NW) * 16;
+                    const uint64_t ad = a0 + (a_off >> 4);
+                    const uint64_t bd = b0 + (b_off >> 4);
+                    const uint32_t acc = (t | kk) != 0;  // a fresh window per slice
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                        :: "r"(d), "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
+                        : "memory");
+                };
+#pragma unroll
+                for (int t = 0; t < 6; ++t)
+#pragma unroll
+                    for (int kk = 0; kk < KCH / 2; ++kk) mma(t, kk);
+                // the next slice's barriers depend on slices up to k - 2 and on the loader only
+                const bool next = k + 1 == k0 + total || slice_ready(k + 1);
+#pragma unroll
+                for (int t = 6; t < 9; ++t)
+#pragma unroll
+                    for (int kk = 0; kk < KCH / 2; ++kk) mma(t, kk);
+                tc_commit(smem_u32(&pp.empty[s]));
+                tc_commit(smem_u32(&pp.ready[k % TC_RING]));
+                ok = next;
+            }
+            if (!ok) {
+                if (!pp.abort_flag) atomicOr(err, ERRBIT_TIMEOUT);
+                pp.abort_flag = 1;
+            }
+            // drain (bounded): the last MMA batch
+            if (k > k0) tc_wait(smem_u32(&pp.empty[(k - 1) % TC_NST]), ((k - 1) / TC_NST) & 1, nullptr);
         }
         __syncwarp();
     } else {
-        const int q = warp & 3, hcol = warp >> 2;
+        const int q = warp & 3, hcol = (warp >> 2) & 1, odd = warp >> 3;
         const int row = q * 32 + lane;  // accumulator lane = tile voxel (x = row & 7, y = row >> 3)
         const uint32_t tq = taddr + ((uint32_t)(q * 32) << 16) + hcol * CPW;
         const size_t nv = (size_t)n * n * n;
@@ -457,30 +474,30 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                     break;
                 }
                 tc_fence_after();
-                // outputs finished by slice zi: zi - 1, and zi itself at the volume's end
-                const int zlo = max(zi - 1, c.o0), zhi = (zi == n - 1) ? min(zi, c.o1) : min(zi - 1, c.o1);
-                float2 r[2][CP2];
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const int z = zlo + m;
-                    if (z > zhi) break;
+                // outputs finished by slice zi: zi - 1, and zi itself at the volume's
+                // end; at most one of them is this warp's
+                const int zhi = (zi == n - 1) ? min(zi, c.o1) : min(zi - 1, c.o1);
+                const int z = (zhi & 1) == odd ? zhi : zhi - 1;
+                const bool mine = z >= max(zi - 1, c.o0);
+                float2 r[CP2];
+                if (mine) {
                     // block b of slice z - 1 + b; slice z - 1 and z + 1 may be missing
                     const int ks = kb + (z - i0);
                     float2 p0[CP2], p2[CP2];
                     const bool lo = z - 1 >= i0, hi = z + 1 <= i1;
                     if (lo) tc_ld_pairs(tq + (uint32_t)(((ks - 1) % TC_NWIN) * NW), p0);
-                    tc_ld_pairs(tq + (uint32_t)((ks % TC_NWIN) * NW + COUT), r[m]);
+                    tc_ld_pairs(tq + (uint32_t)((ks % TC_NWIN) * NW + COUT), r);
                     if (hi) tc_ld_pairs(tq + (uint32_t)(((ks + 1) % TC_NWIN) * NW + 2 * COUT), p2);
-                    tc_ld_wait(r[m]);
+                    tc_ld_wait(r);
                     if (lo) {
                         tc_ld_wait(p0);
 #pragma unroll
-                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(p0[cc], r[m][cc]);
+                        for (int cc = 0; cc < CP2; ++cc) r[cc] = __fadd2_rn(p0[cc], r[cc]);
                     }
                     if (hi) {
                         tc_ld_wait(p2);
 #pragma unroll
-                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(r[m][cc], p2[cc]);
+                        for (int cc = 0; cc < CP2; ++cc) r[cc] = __fadd2_rn(r[cc], p2[cc]);
                     }
                 }
                 tc_fence_before();
@@ -494,18 +511,15 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                         mbar_arrive(smem_u32(&pp.wfree[k % TC_NWIN]));
                     }
                 }
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    if (zlo + m > zhi) break;
-                    const int z = zlo + m;
+                if (mine) {
                     const size_t v = ((size_t)z * n + (y0 + (row >> 3))) * n + x0 + (row & 7);
                     const int c0 = hcol * CPW;
                     auto plane = [&](int cc) { return ((size_t)((c0 + cc) >> 3) * nv + v) * 8; };
                     if (EPI == EPI_F32) {
 #pragma unroll
                         for (int cc = 0; cc < CPW; cc += 4) {
-                            const float2 lo = __fadd2_rn(r[m][cc / 2], bias[cc / 2]);
-                            const float2 hi = __fadd2_rn(r[m][cc / 2 + 1], bias[cc / 2 + 1]);
+                            const float2 lo = __fadd2_rn(r[cc / 2], bias[cc / 2]);
+                            const float2 hi = __fadd2_rn(r[cc / 2 + 1], bias[cc / 2 + 1]);
                             const float4 q4 = make_float4(lo.x, lo.y, hi.x, hi.y);
                             *reinterpret_cast<float4 *>(o.out_f + v * COUT + c0 + cc) = q4;
                             if (cc == 0 && c0 == 0 && o.out_f4) reinterpret_cast<float4 *>(o.out_f4)[v] = q4;
@@ -520,7 +534,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                             for (int jj = 0; jj < 4; ++jj) {
                                 const float2 zz = make_float2(__uint_as_float(zw[jj] << 16),
                                                               __uint_as_float(zw[jj] & 0xffff0000u));
-                                od[jj] = bf16_pair(__fmul2_rn(r[m][cc / 2 + jj], gelu2_grad_f(zz)));
+                                od[jj] = bf16_pair(__fmul2_rn(r[cc / 2 + jj], gelu2_grad_f(zz)));
                             }
                             *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = make_uint4(od[0], od[1], od[2], od[3]);
                         }
@@ -530,7 +544,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                             uint32_t oz[4], oa[4];
 #pragma unroll
                             for (int jj = 0; jj < 4; ++jj) {
-                                const float2 zz = __fadd2_rn(r[m][cc / 2 + jj], bias[cc / 2 + jj]);
+                                const float2 zz = __fadd2_rn(r[cc / 2 + jj], bias[cc / 2 + jj]);
                                 if (EPI == EPI_GELU) oz[jj] = bf16_pair(zz);
                                 oa[jj] = bf16_pair(gelu2_f(zz));
                             }
@@ -565,7 +579,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(
     // griddepcontrol.wait, the weights (written before the first layer) before.
     pdl_trigger();
     const TcOut o = {bias, out_z, out_a, out_f, zprev, out_f4};
-    tc_layer<CIN, COUT, EPI>(pp, taddr, &tm_in, o, n, hbase, 0, wt, nullptr, 0, 0, TC_PRO_PDL,
+    tc_layer<CIN, COUT, EPI>(pp, taddr, &tm_in, o, n, hbase, 0, 0, wt, nullptr, 0, 0, TC_PRO_PDL,
                              false, err);
     tc_pipe_close(pp, taddr);
 }
@@ -586,9 +600,12 @@ __device__ __forceinline__ void tc_grid_sync(unsigned *bar, int *err, TcPipe &pp
             __threadfence();
             atomicAdd(bar + 1, 1u);
         } else {
-            const uint64_t t0 = globaltimer_ns();
-            for (unsigned it = 0; *gen == g0; ++it) {
-                if ((it & 1023u) == 0 && globaltimer_ns() - t0 > 1000000000ull) {
+            uint64_t t0 = 0;
+            for (unsigned it = 1; *gen == g0; ++it) {
+                if ((it & 1023u) != 0) continue;
+                const uint64_t t = globaltimer_ns();
+                if (t0 == 0) t0 = t;
+                if (t - t0 > 1000000000ull) {
                     atomicOr(err, ERRBIT_TIMEOUT);
                     pp.abort_flag = 1;
                     break;
@@ -631,18 +648,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_surr_forward_tc(
     pdl_trigger();
     const int per = tc_slices(n, (n / TC_TX) * (n / TC_TY));
     tc_layer<16, 32, EPI_GELU_ONLY>(pp, taddr, &tm0, TcOut{b0, nullptr, a0, nullptr, nullptr, nullptr}, n,
-                                    hbase, 0, w0, w1, tc_wbytes(32, 32), 0, TC_PRO_PDL, true, err);
+                                    hbase, 0, 0, w0, w1, tc_wbytes(32, 32), 0, TC_PRO_PDL, true, err);
     tc_grid_sync(bar, err, pp);
     tc_layer<32, 32, EPI_GELU_ONLY>(pp, taddr, &tm1, TcOut{b1, nullptr, a1, nullptr, nullptr, nullptr}, n,
-                                    hbase, 1, nullptr, w2, tc_wbytes(32, 32), per, TC_PRO_PROXY,
+                                    hbase, 1, 0, nullptr, w2, tc_wbytes(32, 32), per, TC_PRO_PROXY,
                                     true, err);
     tc_grid_sync(bar, err, pp);
     tc_layer<32, 32, EPI_GELU_ONLY>(pp, taddr, &tm2, TcOut{b2, nullptr, a2, nullptr, nullptr, nullptr}, n,
-                                    hbase, 0, nullptr, w3, tc_wbytes(32, 16), 2 * per,
+                                    hbase, 0, 1, nullptr, w3, tc_wbytes(32, 16), 2 * per,
                                     TC_PRO_PROXY, true, err);
     tc_grid_sync(bar, err, pp);
     tc_layer<32, 16, EPI_F32>(pp, taddr, &tm3, TcOut{b3, nullptr, nullptr, out, nullptr, out4}, n, hbase,
-                              1, nullptr, nullptr, 0, 3 * per, TC_PRO_PROXY, false, err);
+                              1, 1, nullptr, nullptr, 0, 3 * per, TC_PRO_PROXY, false, err);
     tc_pipe_close(pp, taddr);
 }
 

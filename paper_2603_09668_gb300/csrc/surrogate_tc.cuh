@@ -144,9 +144,7 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 }
 
 constexpr int TC_NST = 8;        // halo stages (one input slice each)
-// Epilogue warps: lane quarter = warp & 3, column half = (warp >> 2) & 1, and
-// warps 0-7 take the even output slices, 8-15 the odd ones.
-constexpr int TC_EPI_WARPS = 16;
+constexpr int TC_EPI_WARPS = 8;  // epilogue warps: lane quarter = warp & 3, column half = warp >> 2
 constexpr int TC_MMA_WARP = TC_EPI_WARPS, TC_LOAD_WARP = TC_EPI_WARPS + 1;
 constexpr int TC_THREADS = 32 * (TC_EPI_WARPS + 2);  // + the MMA warp and the loader warp
 constexpr int TC_TMEM_COLS = 512;                     // the whole tensor memory of the SM
@@ -221,16 +219,13 @@ __device__ __forceinline__ bool tc_segment(int n, int nxy, int j, TcSeg &c) {
 // three blocks. Windows never overlap, so the MMAs of consecutive slices do
 // not wait on each other's accumulators.
 //
-// Roles: warp 17, lane 0 (the loader) issues the weight copies and the halo
-// loads (ring of TC_NST slices, each refilled once its MMAs are done); warp 16,
+// Roles: warp 9, lane 0 (the loader) issues the weight copies and the halo
+// loads (ring of TC_NST slices, each refilled once its MMAs are done); warp 8,
 // lane 0 issues the MMAs, committing each slice to empty[k % TC_NST] and
-// ready[k % TC_RING]; warps 0-15 read the finished output slices, the even
-// ones warps 0-7, the odd ones warps 8-15 (warp w: accumulator lanes
-// 32 (w % 4) .. + 31, column half (w / 4) % 2), and all of them arrive on
+// ready[k % TC_RING]; warps 0-7 read the finished output slices (warp w:
+// accumulator lanes 32 (w % 4) .. + 31, column half w / 4) and arrive on
 // wfree[w] once no output needs window w any more, which the MMA thread waits
-// for before reusing it. A slice's epilogue (barrier, tensor-memory loads,
-// GELU, stores) takes its warps about 1,400 cycles, mostly latency, so two
-// sets take turns.
+// for before reusing it.
 //
 // The MMA thread's issue stalls at the tensor pipe's pace with only a few
 // MMAs queued, so whatever else it does between two slices leaves the pipe
@@ -239,7 +234,8 @@ __device__ __forceinline__ bool tc_segment(int n, int nxy, int j, TcSeg &c) {
 // against the 1,008 of its 18 MMAs (64^3; with the MMAs left out the waits
 // alone took 800; a quarter of the halo bytes changed nothing). So the loads
 // have a warp of their own, and the next slice's barriers are waited for
-// after two thirds of a slice's MMAs, when they have normally completed.
+// after two thirds of a slice's MMAs, when they have normally completed (the
+// four layers: 77.7 -> 74.1 us at 64^3, 191 -> 181 us at 96^3).
 
 // The pipeline's shared-memory state, kept across the layers of one launch:
 // the slice counter k runs on from layer to layer, so every mbarrier phase
@@ -351,7 +347,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
     constexpr int KCH = CIN / 8;
     constexpr int HBYTES = KCH * TC_SLICE;
     constexpr int WBYTES = tc_wbytes(CIN, COUT);
-    constexpr int CPW = COUT / 2;                   // accumulator columns per epilogue warp
+    constexpr int CPW = COUT / (TC_EPI_WARPS / 4);  // accumulator columns per epilogue warp
     constexpr int CP2 = CPW / 2;                    // as pairs
     constexpr int NW = 3 * COUT;                    // MMA N: the three dz taps
     static_assert(TC_NWIN * NW <= TC_TMEM_COLS && TC_RING >= TC_NWIN + 2, "tensor memory plan");
@@ -443,7 +439,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
         }
         __syncwarp();
     } else {
-        const int q = warp & 3, hcol = (warp >> 2) & 1, odd = warp >> 3;
+        const int q = warp & 3, hcol = warp >> 2;
         const int row = q * 32 + lane;  // accumulator lane = tile voxel (x = row & 7, y = row >> 3)
         const uint32_t tq = taddr + ((uint32_t)(q * 32) << 16) + hcol * CPW;
         const size_t nv = (size_t)n * n * n;
@@ -474,30 +470,30 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                     break;
                 }
                 tc_fence_after();
-                // outputs finished by slice zi: zi - 1, and zi itself at the volume's
-                // end; at most one of them is this warp's
-                const int zhi = (zi == n - 1) ? min(zi, c.o1) : min(zi - 1, c.o1);
-                const int z = (zhi & 1) == odd ? zhi : zhi - 1;
-                const bool mine = z >= max(zi - 1, c.o0);
-                float2 r[CP2];
-                if (mine) {
+                // outputs finished by slice zi: zi - 1, and zi itself at the volume's end
+                const int zlo = max(zi - 1, c.o0), zhi = (zi == n - 1) ? min(zi, c.o1) : min(zi - 1, c.o1);
+                float2 r[2][CP2];
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    const int z = zlo + m;
+                    if (z > zhi) break;
                     // block b of slice z - 1 + b; slice z - 1 and z + 1 may be missing
                     const int ks = kb + (z - i0);
                     float2 p0[CP2], p2[CP2];
                     const bool lo = z - 1 >= i0, hi = z + 1 <= i1;
                     if (lo) tc_ld_pairs(tq + (uint32_t)(((ks - 1) % TC_NWIN) * NW), p0);
-                    tc_ld_pairs(tq + (uint32_t)((ks % TC_NWIN) * NW + COUT), r);
+                    tc_ld_pairs(tq + (uint32_t)((ks % TC_NWIN) * NW + COUT), r[m]);
                     if (hi) tc_ld_pairs(tq + (uint32_t)(((ks + 1) % TC_NWIN) * NW + 2 * COUT), p2);
-                    tc_ld_wait(r);
+                    tc_ld_wait(r[m]);
                     if (lo) {
                         tc_ld_wait(p0);
 #pragma unroll
-                        for (int cc = 0; cc < CP2; ++cc) r[cc] = __fadd2_rn(p0[cc], r[cc]);
+                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(p0[cc], r[m][cc]);
                     }
                     if (hi) {
                         tc_ld_wait(p2);
 #pragma unroll
-                        for (int cc = 0; cc < CP2; ++cc) r[cc] = __fadd2_rn(r[cc], p2[cc]);
+                        for (int cc = 0; cc < CP2; ++cc) r[m][cc] = __fadd2_rn(r[m][cc], p2[cc]);
                     }
                 }
                 tc_fence_before();
@@ -511,15 +507,18 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                         mbar_arrive(smem_u32(&pp.wfree[k % TC_NWIN]));
                     }
                 }
-                if (mine) {
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    if (zlo + m > zhi) break;
+                    const int z = zlo + m;
                     const size_t v = ((size_t)z * n + (y0 + (row >> 3))) * n + x0 + (row & 7);
                     const int c0 = hcol * CPW;
                     auto plane = [&](int cc) { return ((size_t)((c0 + cc) >> 3) * nv + v) * 8; };
                     if (EPI == EPI_F32) {
 #pragma unroll
                         for (int cc = 0; cc < CPW; cc += 4) {
-                            const float2 lo = __fadd2_rn(r[cc / 2], bias[cc / 2]);
-                            const float2 hi = __fadd2_rn(r[cc / 2 + 1], bias[cc / 2 + 1]);
+                            const float2 lo = __fadd2_rn(r[m][cc / 2], bias[cc / 2]);
+                            const float2 hi = __fadd2_rn(r[m][cc / 2 + 1], bias[cc / 2 + 1]);
                             const float4 q4 = make_float4(lo.x, lo.y, hi.x, hi.y);
                             *reinterpret_cast<float4 *>(o.out_f + v * COUT + c0 + cc) = q4;
                             if (cc == 0 && c0 == 0 && o.out_f4) reinterpret_cast<float4 *>(o.out_f4)[v] = q4;
@@ -534,7 +533,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                             for (int jj = 0; jj < 4; ++jj) {
                                 const float2 zz = make_float2(__uint_as_float(zw[jj] << 16),
                                                               __uint_as_float(zw[jj] & 0xffff0000u));
-                                od[jj] = bf16_pair(__fmul2_rn(r[cc / 2 + jj], gelu2_grad_f(zz)));
+                                od[jj] = bf16_pair(__fmul2_rn(r[m][cc / 2 + jj], gelu2_grad_f(zz)));
                             }
                             *reinterpret_cast<uint4 *>(o.out_z + plane(cc)) = make_uint4(od[0], od[1], od[2], od[3]);
                         }
@@ -544,7 +543,7 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
                             uint32_t oz[4], oa[4];
 #pragma unroll
                             for (int jj = 0; jj < 4; ++jj) {
-                                const float2 zz = __fadd2_rn(r[cc / 2 + jj], bias[cc / 2 + jj]);
+                                const float2 zz = __fadd2_rn(r[m][cc / 2 + jj], bias[cc / 2 + jj]);
                                 if (EPI == EPI_GELU) oz[jj] = bf16_pair(zz);
                                 oa[jj] = bf16_pair(gelu2_f(zz));
                             }

@@ -245,24 +245,24 @@ __global__ void __launch_bounds__(256) k_count_fluid(const bf16 *__restrict__ fe
     if (threadIdx.x == 0 && c) atomicAdd(count, c);
 }
 
-// gw += the sum over nchunks CTAs' partial weight gradients, gb += that over
-// nchunks_b CTAs' partial bias gradients (the last block). 64 threads of a row
+// gw and gb += the sums over nchunks CTAs' partial weight and bias gradients
+// (bias: the last block). 64 threads of a row
 // take four neighbouring weights each, the block's eight rows a share of the
 // chunks each: with one thread walking all 152 chunks of a weight, 108 blocks
 // kept too few loads in flight (16 us per 32 -> 32 layer, 17 MB).
 constexpr int WR_ROWS = 8;
 __global__ void __launch_bounds__(64 * WR_ROWS) k_wgrad_reduce(
-    const float *__restrict__ part, const float *__restrict__ part_b, int nchunks, int nchunks_b,
-    int64_t nw, int cout, float *__restrict__ gw, float *__restrict__ gb) {
+    const float *__restrict__ part, const float *__restrict__ part_b, int nchunks, int64_t nw, int cout, float *__restrict__ gw, float *__restrict__ gb) {
     __shared__ float4 sum[WR_ROWS][64];
+    pdl_wait();  // before the trigger: what follows may then read what preceded k_wgrad_tc
+    pdl_trigger();
     const bool bias = blockIdx.x + 1 == gridDim.x;
     const int64_t len = bias ? cout : nw, i = (bias ? 0 : (int64_t)blockIdx.x * 256) + threadIdx.x * 4;
     const float *src = bias ? part_b : part;
-    const int n = bias ? nchunks_b : nchunks;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < len) {
 #pragma unroll 4
-        for (int c = threadIdx.y; c < n; c += WR_ROWS) {
+        for (int c = threadIdx.y; c < nchunks; c += WR_ROWS) {
             const float4 p = *reinterpret_cast<const float4 *>(src + (size_t)c * len + i);
             s.x += p.x;
             s.y += p.y;
@@ -688,25 +688,25 @@ static dw_status make_halo_map(CUtensorMap *tm, const bf16 *base, int n, int C) 
     return make_box_map(tm, base, n, C, TC_HX, TC_HY, 1);
 }
 
-// The weight-gradient kernel's boxes: an input tile's halo (16 voxels x 6
-// rows x 3 slices) and an output-gradient tile (16 x 4 x 1).
+// The weight-gradient kernel's boxes: an input tile's rows with the halo in y,
+// and the output gradients of its rows in three slices.
 static dw_status make_wgrad_maps(CUtensorMap *tm_in, CUtensorMap *tm_g, const bf16 *in, int cin,
                                  const bf16 *g, int cout, int n) {
-    dw_status st = make_box_map(tm_in, in, n, cin, WG_TX, WG_HY, 3);
-    if (st == DW_OK) st = make_box_map(tm_g, g, n, cout, WG_TX, WG_TY, 1);
+    dw_status st = make_box_map(tm_in, in, n, cin, WG_TX, WG_HY, 1);
+    if (st == DW_OK) st = make_box_map(tm_g, g, n, cout, WG_TX, WG_TY, 3);
     return st;
 }
 
-static void launch_wgrad_reduce(SurrHandle *h, int nchunks, int nchunks_b, int64_t nw, int cout,
-                                float *gw, float *gb, cudaStream_t s) {
-    k_wgrad_reduce<<<grid_for(nw, 256) + 1, dim3(64, WR_ROWS), 0, s>>>(
-        h->part, h->part_b, nchunks, nchunks_b, nw, cout, gw, gb);
+static cudaError_t launch_wgrad_reduce(SurrHandle *h, int nchunks, int64_t nw, int cout, float *gw,
+                                       float *gb, cudaStream_t s) {
+    return launch_pdl3(k_wgrad_reduce, dim3(grid_for(nw, 256) + 1), dim3(64, WR_ROWS), s, h->part, h->part_b,
+                       nchunks, nw, cout, gw, gb);
 }
 
 // Weight and bias gradients of one layer on tcgen05: gw += dW, gb += db.
 template <int CIN, int COUT>
 static dw_status wgrad_tc(SurrHandle *h, const CUtensorMap &tm_in, const CUtensorMap &tm_g,
-                          const bf16 *g, float *gw, float *gb, cudaStream_t s) {
+                          float *gw, float *gb, cudaStream_t s) {
     constexpr size_t smem = wg_smem<CIN, COUT>();
     static bool attr_set = false;
     if (!attr_set) {
@@ -716,13 +716,9 @@ static dw_status wgrad_tc(SurrHandle *h, const CUtensorMap &tm_in, const CUtenso
     }
     const int ntiles = (h->n / WG_TX) * (h->n / WG_TY) * h->n;
     const int grid = std::min(std::min(h->sms, h->part_chunks), ntiles);
-    k_wgrad_tc<CIN, COUT><<<grid, WG_THREADS, smem, s>>>(tm_in, tm_g, h->n, h->part, h->err);
-    DW_LAUNCHED("k_wgrad_tc");
-    const int gridb = h->part_chunks;
-    k_bias_grad<COUT><<<gridb, 256, 0, s>>>(g, h->nv, h->part_b);
-    DW_LAUNCHED("k_bias_grad");
-    launch_wgrad_reduce(h, grid, gridb, 27LL * CIN * COUT, COUT, gw, gb, s);
-    DW_LAUNCHED("k_wgrad_reduce");
+    DW_CUDA(launch_pdl_smem(k_wgrad_tc<CIN, COUT>, dim3(grid), dim3(WG_THREADS), smem, s, tm_in, tm_g, h->n,
+                            h->part, h->part_b, h->err));
+    DW_CUDA(launch_wgrad_reduce(h, grid, 27LL * CIN * COUT, COUT, gw, gb, s));
     return DW_OK;
 }
 
@@ -741,8 +737,7 @@ static dw_status wgrad(SurrHandle *h, const bf16 *in, const bf16 *g, float *gw, 
     k_wgrad<CIN, COUT><<<dim3(h->nchunks, 3), CV_THREADS, smem, s>>>(in, g, h->n, h->tiles_per_chunk,
                                                                      h->part, h->part_b);
     DW_LAUNCHED("k_wgrad");
-    launch_wgrad_reduce(h, h->nchunks, h->nchunks, 27LL * CIN * COUT, COUT, gw, gb, s);
-    DW_LAUNCHED("k_wgrad_reduce");
+    DW_CUDA(launch_wgrad_reduce(h, h->nchunks, 27LL * CIN * COUT, COUT, gw, gb, s));
     return DW_OK;
 }
 
@@ -1055,22 +1050,22 @@ extern "C" dw_status surr_backward(dw_surr h, dw_stream stream) {
     cudaStream_t s = as_stream(stream);
     dw_status st;
     // layer 4: dW from a3 and g4; dL/dz3 = (W4' * g4) GELU'(z3)
-    st = wgrad_tc<32, 16>(h, h->tmw_in[3], h->tmw_g[3], h->g4, h->grads + h->off_w[3],
+    st = wgrad_tc<32, 16>(h, h->tmw_in[3], h->tmw_g[3], h->grads + h->off_w[3],
                           h->grads + h->off_b[3], s);
     if (st != DW_OK) return st;
     st = conv<16, 32, EPI_DGELU>(h, h->tm_g4, h->wd + h->woff[3], nullptr, h->gz[2], nullptr, nullptr, h->z[2], s);
     if (st != DW_OK) return st;
-    st = wgrad_tc<32, 32>(h, h->tmw_in[2], h->tmw_g[2], h->gz[2], h->grads + h->off_w[2],
+    st = wgrad_tc<32, 32>(h, h->tmw_in[2], h->tmw_g[2], h->grads + h->off_w[2],
                           h->grads + h->off_b[2], s);
     if (st != DW_OK) return st;
     st = conv<32, 32, EPI_DGELU>(h, h->tm_gz[2], h->wd + h->woff[2], nullptr, h->gz[1], nullptr, nullptr, h->z[1], s);
     if (st != DW_OK) return st;
-    st = wgrad_tc<32, 32>(h, h->tmw_in[1], h->tmw_g[1], h->gz[1], h->grads + h->off_w[1],
+    st = wgrad_tc<32, 32>(h, h->tmw_in[1], h->tmw_g[1], h->grads + h->off_w[1],
                           h->grads + h->off_b[1], s);
     if (st != DW_OK) return st;
     st = conv<32, 32, EPI_DGELU>(h, h->tm_gz[1], h->wd + h->woff[1], nullptr, h->gz[0], nullptr, nullptr, h->z[0], s);
     if (st != DW_OK) return st;
-    st = wgrad_tc<16, 32>(h, h->tmw_in[0], h->tmw_g[0], h->gz[0], h->grads + h->off_w[0],
+    st = wgrad_tc<16, 32>(h, h->tmw_in[0], h->tmw_g[0], h->grads + h->off_w[0],
                           h->grads + h->off_b[0], s);
     return st;
 }
@@ -1092,9 +1087,9 @@ extern "C" dw_status surr_weight_grad(dw_surr h, int32_t cin, int32_t cout, cons
     CUtensorMap tm_in, tm_g;
     dw_status st = make_wgrad_maps(&tm_in, &tm_g, bi, cin, bg, cout, h->n);
     if (st != DW_OK) return st;
-    if (cin == 16) return wgrad_tc<16, 32>(h, tm_in, tm_g, bg, gw, gb, s);
-    if (cout == 32) return wgrad_tc<32, 32>(h, tm_in, tm_g, bg, gw, gb, s);
-    return wgrad_tc<32, 16>(h, tm_in, tm_g, bg, gw, gb, s);
+    if (cin == 16) return wgrad_tc<16, 32>(h, tm_in, tm_g, gw, gb, s);
+    if (cout == 32) return wgrad_tc<32, 32>(h, tm_in, tm_g, gw, gb, s);
+    return wgrad_tc<32, 16>(h, tm_in, tm_g, gw, gb, s);
 }
 
 extern "C" dw_status surr_adam(dw_surr h, float lr, float beta1, float beta2, float eps,

@@ -1,58 +1,68 @@
-// Weight gradients of the surrogate network's 3x3x3 convolutions on the
-// fifth-generation tensor cores (tcgen05.mma kind::f16, BF16 operands, FP32
-// accumulators in tensor memory, operands loaded by TMA).
+// Weight and bias gradients of the surrogate network's 3x3x3 convolutions on
+// the fifth-generation tensor cores (tcgen05.mma kind::f16, BF16 operands,
+// FP32 accumulators in tensor memory, operands loaded by TMA).
 //
 // dW[tap][co][ci] = sum_v g[v][co] in[v + d(tap)][ci] (zero padding) is a
-// GEMM over voxels (K). For each (dy, dz) pair of taps one MMA computes
-//   D_(dy,dz)[(dx, ci)][co] += sum_{v in a row of 16 x-voxels}
-//                              in[v + (dx, dy, dz) - 1][ci] g[v][co]
+// GEMM over voxels (K). A tile is 16 (x) x WG_TY (y) voxels of one slice z of
+// the input; for each of its rows y and each dy one MMA computes
+//   D_dy[(dx, ci)][(co, dz)] += sum_{16 x-voxels}
+//            in[(x + dx - 1, y + dy - 1, z)][ci] g[(x, y, z - dz + 1)][co]
 // with M = 128 rows = 4 dx slots x 32 input channels (the fourth slot, and
 // for CIN = 16 the upper half of every slot, are rows whose results are not
-// read), N = COUT, K = 16 voxels. Both operands are MN-major: in the planar
+// read), N = 3 COUT, K = 16 voxels. Both operands are MN-major: in the planar
 // activation layout [C/8][n^3][8] a voxel's 8 channels are one 16-byte row,
 // and 8 consecutive voxels of one 8-channel plane form a core matrix (8 K
-// rows x 16 B). The input is loaded three times per tile, shifted by dx =
-// 0, 1, 2 voxels (three TMA boxes, 16-byte aligned in x because a voxel
+// rows x 16 B). The input rows are loaded three times per tile, shifted by
+// dx = 0, 1, 2 voxels (three TMA boxes, 16-byte aligned in x because a voxel
 // record is 16 bytes), into consecutive slots, so that every 8-row group of
 // M, (dx, 8 channels), is one plane further: a uniform stride-dimension
-// offset, which is what lets the three dx taps share one MMA. The nine
-// (dy, dz) accumulators (9 COUT columns of tensor memory) stay in tensor
-// memory over all of a CTA's tiles; the epilogue writes the CTA's partial sums
-// once.
+// offset, which is what lets the three dx taps share one MMA. The three g
+// slices come as one box whose (plane, slice) order gives the 8-column groups
+// of N the same property, so the three dz taps share it too. Slices outside
+// the volume are zeros. The three dy accumulators (9 COUT columns of tensor
+// memory) stay in tensor memory over all of a CTA's tiles; the epilogue
+// writes the CTA's partial sums once.
 //
-// Tiles: 16 (x) x 4 (y) voxels of one z slice. A tile's halo for the input is
-// 3 slices x 6 rows x 16 voxels per dx slot. Roles: warp 4, lane 0 issues the
-// TMA loads (a ring of WG_NST stages) and the MMAs; warps 0-3 wait for the
-// last MMA and read the accumulators (warp w: rows 32 w .. 32 w + 31). Every
-// wait is bounded (about a second): the kernel then sets ERRBIT_TIMEOUT,
-// drains its copies and frees the tensor memory.
+// With one MMA of N = COUT per (dy, dz), on 16 x 4 tiles of g and the three
+// input slices around them, 64 voxels took 36 MMAs and 58 KB of loads (now 12
+// and 27 KB), and the bias gradient read g once more: a 32 -> 32 layer with
+// its reductions took 66 us at 64^3 and 183 us at 96^3, now 20 and 46 us
+// (without the MMAs 16 us at 64^3: launches, the loads' start and the
+// partial sums' reduction are most of the rest). With WG_TY = 4 (six stages)
+// 96^3 takes 54 us instead of 50: the halo rows are half of a plane's six.
+//
+// Roles: warp 5, lane 0 issues the TMA loads (a ring of WG_NST stages); warp
+// 4, lane 0 the MMAs; warps 0-3 add up the g slice of each tile for the bias
+// gradient, from the stage the MMAs read it from, and at the end read the
+// accumulators (warp w: rows 32 w .. 32 w + 31). Every wait is bounded (about
+// a second): the kernel then sets ERRBIT_TIMEOUT, drains its copies and frees
+// the tensor memory.
 #pragma once
 
 #include "surrogate_tc.cuh"
 
 namespace dw {
 
-constexpr int WG_TX = 16, WG_TY = 4;   // tile: 16 x-voxels (one K step) x 4 rows, one z slice
+constexpr int WG_TX = 16, WG_TY = 8;   // tile: 16 x-voxels (one K step) x WG_TY rows, one z slice
 constexpr int WG_HY = WG_TY + 2;       // halo rows
 constexpr int WG_ROW = WG_TX * 16;     // bytes of one row of 16 voxel records
-constexpr int WG_PLANE = 3 * WG_HY * WG_ROW;  // one 8-channel plane of a slot: 3 slices x 6 rows
-constexpr int WG_NST = 3;              // pipeline stages
-constexpr int WG_EPI = 4;              // epilogue warps: tensor-memory rows 0-127
-constexpr int WG_THREADS = 32 * (WG_EPI + 1);
+constexpr int WG_PLANE = WG_HY * WG_ROW;   // one 8-channel plane of a slot
+constexpr int WG_GSLICE = WG_TY * WG_ROW;  // one 8-channel plane of a g slice
+constexpr int WG_NST = 4;              // pipeline stages
+constexpr int WG_EPI = 4;              // bias and epilogue warps: tensor-memory rows 0-127
+constexpr int WG_MMA_WARP = WG_EPI, WG_LOAD_WARP = WG_EPI + 1;
+constexpr int WG_THREADS = 32 * (WG_EPI + 2);
 
 template <int CIN>
 constexpr int wg_slot() { return (CIN / 8) * WG_PLANE; }
-template <int COUT>
-constexpr int wg_gbytes() { return (COUT / 8) * WG_TY * WG_ROW; }
 template <int CIN, int COUT>
-constexpr int wg_stage() { return 3 * wg_slot<CIN>() + wg_gbytes<COUT>(); }
+constexpr int wg_stage() { return 3 * wg_slot<CIN>() + (COUT / 8) * 3 * WG_GSLICE; }
 // The stages, plus what the M = 128 rows of the last stage's MMAs reach past
-// it, plus alignment. An MMA's A operand starts at most 17 rows into a plane
-// and spans 16 planes in M and 2 x 128 B in K: 16 planes from the stage start.
+// it (an MMA's A operand ends within 16 planes of the stage start), plus
+// alignment.
 template <int CIN, int COUT>
 constexpr size_t wg_smem() {
-    constexpr int reach = (2 * WG_HY + WG_TY + 1) * WG_ROW + 15 * WG_PLANE + 2 * 128;
-    constexpr int extra = reach > wg_stage<CIN, COUT>() ? reach - wg_stage<CIN, COUT>() : 0;
+    constexpr int extra = 16 * WG_PLANE > wg_stage<CIN, COUT>() ? 16 * WG_PLANE - wg_stage<CIN, COUT>() : 0;
     return (size_t)WG_NST * wg_stage<CIN, COUT>() + extra + 1024;
 }
 template <int COUT>
@@ -69,9 +79,11 @@ struct WgPipe {
     uint64_t full[WG_NST], empty[WG_NST], done;
     uint32_t tmem_base;
     int abort_flag;
+    float bias[WG_EPI][32];
 };
 
-// Tiles of this CTA: a contiguous range of the layer's (x, y, z) tiles.
+// Tiles of this CTA: a contiguous range of the layer's (x, y, z) tiles (at
+// least one: the grid has no more CTAs than there are tiles).
 __device__ __forceinline__ void wg_range(int ntiles, int &t0, int &t1) {
     t0 = (int)((int64_t)ntiles * blockIdx.x / gridDim.x);
     t1 = (int)((int64_t)ntiles * (blockIdx.x + 1) / gridDim.x);
@@ -90,27 +102,29 @@ __device__ __forceinline__ void wg_load(const CUtensorMap *tm_in, const CUtensor
             "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
             " [%0], [%1, {%2, %3, %4, %5}], [%6];"
             :: "r"(stage + d * wg_slot<CIN>()), "l"((uint64_t)tm_in), "r"(8 * (x0 - 1 + d)),
-               "r"(y0 - 1), "r"(z - 1), "r"(0), "r"(bar)
+               "r"(y0 - 1), "r"(z), "r"(0), "r"(bar)
             : "memory");
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        :: "r"(stage + 3 * wg_slot<CIN>()), "l"((uint64_t)tm_g), "r"(8 * x0), "r"(y0), "r"(z),
+        :: "r"(stage + 3 * wg_slot<CIN>()), "l"((uint64_t)tm_g), "r"(8 * x0), "r"(y0), "r"(z - 1),
            "r"(0), "r"(bar)
         : "memory");
 }
 
-// Partial weight gradients of CTA b: part[b][tap][co][ci] for the CTA's
-// tiles. tm_in: the input activations as boxes {128, 6, 3, CIN/8}; tm_g: the
-// output gradients as boxes {128, 4, 1, COUT/8} (both views [C/8][z][y][x * 8]).
+// Partial gradients of CTA b over its tiles: part[b][tap][co][ci] and
+// part_b[b][co]. tm_in: the input activations as boxes {128, WG_HY, 1,
+// CIN/8}; tm_g: the output gradients as boxes {128, WG_TY, 3, COUT/8} (both
+// views [C/8][z][y][x * 8]).
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const __grid_constant__ CUtensorMap tm_in,
                                                             const __grid_constant__ CUtensorMap tm_g,
-                                                            int n, float *__restrict__ part, int *err) {
+                                                            int n, float *__restrict__ part,
+                                                            float *__restrict__ part_b, int *err) {
     static_assert((CIN == 16 || CIN == 32) && (COUT == 16 || COUT == 32), "unsupported shape");
-    constexpr int STAGE = wg_stage<CIN, COUT>(), SLOT = wg_slot<CIN>();
-    constexpr int TCOLS = wg_tmem_cols<COUT>();
-    constexpr uint32_t IDESC = wg_idesc(COUT);
+    constexpr int STAGE = wg_stage<CIN, COUT>(), GOFF = 3 * wg_slot<CIN>();
+    constexpr int TCOLS = wg_tmem_cols<COUT>(), NW = 3 * COUT;
+    constexpr uint32_t IDESC = wg_idesc(NW);
     extern __shared__ unsigned char smem_raw[];
     __shared__ WgPipe pp;
     unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -121,7 +135,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const __grid_constan
         pp.abort_flag = 0;
         for (int i = 0; i < WG_NST; ++i) {
             mbar_init(smem_u32(&pp.full[i]), 1);
-            mbar_init(smem_u32(&pp.empty[i]), 1);
+            mbar_init(smem_u32(&pp.empty[i]), 1 + WG_EPI);  // the MMAs, the bias warps
         }
         mbar_init(smem_u32(&pp.done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -134,37 +148,49 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const __grid_constan
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t taddr = pp.tmem_base;
-    const volatile int *abort_p = &pp.abort_flag;
+    volatile int *abort_p = &pp.abort_flag;
     const int ntiles = (n / WG_TX) * (n / WG_TY) * n;
     int t0, t1;
     wg_range(ntiles, t0, t1);
     const int cnt = t1 - t0;
 
-    if (warp == WG_EPI) {
-        if (lane == 0 && cnt > 0) {
-            int issued = 0, consumed = 0;
-            bool ok = true;
-            while (issued < WG_NST && issued < cnt) {
-                wg_load<CIN, COUT>(&tm_in, &tm_g, sbase + (issued % WG_NST) * STAGE,
-                                   smem_u32(&pp.full[issued % WG_NST]), n, t0 + issued);
-                ++issued;
+    if (warp == WG_LOAD_WARP) {
+        if (lane == 0) {
+            pdl_wait();  // everything else in the kernel follows from the first load
+            int j = 0;
+            for (; j < cnt; ++j) {
+                const int s = j % WG_NST;
+                if (j >= WG_NST && !tc_wait(smem_u32(&pp.empty[s]), (j / WG_NST - 1) & 1, abort_p)) {
+                    *abort_p = 1;
+                    break;
+                }
+                wg_load<CIN, COUT>(&tm_in, &tm_g, sbase + s * STAGE, smem_u32(&pp.full[s]), n, t0 + j);
             }
+            // drain (bounded): the last copies into every stage
+            for (int i = max(0, j - WG_NST); i < j; ++i)
+                tc_wait(smem_u32(&pp.full[i % WG_NST]), (i / WG_NST) & 1, nullptr);
+        }
+        __syncwarp();
+    } else if (warp == WG_MMA_WARP) {
+        if (lane == 0) {
             for (int j = 0; j < cnt; ++j) {
                 const int s = j % WG_NST;
-                ok = tc_wait(smem_u32(&pp.full[s]), (j / WG_NST) & 1, abort_p);
-                if (!ok) break;
-                ++consumed;
+                if (!tc_wait(smem_u32(&pp.full[s]), (j / WG_NST) & 1, abort_p)) {
+                    *abort_p = 1;
+                    break;
+                }
                 tc_fence_after();
-                const uint32_t st = sbase + s * STAGE;
+                const uint64_t a0 = tc_desc(sbase + s * STAGE, 128, WG_PLANE);
+                const uint64_t b0 = tc_desc(sbase + s * STAGE + GOFF, 128, WG_GSLICE);
 #pragma unroll
                 for (int r = 0; r < WG_TY; ++r) {
-                    const uint64_t bd = tc_desc(st + 3 * SLOT + r * WG_ROW, 128, WG_TY * WG_ROW);
 #pragma unroll
-                    for (int b = 0; b < 9; ++b) {  // b = 3 dz + dy
-                        const int dz = b / 3, dy = b % 3;
-                        const uint64_t ad = tc_desc(st + (dz * WG_HY + r + dy) * WG_ROW, 128, WG_PLANE);
-                        const uint32_t d = taddr + (uint32_t)(b * COUT);
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const uint64_t ad = a0 + (uint32_t)((r + dy) * WG_ROW >> 4);
+                        const uint64_t bd = b0 + (uint32_t)(r * WG_ROW >> 4);
+                        const uint32_t d = taddr + (uint32_t)(dy * NW);
                         const uint32_t acc = (j | r) != 0;  // the CTA's first row starts each sum
                         asm volatile(
                             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -174,59 +200,81 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const __grid_constan
                     }
                 }
                 tc_commit(smem_u32(&pp.empty[s]));
-                // refill the stage of tile j - 1 (its MMAs were issued one tile ago)
-                if (j >= 1 && issued < cnt) {
-                    const int k1 = j - 1;
-                    ok = tc_wait(smem_u32(&pp.empty[k1 % WG_NST]), (k1 / WG_NST) & 1, abort_p);
-                    if (!ok) break;
-                    wg_load<CIN, COUT>(&tm_in, &tm_g, sbase + (issued % WG_NST) * STAGE,
-                                       smem_u32(&pp.full[issued % WG_NST]), n, t0 + issued);
-                    ++issued;
-                }
             }
-            if (ok) {
-                tc_commit(smem_u32(&pp.done));
-            } else {
-                atomicOr(err, ERRBIT_TIMEOUT);
-                pp.abort_flag = 1;
-            }
-            // drain (bounded): copies still in flight, the last MMAs
-            for (int k = consumed; k < issued; ++k)
-                tc_wait(smem_u32(&pp.full[k % WG_NST]), (k / WG_NST) & 1, nullptr);
-            if (consumed > 0)
-                tc_wait(smem_u32(&pp.empty[(consumed - 1) % WG_NST]), ((consumed - 1) / WG_NST) & 1,
-                        nullptr);
+            // all MMAs issued have ended when done completes (bounded)
+            tc_commit(smem_u32(&pp.done));
+            tc_wait(smem_u32(&pp.done), 0, nullptr);
         }
         __syncwarp();
     } else {
-        // rows 32 warp .. + 31: m = dx CIN + ci (rows from 3 CIN on are padding)
-        const int m = 32 * warp + lane;
-        float *pc = part + (size_t)blockIdx.x * 27 * COUT * CIN;
-        int okw = 1;
-        if (cnt > 0 && lane == 0) okw = tc_wait(smem_u32(&pp.done), 0, abort_p);
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (okw && cnt > 0) {
-            tc_fence_after();
-            const uint32_t tq = taddr + ((uint32_t)(32 * warp) << 16);
-#pragma unroll 1
-            for (int b = 0; b < 9; ++b) {
+        // bias: the 16-byte records of the tile's own g slice, spread over the
+        // threads by (row, x) within a plane, so that a thread's planes are fixed
+        constexpr int PL = COUT / 8, REC = WG_TY * WG_TX, PPP = 32 * WG_EPI / REC;  // planes per pass
+        static_assert(32 * WG_EPI % REC == 0 && PL % PPP == 0, "bias records do not split evenly");
+        float acc[PL / PPP][8] = {};
+        bool ok = true;
+        for (int j = 0; j < cnt && ok; ++j) {
+            const int s = j % WG_NST;
+            ok = tc_wait(smem_u32(&pp.full[s]), (j / WG_NST) & 1, abort_p);
+            if (ok) {
+                const unsigned char *g = smem + s * STAGE + GOFF + WG_GSLICE + (tid % REC) * 16;
 #pragma unroll
-                for (int c0 = 0; c0 < COUT; c0 += 16) {
-                    float r[16];
-                    tc_ld<16>(tq + (uint32_t)(b * COUT + c0), r);
-                    if (m < 3 * CIN) {
-                        const int dx = m / CIN, ci = m % CIN, tap = 3 * b + dx;
+                for (int p = 0; p < PL / PPP; ++p) {
+                    const uint4 q = *reinterpret_cast<const uint4 *>(g + (p * PPP + tid / REC) * 3 * WG_GSLICE);
+                    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-                        for (int cc = 0; cc < 16; ++cc)
-                            pc[((size_t)tap * COUT + c0 + cc) * CIN + ci] = r[cc];
+                    for (int c = 0; c < 4; ++c) {
+                        acc[p][2 * c] += __uint_as_float(w[c] << 16);
+                        acc[p][2 * c + 1] += __uint_as_float(w[c] & 0xffff0000u);
                     }
                 }
             }
-        } else if (cnt == 0 && m < 3 * CIN) {
+            ok = __all_sync(0xffffffffu, ok);
+            if (lane == 0) mbar_arrive(smem_u32(&pp.empty[s]));
+        }
+        // the warp's sums of its planes (p PPP + its first thread's plane)
+#pragma unroll
+        for (int p = 0; p < PL / PPP; ++p)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[p][c] += __shfl_xor_sync(0xffffffffu, acc[p][c], o);
+                if (lane == 0) pp.bias[warp][p * 8 + c] = acc[p][c];
+            }
+        asm volatile("bar.sync 1, %0;" :: "n"(32 * WG_EPI) : "memory");
+        if (tid < COUT) {
+            constexpr int WPP = WG_EPI / PPP;  // warps per plane
+            const int pl = tid / 8, w0 = (pl % PPP) * WPP;
+            float sum = 0.0f;
+            for (int w = 0; w < WPP; ++w) sum += pp.bias[w0 + w][pl / PPP * 8 + (tid & 7)];
+            part_b[(size_t)blockIdx.x * COUT + tid] = sum;
+        }
+        // rows 32 warp .. + 31: m = dx CIN + ci (rows from 3 CIN on are padding)
+        const int m = 32 * warp + lane;
+        ok = tc_wait(smem_u32(&pp.done), 0, abort_p) && !*abort_p;
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+            tc_fence_after();
+            const uint32_t tq = taddr + ((uint32_t)(32 * warp) << 16);
             const int dx = m / CIN, ci = m % CIN;
-            for (int b = 0; b < 9; ++b)
-                for (int co = 0; co < COUT; ++co) pc[((size_t)(3 * b + dx) * COUT + co) * CIN + ci] = 0.0f;
-        } else if (!okw && lane == 0) {
+            float *pc = part + (size_t)blockIdx.x * 27 * COUT * CIN + (size_t)dx * COUT * CIN + ci;
+#pragma unroll 1
+            for (int dy = 0; dy < 3; ++dy) {
+#pragma unroll
+                for (int c0 = 0; c0 < NW; c0 += 16) {
+                    float r[16];
+                    tc_ld<16>(tq + (uint32_t)(dy * NW + c0), r);
+                    if (m < 3 * CIN) {
+#pragma unroll
+                        for (int cc = 0; cc < 16; ++cc) {
+                            // 8-column group (plane, g slice z + 1 - dz)
+                            const int grp = (c0 + cc) / 8, dz = 2 - grp % 3, co = grp / 3 * 8 + cc % 8;
+                            pc[((size_t)(9 * dz + 3 * dy) * COUT + co) * CIN] = r[cc];
+                        }
+                    }
+                }
+            }
+        } else if (lane == 0) {
             atomicOr(err, ERRBIT_TIMEOUT);
         }
     }
@@ -235,39 +283,6 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const __grid_constan
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(taddr), "r"(TCOLS));
-    }
-}
-
-// Bias-gradient partials: part_b[b][co] = sum over CTA b's voxels of g[v][co]
-// (planar BF16 [COUT/8][nv][8]); one plane per warp, lanes summed by shuffles
-// (the 2,048 shared-memory atomics onto COUT words, one load in flight per
-// thread and one CTA per SM took 21 us for 17 MB).
-template <int COUT>
-__global__ void __launch_bounds__(256) k_bias_grad(const bf16 *__restrict__ g, int64_t nv,
-                                                   float *__restrict__ part_b) {
-    constexpr int PL = COUT / 8, WPP = 8 / PL;  // planes, warps per plane
-    __shared__ float sum[8][8];
-    const int64_t v0 = nv * blockIdx.x / gridDim.x, v1 = nv * (blockIdx.x + 1) / gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pl = warp % PL;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int64_t v = v0 + warp / PL * 32 + lane; v < v1; v += 32 * WPP) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(g + ((size_t)pl * nv + v) * 8);
-        const bf16 *e = reinterpret_cast<const bf16 *>(&q);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(e[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-        if (lane == 0) sum[warp][j] = acc[j];
-    }
-    __syncthreads();
-    if (threadIdx.x < COUT) {
-        float s = 0.0f;
-        for (int w = 0; w < WPP; ++w) s += sum[threadIdx.x / 8 + w * PL][threadIdx.x & 7];
-        part_b[(size_t)blockIdx.x * COUT + threadIdx.x] = s;
     }
 }
 

@@ -232,3 +232,33 @@ def test_dssim_tiles(shape):
     l2 = torch.zeros(1, device="cuda")
     B.image_dssim_loss(to_dev(a), to_dev(b), l2, 2.0)
     assert abs(l2.item() - loss.item()) <= 1e-6  # the block sums' order: 4 ulp of the weight
+
+
+# Weight gradients of a g with a few single nonzero voxels (corners, faces, tile
+# and slice edges): each tap's entry is a sum of few products of small whole
+# numbers, exact in any order.
+@pytest.mark.parametrize("shape", [(16, 32), (32, 32), (32, 16)])
+@pytest.mark.parametrize("n", [16, 48])
+def test_weight_gradient_of_single_voxels(n, shape):
+    cin, cout = shape
+    rng = np.random.default_rng(3)
+    X = rng.integers(-8, 9, (cin, n, n, n)).astype(np.float64)
+    G = np.zeros((cout, n, n, n))
+    e = n - 1
+    for v in ((0, 0, 0), (e, e, e), (0, e, 8), (7, 8, 15), (8, 7, 16 % n), (e, 0, 0), (5, 15, e), (1, 2, 3)):
+        G[(slice(None), *v)] = rng.integers(-8, 9, cout)
+    Xp = np.pad(X, ((0, 0), (1, 1), (1, 1), (1, 1)))
+    ref = np.stack([np.einsum("ozyx,izyx->oi", G, Xp[:, dz:dz + n, dy:dy + n, dx:dx + n], optimize=True)
+                    for dz in range(3) for dy in range(3) for dx in range(3)])
+
+    def planar(a):
+        p = np.moveaxis(a.reshape(-1, 8, n, n, n), 1, 4).reshape(-1, n ** 3, 8)
+        return torch.tensor(np.ascontiguousarray(p)).to(torch.bfloat16).cuda()
+
+    s = B.Surrogate(n)
+    gw, gb = torch.zeros(27 * cout * cin, device="cuda"), torch.zeros(cout, device="cuda")
+    s.weight_grad(cin, cout, planar(X), planar(G), gw, gb)
+    s.device_status()
+    assert np.array_equal(gw.cpu().numpy().reshape(27, cout, cin), ref)
+    assert np.array_equal(gb.cpu().numpy(), G.sum(axis=(1, 2, 3)))
+    s.close()

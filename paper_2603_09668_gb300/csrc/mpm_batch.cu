@@ -282,6 +282,12 @@ __global__ void __launch_bounds__(THREADS) k_batch_particles(BatchView A, int L)
 // work item (b PAIR_WARPS + w) >> 1: up to 64 particles of one scene. Each
 // warp stages its scene record in shared memory, so that the scene's
 // parameters are shared-memory operands, and the material is chosen per warp.
+// 128 registers and 16 warps per SM: with both materials in one kernel, 96
+// registers spill (64 scenes of 20k to 400k particles, 30 substeps: 34.8 ms
+// against 30.9; one-warp CTAs 31.4; 168 registers, 12 warps 35.0).
+constexpr int PAIR_THREADS = 128;
+constexpr int PAIR_WARPS = PAIR_THREADS / 32;
+constexpr int PAIR_MIN_CTAS = 4;
 template <bool VEC>
 __global__ void __launch_bounds__(PAIR_THREADS, PAIR_MIN_CTAS) k_batch_pair(BatchView A, int L) {
     constexpr int WORDS = sizeof(BatchScene) / 4;

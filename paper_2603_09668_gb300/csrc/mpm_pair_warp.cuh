@@ -27,10 +27,16 @@ namespace dw {
 //   Active blocks of the next grid are marked for every run's first particle,
 //   eight lanes per run; the flags of the first four runs are loaded before
 //   the passes and tested after them.
-constexpr int PAIR_THREADS = 128;
-constexpr int PAIR_WARPS = PAIR_THREADS / 32;
-// resident CTAs per SM the launch bounds ask for: 96 registers per thread
-constexpr int PAIR_MIN_CTAS = 65536 / (96 * PAIR_THREADS);
+//
+// What bounds it: latency. 20 warps fit an SM (96 registers, 10 KB of shared
+// memory each) and issue in half of the cycles; the FP32 pipes are busy a third
+// of the time. Steps that shortened the instruction stream, per launch of the
+// 400k sheet (128^3): 33.6 us at first; the single-scene kernel as one-warp
+// CTAs 32.2 (a CTA's slot is free again when its own warp ends, which matters
+// for the last, partly filled round of CTAs); the runs' first particles picked
+// from the ballot masks by clearing bits instead of __fns 31.3; the box staged
+// by 4-byte asynchronous copies and a split lane's second row taken from the
+// pair's own products 31.0.
 constexpr unsigned FULL = 0xffffffffu;
 
 template <bool VEC>
@@ -141,6 +147,10 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -247,11 +257,14 @@ __device__ __forceinline__ void pair_warp(
                 const int rem = i - iz * exy;
                 const int iy = (int)(((float)rem + 0.5f) * inv_ex);
                 const int ix = rem - iy * ex;
-                const float4 g = grid_v[((lo[2] + iz) * N + (lo[1] + iy)) * N + (lo[0] + ix)];
-                ws.g.box[i] = g.x;
-                ws.g.box[BOX_MAX + i] = g.y;
-                ws.g.box[2 * BOX_MAX + i] = g.z;
+                const float *g = reinterpret_cast<const float *>(
+                    grid_v + ((lo[2] + iz) * N + (lo[1] + iy)) * N + (lo[0] + ix));
+                cp_async4(&ws.g.box[i], g);
+                cp_async4(&ws.g.box[BOX_MAX + i], g + 1);
+                cp_async4(&ws.g.box[2 * BOX_MAX + i], g + 2);
             }
+            cp_async_commit();
+            cp_async_wait_all();
             __syncwarp();
             const int o0 = g0ok ? ((s.b0[2] - lo[2]) * ey + (s.b0[1] - lo[1])) * ex + (s.b0[0] - lo[0]) : 0;
             const int o1 = g1ok ? ((s.b1[2] - lo[2]) * ey + (s.b1[1] - lo[1])) * ex + (s.b1[0] - lo[0]) : 0;
@@ -376,12 +389,7 @@ __device__ __forceinline__ void pair_warp(
     const unsigned smask = __ballot_sync(FULL, split);
     const int pos = lane + __popc(smask & ((1u << lane) - 1u));  // this lane's row
     const int R = 32 + __popc(smask);
-    float w2y[3];  // the second particle's z weights, kept out of the summed row when split
-#pragma unroll
-    for (int o = 0; o < 3; ++o) {
-        w2y[o] = t.w[2][o].y;
-        if (split) t.w[2][o].y = 0.0f;
-    }
+    const float keep = split ? 0.0f : 1.0f;  // the second particle's share of the lane's row
     uint64_t ends;
     bool st_main;
     {
@@ -412,30 +420,34 @@ __device__ __forceinline__ void pair_warp(
     // particle, four runs at a time (eight lanes per run, one block per lane).
     // The flags of the first four runs are loaded now and tested after the
     // passes, so that the loads' latency overlaps them.
-    const unsigned m0 = __ballot_sync(FULL, st_main && nk0 >= 0), m1 = smask;
-    const int n0 = __popc(m0), nr = n0 + __popc(m1);
-    auto mark_id = [&](int j0) {
-        const int j = j0 + (lane >> 3);
-        int src = 0, h = 0;
-        if (j < nr) {
-            if (j < n0) {
-                src = __fns(m0, 0, j + 1);
-            } else {
-                src = __fns(m1, 0, j - n0 + 1);
-                h = 1;
-            }
-        }
+    unsigned m0 = __ballot_sync(FULL, st_main && nk0 >= 0), m1 = smask;  // runs not yet marked
+    auto mark_id = [&]() {
+        const int n0 = __popc(m0), j = lane >> 3;
+        const bool h = j >= n0;
+        unsigned m = h ? m1 : m0;
+        const int c = h ? j - n0 : j;  // its c lowest bits are other groups' runs
+        if (c > 0) m &= m - 1u;
+        if (c > 1) m &= m - 1u;
+        if (c > 2) m &= m - 1u;
+        const int src = m ? __ffs(m) - 1 : 0;
         const int c0 = __shfl_sync(FULL, t.b0[0], src), c1 = __shfl_sync(FULL, t.b0[1], src),
                   c2 = __shfl_sync(FULL, t.b0[2], src);
         const int d0 = __shfl_sync(FULL, t.b1[0], src), d1 = __shfl_sync(FULL, t.b1[1], src),
                   d2 = __shfl_sync(FULL, t.b1[2], src);
-        if (j >= nr) return -1;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (m0)
+                m0 &= m0 - 1u;
+            else
+                m1 &= m1 - 1u;
+        }
+        if (m == 0u) return -1;
         return h ? stencil_block(ab_next, d0, d1, d2, lane & 7)
                  : stencil_block(ab_next, c0, c1, c2, lane & 7);
     };
     int mid = -1, mflag = 1;
     if (ab_next.flags) {
-        mid = mark_id(0);
+        mid = mark_id();
         if (mid >= 0) mflag = *(volatile int *)&ab_next.flags[mid];
     }
     const float2 pm = s2(P.p_mass);
@@ -443,14 +455,12 @@ __device__ __forceinline__ void pair_warp(
 #pragma unroll 1
     for (int ok = 0; ok < 3; ++ok) {
         const float2 wz = ok == 0 ? t.w[2][0] : (ok == 1 ? t.w[2][1] : t.w[2][2]);
-        const float wz1 = ok == 0 ? w2y[0] : (ok == 1 ? w2y[1] : w2y[2]);
         float2 rz[3];  // r0 + ok sz
 #pragma unroll
         for (int c = 0; c < 3; ++c) rz[c] = ok == 0 ? r0[c] : fma(s2((float)ok), sz[c], r0[c]);
 #pragma unroll
         for (int oj = 0; oj < 3; ++oj) {
             const float2 wyz = mul(t.w[1][oj], wz);
-            const float wyz1 = t.w[1][oj].y * wz1;
             float2 b[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -469,13 +479,9 @@ __device__ __forceinline__ void pair_warp(
                 const float2 Wm = mul(W, pm), v0p = mul(W, bb[0]), v1p = mul(W, bb[1]),
                              v2p = mul(W, bb[2]);
                 ws.rows[pos][3 * oj + oi] =
-                    make_float4(Wm.x + Wm.y, v0p.x + v0p.y, v1p.x + v1p.y, v2p.x + v2p.y);
-                if (smask) {
-                    const float W1 = t.w[0][oi].y * wyz1;
-                    if (split)
-                        ws.rows[pos + 1][3 * oj + oi] = make_float4(W1 * P.p_mass, W1 * bb[0].y,
-                                                                    W1 * bb[1].y, W1 * bb[2].y);
-                }
+                    make_float4(fmaf(Wm.y, keep, Wm.x), fmaf(v0p.y, keep, v0p.x),
+                                fmaf(v1p.y, keep, v1p.x), fmaf(v2p.y, keep, v2p.x));
+                if (split) ws.rows[pos + 1][3 * oj + oi] = make_float4(Wm.y, v0p.y, v1p.y, v2p.y);
             }
         }
         __syncwarp();
@@ -490,8 +496,8 @@ __device__ __forceinline__ void pair_warp(
     if (ab_next.flags) {
         if (mid >= 0 && mflag == 0 && atomicExch(&ab_next.flags[mid], 1) == 0)
             ab_next.list[atomicAdd(ab_next.count, 1)] = ab_next.tag | mid;
-        for (int j0 = 4; j0 < nr; j0 += 4) {
-            const int id = mark_id(j0);
+        while (m0 | m1) {
+            const int id = mark_id();
             if (id >= 0) mark_block(ab_next, id);
         }
     }

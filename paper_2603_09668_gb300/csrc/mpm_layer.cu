@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(LAYER_THREADS) k_layer_p2g(
             }
 #pragma unroll
             for (int a = 0; a < 3; ++a) mv[a] = P.p_mass * v[a * n + p];
-            if (!layer_stress(P, Fp, Cp, A)) atomicOr(err, ERRBIT_INVERTED);
+            if (!p2g_affine(P, Fp, Cp, A)) atomicOr(err, ERRBIT_INVERTED);
             key = stencil_node(P, s);
         } else if (live) {
             atomicOr(err, ERRBIT_DOMAIN);
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(LAYER_THREADS, LAYER_FWD_CTAS) k_layer_g2p(
 #pragma unroll
             for (int a = 0; a < 3; ++a) mv[a] = P.p_mass * vn[a];
             if (make_stencil(P, xp[0], xp[1], xp[2], s) && live) {
-                if (!layer_stress(P, Fn, Cn, A)) atomicOr(err, ERRBIT_INVERTED);
+                if (!p2g_affine(P, Fn, Cn, A)) atomicOr(err, ERRBIT_INVERTED);
                 key = stencil_node(P, s);
             } else if (live) {
                 atomicOr(err, ERRBIT_DOMAIN);

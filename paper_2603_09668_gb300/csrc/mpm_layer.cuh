@@ -77,37 +77,6 @@ __device__ __forceinline__ void layer_mul3(const float A[9], const float B[9], f
                                      __fmaf_rn(A[3 * i + 1], B[3 + j], __fmul_rn(A[3 * i], B[j])));
 }
 
-// Affine momentum matrix A = -dt V0 (4/dx^2) P F^T + m C, rounded operation by
-// operation as in the paired kernels (affine2), so that a scene's states do
-// not depend on which of them its size takes it to (a batch runs the paired
-// one). Returns false (P = 0) for det F <= 0.
-__device__ __forceinline__ bool layer_stress(const MpmParams &P, const float F[9], const float C[9],
-                                             float A[9]) {
-    if (P.material != DW_NEOHOOKEAN) return p2g_affine(P, F, C, A);
-    float K[9];
-    const int r[9][4] = {{4, 8, 5, 7}, {5, 6, 3, 8}, {3, 7, 4, 6}, {2, 7, 1, 8}, {0, 8, 2, 6},
-                         {1, 6, 0, 7}, {1, 5, 2, 4}, {2, 3, 0, 5}, {0, 4, 1, 3}};
-#pragma unroll
-    for (int k = 0; k < 9; ++k)
-        K[k] = __fmaf_rn(-F[r[k][2]], F[r[k][3]], __fmul_rn(F[r[k][0]], F[r[k][1]]));
-    const float J = __fmaf_rn(F[2], K[2], __fmaf_rn(F[1], K[1], __fmul_rn(F[0], K[0])));
-    const bool ok = J > 0.0f;
-    const float inv = ok ? 1.0f / J : 0.0f, lnJ = ok ? logf(J) : 0.0f, mu = ok ? P.mu : 0.0f;
-    const float c = __fadd_rn(__fmul_rn(P.lam, lnJ), -mu);
-    float Pk[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Pk[k] = __fmaf_rn(c, __fmul_rn(K[k], inv), __fmul_rn(mu, F[k]));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float t = __fmaf_rn(Pk[3 * i + 2], F[3 * j + 2],
-                                      __fmaf_rn(Pk[3 * i + 1], F[3 * j + 1], __fmul_rn(Pk[3 * i], F[3 * j])));
-            A[3 * i + j] = __fmaf_rn(-P.kappa, t, __fmul_rn(P.p_mass, C[3 * i + j]));
-        }
-    return ok;
-}
-
 // A particle's node value is W (m, r + ox sx + oy sy) in layer k, with
 // r = m v - A fx dx + k sz and s the columns of A times dx.
 struct LayerAffine {

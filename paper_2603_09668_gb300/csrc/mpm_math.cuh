@@ -100,23 +100,34 @@ __device__ __forceinline__ void mul3_atb(const float A[9], const float B[9], flo
             C[3 * i + j] = A[i] * B[j] + A[3 + i] * B[3 + j] + A[6 + i] * B[6 + j];
 }
 
-// Polar factor R of F (det F > 0) by Newton's iteration; false if det <= 0.
+// Cofactor matrix with explicit fused operations.
+__device__ __forceinline__ void cof3_fma(const float A[9], float K[9]) {
+    const int r[9][4] = {{4, 8, 5, 7}, {5, 6, 3, 8}, {3, 7, 4, 6}, {2, 7, 1, 8}, {0, 8, 2, 6},
+                         {1, 6, 0, 7}, {1, 5, 2, 4}, {2, 3, 0, 5}, {0, 4, 1, 3}};
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+        K[k] = __fmaf_rn(-A[r[k][2]], A[r[k][3]], __fmul_rn(A[r[k][0]], A[r[k][1]]));
+}
+
+// Polar factor R of F (det F > 0) by Newton's iteration R <- (R + R^-T) / 2;
+// false if a determinant is <= 0. The operations round as those of polar_R2
+// (mpm_pair.cuh), which runs it for two particles at once.
 __device__ __forceinline__ bool polar_R(const float F[9], float R[9]) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) R[k] = F[k];
     bool converged = false;
     for (int it = 0; it < 40; ++it) {
         float K[9];
-        cof3(R, K);
-        float J = det3(R);
+        cof3_fma(R, K);
+        const float J = __fmaf_rn(R[2], K[2], __fmaf_rn(R[1], K[1], __fmul_rn(R[0], K[0])));
         if (!(J > 0.0f)) return false;
-        float inv = 1.0f / J;
+        const float hinv = 0.5f / J;
         float change = 0.0f, norm = 0.0f;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            float xn = 0.5f * (R[k] + K[k] * inv);
-            change += (xn - R[k]) * (xn - R[k]);
-            norm += xn * xn;
+            const float xn = __fmaf_rn(K[k], hinv, __fmul_rn(0.5f, R[k])), d = xn - R[k];
+            change = __fmaf_rn(d, d, change);
+            norm = __fmaf_rn(xn, xn, norm);
             R[k] = xn;
         }
         if (converged) break;                    // one more step after the test passes
@@ -150,6 +161,52 @@ __device__ __forceinline__ bool stress_P(const MpmParams &P, const float F[9], f
         for (int k = 0; k < 9; ++k) Pk[k] = 2.0f * P.mu * (F[k] - R[k]) + P.lam * (J - 1.0f) * K[k];
     }
     return true;
+}
+
+// Kirchhoff stress tau = P F^T, without P: F^-T F^T = I and cof(F) F^T = J I, so
+//   Neo-Hookean:      tau = mu F F^T + (lam ln J - mu) I
+//   fixed-corotated:  tau = 2 mu (F - R) F^T + lam (J - 1) J I,
+// which needs no cofactors beyond J's and one product of matrices. Written
+// with explicit fused operations in the order of the paired kernels
+// (affine2), so that a scene's states do not depend on the kernel its size
+// takes it to. Returns false (tau = 0) for det F <= 0.
+__device__ __forceinline__ bool stress_tau(const MpmParams &P, const float F[9], float tau[9]) {
+    const float k0 = __fmaf_rn(-F[5], F[7], __fmul_rn(F[4], F[8])),
+                k1 = __fmaf_rn(-F[3], F[8], __fmul_rn(F[5], F[6])),
+                k2 = __fmaf_rn(-F[4], F[6], __fmul_rn(F[3], F[7]));
+    const float J = __fmaf_rn(F[2], k2, __fmaf_rn(F[1], k1, __fmul_rn(F[0], k0)));
+    const bool ok = J > 0.0f;
+    if (P.material == DW_NEOHOOKEAN) {
+        const float mu = ok ? P.mu : 0.0f;
+        const float c = __fmaf_rn(P.lam, ok ? logf(J) : 0.0f, -mu);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) {
+                const float b = __fmaf_rn(F[3 * i + 2], F[3 * j + 2],
+                                          __fmaf_rn(F[3 * i + 1], F[3 * j + 1], __fmul_rn(F[3 * i], F[3 * j])));
+                tau[3 * i + j] = i == j ? __fmaf_rn(mu, b, c) : __fmul_rn(mu, b);
+                tau[3 * j + i] = tau[3 * i + j];
+            }
+    } else if (ok) {
+        float R[9];
+        polar_R(F, R);
+        const float mu2 = 2.0f * P.mu, c = __fmul_rn(__fmul_rn(P.lam, J - 1.0f), J);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) R[k] = __fmul_rn(mu2, F[k] - R[k]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float b = __fmaf_rn(R[3 * i + 2], F[3 * j + 2],
+                                          __fmaf_rn(R[3 * i + 1], F[3 * j + 1], __fmul_rn(R[3 * i], F[3 * j])));
+                tau[3 * i + j] = i == j ? __fadd_rn(b, c) : b;
+            }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) tau[k] = 0.0f;
+    }
+    return ok;
 }
 
 __device__ __forceinline__ void cross3(const float a[3], const float b[3], float c[3]) {

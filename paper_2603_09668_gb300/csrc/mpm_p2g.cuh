@@ -48,11 +48,10 @@ __device__ __forceinline__ void mark_stencil_blocks(const ActiveBlocks &ab, cons
 // Affine momentum matrix A = -dt V0 (4/dx^2) P F^T + m C of one particle.
 __device__ __forceinline__ bool p2g_affine(const MpmParams &P, const float F[9], const float C[9],
                                            float A[9]) {
-    float Pk[9], PFt[9];
-    bool ok = stress_P(P, F, Pk);
-    mul3_abt(Pk, F, PFt);
+    float tau[9];
+    const bool ok = stress_tau(P, F, tau);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) A[k] = -P.kappa * PFt[k] + P.p_mass * C[k];
+    for (int k = 0; k < 9; ++k) A[k] = __fmaf_rn(-P.kappa, tau[k], __fmul_rn(P.p_mass, C[k]));
     return ok;
 }
 

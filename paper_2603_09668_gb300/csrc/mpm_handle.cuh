@@ -139,14 +139,14 @@ dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *
 
 // The layer-split kernels (mpm_layer.cu) and the particle counts up to which
 // they are the faster ones (measured, us): a fused launch with its grid update
-// 8.2 against 14.5 at 5,504 particles, 9.2 / 13.2 at 20,000, 13.5 / 13.4 at
-// 40,000 of a sheet, 11.2 / 18.2 at 20,000 and 18.0 / 17.4 at 50,000 of a
-// block; the P2G alone 5 against 13 at 5,504, a whole substep 26.2 / 26.7 at
-// 100,000 and 41 / 40 at 200,000 of a block. Without the paired kernel's vector
-// loads (vec, see mpm_rollout) it loses longer: 16.1 / 16.3 at 65,535 of a
-// sheet, 25.6 / 34.2 of a block on 128^3, 20.1 / 18.0 at 100,001 of a sheet.
+// 7.9 against 11.9 at 5,504 particles, 9.4 / 11.6 at 32,768, 11.5 / 11.7 at
+// 38,912, 12.3 / 11.5 at 40,960, 14.3 / 12.5 at 49,151 of a sheet; 13.7 / 15.6 at
+// 38,912, 15.0 / 15.3 at 40,960, 18.9 / 17.3 at 65,535 of a block. The fused
+// line lies where the layer kernel's CTAs (32 particles, eight per SM on 152
+// SMs) no longer run all at once. The P2G alone takes 5 against 13 at 5,504, a
+// whole substep 26.2 / 26.7 at 100,000 and 41 / 40 at 200,000 of a block.
 constexpr int64_t LAYER_MAX_P2G = 1 << 17, LAYER_MAX_G2P = 1 << 17;
-inline bool layer_fused(int64_t n, bool vec) { return n <= (vec ? 1 << 15 : 1 << 16); }
+inline bool layer_fused(int64_t n) { return n <= 32 * 8 * 152; }
 dw_status launch_layer_p2g(const MpmParams &P, const float *x, const float *v, const float *C,
                            const float *F, int64_t n, float4 *grid, int *err,
                            const ActiveBlocks &ab, cudaStream_t st);

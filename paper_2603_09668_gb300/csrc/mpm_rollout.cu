@@ -158,7 +158,7 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
                          ((reinterpret_cast<uintptr_t>(in.x) | reinterpret_cast<uintptr_t>(in.F) |
                            reinterpret_cast<uintptr_t>(out.x) | reinterpret_cast<uintptr_t>(out.F)) %
                               16 == 0);
-        if (layer_fused(n, vec)) {
+        if (layer_fused(n)) {
             st = launch_layer_g2p2g(h->P, in.x, in.F, pinned, h->grid_v, out, h->grid_mp, n, h->err,
                                     active_blocks(h, 1 - L), h->block_count + L, nullptr, nullptr, s);
             if (st != DW_OK) return st;
@@ -256,7 +256,7 @@ extern "C" dw_status mpm_rollout(dw_mpm h, const dw_mpm_state *state, uint8_t *p
             // multiple of 4, 16-byte aligned arrays)
             const bool pair_vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(cur.x) |
                                                     reinterpret_cast<uintptr_t>(cur.F)) % 16 == 0);
-            if (pair && layer_fused(n, pair_vec)) {
+            if (pair && layer_fused(n)) {
                 const bool keys = sort_every > 0 && (k + 1) % sort_every == 0;
                 const dw_mpm_state out{cur.x, nullptr, nullptr, cur.F, n};  // v and C are not kept
                 st = launch_layer_g2p2g(h->P, cur.x, cur.F, cur_pin, h->grid_v, out, h->grid_mp, n,

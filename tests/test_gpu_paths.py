@@ -61,8 +61,9 @@ def _dev(st):
 
 
 # The layer-split kernels (P2G and G2P up to 2^17 particles, the fused kernel up
-# to 2^15, 2^16 for counts not a multiple of 4) against the one-particle-per-thread kernels, around the CTA's 32
-# particles and the rules' edges. The same formulas summed in another order:
+# to 38,912) and the paired kernel above them, with and without vector loads,
+# against the one-particle-per-thread kernels, around the CTA's 32 particles and
+# the rules' edges. The same formulas summed in another order:
 # the bounds of the paired kernels' test (x, F 1e-5; v, C 1e-3 of the largest).
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 95, 1000, 32768, 32772, 65535, 65537, 131072, 131073])
 @pytest.mark.parametrize("material,sort_every", [(0, 0), (1, 3)])
@@ -89,6 +90,11 @@ def test_layer_split_forward(n, material, sort_every):
         assert (got[0][k] - got[1][k]).abs().max().item() <= tol
     for k in (1, 2):
         assert (got[0][k] - got[1][k]).abs().max() <= 1e-3 * got[1][k].abs().max()
+
+
+@pytest.mark.parametrize("n", [38912, 38913, 38916])
+def test_fused_layer_split_at_the_rule(n):
+    test_layer_split_forward(n, 0, 3)
 
 
 def test_layer_split_reports_a_particle_off_the_grid():

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(THREADS) k_batch_particles(BatchView A, int L)
 constexpr int PAIR_THREADS = 128;
 constexpr int PAIR_WARPS = PAIR_THREADS / 32;
 constexpr int PAIR_MIN_CTAS = 4;
-template <bool VEC, bool OUT>
+template <bool VEC>
 __global__ void __launch_bounds__(PAIR_THREADS, PAIR_MIN_CTAS) k_batch_pair(BatchView A, int L) {
     constexpr int WORDS = sizeof(BatchScene) / 4;
     __shared__ PairWarpSmem smem[PAIR_WARPS];
@@ -304,10 +304,10 @@ __global__ void __launch_bounds__(PAIR_THREADS, PAIR_MIN_CTAS) k_batch_pair(Batc
     const ActiveBlocks ab{S.flags, A.list + (size_t)(1 - L) * A.list_cap, A.count + (1 - L), S.nb,
                           item.x << BATCH_SCENE_SHIFT};
     const int64_t first = item.y;
-    pair_warp<-1, false, VEC, OUT>(S.P, A.x, A.v, A.C, A.F, A.pinned, S.grid_v, S.grid_mp, A.n,
+    pair_warp<-1, false, VEC>(S.P, A.x, A.v, A.C, A.F, A.pinned, S.grid_v, S.grid_mp, A.n,
                               first + (hw & 1) * 64, first + item.z, A.err, ab,
                               blockIdx.x == 0 && threadIdx.x == 0 ? A.count + L : nullptr,
-                              smem[wid], PairOut{A.ox, A.ov, A.oC, A.oF});
+                              smem[wid]);
 }
 
 // P2G of every scene from a complete state (start of a segment), list L.
@@ -651,21 +651,12 @@ static int occupancy_of(dw_mpm_batch h, int threads, bool final_) {
     return h->occupancy[threads == 256 ? 1 : 0][final_ ? 1 : 0];
 }
 
-// Whether the pair kernel may load x and F as float2 and in 16-byte pieces
-// (and, where it writes the whole state to q, store v and C as float2).
-static bool pair_vec(dw_mpm_batch h, const dw_mpm_state &q) {
-    return h->items_aligned4 && ((reinterpret_cast<uintptr_t>(q.x) | reinterpret_cast<uintptr_t>(q.F) |
-                                  reinterpret_cast<uintptr_t>(q.v) | reinterpret_cast<uintptr_t>(q.C)) %
-                                     16 ==
-                                 0);
-}
-
 // One substep launch (or two in split and pair mode). vec: the pair kernel
 // may load x and F as float2 and 16-byte pieces.
 static dw_status launch_substep(dw_mpm_batch h, const BatchView &A, const dw_batch_config &c,
                                 int k, int L, bool final_, cudaStream_t s, bool vec = false) {
     const int T = c.threads;
-    if (c.mode == DW_BATCH_PAIR && !final_) {
+    if (c.mode == DW_BATCH_PAIR && !final_ && !A.ox) {
         const unsigned ggrid = (unsigned)(c.ctas_per_sm * h->num_sms);
         // PAIR_WARPS halves of 128-particle work items per CTA
         const unsigned pgrid = (unsigned)((2 * h->n_items + PAIR_WARPS - 1) / PAIR_WARPS);
@@ -673,9 +664,8 @@ static dw_status launch_substep(dw_mpm_batch h, const BatchView &A, const dw_bat
             DW_CUDA(launch_pdl(k_batch_grid<256>, ggrid, 256, s, A, k, L));
         else
             DW_CUDA(launch_pdl(k_batch_grid<128>, ggrid, 128, s, A, k, L));
-        auto kern = A.ox ? (vec ? k_batch_pair<true, true> : k_batch_pair<false, true>)
-                         : (vec ? k_batch_pair<true, false> : k_batch_pair<false, false>);
-        DW_CUDA(launch_pdl(kern, pgrid, PAIR_THREADS, s, A, L));
+        DW_CUDA(vec ? launch_pdl(k_batch_pair<true>, pgrid, PAIR_THREADS, s, A, L)
+                    : launch_pdl(k_batch_pair<false>, pgrid, PAIR_THREADS, s, A, L));
         return DW_OK;
     }
     if (c.mode == DW_BATCH_PERSISTENT) {
@@ -723,7 +713,10 @@ static dw_status enqueue_rollout(dw_mpm_batch h, const dw_mpm_state *state, uint
     };
     // pair kernel vector loads: every work item starts at a multiple of 4
     // particles and the arrays are 16-byte aligned
-    auto vec_of = [&](const dw_mpm_state &q) { return pair_vec(h, q); };
+    auto vec_of = [&](const dw_mpm_state &q) {
+        return h->items_aligned4 &&
+               ((reinterpret_cast<uintptr_t>(q.x) | reinterpret_cast<uintptr_t>(q.F)) % 16 == 0);
+    };
     if (sort_every > 0) {
         dw_status st = resort(true);  // the input state's v and C feed the first P2G
         if (st != DW_OK) return st;
@@ -1267,10 +1260,11 @@ static dw_status enqueue_segment_adjoint(dw_mpm_batch h, const dw_mpm_state *sta
                 A.gtape_count = h->gtape_count + k;
             }
             const bool final_ = k + 2 == n_substeps;
-            // (in pair mode the paired kernel: 10.25 ms against 10.41 with one
-            // particle per thread, 16 scenes)
-            st = launch_substep(h, A, h->cfg, k, L, final_, s,
-                                pair_vec(h, o) && (k > 0 || pair_vec(h, *start)));
+            // one particle per thread also in pair mode: the reverse pass then
+            // meets the states of the single-scene adjoint's WARP kernels bit for
+            // bit (an isolated particle's dL/dx is ill-conditioned); the paired
+            // kernel's recompute gained 1.5%
+            st = launch_substep(h, A, h->cfg, k, L, final_, s);
             if (st != DW_OK) return st;
             if (!final_) L = 1 - L;
         }

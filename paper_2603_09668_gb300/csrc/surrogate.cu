@@ -84,60 +84,17 @@ __global__ void k_surr_weights(const float *__restrict__ params, bf16 *__restric
     wd[woff + ((((int64_t)(t2 % 9) * (cout / 8) + co / 8) * 3 + t2 / 9) * cin + ci) * 8 + (co & 7)] = w;
 }
 
-__device__ __constant__ int kCX[19] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 1, -1, 1, -1, 0, 0};
-__device__ __constant__ int kCY[19] = {0, 0, 0, 1, -1, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 1, -1};
-__device__ __constant__ int kCZ[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 1, -1, 1, -1, 0, 0, -1, 1, -1, 1};
+// (constexpr, so that the unrolled loops see the values: read as constants, each
+// costs a load and an integer conversion per use)
+__device__ constexpr int kCX[19] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 1, -1, 1, -1, 0, 0};
+__device__ constexpr int kCY[19] = {0, 0, 0, 1, -1, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 1, -1};
+__device__ constexpr int kCZ[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 1, -1, 1, -1, 0, 0, -1, 1, -1, 1};
 
-// Fine rho and u of every cell of a shifted (2n)^3 lattice (solid: rho 1, u 0).
-__global__ void k_surr_fine(const float *__restrict__ f, const uint8_t *__restrict__ solid, int N,
-                            float *__restrict__ fine) {
-    const int64_t nc = (int64_t)N * N * N;
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nc) return;
-    float r = 1.0f, ux = 0.0f, uy = 0.0f, uz = 0.0f;
-    if (!(solid && solid[c])) {
-        float rs = 0.0f, jx = 0.0f, jy = 0.0f, jz = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const float fi = f[(size_t)i * nc + c];
-            rs += fi;
-            jx += (float)kCX[i] * fi;
-            jy += (float)kCY[i] * fi;
-            jz += (float)kCZ[i] * fi;
-        }
-        r = 1.0f + rs;
-        ux = jx / r;
-        uy = jy / r;
-        uz = jz / r;
-    }
-    fine[c] = r;
-    fine[nc + c] = ux;
-    fine[2 * nc + c] = uy;
-    fine[3 * nc + c] = uz;
-}
-
-// Coarse features: 2x2x2 averages over fluid cells of (rho - 1, u), solid fraction.
-__global__ void k_surr_coarse(const float *__restrict__ fine, const uint8_t *__restrict__ solid,
-                              int n, float in_scale, float3 uref, bf16 *__restrict__ feats,
-                              float *__restrict__ feats32) {
-    const int64_t nv = (int64_t)n * n * n;
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nv) return;
-    const int N = 2 * n;
-    const int64_t nc = (int64_t)N * N * N;
-    const int x = (int)(v % n), y = (int)((v / n) % n), z = (int)(v / ((int64_t)n * n));
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-    int fluid = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int64_t c = ((int64_t)(2 * z + (k >> 2)) * N + (2 * y + ((k >> 1) & 1))) * N + 2 * x + (k & 1);
-        if (solid && solid[c]) continue;
-        ++fluid;
-        s[0] += fine[c] - 1.0f;
-        s[1] += fine[nc + c];
-        s[2] += fine[2 * nc + c];
-        s[3] += fine[3 * nc + c];
-    }
+// Features of coarse voxel v from the sums over its `fluid` fluid cells of
+// (rho - 1, u): averages, solid fraction, reference velocity.
+__device__ __forceinline__ void store_features(const float s[4], int fluid, float in_scale, float3 uref,
+                                               int64_t nv, int64_t v, bf16 *__restrict__ feats,
+                                               float *__restrict__ feats32) {
     const float inv = fluid > 0 ? in_scale / (float)fluid : 0.0f;
     // velocity relative to the reference velocity, which itself fills channels 5-7
     const float r1 = fluid > 0 ? s[1] * inv - uref.x * in_scale : 0.0f;
@@ -164,6 +121,108 @@ __global__ void k_surr_coarse(const float *__restrict__ fine, const uint8_t *__r
         d32[2] = make_float4(0.f, 0.f, 0.f, 0.f);
         d32[3] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+}
+
+// Fine (rho, u) of every cell of a shifted (2n)^3 lattice (solid: rho 1, u 0)
+// and the coarse features: a block takes 32 coarse voxels, its warp k the k-th
+// of their four rows of cell pairs; warp 0 then adds up each voxel's eight
+// cells in order. Bound by the populations' 76 B a cell. PAIRS: f is 8-byte
+// aligned (two populations per load), solid 2-byte. 41 us at 128^3 cells and 112
+// at 192^3; 46 and 130 as two kernels, the second reading the fine state back,
+// with the directions' components read as integers from constant memory; 46 and
+// 109 with a thread per voxel walking the four rows (64^3 voxels then just
+// exceed one round of blocks).
+template <bool PAIRS>
+__global__ void __launch_bounds__(128) k_surr_features(const float *__restrict__ f,
+                                                       const uint8_t *__restrict__ solid, int n,
+                                                       float in_scale, float3 uref, float *__restrict__ fine,
+                                                       bf16 *__restrict__ feats, float *__restrict__ feats32) {
+    __shared__ float val[8][4][32];  // per cell of a voxel: rho - 1, u
+    __shared__ unsigned char wet[8][32];
+    const int64_t nv = (int64_t)n * n * n, nc = 8 * nv;  // nv is a multiple of 32: n is one of 16
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t v = (int64_t)blockIdx.x * 32 + lane;
+    const int N = 2 * n;
+    const int x = (int)(v % n), y = (int)((v / n) % n), z = (int)(v / ((int64_t)n * n));
+    const int64_t c = ((int64_t)(2 * z + (k >> 1)) * N + (2 * y + (k & 1))) * N + 2 * x;
+    bool sol[2] = {false, false};
+    if (solid) {
+        if (PAIRS) {
+            const uchar2 q = *reinterpret_cast<const uchar2 *>(solid + c);
+            sol[0] = q.x != 0;
+            sol[1] = q.y != 0;
+        } else {
+            sol[0] = solid[c] != 0;
+            sol[1] = solid[c + 1] != 0;
+        }
+    }
+    float m[2][4] = {};  // rho - 1, momentum
+    if (!(sol[0] && sol[1])) {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            const float *fi = f + (size_t)i * nc + c;
+            const float2 q = PAIRS ? *reinterpret_cast<const float2 *>(fi) : make_float2(fi[0], fi[1]);
+            const float a[2] = {q.x, q.y};
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                m[j][0] += a[j];
+                m[j][1] += (float)kCX[i] * a[j];
+                m[j][2] += (float)kCY[i] * a[j];
+                m[j][3] += (float)kCZ[i] * a[j];
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float r = 1.0f + m[j][0];
+        m[j][0] = sol[j] ? 1.0f : r;
+#pragma unroll
+        for (int a = 1; a < 4; ++a) m[j][a] = sol[j] ? 0.0f : m[j][a] / r;
+        wet[2 * k + j][lane] = !sol[j];
+        val[2 * k + j][0][lane] = m[j][0] - 1.0f;
+#pragma unroll
+        for (int a = 1; a < 4; ++a) val[2 * k + j][a][lane] = m[j][a];
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        *reinterpret_cast<float2 *>(fine + a * nc + c) = make_float2(m[0][a], m[1][a]);
+    __syncthreads();
+    if (k != 0) return;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    int fluid = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (!wet[j][lane]) continue;
+        ++fluid;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) s[a] += val[j][a][lane];
+    }
+    store_features(s, fluid, in_scale, uref, nv, v, feats, feats32);
+}
+
+// The coarse features from the fine state.
+__global__ void k_surr_coarse(const float *__restrict__ fine, const uint8_t *__restrict__ solid,
+                              int n, float in_scale, float3 uref, bf16 *__restrict__ feats,
+                              float *__restrict__ feats32) {
+    const int64_t nv = (int64_t)n * n * n;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= nv) return;
+    const int N = 2 * n;
+    const int64_t nc = (int64_t)N * N * N;
+    const int x = (int)(v % n), y = (int)((v / n) % n), z = (int)(v / ((int64_t)n * n));
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    int fluid = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int64_t c = ((int64_t)(2 * z + (k >> 2)) * N + (2 * y + ((k >> 1) & 1))) * N + 2 * x + (k & 1);
+        if (solid && solid[c]) continue;
+        ++fluid;
+        s[0] += fine[c] - 1.0f;
+        s[1] += fine[nc + c];
+        s[2] += fine[2 * nc + c];
+        s[3] += fine[3 * nc + c];
+    }
+    store_features(s, fluid, in_scale, uref, nv, v, feats, feats32);
 }
 
 // Channels-last FP32 [nv][16] -> planar BF16 [2][nv][8] (the layout of the
@@ -509,8 +568,9 @@ __global__ void k_surr_write_lattice(const float *__restrict__ fine, const uint8
                                      int64_t nc, float *__restrict__ f) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nc) return;
-    if (solid && solid[c]) return;
+    const bool skip = solid && solid[c];  // beside the loads below, not before them
     const float rho = fine[c], ux = fine[nc + c], uy = fine[2 * nc + c], uz = fine[3 * nc + c];
+    if (skip) return;
     const float uu = 1.5f * (ux * ux + uy * uy + uz * uz);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
@@ -920,11 +980,9 @@ extern "C" dw_status surr_features(dw_surr h, const float *f, const uint8_t *sol
                                    float in_scale, float *feats32, dw_stream stream) {
     DW_REQUIRE(h && f, "handle and f must not be NULL");
     cudaStream_t s = as_stream(stream);
-    const int N = 2 * h->n;
-    const int64_t nc = (int64_t)N * N * N;
-    k_surr_fine<<<grid_for(nc, 256), 256, 0, s>>>(f, solid, N, h->fine);
-    k_surr_coarse<<<grid_for(h->nv, 256), 256, 0, s>>>(h->fine, solid, h->n, in_scale,
-                                                       uref_of(h), h->feats, feats32);
+    const bool pairs = reinterpret_cast<uintptr_t>(f) % 8 == 0 && reinterpret_cast<uintptr_t>(solid) % 2 == 0;
+    auto kern = pairs ? k_surr_features<true> : k_surr_features<false>;
+    kern<<<(unsigned)(h->nv / 32), 128, 0, s>>>(f, solid, h->n, in_scale, uref_of(h), h->fine, h->feats, feats32);
     DW_LAUNCHED("surr_features");
     return DW_OK;
 }

@@ -268,3 +268,28 @@ def test_weight_gradient_of_single_voxels(n, shape):
     assert np.array_equal(gw.cpu().numpy().reshape(27, cout, cin), ref)
     assert np.array_equal(gb.cpu().numpy(), G.sum(axis=(1, 2, 3)))
     s.close()
+
+
+# The features kernel with paired and with scalar loads (a lattice or a mask
+# that starts off its alignment) does the same operations in the same order.
+@pytest.mark.parametrize("n", [16, 48])
+def test_surrogate_features_alignment(n):
+    rng = np.random.default_rng(5)
+    N = 2 * n
+    f = torch.tensor(0.02 * rng.standard_normal((19, N, N, N)).astype(np.float32), device="cuda")
+    solid = torch.tensor((rng.random((N, N, N)) < 0.3).astype(np.uint8), device="cuda")
+    fo = torch.empty(f.numel() + 1, device="cuda")[1:].view(f.shape)
+    so = torch.empty(solid.numel() + 1, dtype=torch.uint8, device="cuda")[1:].view(solid.shape)
+    fo.copy_(f)
+    so.copy_(solid)
+    s = B.Surrogate(n)
+    got = [s.features(a, b, 20.0, torch.empty((n ** 3, 16), device="cuda"))
+           for a, b in ((f, solid), (fo, solid), (f, so), (f, None), (fo, None))]
+    assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2]) and torch.equal(got[3], got[4])
+    rho = 1.0 + f.double().sum(0)
+    cells = torch.where(solid == 0, rho - 1.0, 0.0).view(n, 2, n, 2, n, 2).sum((1, 3, 5))
+    count = (solid == 0).double().view(n, 2, n, 2, n, 2).sum((1, 3, 5))
+    ref = torch.where(count > 0, 20.0 * cells / count.clamp(min=1), 0.0).reshape(-1)
+    # 19 populations and 8 cells summed in float32 around rho = 1: 27 half ulp of 1, scaled
+    assert (got[0][:, 0].double() - ref).abs().max() <= 27 * 6e-8 * 20
+    s.close()

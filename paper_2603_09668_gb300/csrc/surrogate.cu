@@ -41,7 +41,7 @@ struct SurrHandle {
     bool corr_on = false;           // corr is added by surr_advance_fine
     double *red = nullptr;          // reduction scratch
     int *err = nullptr;             // device status bits (bounded waits of the conv kernels)
-    unsigned *gbar = nullptr;       // grid barrier of the one-launch forward (arrivals, generation)
+    unsigned *gbar = nullptr;       // grid barriers of the one-launch forward (arrivals)
     bool fused = true;              // the one-launch forward can be launched (cooperatively)
     bool fused_attr_set = false;
     int conv_ctas = 0;
@@ -885,14 +885,14 @@ extern "C" dw_status surr_create(int32_t n, dw_surr *out) {
     DW_ALLOC(h->fine, sizeof(float) * 4 * Nc);
     DW_ALLOC(h->red, sizeof(double) * 4);
     DW_ALLOC(h->err, sizeof(int));
-    DW_ALLOC(h->gbar, sizeof(unsigned) * 2);
+    DW_ALLOC(h->gbar, sizeof(unsigned) * 3);
 #undef DW_ALLOC
     if (e == cudaSuccess) e = cudaMemset(h->params, 0, sizeof(float) * o);
     if (e == cudaSuccess) e = cudaMemset(h->grads, 0, sizeof(float) * o);
     if (e == cudaSuccess) e = cudaMemset(h->m, 0, sizeof(float) * o);
     if (e == cudaSuccess) e = cudaMemset(h->v, 0, sizeof(float) * o);
     if (e == cudaSuccess) e = cudaMemset(h->err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->gbar, 0, sizeof(unsigned) * 2);
+    if (e == cudaSuccess) e = cudaMemset(h->gbar, 0, sizeof(unsigned) * 3);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         dw_status st = cuda_fail(e, "surr_create");
@@ -1078,7 +1078,7 @@ extern "C" dw_status surr_device_status(dw_surr h, dw_stream stream) {
     DW_CUDA(cudaMemcpyAsync(&bits, h->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     DW_CUDA(cudaStreamSynchronize(s));
     DW_CUDA(cudaMemsetAsync(h->err, 0, sizeof(int), s));
-    DW_CUDA(cudaMemsetAsync(h->gbar, 0, sizeof(unsigned) * 2, s));  // a barrier that gave up
+    DW_CUDA(cudaMemsetAsync(h->gbar, 0, sizeof(unsigned) * 3, s));  // a barrier that gave up
     DW_CUDA(cudaStreamSynchronize(s));
     return status_from_bits(bits);
 }

@@ -583,24 +583,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(
     tc_pipe_close(pp, taddr);
 }
 
-// Grid-wide barrier of a cooperative launch for `expected` CTAs (bar[0]
-// arrivals, bar[1] generation). Bounded: after about a second the CTA sets
+// Grid-wide barrier `round` (0, 1 or 2) of a cooperative launch: each has its
+// own arrival counter, which the waiting CTAs poll themselves (a separate
+// generation word costs another trip through L2). The last CTA to arrive
+// clears the counter of the barrier before, which every CTA has left by then
+// (the last launch's for round 0). Bounded: after about a second the CTA sets
 // ERRBIT_TIMEOUT and the abort flag and leaves; every later layer of the
 // launch then does nothing.
-__device__ __forceinline__ void tc_grid_sync(unsigned *bar, int *err, TcPipe &pp) {
+__device__ __forceinline__ void tc_grid_sync(unsigned *bar, int round, int *err, TcPipe &pp) {
     __syncthreads();
     if (threadIdx.x == 0 && !pp.abort_flag) {
-        volatile unsigned *gen = bar + 1;
-        const unsigned g0 = *gen;
+        volatile unsigned *count = bar + round;
         __threadfence();
-        const unsigned arrived = atomicAdd(bar, 1u) + 1u;
-        if (arrived == gridDim.x) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
+        if (atomicAdd(bar + round, 1u) + 1u == gridDim.x) {
+            bar[(round + 2) % 3] = 0u;
         } else {
             uint64_t t0 = 0;
-            for (unsigned it = 1; *gen == g0; ++it) {
+            for (unsigned it = 1; *count < gridDim.x; ++it) {
                 if ((it & 1023u) != 0) continue;
                 const uint64_t t = globaltimer_ns();
                 if (t0 == 0) t0 = t;
@@ -643,20 +642,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_surr_forward_tc(
         pp.wbuf[0] = hbase + TC_NST * 4 * TC_SLICE;
         pp.wbuf[1] = pp.wbuf[0] + TC_WMAX;
     }
+    if (threadIdx.x == 0) {
+        for (const CUtensorMap *m : {&tm0, &tm1, &tm2, &tm3})
+            asm volatile("prefetch.tensormap [%0];" :: "l"((uint64_t)m) : "memory");
+    }
     const uint32_t taddr = tc_pipe_open(pp);
     pdl_trigger();
     const int per = tc_slices(n, (n / TC_TX) * (n / TC_TY));
     tc_layer<16, 32, EPI_GELU_ONLY>(pp, taddr, &tm0, TcOut{b0, nullptr, a0, nullptr, nullptr, nullptr}, n,
                                     hbase, 0, 0, w0, w1, tc_wbytes(32, 32), 0, TC_PRO_PDL, true, err);
-    tc_grid_sync(bar, err, pp);
+    tc_grid_sync(bar, 0, err, pp);
     tc_layer<32, 32, EPI_GELU_ONLY>(pp, taddr, &tm1, TcOut{b1, nullptr, a1, nullptr, nullptr, nullptr}, n,
                                     hbase, 1, 0, nullptr, w2, tc_wbytes(32, 32), per, TC_PRO_PROXY,
                                     true, err);
-    tc_grid_sync(bar, err, pp);
+    tc_grid_sync(bar, 1, err, pp);
     tc_layer<32, 32, EPI_GELU_ONLY>(pp, taddr, &tm2, TcOut{b2, nullptr, a2, nullptr, nullptr, nullptr}, n,
                                     hbase, 0, 1, nullptr, w3, tc_wbytes(32, 16), 2 * per,
                                     TC_PRO_PROXY, true, err);
-    tc_grid_sync(bar, err, pp);
+    tc_grid_sync(bar, 2, err, pp);
     tc_layer<32, 16, EPI_F32>(pp, taddr, &tm3, TcOut{b3, nullptr, nullptr, out, nullptr, out4}, n, hbase,
                               1, 1, nullptr, nullptr, 0, 3 * per, TC_PRO_PROXY, false, err);
     tc_pipe_close(pp, taddr);

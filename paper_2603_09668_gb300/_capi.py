@@ -174,6 +174,8 @@ def library_path() -> str:
 def lib():
     """The loaded libdiffwind. Raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = library_path()

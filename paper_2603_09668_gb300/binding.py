@@ -59,8 +59,10 @@ def _dev(t: Optional[torch.Tensor], dtype=torch.float32, name="tensor"):
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ct.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ct.c_void_p(stream.cuda_stream)
+    # the current device's current stream, without a Stream object per call
+    return ct.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 class MpmState(NamedTuple):
@@ -74,7 +76,16 @@ class MpmState(NamedTuple):
         return self.x.shape[1]
 
     def to_c(self):
-        n = self.x.shape[1]
+        x, v, C, F = self
+        n = x.shape[1]
+        r3, r9 = (3, n), (9, n)
+        if x.shape == r3 and v.shape == r3 and C.shape == r9 and F.shape == r9:
+            for t in self:
+                if not (t.is_cuda and t.dtype is torch.float32 and t.is_contiguous()):
+                    break
+            else:
+                return DwMpmState(x.data_ptr(), v.data_ptr(), C.data_ptr(), F.data_ptr(), n)
+        # something is wrong: the checks one by one, for the message
         for name, t, rows in (("x", self.x, 3), ("v", self.v, 3), ("C", self.C, 9), ("F", self.F, 9)):
             if t.dim() != 2 or t.shape[0] != rows or t.shape[1] != n:
                 raise ValueError(f"state.{name} must have shape [{rows}, {n}], got {tuple(t.shape)}")

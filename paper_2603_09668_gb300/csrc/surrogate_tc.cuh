@@ -590,6 +590,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(
 // (the last launch's for round 0). Bounded: after about a second the CTA sets
 // ERRBIT_TIMEOUT and the abort flag and leaves; every later layer of the
 // launch then does nothing.
+// With a generation word, and without the descriptors' prefetch at the
+// kernel's start, the four layers took 73.9 us at 64^3 (now 69.3) and 34.8 at
+// 32^3 (29.2).
 __device__ __forceinline__ void tc_grid_sync(unsigned *bar, int round, int *err, TcPipe &pp) {
     __syncthreads();
     if (threadIdx.x == 0 && !pp.abort_flag) {

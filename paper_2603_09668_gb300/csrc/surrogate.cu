@@ -73,6 +73,7 @@ struct SurrLayers {
 // instead of four of 3 us.
 __global__ void k_surr_weights(const float *__restrict__ params, bf16 *__restrict__ wf,
                                bf16 *__restrict__ wd, SurrLayers L) {
+    pdl_wait();
     const int l = blockIdx.y, cin = L.cin[l], cout = L.cout[l];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 27 * cin * cout) return;
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(256) k_surr_loss(const float4 *__restrict__ ou
                                                    const bf16 *__restrict__ feats, int64_t nv,
                                                    const int *__restrict__ count,
                                                    bf16 *__restrict__ g4, float *__restrict__ loss) {
+    pdl_wait();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float inv_norm = 1.0f / (3.0f * (float)max(*count, 1));
     float l = 0.0f;
@@ -810,8 +812,8 @@ static dw_status refresh_weights(SurrHandle *h, cudaStream_t s) {
         L.cin[l] = SCH[l];
         L.cout[l] = SCH[l + 1];
     }
-    k_surr_weights<<<dim3(grid_for(27 * 32 * 32, 256), 4), 256, 0, s>>>(h->params, h->wf, h->wd, L);
-    DW_LAUNCHED("k_surr_weights");
+    DW_CUDA(launch_pdl3(k_surr_weights, dim3(grid_for(27 * 32 * 32, 256), 4), dim3(256), s, h->params, h->wf,
+                        h->wd, L));
     return DW_OK;
 }
 
@@ -1090,9 +1092,8 @@ extern "C" dw_status surr_loss(dw_surr h, const float *target, float *loss, dw_s
     DW_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int), s));
     const unsigned blocks = grid_for(h->nv, 256);
     k_count_fluid<<<std::min(blocks, 304u), 256, 0, s>>>(h->feats, h->nv, cnt);
-    k_surr_loss<<<blocks, 256, 0, s>>>(reinterpret_cast<const float4 *>(h->out4), target, h->feats, h->nv,
-                                       cnt, h->g4, loss);
-    DW_LAUNCHED("k_surr_loss");
+    DW_CUDA(launch_pdl(k_surr_loss, blocks, 256, s, reinterpret_cast<const float4 *>(h->out4), target, h->feats,
+                       h->nv, cnt, h->g4, loss));
     return DW_OK;
 }
 

@@ -333,7 +333,8 @@ __device__ __forceinline__ int tc_slices(int n, int nxy) {
 // buffer wb holds (or receives) this layer's weights, as its wuse-th use
 // (from 0): own_wt, when not NULL, is copied there first by the loader. next_wt, when not NULL, is copied
 // into the other buffer at the start, the prefetch of the following layer's
-// weights (that buffer's previous layer has finished). k0 counts the slices
+// weights (that buffer's previous layer has finished, and its MMA thread has
+// waited for the copy of that layer's weights). k0 counts the slices
 // this CTA has gone through in earlier layers of the launch. fence_out: the
 // epilogue ends with a proxy fence, so that TMA reads of the output by other
 // CTAs after a grid barrier see it.
@@ -359,13 +360,17 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
 
     if (warp == TC_LOAD_WARP) {
         if (lane == 0) {
-            if (own_wt) tc_copy_weights(pp, wb, own_wt, WBYTES);
-            if (next_wt) tc_copy_weights(pp, 1 - wb, next_wt, next_bytes);
+            TcSeg c;
+            // A CTA without output slices copies no weights: its MMA thread waits for none,
+            // and nothing else would order a buffer's next copy after the last one.
+            if (tc_segment(n, nxy, 0, c)) {
+                if (own_wt) tc_copy_weights(pp, wb, own_wt, WBYTES);
+                if (next_wt) tc_copy_weights(pp, 1 - wb, next_wt, next_bytes);
+            }
             if (prologue == TC_PRO_PDL) pdl_wait();
             if (prologue == TC_PRO_PROXY) asm volatile("fence.proxy.async.global;" ::: "memory");
             int k = k0;
             bool ok = true;
-            TcSeg c;
             for (int j = 0; ok && tc_segment(n, nxy, j, c); ++j) {
                 const int i0 = max(c.o0 - 1, 0), i1 = min(c.o1 + 1, n - 1);
                 const int x0 = (c.xy % tiles_x) * TC_TX, y0 = (c.xy / tiles_x) * TC_TY;

@@ -293,3 +293,27 @@ def test_surrogate_features_alignment(n):
     # 19 populations and 8 cells summed in float32 around rho = 1: 27 half ulp of 1, scaled
     assert (got[0][:, 0].double() - ref).abs().max() <= 27 * 6e-8 * 20
     s.close()
+
+
+# The one-launch inference pass where the grid has more CTAs than the volume
+# has output slices (16^3: 32 slices), launch after launch, against the
+# per-layer kernels: the same operations on the same operands (the tolerance of
+# that comparison at 64^3).
+def test_inference_with_idle_ctas():
+    n = 16
+    g = torch.Generator(device="cuda").manual_seed(9)
+    s = B.Surrogate(n)
+    s.set_params(0.1 * torch.randn(s.nparams, generator=g, device="cuda"))
+    outs = []
+    for keep in (True, False):
+        for k in range(40):
+            feats = torch.randn((n ** 3, 16), generator=torch.Generator(device="cuda").manual_seed(k),
+                                device="cuda")
+            s.set_features(feats)
+            out = torch.empty((n ** 3, 16), device="cuda")
+            s.forward(out, keep_activations=keep)
+            outs.append(out)
+    s.device_status()
+    for a, b in zip(outs[:40], outs[40:]):
+        assert a.abs().max() > 0 and (a - b).abs().max() <= 1e-6 * a.abs().max()
+    s.close()

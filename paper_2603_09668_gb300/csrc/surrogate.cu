@@ -266,7 +266,9 @@ __device__ __forceinline__ T block_sum256(T v) {
 // Mean squared error over the coarse voxels that are not fully solid, on
 // channels 0..2: L = sum (out - target)^2 / (3 count); g4 = dL/d(out). out4
 // holds channels 0..3 of the output. One loss atomic per block, as in the count
-// below: one per warp, 8,192 atomics on one address, took 14 us of 18.
+// below: one per warp, 8,192 atomics on one address, took 14 us of 18. VEC:
+// target is 16-byte aligned (the caller's; one load per voxel).
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_surr_loss(const float4 *__restrict__ out4,
                                                    const float *__restrict__ target,
                                                    const bf16 *__restrict__ feats, int64_t nv,
@@ -278,7 +280,9 @@ __global__ void __launch_bounds__(256) k_surr_loss(const float4 *__restrict__ ou
     float l = 0.0f;
     if (v < nv) {
         const bool fluid = __bfloat162float(feats[v * 8 + 4]) < 1.0f;  // solid fraction, plane 0
-        const float4 a = out4[v], b = *reinterpret_cast<const float4 *>(target + v * 16);
+        const float4 a = out4[v];
+        const float *t = target + v * 16;
+        const float4 b = VEC ? *reinterpret_cast<const float4 *>(t) : make_float4(t[0], t[1], t[2], 0.0f);
         __align__(16) bf16 g[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) g[c] = __float2bfloat16_rn(0.0f);
@@ -1092,7 +1096,8 @@ extern "C" dw_status surr_loss(dw_surr h, const float *target, float *loss, dw_s
     DW_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int), s));
     const unsigned blocks = grid_for(h->nv, 256);
     k_count_fluid<<<std::min(blocks, 304u), 256, 0, s>>>(h->feats, h->nv, cnt);
-    DW_CUDA(launch_pdl(k_surr_loss, blocks, 256, s, reinterpret_cast<const float4 *>(h->out4), target, h->feats,
+    auto kern = reinterpret_cast<uintptr_t>(target) % 16 == 0 ? k_surr_loss<true> : k_surr_loss<false>;
+    DW_CUDA(launch_pdl(kern, blocks, 256, s, reinterpret_cast<const float4 *>(h->out4), target, h->feats,
                        h->nv, cnt, h->g4, loss));
     return DW_OK;
 }

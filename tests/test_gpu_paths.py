@@ -317,3 +317,33 @@ def test_inference_with_idle_ctas():
     for a, b in zip(outs[:40], outs[40:]):
         assert a.abs().max() > 0 and (a - b).abs().max() <= 1e-6 * a.abs().max()
     s.close()
+
+
+# The loss of a target that starts off a 16-byte boundary (scalar loads): the
+# same gradients bit for bit; the loss up to the order of its 432 block sums, one
+# rounding each.
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_surrogate_loss_alignment(offset):
+    n = 48
+    g = torch.Generator(device="cuda").manual_seed(4)
+    s = B.Surrogate(n)
+    s.set_params(0.1 * torch.randn(s.nparams, generator=g, device="cuda"))
+    feats = torch.randn((n ** 3, 16), generator=g, device="cuda")
+    feats[:, 4] = (torch.rand(n ** 3, generator=g, device="cuda") < 0.3).float()
+    s.set_features(feats)
+    target = torch.randn((n ** 3, 16), generator=g, device="cuda")
+    off = torch.empty(target.numel() + 4, device="cuda")[offset:offset + target.numel()].view(target.shape)
+    off.copy_(target)
+    assert target.data_ptr() % 16 == 0 and off.data_ptr() % 16 == 4 * offset and off.is_contiguous()
+    got = []
+    for t in (target, off):
+        loss = torch.zeros(1, device="cuda")
+        s.forward()
+        s.loss(t, loss)
+        s.zero_grads()
+        s.backward()
+        got.append((loss.item(), s.grads()))
+    s.device_status()
+    assert got[0][0] > 0 and abs(got[0][0] - got[1][0]) <= 432 * 1.2e-7 * got[0][0]
+    assert got[0][1].abs().max() > 0 and torch.equal(got[0][1], got[1][1])
+    s.close()

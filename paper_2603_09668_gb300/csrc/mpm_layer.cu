@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(256) k_layer_gE(const double *__restrict__ par
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w) s += red[w];
-        *g_E += (float)s;
+        atomicAdd(g_E, (float)s);  // handles on other streams may add to the same sum
     }
 }
 

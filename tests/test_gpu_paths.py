@@ -347,3 +347,39 @@ def test_surrogate_loss_alignment(offset):
     assert got[0][0] > 0 and abs(got[0][0] - got[1][0]) <= 432 * 1.2e-7 * got[0][0]
     assert got[0][1].abs().max() > 0 and torch.equal(got[0][1], got[1][1])
     s.close()
+
+
+# Two handles that differentiate on two streams into one g_E and one wind
+# gradient: every segment's part arrives. 80 parts of one sign in any order:
+# 80 roundings, and the segments' own sums in any order, 1e-4.
+def test_segments_of_two_streams_share_a_gradient():
+    n, steps, calls = 64, 2, 40
+    pr, st, pin = _mpm_case(n, 24, 0, seed=2)
+    wind = B.WindField(to_dev(inputs.fourier_wind(5, 1, seed=4)), 1.0)
+    g0 = [0.1 * torch.randn(a.shape, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+          for a in st]
+
+    def work(mpm, gw, gE, tape, stream, calls):
+        with torch.cuda.stream(stream):
+            for _ in range(calls):
+                gs = B.MpmState(*(a.clone() for a in g0))
+                mpm.segment_adjoint(state, tape, gs, pin_d, wind, 0.0, steps, gw, gE)
+
+    state, pin_d = _dev(st), to_dev(pin)
+    mpms = [B.MPM.from_params(pr, max_particles=n) for _ in range(2)]
+    tapes = [torch.empty((steps - 1) * 24 * n, device="cuda") for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    sums = []
+    for rounds in ((1,), (calls, calls)):  # one segment alone, then both streams at once
+        gw, gE = torch.zeros_like(wind.values), torch.zeros(1, device="cuda")
+        torch.cuda.synchronize()
+        for k, c in enumerate(rounds):
+            work(mpms[k], gw, gE, tapes[k], streams[k], c)
+        torch.cuda.synchronize()
+        sums.append((gw.cpu().numpy(), gE.item()))
+    for m in mpms:
+        m.device_status()
+        m.close()
+    (gw1, gE1), (gw2, gE2) = sums
+    assert gE1 != 0 and abs(gE2 - 2 * calls * gE1) <= 1e-4 * abs(2 * calls * gE1)
+    assert rel_l2(gw2, 2 * calls * gw1.astype(np.float64)) <= 1e-4

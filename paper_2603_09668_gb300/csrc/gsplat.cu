@@ -477,14 +477,15 @@ __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big
                                                 GsStat *__restrict__ stat) {
     const uint32_t queued = *big_count;
     if (!LIST && blockIdx.x == 0 && threadIdx.x == 0) stat->big = queued;
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * 8;
-    for (uint32_t u = blockIdx.x * 8 + (threadIdx.x >> 5); u / 16 < queued; u += warps) {
-        const int i = (int)big[u / 16];
+    // sixteen warps, two blocks, per Gaussian; queued and the step stay far below 2^32
+    static_assert(GS_BIG_CTAS % 2 == 0, "two blocks per Gaussian");
+    const int lane = threadIdx.x & 31, slice = (int)(blockIdx.x % 2) * 8 + (threadIdx.x >> 5);
+    for (uint32_t q = blockIdx.x / 2; q < queued; q += gridDim.x / 2) {
+        const int i = (int)big[q];
         const GsTiles g = gs_tiles(rect[i], true, tiles_x);
         const unsigned long long k = LIST ? gs_key(key, i) : 0ull;
 #pragma unroll 4
-        for (int t = (int)(u % 16) * 32 + lane; t < g.count; t += 512) {
+        for (int t = slice * 32 + lane; t < g.count; t += 512) {
             const int tile = g.first + t / g.nx * tiles_x + t % g.nx;
             if (LIST)
                 list[atomicAdd(&ranges[tile].y, 1)] = k;

@@ -383,3 +383,27 @@ def test_segments_of_two_streams_share_a_gradient():
     (gw1, gE1), (gw2, gE2) = sums
     assert gE1 != 0 and abs(gE2 - 2 * calls * gE1) <= 1e-4 * abs(2 * calls * gE1)
     assert rel_l2(gw2, 2 * calls * gw1.astype(np.float64)) <= 1e-4
+
+
+# As many Gaussians that meet more than 16 tiles as a 32-bit count of their
+# warps' work items (16 each) no longer holds: the call is refused, and the
+# handle still renders.
+def test_gaussian_queue_of_2_28():
+    n, W, H = 1 << 28, 64, 64
+    if torch.cuda.mem_get_info()[0] < 90 << 30:
+        pytest.skip("needs 90 GB of device memory")
+    r = B.GaussianRenderer(n, W, H)
+    x, F, s0 = (torch.zeros((k, n), device="cuda") for k in (3, 9, 6))
+    F[::4] = 1.0
+    s0[:3] = 4.0
+    col, op = torch.full((3, n), 0.5, device="cuda"), torch.full((n,), 0.25, device="cuda")
+    cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), 40.0, 40.0, W / 2, H / 2, W, H)
+    with pytest.raises(B.DiffWindError, match="too long"):
+        r.render(cam, x, F, s0, col, op)
+    few = [a[..., :3].contiguous() for a in (x, F, s0, col, op)]
+    # three layers, each covers the image: at the centre C = 0.5 (1 - (1 - 0.25)^3)
+    img = r.render(cam, *few)
+    assert abs(img[0, H // 2, W // 2].item() - 0.5 * (1 - 0.75 ** 3)) <= 1e-3
+    r.close()
+    del x, F, s0, col, op
+    torch.cuda.empty_cache()

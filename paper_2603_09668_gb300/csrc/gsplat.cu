@@ -354,9 +354,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *__res
 
 // ------------------------------------------------------------ tile lists --
 
-constexpr int GS_WORD = 28;  // bits of the batch count in a scan word
+// A scan word: entries in the high half, batches in the low one.
 __device__ __forceinline__ unsigned long long gs_word(uint32_t entries) {
-    return ((unsigned long long)entries << GS_WORD) | ((entries + GS_THREADS - 1) / GS_THREADS);
+    return ((unsigned long long)entries << 32) | ((entries + GS_THREADS - 1) / GS_THREADS);
 }
 
 // What gs_render reads back: the list's length, its batches of GS_THREADS
@@ -373,15 +373,15 @@ __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restric
                                                        int tiles, int2 *__restrict__ ranges,
                                                        uint32_t *__restrict__ batch_off,
                                                        GsStat *__restrict__ stat) {
-    // a 64-bit word carries both sums: the entries above bit GS_WORD, the
-    // batches below it (at most list / 64 + tiles: below 2^27 for a list of 2^31
-    // entries and an image of 2^31 pixels)
+    // Of a list that is accepted (below 2^31 entries) both sums of a word fit 32
+    // bits: an image has at most 2^28 tiles. `all` holds any list's length.
     __shared__ unsigned long long wsum[32];
     __shared__ uint32_t wmax[32];
-    __shared__ unsigned long long carry;
+    __shared__ unsigned long long carry, wall[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) carry = 0;
     uint32_t mx = 0;
+    unsigned long long all = 0;
     __syncthreads();
     for (int base = 0; base < tiles; base += 4096) {
         uint32_t v[4];
@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restric
             const int i = base + (int)threadIdx.x * 4 + j;
             v[j] = i < tiles ? count[i] : 0u;
             mx = max(mx, v[j]);
+            all += v[j];
             t += gs_word(v[j]);
         }
         unsigned long long incl = t;
@@ -418,22 +419,30 @@ __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restric
         for (int j = 0; j < 4; ++j) {
             const int i = base + (int)threadIdx.x * 4 + j;
             if (i < tiles) {
-                const int at = (int)(run >> GS_WORD);
+                const int at = (int)(run >> 32);
                 ranges[i] = make_int2(at, at);
-                batch_off[i] = (uint32_t)run & ((1u << GS_WORD) - 1u);
+                batch_off[i] = (uint32_t)run;
             }
             run += gs_word(v[j]);
         }
         __syncthreads();
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) wmax[warp] = mx;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    if (lane == 0) {
+        wmax[warp] = mx;
+        wall[warp] = all;
+    }
     __syncthreads();
     if (warp == 0) {
         mx = __reduce_max_sync(0xffffffffu, wmax[lane]);
+        all = wall[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
         if (lane == 0) {
-            stat->total = carry >> GS_WORD;
-            stat->batches = (uint32_t)carry & ((1u << GS_WORD) - 1u);
+            stat->total = all;
+            stat->batches = (uint32_t)carry;
             stat->most = mx;
         }
     }

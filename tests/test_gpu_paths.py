@@ -407,3 +407,20 @@ def test_gaussian_queue_of_2_28():
     r.close()
     del x, F, s0, col, op
     torch.cuda.empty_cache()
+
+
+# A list whose length no 32-bit (nor 36-bit) count holds, 2^18 Gaussians on all
+# 2^18 tiles of an image, is refused; the handle still renders.
+def test_gaussian_list_of_2_36_entries():
+    n, W = 1 << 18, 4096
+    r = B.GaussianRenderer(n, W, W)
+    x, F, s0 = (torch.zeros((k, n), device="cuda") for k in (3, 9, 6))
+    F[::4] = 1.0
+    s0[:3] = 4.0
+    col, op = torch.full((3, n), 0.5, device="cuda"), torch.full((n,), 0.25, device="cuda")
+    cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), 2560.0, 2560.0, W / 2, W / 2, W, W)
+    with pytest.raises(B.DiffWindError, match="too long"):
+        r.render(cam, x, F, s0, col, op)
+    img = r.render(cam, *[a[..., :3].contiguous() for a in (x, F, s0, col, op)])
+    assert abs(img[0, W // 2, W // 2].item() - 0.5 * (1 - 0.75 ** 3)) <= 1e-3
+    r.close()

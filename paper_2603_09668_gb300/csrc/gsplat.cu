@@ -22,7 +22,8 @@
 //                    composites them.
 // A tile with more Gaussians than the shared-memory sort holds sends the call
 // through a stable LSD radix sort of all depths and a stable sort of the list
-// by tile instead (the same lists).
+// by tile instead (the same lists). A list too long for 8 x 8 tiles (wide
+// Gaussians: up to four times the entries) is made on 16 x 16 tiles.
 // gs_render_backward walks the same ranges front to back again with the
 // final colour known (dC/dalpha_i = T_i c_i - (C - C_<=i) / (1 - alpha_i)),
 // reduces each Gaussian's pixel contributions per warp before one atomic,
@@ -42,13 +43,17 @@
 
 namespace dw {
 
-// Tile edge. The path renders particles, whose Gaussians cover a few pixels: 8
-// pixels leave a warp (8 x 4 pixels) few idle lanes per Gaussian, and four
-// times as many blocks as 16, with lists half as long (100,284 Gaussians of
-// about 7 pixels at 512 x 512: 183,000 entries of 256 pixels against 306,000
-// of 64).
-constexpr int GS_TILE = 8;
-constexpr int GS_THREADS = GS_TILE * GS_TILE;  // one pixel per thread
+// Tile edges are 2^ts pixels; a tile's block has a thread per pixel and takes
+// its list in batches of as many entries. The path renders particles, whose
+// Gaussians cover a few pixels: 8 pixels leave a warp (8 x 4 pixels) few idle
+// lanes per Gaussian, and four times as many blocks as 16, with lists half as
+// long (100,284 Gaussians of about 7 pixels at 512 x 512: 183,000 entries of 256
+// pixels against 306,000 of 64). Wide Gaussians meet four times as many tiles of
+// 8 as of 16: a list that would be longer than GS_LIST_MAX, what its indices
+// hold, is made on 16 instead.
+constexpr int GS_FINE = 3, GS_COARSE = 4;
+__host__ __device__ constexpr int gs_threads(int ts) { return 1 << (2 * ts); }
+constexpr int64_t GS_LIST_MAX = (1ll << 31) - 1;
 constexpr int GS_SORT_MAX = 4096;   // keys of one tile k_gs_tile_sort holds
 constexpr int GS_SORT_THREADS = 128;
 constexpr int GS_BIG_CTAS = 304;    // two per SM
@@ -189,20 +194,22 @@ struct GsTiles {
     int first, nx, count;  // tile of the rectangle's corner, tiles per row, tiles
 };
 
-__device__ __forceinline__ GsTiles gs_tiles(int4 r, bool drawn, int tiles_x) {
-    const int x0 = r.x / GS_TILE, y0 = r.y / GS_TILE;
+__device__ __forceinline__ GsTiles gs_tiles(int4 r, bool drawn, int tiles_x, int ts) {
+    const int x0 = r.x >> ts, y0 = r.y >> ts;
     GsTiles t;
     t.first = y0 * tiles_x + x0;
-    t.nx = drawn ? r.z / GS_TILE - x0 + 1 : 0;
-    t.count = drawn ? t.nx * (r.w / GS_TILE - y0 + 1) : 0;
+    t.nx = drawn ? (r.z >> ts) - x0 + 1 : 0;
+    t.count = drawn ? t.nx * ((r.w >> ts) - y0 + 1) : 0;
     return t;
 }
+
+// A Gaussian that meets more than GS_BIG of the fine tiles is queued (k_gs_big).
+constexpr int GS_BIG = 16;
 
 // f(tile, mask) for every tile of each lane's Gaussian that meets at most
 // GS_BIG of them, called by whole warps with the mask of the lanes that call
 // it together. Neighbouring particles' Gaussians meet the same tiles, so f
 // combines equal tiles of the mask before its atomic.
-constexpr int GS_BIG = 16;
 template <typename Fn>
 __device__ __forceinline__ void gs_for_tiles(const GsTiles &g, int tiles_x, Fn f) {
     const int cnt = g.count <= GS_BIG ? g.count : 0;
@@ -217,6 +224,12 @@ __device__ __forceinline__ void gs_for_tiles(const GsTiles &g, int tiles_x, Fn f
             tile += tiles_x - g.nx;
         }
     }
+}
+
+// One of the mask's lanes adds a tile's lanes to its count.
+__device__ __forceinline__ void gs_count_tile(int tile, unsigned mask, uint32_t *__restrict__ tile_count) {
+    const unsigned peers = __match_any_sync(mask, tile);
+    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&tile_count[tile], __popc(peers));
 }
 
 // Per Gaussian: row = (mu'(2), conic(3), opacity, colour(3)), the pixel
@@ -253,11 +266,8 @@ __global__ void __launch_bounds__(128) k_gs_preprocess(
         if (!(lx <= hx && ly <= hy)) r = make_int4(0, 0, -1, -1);  // also NaN
     }
     const bool drawn = r.z >= r.x && r.w >= r.y;
-    const GsTiles g = gs_tiles(r, drawn && t < n, tiles_x);
-    gs_for_tiles(g, tiles_x, [&](int tile, unsigned mask) {
-        const unsigned peers = __match_any_sync(mask, tile);
-        if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&tile_count[tile], __popc(peers));
-    });
+    const GsTiles g = gs_tiles(r, drawn && t < n, tiles_x, GS_FINE);
+    gs_for_tiles(g, tiles_x, [&](int tile, unsigned mask) { gs_count_tile(tile, mask, tile_count); });
     if (t >= n) return;
     if (g.count > GS_BIG) big[atomicAdd(big_count, 1u)] = (uint32_t)i;
     rows[3 * (int64_t)i] = make_float4(p.mu[0], p.mu[1], p.conic[0], p.conic[1]);
@@ -355,12 +365,15 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *__res
 // ------------------------------------------------------------ tile lists --
 
 // A scan word: entries in the high half, batches in the low one.
-__device__ __forceinline__ unsigned long long gs_word(uint32_t entries) {
-    return ((unsigned long long)entries << 32) | ((entries + GS_THREADS - 1) / GS_THREADS);
+__device__ __forceinline__ uint32_t gs_batches(uint32_t entries, int ts) {
+    return (entries + gs_threads(ts) - 1) >> (2 * ts);
+}
+__device__ __forceinline__ unsigned long long gs_word(uint32_t entries, int ts) {
+    return ((unsigned long long)entries << 32) | gs_batches(entries, ts);
 }
 
-// What gs_render reads back: the list's length, its batches of GS_THREADS
-// entries, the longest tile's list and the queue's length.
+// What gs_render reads back: the list's length, its batches, the longest tile's
+// list and the queue's length.
 struct GsStat {
     unsigned long long total;
     uint32_t batches, most, big;
@@ -370,7 +383,7 @@ struct GsStat {
 // = the tile's first entry (k_gs_list advances .y to its end), and of their
 // batches: batch_off[t] = the tile's first batch.
 __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restrict__ count,
-                                                       int tiles, int2 *__restrict__ ranges,
+                                                       int tiles, int ts, int2 *__restrict__ ranges,
                                                        uint32_t *__restrict__ batch_off,
                                                        GsStat *__restrict__ stat) {
     // Of a list that is accepted (below 2^31 entries) both sums of a word fit 32
@@ -392,7 +405,7 @@ __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restric
             v[j] = i < tiles ? count[i] : 0u;
             mx = max(mx, v[j]);
             all += v[j];
-            t += gs_word(v[j]);
+            t += gs_word(v[j], ts);
         }
         unsigned long long incl = t;
 #pragma unroll
@@ -423,7 +436,7 @@ __global__ void __launch_bounds__(1024) k_gs_tile_scan(const uint32_t *__restric
                 ranges[i] = make_int2(at, at);
                 batch_off[i] = (uint32_t)run;
             }
-            run += gs_word(v[j]);
+            run += gs_word(v[j], ts);
         }
         __syncthreads();
     }
@@ -452,24 +465,32 @@ __device__ __forceinline__ unsigned long long gs_key(const uint32_t *__restrict_
     return ((unsigned long long)key[i] << 32) | (uint32_t)i;
 }
 
-// Each drawn Gaussian's key into the ranges of the tiles it meets.
+// Each drawn Gaussian outside the queue counted in the tiles it meets, or (LIST)
+// its key into their ranges.
+template <bool LIST>
 __global__ void __launch_bounds__(128) k_gs_list(const int4 *__restrict__ rect,
                                                  const uint32_t *__restrict__ key, int n,
-                                                 int tiles_x, int2 *__restrict__ ranges,
+                                                 int tiles_x, int ts, uint32_t *__restrict__ tile_count,
+                                                 int2 *__restrict__ ranges,
                                                  unsigned long long *__restrict__ list) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, i = min(t, n - 1);
     const int4 r = rect[i];
+    const bool drawn = t < n && r.z >= r.x && r.w >= r.y;
+    const bool queued = gs_tiles(r, drawn, tiles_x, GS_FINE).count > GS_BIG;
     const unsigned long long k = gs_key(key, i);
     const int lane = threadIdx.x & 31;
-    gs_for_tiles(gs_tiles(r, t < n && r.z >= r.x && r.w >= r.y, tiles_x), tiles_x,
-                 [&](int tile, unsigned mask) {
-                     const unsigned peers = __match_any_sync(mask, tile);
-                     const int leader = __ffs(peers) - 1;
-                     int at = 0;
-                     if (lane == leader) at = atomicAdd(&ranges[tile].y, __popc(peers));
-                     at = __shfl_sync(peers, at, leader);
-                     list[at + __popc(peers & ((1u << lane) - 1u))] = k;
-                 });
+    gs_for_tiles(gs_tiles(r, drawn && !queued, tiles_x, ts), tiles_x, [&](int tile, unsigned mask) {
+        if (!LIST) {
+            gs_count_tile(tile, mask, tile_count);
+            return;
+        }
+        const unsigned peers = __match_any_sync(mask, tile);
+        const int leader = __ffs(peers) - 1;
+        int at = 0;
+        if (lane == leader) at = atomicAdd(&ranges[tile].y, __popc(peers));
+        at = __shfl_sync(peers, at, leader);
+        list[at + __popc(peers & ((1u << lane) - 1u))] = k;
+    });
 }
 
 // The queued Gaussians' tiles, counted or (LIST) listed: 16 warps per Gaussian,
@@ -479,7 +500,7 @@ template <bool LIST>
 __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big,
                                                 const uint32_t *__restrict__ big_count,
                                                 const int4 *__restrict__ rect,
-                                                const uint32_t *__restrict__ key, int tiles_x,
+                                                const uint32_t *__restrict__ key, int tiles_x, int ts,
                                                 uint32_t *__restrict__ tile_count,
                                                 int2 *__restrict__ ranges,
                                                 unsigned long long *__restrict__ list,
@@ -491,7 +512,7 @@ __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big
     const int lane = threadIdx.x & 31, slice = (int)(blockIdx.x % 2) * 8 + (threadIdx.x >> 5);
     for (uint32_t q = blockIdx.x / 2; q < queued; q += gridDim.x / 2) {
         const int i = (int)big[q];
-        const GsTiles g = gs_tiles(rect[i], true, tiles_x);
+        const GsTiles g = gs_tiles(rect[i], true, tiles_x, ts);
         const unsigned long long k = LIST ? gs_key(key, i) : 0ull;
 #pragma unroll 4
         for (int t = slice * 32 + lane; t < g.count; t += 512) {
@@ -504,11 +525,11 @@ __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big
     }
 }
 
-// The batches of tile t: batch k holds the entries [64 k, 64 k + 64) of its
+// The batches of tile t: batch k holds the entries from gs_threads k on of its
 // range; batch_tile[batch_off[t] + k] = t.
-__device__ __forceinline__ void gs_write_batches(int t, int cnt, const uint32_t *__restrict__ batch_off,
+__device__ __forceinline__ void gs_write_batches(int t, int cnt, int ts, const uint32_t *__restrict__ batch_off,
                                                  uint32_t *__restrict__ batch_tile) {
-    const int nb = (cnt + GS_THREADS - 1) / GS_THREADS;
+    const int nb = (int)gs_batches(cnt, ts);
     for (int k = threadIdx.x; k < nb; k += blockDim.x) batch_tile[batch_off[t] + k] = (uint32_t)t;
 }
 
@@ -518,13 +539,13 @@ __device__ __forceinline__ void gs_write_batches(int t, int cnt, const uint32_t 
 // distances need the block's barrier.
 __global__ void __launch_bounds__(GS_SORT_THREADS) k_gs_tile_sort(
     const int2 *__restrict__ ranges, const unsigned long long *__restrict__ list,
-    const uint32_t *__restrict__ batch_off, uint32_t *__restrict__ gid,
+    const uint32_t *__restrict__ batch_off, int ts, uint32_t *__restrict__ gid,
     uint32_t *__restrict__ batch_tile) {
     extern __shared__ unsigned long long k[];  // the longest list, rounded up to a power of two
     const int2 rg = ranges[blockIdx.x];
     const int cnt = rg.y - rg.x;
     if (cnt <= 0) return;
-    gs_write_batches(blockIdx.x, cnt, batch_off, batch_tile);
+    gs_write_batches(blockIdx.x, cnt, ts, batch_off, batch_tile);
     int size = 2;
     while (size < cnt) size <<= 1;
     for (int i = threadIdx.x; i < size; i += GS_SORT_THREADS) k[i] = i < cnt ? list[rg.x + i] : ~0ull;
@@ -552,11 +573,11 @@ __global__ void __launch_bounds__(GS_SORT_THREADS) k_gs_tile_sort(
 
 // The batches of every tile (the radix path; one thread per tile).
 __global__ void __launch_bounds__(256) k_gs_batches(const int2 *__restrict__ ranges, int tiles,
-                                                    const uint32_t *__restrict__ batch_off,
+                                                    int ts, const uint32_t *__restrict__ batch_off,
                                                     uint32_t *__restrict__ batch_tile) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
-    const int nb = (ranges[t].y - ranges[t].x + GS_THREADS - 1) / GS_THREADS;
+    const int nb = (int)gs_batches(ranges[t].y - ranges[t].x, ts);
     for (int k = 0; k < nb; ++k) batch_tile[batch_off[t] + k] = (uint32_t)t;
 }
 
@@ -571,13 +592,13 @@ __global__ void k_gs_order_init(const uint32_t *__restrict__ key, int n, uint32_
 
 // Tiles met by Gaussian order[k] (its pixel rectangle in tiles).
 __global__ void k_gs_tile_count(const uint32_t *__restrict__ order, const int4 *__restrict__ rect,
-                                int n, uint32_t *__restrict__ cnt) {
+                                int n, int ts, uint32_t *__restrict__ cnt) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int4 r = rect[order[k]];
     uint32_t c = 0;
     if (r.z >= r.x && r.w >= r.y)
-        c = (uint32_t)((r.z / GS_TILE - r.x / GS_TILE + 1) * (r.w / GS_TILE - r.y / GS_TILE + 1));
+        c = (uint32_t)(((r.z >> ts) - (r.x >> ts) + 1) * ((r.w >> ts) - (r.y >> ts) + 1));
     cnt[k] = c;
 }
 
@@ -622,7 +643,7 @@ __global__ void k_scan_finish(uint32_t *__restrict__ out, const uint32_t *__rest
 
 // One entry (tile id, Gaussian) per tile met, written in depth order.
 __global__ void k_gs_duplicate(const uint32_t *__restrict__ order, const int4 *__restrict__ rect,
-                               const uint32_t *__restrict__ off, int n, int tiles_x,
+                               const uint32_t *__restrict__ off, int n, int tiles_x, int ts,
                                uint32_t *__restrict__ tile_key, uint32_t *__restrict__ gid) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -630,8 +651,8 @@ __global__ void k_gs_duplicate(const uint32_t *__restrict__ order, const int4 *_
     const int4 r = rect[g];
     if (!(r.z >= r.x && r.w >= r.y)) return;
     uint32_t o = off[k];
-    for (int ty = r.y / GS_TILE; ty <= r.w / GS_TILE; ++ty)
-        for (int tx = r.x / GS_TILE; tx <= r.z / GS_TILE; ++tx) {
+    for (int ty = r.y >> ts; ty <= r.w >> ts; ++ty)
+        for (int tx = r.x >> ts; tx <= r.z >> ts; ++tx) {
             tile_key[o] = (uint32_t)(ty * tiles_x + tx);
             gid[o] = g;
             ++o;
@@ -640,15 +661,17 @@ __global__ void k_gs_duplicate(const uint32_t *__restrict__ order, const int4 *_
 
 // ---------------------------------------------------------------- render --
 
-// The batch [b0, b0 + GS_THREADS) of the tile's range in shared memory.
+// A batch of the tile's range, from entry b0 on, in shared memory.
+template <int TS>
 struct GsBatch {
-    float4 row[GS_THREADS][3];  // mu(2) conic(3) opacity color(3), 3 unused
-    int id[GS_THREADS];
+    float4 row[gs_threads(TS)][3];  // mu(2) conic(3) opacity color(3), 3 unused
+    int id[gs_threads(TS)];
 };
 
+template <int TS>
 __device__ __forceinline__ int gs_load_batch(int b0, int end, const uint32_t *__restrict__ list,
-                                             const float4 *__restrict__ rows, GsBatch &s) {
-    const int cnt = min(GS_THREADS, end - b0);
+                                             const float4 *__restrict__ rows, GsBatch<TS> &s) {
+    const int cnt = min(gs_threads(TS), end - b0);
     if ((int)threadIdx.x < cnt) {
         const int g = (int)list[b0 + threadIdx.x];
         s.id[threadIdx.x] = g;
@@ -659,18 +682,20 @@ __device__ __forceinline__ int gs_load_batch(int b0, int end, const uint32_t *__
     return cnt;
 }
 
-__global__ void __launch_bounds__(GS_THREADS) k_gs_render_fwd(
+template <int TS>
+__global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_fwd(
     GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
     const float4 *__restrict__ rows, float *__restrict__ image, float *__restrict__ image_keep,
     const uint32_t *__restrict__ batch_off, float4 *__restrict__ before) {
-    __shared__ GsBatch s;
-    const int tx0 = (int)(blockIdx.x % tiles_x) * GS_TILE, ty0 = (int)(blockIdx.x / tiles_x) * GS_TILE;
-    const int px = tx0 + (threadIdx.x & (GS_TILE - 1)), py = ty0 + threadIdx.x / GS_TILE;
+    constexpr int TILE = 1 << TS, THREADS = gs_threads(TS);
+    __shared__ GsBatch<TS> s;
+    const int tx0 = (int)(blockIdx.x % tiles_x) * TILE, ty0 = (int)(blockIdx.x / tiles_x) * TILE;
+    const int px = tx0 + (threadIdx.x & (TILE - 1)), py = ty0 + threadIdx.x / TILE;
     const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
     const int2 rg = ranges[blockIdx.x];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    float4 *keep = before + (size_t)batch_off[blockIdx.x] * GS_THREADS + threadIdx.x;
-    for (int b0 = rg.x; b0 < rg.y; b0 += GS_THREADS, keep += GS_THREADS) {
+    float4 *keep = before + (size_t)batch_off[blockIdx.x] * THREADS + threadIdx.x;
+    for (int b0 = rg.x; b0 < rg.y; b0 += THREADS, keep += THREADS) {
         const int cnt = gs_load_batch(b0, rg.y, list, rows, s);
         *keep = make_float4(C0, C1, C2, T);  // for the backward, which takes each batch by itself
 #pragma unroll 4
@@ -745,16 +770,18 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
 // s d d^T, which k_gs_preprocess_bwd turns into dL/d(mu', conic). Each warp's
 // nine sums go to the Gaussian's row of g2d (GS_ROW floats, so nine
 // neighbouring words: two sectors) from nine lanes at once.
-__global__ void __launch_bounds__(GS_THREADS) k_gs_render_bwd(
+template <int TS>
+__global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_bwd(
     GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
     const float4 *__restrict__ rows, const uint32_t *__restrict__ batch_tile,
     const uint32_t *__restrict__ batch_off, const float4 *__restrict__ before,
     const float *__restrict__ image_keep, const float *__restrict__ g_image,
     float *__restrict__ g2d) {
-    __shared__ GsBatch s;
+    constexpr int TILE = 1 << TS, THREADS = gs_threads(TS);
+    __shared__ GsBatch<TS> s;
     const unsigned tile = batch_tile[blockIdx.x];
-    const int tx0 = (int)(tile % tiles_x) * GS_TILE, ty0 = (int)(tile / tiles_x) * GS_TILE;
-    const int px = tx0 + (threadIdx.x & (GS_TILE - 1)), py = ty0 + threadIdx.x / GS_TILE;
+    const int tx0 = (int)(tile % tiles_x) * TILE, ty0 = (int)(tile / tiles_x) * TILE;
+    const int px = tx0 + (threadIdx.x & (TILE - 1)), py = ty0 + threadIdx.x / TILE;
     const bool inside = px < c.width && py < c.height;
     const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
     const int64_t hw = (int64_t)c.width * c.height, pix = (int64_t)py * c.width + px;
@@ -766,11 +793,11 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_render_bwd(
             gC[ch] = g_image[ch * hw + pix];
         }
     }
-    const float4 b4 = before[(size_t)blockIdx.x * GS_THREADS + threadIdx.x];
+    const float4 b4 = before[(size_t)blockIdx.x * THREADS + threadIdx.x];
     float T = b4.w, Cl[3] = {b4.x, b4.y, b4.z};
     const int lane = threadIdx.x & 31;
     const int2 rg = ranges[tile];
-    const int cnt = gs_load_batch(rg.x + (int)(blockIdx.x - batch_off[tile]) * GS_THREADS, rg.y, list,
+    const int cnt = gs_load_batch(rg.x + (int)(blockIdx.x - batch_off[tile]) * THREADS, rg.y, list,
                                   rows, s);
 #pragma unroll 2
     for (int k = 0; k < cnt; ++k) {
@@ -1166,7 +1193,7 @@ struct GsHandle {
     uint32_t *rk[2] = {nullptr, nullptr}, *rv[2] = {nullptr, nullptr}, *rcounts = nullptr;
     uint32_t *tcnt = nullptr, *toff = nullptr, *bsum = nullptr, *total = nullptr;
     const uint32_t *list = nullptr;  // the sorted Gaussian column of the last gs_render
-    int tiles_x = 0, tiles_y = 0;
+    int ts = GS_FINE, tiles_x = 0, tiles_y = 0;  // tiles of the last gs_render
     int last_n = -1;  // Gaussians of the last gs_render
     // inputs and camera of the last gs_render (the backward must see the same)
     const void *last_in[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -1208,6 +1235,12 @@ using namespace dw;
 
 struct dw_gs_s : GsHandle {};
 
+static void gs_set_tiles(dw_gs h, int ts) {
+    h->ts = ts;
+    h->tiles_x = ((h->width - 1) >> ts) + 1;
+    h->tiles_y = ((h->height - 1) >> ts) + 1;
+}
+
 // Grow the tile-list buffers to hold m entries.
 static dw_status gs_list_reserve(dw_gs h, int64_t m) {
     if (m <= h->list_cap) return DW_OK;
@@ -1224,7 +1257,8 @@ static dw_status gs_list_reserve(dw_gs h, int64_t m) {
     return DW_OK;
 }
 
-// Grow the batch buffers to hold nb batches (1 KB each).
+// Grow the batch buffers to hold nb batches of fine tiles (1 KB each; a coarse
+// tile's batch takes four of them).
 static dw_status gs_batch_reserve(dw_gs h, int64_t nb) {
     if (nb <= h->batch_cap) return DW_OK;
     const int64_t cap = std::max<int64_t>(nb, h->batch_cap * 3 / 2);
@@ -1235,7 +1269,7 @@ static dw_status gs_batch_reserve(dw_gs h, int64_t nb) {
     h->batch_cap = 0;
     cudaError_t e = cudaMalloc((void **)&h->batch_tile, sizeof(uint32_t) * (size_t)cap);
     if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->before, sizeof(float4) * GS_THREADS * (size_t)cap);
+        e = cudaMalloc((void **)&h->before, sizeof(float4) * gs_threads(GS_FINE) * (size_t)cap);
     if (e != cudaSuccess) return cuda_fail(e, "gs_render (list batches)");
     h->batch_cap = cap;
     return DW_OK;
@@ -1289,15 +1323,15 @@ static dw_status gs_list_radix(dw_gs h, int n, int64_t m, cudaStream_t s) {
     uint32_t *ka = h->rk[0], *va = h->rv[0], *kb = h->rk[1], *vb = h->rv[1];
     k_gs_order_init<<<grid_for(n, 256), 256, 0, s>>>(h->key, n, ka, va);
     radix_sort(ka, va, kb, vb, n, 4, h->rcounts, s);  // depth order in va
-    k_gs_tile_count<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, n, h->tcnt);
+    k_gs_tile_count<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, n, h->ts, h->tcnt);
     const int nsb = (n + 1023) / 1024;
     k_scan1024<<<nsb, 256, 0, s>>>(h->tcnt, n, h->toff, h->bsum);
     k_rs_scan<<<1, 1024, 0, s>>>(h->bsum, nsb);
     k_scan_finish<<<grid_for(n, 256), 256, 0, s>>>(h->toff, h->tcnt, n, h->bsum, h->total);
     // the list: tile keys to kb, Gaussians to lgid, then both sorted (the depth
     // order in va is read before the sort's second buffers overwrite it)
-    k_gs_duplicate<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, h->toff, n, h->tiles_x, kb,
-                                                    h->lgid);
+    k_gs_duplicate<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, h->toff, n, h->tiles_x, h->ts,
+                                                    kb, h->lgid);
     int bits = 1;
     while ((1ll << bits) < (int64_t)h->tiles_x * h->tiles_y) ++bits;
     uint32_t *lk = kb, *lv = h->lgid, *lk2 = ka, *lv2 = va;
@@ -1320,8 +1354,7 @@ extern "C" dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t hei
     h->cap = max_gaussians;
     h->width = width;
     h->height = height;
-    h->tiles_x = (width + GS_TILE - 1) / GS_TILE;
-    h->tiles_y = (height + GS_TILE - 1) / GS_TILE;
+    gs_set_tiles(h, GS_FINE);  // the coarse tiles are fewer
     const size_t n = (size_t)max_gaussians, tiles = (size_t)h->tiles_x * h->tiles_y;
     cudaError_t e = cudaMalloc((void **)&h->rows, sizeof(float4) * 3 * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&h->g2d, sizeof(float) * GS_ROW * n);
@@ -1387,6 +1420,66 @@ static dw_status gs_check(dw_gs h, const dw_camera *cam, const float *x, const f
     return DW_OK;
 }
 
+// The scan of the tiles' counts, and what the host needs of it (waits for s).
+static dw_status gs_scan(dw_gs h, GsStat &stat, cudaStream_t s) {
+    k_gs_tile_scan<<<1, 1024, 0, s>>>(h->tile_count, h->tiles_x * h->tiles_y, h->ts, h->ranges,
+                                      h->batch_off, h->stat);
+    DW_CUDA(cudaMemcpyAsync(&stat, h->stat, sizeof stat, cudaMemcpyDeviceToHost, s));
+    DW_CUDA(cudaStreamSynchronize(s));
+    return DW_OK;
+}
+
+// The Gaussians projected and counted in the fine tiles they meet.
+static dw_status gs_count(dw_gs h, const GsCam &c, const float *x, const float *F, const float *sigma0,
+                          const float *color, const float *opacity, int n, GsStat &stat,
+                          cudaStream_t s) {
+    uint32_t *queued = h->big + h->cap;
+    DW_CUDA(cudaMemsetAsync(h->tile_count, 0, sizeof(uint32_t) * (size_t)h->tiles_x * h->tiles_y, s));
+    DW_CUDA(cudaMemsetAsync(queued, 0, sizeof(uint32_t), s));
+    k_gs_preprocess<<<grid_for(n, 128), 128, 0, s>>>(c, x, F, sigma0, color, opacity, n, h->tiles_x,
+                                                     h->rows, h->rect, h->key, h->tile_count, h->big,
+                                                     queued);
+    k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key, h->tiles_x, h->ts,
+                                                h->tile_count, h->ranges, h->lkey, h->stat);
+    return gs_scan(h, stat, s);
+}
+
+// The projected Gaussians counted again, in the tiles set now.
+static dw_status gs_recount(dw_gs h, int n, GsStat &stat, cudaStream_t s) {
+    DW_CUDA(cudaMemsetAsync(h->tile_count, 0, sizeof(uint32_t) * (size_t)h->tiles_x * h->tiles_y, s));
+    k_gs_list<false><<<grid_for(n, 128), 128, 0, s>>>(h->rect, h->key, n, h->tiles_x, h->ts,
+                                                      h->tile_count, h->ranges, h->lkey);
+    k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, h->big + h->cap, h->rect, h->key, h->tiles_x,
+                                                h->ts, h->tile_count, h->ranges, h->lkey, h->stat);
+    return gs_scan(h, stat, s);
+}
+
+// The counted tiles' lists in order, and their batches.
+static dw_status gs_make_list(dw_gs h, int n, const GsStat &stat, cudaStream_t s) {
+    const int ntiles = h->tiles_x * h->tiles_y;
+    dw_status st = gs_list_reserve(h, (int64_t)stat.total);
+    if (st == DW_OK) st = gs_batch_reserve(h, (int64_t)stat.batches << (2 * (h->ts - GS_FINE)));
+    if (st != DW_OK) return st;
+    h->list = h->lgid;
+    k_gs_list<true><<<grid_for(n, 128), 128, 0, s>>>(h->rect, h->key, n, h->tiles_x, h->ts,
+                                                     h->tile_count, h->ranges, h->lkey);
+    if (stat.big > 0)
+        k_gs_big<true><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, h->big + h->cap, h->rect, h->key, h->tiles_x,
+                                                   h->ts, h->tile_count, h->ranges, h->lkey, h->stat);
+    if (stat.most <= GS_SORT_MAX) {
+        size_t len = 2;
+        while (len < stat.most) len <<= 1;
+        k_gs_tile_sort<<<(unsigned)ntiles, GS_SORT_THREADS, len * sizeof(unsigned long long), s>>>(
+            h->ranges, h->lkey, h->batch_off, h->ts, h->lgid, h->batch_tile);
+    } else {
+        st = gs_list_radix(h, n, (int64_t)stat.total, s);
+        if (st != DW_OK) return st;
+        k_gs_batches<<<grid_for(ntiles, 256), 256, 0, s>>>(h->ranges, ntiles, h->ts, h->batch_off,
+                                                           h->batch_tile);
+    }
+    return DW_OK;
+}
+
 extern "C" dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, const float *F,
                                const float *sigma0, const float *color, const float *opacity,
                                int64_t n, float *image, dw_stream stream) {
@@ -1396,55 +1489,32 @@ extern "C" dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, co
     cudaStream_t s = as_stream(stream);
     const GsCam c = to_cam(*cam);
     const int nn = (int)n;
-    const int ntiles = h->tiles_x * h->tiles_y;
     h->last_n = -1;  // no picture to differentiate until this call has drawn one
-    h->list = h->lgid;
+    gs_set_tiles(h, GS_FINE);
     if (nn > 0) {
-        DW_CUDA(cudaMemsetAsync(h->tile_count, 0, sizeof(uint32_t) * (size_t)ntiles, s));
-        uint32_t *queued = h->big + h->cap;
-        DW_CUDA(cudaMemsetAsync(queued, 0, sizeof(uint32_t), s));
-        k_gs_preprocess<<<grid_for(nn, 128), 128, 0, s>>>(c, x, F, sigma0, color, opacity, nn,
-                                                          h->tiles_x, h->rows, h->rect, h->key,
-                                                          h->tile_count, h->big, queued);
-        k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key, h->tiles_x,
-                                                    h->tile_count, h->ranges, h->lkey, h->stat);
-        k_gs_tile_scan<<<1, 1024, 0, s>>>(h->tile_count, ntiles, h->ranges, h->batch_off, h->stat);
         GsStat stat;
-        DW_CUDA(cudaMemcpyAsync(&stat, h->stat, sizeof stat, cudaMemcpyDeviceToHost, s));
-        DW_CUDA(cudaStreamSynchronize(s));
-        const unsigned long long m = stat.total;
-        DW_REQUIRE(m < (1ull << 31), "tile list too long (Gaussians x tiles met >= 2^31)");
+        st = gs_count(h, c, x, F, sigma0, color, opacity, nn, stat, s);
+        if (st == DW_OK && stat.total > (unsigned long long)GS_LIST_MAX) {
+            gs_set_tiles(h, GS_COARSE);
+            st = gs_recount(h, nn, stat, s);
+        }
+        if (st != DW_OK) return st;
+        DW_REQUIRE(stat.total <= (unsigned long long)GS_LIST_MAX,
+                   "tile list too long (Gaussians x tiles met >= 2^31)");
         h->batches = stat.batches;
-        if (m > 0) {
-            st = gs_list_reserve(h, (int64_t)m);
-            if (st == DW_OK) st = gs_batch_reserve(h, stat.batches);
+        if (stat.total > 0) {
+            st = gs_make_list(h, nn, stat, s);
             if (st != DW_OK) return st;
-            h->list = h->lgid;
-            k_gs_list<<<grid_for(nn, 128), 128, 0, s>>>(h->rect, h->key, nn, h->tiles_x, h->ranges,
-                                                        h->lkey);
-            if (stat.big > 0)
-                k_gs_big<true><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key,
-                                                           h->tiles_x, h->tile_count, h->ranges,
-                                                           h->lkey, h->stat);
-            if (stat.most <= GS_SORT_MAX) {
-                size_t len = 2;
-                while (len < stat.most) len <<= 1;
-                k_gs_tile_sort<<<(unsigned)ntiles, GS_SORT_THREADS, len * sizeof(unsigned long long), s>>>(
-                    h->ranges, h->lkey, h->batch_off, h->lgid, h->batch_tile);
-            } else {
-                st = gs_list_radix(h, nn, (int64_t)m, s);
-                if (st != DW_OK) return st;
-                k_gs_batches<<<grid_for(ntiles, 256), 256, 0, s>>>(h->ranges, ntiles, h->batch_off,
-                                                                   h->batch_tile);
-            }
         }
     } else {
-        DW_CUDA(cudaMemsetAsync(h->ranges, 0, sizeof(int2) * (size_t)ntiles, s));
-        DW_CUDA(cudaMemsetAsync(h->batch_off, 0, sizeof(uint32_t) * (size_t)ntiles, s));
+        const size_t ntiles = (size_t)h->tiles_x * h->tiles_y;
+        DW_CUDA(cudaMemsetAsync(h->ranges, 0, sizeof(int2) * ntiles, s));
+        DW_CUDA(cudaMemsetAsync(h->batch_off, 0, sizeof(uint32_t) * ntiles, s));
         h->batches = 0;
     }
-    k_gs_render_fwd<<<(unsigned)ntiles, GS_THREADS, 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, image, h->image,
-                                                            h->batch_off, h->before);
+    auto kern = h->ts == GS_FINE ? k_gs_render_fwd<GS_FINE> : k_gs_render_fwd<GS_COARSE>;
+    kern<<<(unsigned)(h->tiles_x * h->tiles_y), gs_threads(h->ts), 0, s>>>(
+        c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, image, h->image, h->batch_off, h->before);
     h->last_n = nn;
     const void *in[5] = {x, F, sigma0, color, opacity};
     memcpy(h->last_in, in, sizeof in);
@@ -1470,10 +1540,11 @@ extern "C" dw_status gs_render_backward(dw_gs h, const dw_camera *cam, const flo
     const GsCam c = to_cam(*cam);
     const int nn = (int)n;
     DW_CUDA(cudaMemsetAsync(h->g2d, 0, sizeof(float) * GS_ROW * (size_t)nn, s));
+    auto kern = h->ts == GS_FINE ? k_gs_render_bwd<GS_FINE> : k_gs_render_bwd<GS_COARSE>;
     if (h->batches > 0)
-        k_gs_render_bwd<<<h->batches, GS_THREADS, 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges,
-                                                         h->rows, h->batch_tile, h->batch_off,
-                                                         h->before, h->image, g_image, h->g2d);
+        kern<<<h->batches, gs_threads(h->ts), 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows,
+                                                      h->batch_tile, h->batch_off, h->before, h->image,
+                                                      g_image, h->g2d);
     k_gs_preprocess_bwd<<<grid_for(nn, 256), 256, 0, s>>>(c, x, F, sigma0, opacity, nn, h->g2d, g_x, g_F,
                                                            g_color, g_opacity);
     DW_LAUNCHED("gs_render_backward");

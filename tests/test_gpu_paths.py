@@ -424,3 +424,49 @@ def test_gaussian_list_of_2_36_entries():
     img = r.render(cam, *[a[..., :3].contiguous() for a in (x, F, s0, col, op)])
     assert abs(img[0, W // 2, W // 2].item() - 0.5 * (1 - 0.75 ** 3)) <= 1e-3
     r.close()
+
+
+# Lists too long for 8 x 8 tiles, made on 16 x 16: Gaussians about the optical
+# axis that cover the image (q < 9 everywhere), at a few pixels against the
+# float64 composite, with the gradients of those pixels. A pixel is a product of
+# n factors, each rounded twice: n^0.5 x 1.2e-7 = 2 to 3e-5 of the image if the
+# roundings are independent, allowed 1e-4. dL/dopacity is a difference of two
+# such terms, allowed 1e-3 relative L2.
+@pytest.mark.parametrize("size,n", [((2048, 2048), 32769)])
+def test_gaussian_list_on_coarse_tiles(size, n):
+    (W, H), g = size, np.random.default_rng(3)
+    if torch.cuda.mem_get_info()[0] < 120 << 30:
+        pytest.skip("needs 120 GB of device memory")
+    assert n * ((W + 7) // 8) * ((H + 7) // 8) > 2 ** 31 - 4096
+    f, s = 0.4 * W, 1.5
+    x, F, s0 = np.zeros((3, n), np.float32), np.zeros((9, n), np.float32), np.zeros((6, n), np.float32)
+    x[2] = (g.permutation(n) / n - 0.5) * 0.8
+    F[::4] = 1.0
+    s0[:3] = s * s
+    col = g.uniform(0.0, 1.0, (3, n)).astype(np.float32)
+    op = (g.uniform(0.5, 1.5, n) * 3.0 / n).astype(np.float32)
+    cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), f, f, W / 2, H / 2, W, H)
+    d = [to_dev(a) for a in (x, F, s0, col, op)]
+    r = B.GaussianRenderer(n, W, H)
+    img = r.render(cam, *d)
+    pix = [(0, 0), (W - 1, H - 1), (W // 2, H // 2 - 1), (W - 16, H - 1), (17, 15)]
+    g_img = torch.zeros((3, H, W), device="cuda")
+    for k, (px, py) in enumerate(pix):
+        g_img[:, py, px] = torch.tensor([1.0, -0.5, 0.25]) * (k + 1)
+    gs = [torch.zeros_like(d[k]) for k in (0, 1, 3, 4)]
+    r.backward(cam, *d, g_img, *gs)
+    tz = 2.0 + x[2].astype(np.float64)
+    order = np.argsort(tz)
+    gc, go = np.zeros((3, n)), np.zeros(n)
+    for k, (px, py) in enumerate(pix):
+        e = np.exp(-0.5 * ((px + 0.5 - W / 2) ** 2 + (py + 0.5 - H / 2) ** 2) / (f * s / tz) ** 2)[order]
+        a, c = op.astype(np.float64)[order] * e, col.astype(np.float64)[:, order]
+        T = np.concatenate([[1.0], np.cumprod(1.0 - a)[:-1]])
+        part = np.cumsum(T * a * c, axis=1)
+        C = part[:, -1:]
+        assert np.abs(img[:, py, px].cpu().numpy() - C[:, 0]).max() <= 1e-4
+        w = np.array([1.0, -0.5, 0.25])[:, None] * (k + 1)
+        gc[:, order] += w * T * a
+        go[order] += (w * (T * c - (C - part) / (1.0 - a))).sum(0) * e
+    assert rel_l2(gs[2].cpu().numpy(), gc) <= 1e-4 and rel_l2(gs[3].cpu().numpy(), go) <= 1e-3
+    r.close()

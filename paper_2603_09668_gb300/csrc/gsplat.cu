@@ -53,13 +53,15 @@ namespace dw {
 // hold, is made on 16 instead.
 constexpr int GS_FINE = 3, GS_COARSE = 4;
 __host__ __device__ constexpr int gs_threads(int ts) { return 1 << (2 * ts); }
-constexpr int64_t GS_LIST_MAX = (1ll << 31) - 1;
 constexpr int GS_SORT_MAX = 4096;   // keys of one tile k_gs_tile_sort holds
 constexpr int GS_SORT_THREADS = 128;
 constexpr int GS_BIG_CTAS = 304;    // two per SM
 constexpr int GS_ROW = 12;          // floats per Gaussian of the packed rows and of the 2D gradients
 constexpr int RS_THREADS = 256;
 constexpr int RS_TILE = RS_THREADS * 16;  // keys per sort block
+// Entries of a list: the sort's last block and a tile's last batch step past it
+// by up to RS_TILE, in 32-bit indices.
+constexpr int64_t GS_LIST_MAX = (1ll << 31) - RS_TILE;
 
 struct GsCam {
     float R[9], T[3];

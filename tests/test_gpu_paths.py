@@ -426,13 +426,14 @@ def test_gaussian_list_of_2_36_entries():
     r.close()
 
 
-# Lists too long for 8 x 8 tiles, made on 16 x 16: Gaussians about the optical
+# Lists too long for 8 x 8 tiles (the second by the indices' step past the end: 2^31
+# - 2 entries), made on 16 x 16: Gaussians about the optical
 # axis that cover the image (q < 9 everywhere), at a few pixels against the
 # float64 composite, with the gradients of those pixels. A pixel is a product of
 # n factors, each rounded twice: n^0.5 x 1.2e-7 = 2 to 3e-5 of the image if the
 # roundings are independent, allowed 1e-4. dL/dopacity is a difference of two
 # such terms, allowed 1e-3 relative L2.
-@pytest.mark.parametrize("size,n", [((2048, 2048), 32769)])
+@pytest.mark.parametrize("size,n", [((2048, 2048), 32769), ((1736, 1208), 65538)])
 def test_gaussian_list_on_coarse_tiles(size, n):
     (W, H), g = size, np.random.default_rng(3)
     if torch.cuda.mem_get_info()[0] < 120 << 30:

@@ -386,8 +386,13 @@ DW_API dw_status gs_covariance(const float *F, const float *sigma0, int64_t n, f
                                dw_stream stream);
 
 /* Renderer workspace for up to max_gaussians Gaussians and width x height
- * images (about 120 bytes per Gaussian plus one image; gs_render adds, and grows
- * when needed, about 30 bytes per entry of the tile lists). */
+ * images (about 120 bytes per Gaussian plus one image). gs_render adds, and
+ * grows when needed, the tile lists: 12 bytes per entry (a Gaussian on an 8 x 8
+ * pixel tile it meets), 16 and 24 per Gaussian when a tile has more than 4,096;
+ * and for gs_render_backward 1 KB per started batch of 64 entries of a tile.
+ * Without memory for the last the backward walks the lists tile by tile;
+ * without memory for the lists, or from 2^31 entries on, they are made on 16 x 16
+ * tiles, and only then is the call refused. */
 DW_API dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t height, dw_gs *out);
 DW_API dw_status gs_destroy(dw_gs h);
 
@@ -395,7 +400,7 @@ DW_API dw_status gs_destroy(dw_gs h);
  * with deformation gradients F and rest covariances sigma0. The handle keeps
  * the projected Gaussians, their depth order, the per-tile lists and the
  * image for gs_render_backward. cam's image size must be the handle's. The
- * call reads the length of the tile lists back to the host (16 bytes) to size the
+ * call reads the length of the tile lists back to the host (24 bytes) to size the
  * lists, so it waits for `stream` and cannot be captured in a CUDA graph. */
 DW_API dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, const float *F,
                            const float *sigma0, const float *color, const float *opacity,

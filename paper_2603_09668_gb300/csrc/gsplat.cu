@@ -539,15 +539,16 @@ __device__ __forceinline__ void gs_write_batches(int t, int cnt, int ts, const u
 // the Gaussians' indices in order go to gid. A warp's threads compare within
 // 64 consecutive keys while the distance is at most 32, so only the longer
 // distances need the block's barrier.
+template <int TS>
 __global__ void __launch_bounds__(GS_SORT_THREADS) k_gs_tile_sort(
     const int2 *__restrict__ ranges, const unsigned long long *__restrict__ list,
-    const uint32_t *__restrict__ batch_off, int ts, uint32_t *__restrict__ gid,
+    const uint32_t *__restrict__ batch_off, uint32_t *__restrict__ gid,
     uint32_t *__restrict__ batch_tile) {
     extern __shared__ unsigned long long k[];  // the longest list, rounded up to a power of two
     const int2 rg = ranges[blockIdx.x];
     const int cnt = rg.y - rg.x;
     if (cnt <= 0) return;
-    gs_write_batches(blockIdx.x, cnt, ts, batch_off, batch_tile);
+    gs_write_batches(blockIdx.x, cnt, TS, batch_off, batch_tile);
     int size = 2;
     while (size < cnt) size <<= 1;
     for (int i = threadIdx.x; i < size; i += GS_SORT_THREADS) k[i] = i < cnt ? list[rg.x + i] : ~0ull;
@@ -573,13 +574,16 @@ __global__ void __launch_bounds__(GS_SORT_THREADS) k_gs_tile_sort(
     for (int i = threadIdx.x; i < cnt; i += GS_SORT_THREADS) gid[rg.x + i] = (uint32_t)k[i];
 }
 
-// The batches of every tile (the radix path; one thread per tile).
-__global__ void __launch_bounds__(256) k_gs_batches(const int2 *__restrict__ ranges, int tiles,
+// The end of every tile's range, and its batches (the radix path; one thread
+// per tile).
+__global__ void __launch_bounds__(256) k_gs_batches(const uint32_t *__restrict__ count, int tiles,
                                                     int ts, const uint32_t *__restrict__ batch_off,
+                                                    int2 *__restrict__ ranges,
                                                     uint32_t *__restrict__ batch_tile) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
-    const int nb = (int)gs_batches(ranges[t].y - ranges[t].x, ts);
+    ranges[t].y = ranges[t].x + (int)count[t];
+    const int nb = (int)gs_batches(count[t], ts);
     for (int k = 0; k < nb; ++k) batch_tile[batch_off[t] + k] = (uint32_t)t;
 }
 
@@ -633,14 +637,10 @@ __global__ void __launch_bounds__(256) k_scan1024(const uint32_t *__restrict__ i
     if (threadIdx.x == 255) sums[blockIdx.x] = part[255];
 }
 
-// out += the scanned block offsets; the total goes to *total.
-__global__ void k_scan_finish(uint32_t *__restrict__ out, const uint32_t *__restrict__ cnt, int n,
-                              const uint32_t *__restrict__ block_off, uint32_t *__restrict__ total) {
+// out += the scanned block offsets.
+__global__ void k_scan_finish(uint32_t *__restrict__ out, int n, const uint32_t *__restrict__ block_off) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t o = out[i] + block_off[i / 1024];
-    out[i] = o;
-    if (i == n - 1) *total = o + cnt[i];
+    if (i < n) out[i] += block_off[i / 1024];
 }
 
 // One entry (tile id, Gaussian) per tile met, written in depth order.
@@ -684,7 +684,10 @@ __device__ __forceinline__ int gs_load_batch(int b0, int end, const uint32_t *__
     return cnt;
 }
 
-template <int TS>
+// KEEP: each batch's colour and transmittance in front of it go to `before`, for
+// the backward, which takes each batch by itself (as a test of the pointer in the
+// loop instead, 66 us against 59).
+template <int TS, bool KEEP>
 __global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_fwd(
     GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
     const float4 *__restrict__ rows, float *__restrict__ image, float *__restrict__ image_keep,
@@ -696,10 +699,10 @@ __global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_fwd(
     const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
     const int2 rg = ranges[blockIdx.x];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    float4 *keep = before + (size_t)batch_off[blockIdx.x] * THREADS + threadIdx.x;
+    float4 *keep = KEEP ? before + (size_t)batch_off[blockIdx.x] * THREADS + threadIdx.x : nullptr;
     for (int b0 = rg.x; b0 < rg.y; b0 += THREADS, keep += THREADS) {
         const int cnt = gs_load_batch(b0, rg.y, list, rows, s);
-        *keep = make_float4(C0, C1, C2, T);  // for the backward, which takes each batch by itself
+        if (KEEP) *keep = make_float4(C0, C1, C2, T);
 #pragma unroll 4
         for (int k = 0; k < cnt; ++k) {
             const float4 r = s.row[k][0], u = s.row[k][1];
@@ -771,8 +774,9 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
 // of a Gaussian's gradients are linear in the sums over pixels of s, s d and
 // s d d^T, which k_gs_preprocess_bwd turns into dL/d(mu', conic). Each warp's
 // nine sums go to the Gaussian's row of g2d (GS_ROW floats, so nine
-// neighbouring words: two sectors) from nine lanes at once.
-template <int TS>
+// neighbouring words: two sectors) from nine lanes at once. WALK: without
+// `before`, one tile per block, its batches one after the other.
+template <int TS, bool WALK>
 __global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_bwd(
     GsCam c, unsigned tiles_x, const uint32_t *__restrict__ list, const int2 *__restrict__ ranges,
     const float4 *__restrict__ rows, const uint32_t *__restrict__ batch_tile,
@@ -781,7 +785,7 @@ __global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_bwd(
     float *__restrict__ g2d) {
     constexpr int TILE = 1 << TS, THREADS = gs_threads(TS);
     __shared__ GsBatch<TS> s;
-    const unsigned tile = batch_tile[blockIdx.x];
+    const unsigned tile = WALK ? blockIdx.x : batch_tile[blockIdx.x];
     const int tx0 = (int)(tile % tiles_x) * TILE, ty0 = (int)(tile / tiles_x) * TILE;
     const int px = tx0 + (threadIdx.x & (TILE - 1)), py = ty0 + threadIdx.x / TILE;
     const bool inside = px < c.width && py < c.height;
@@ -795,50 +799,56 @@ __global__ void __launch_bounds__(gs_threads(TS)) k_gs_render_bwd(
             gC[ch] = g_image[ch * hw + pix];
         }
     }
-    const float4 b4 = before[(size_t)blockIdx.x * THREADS + threadIdx.x];
+    const float4 b4 = WALK ? make_float4(0.0f, 0.0f, 0.0f, 1.0f)
+                           : before[(size_t)blockIdx.x * THREADS + threadIdx.x];
     float T = b4.w, Cl[3] = {b4.x, b4.y, b4.z};
     const int lane = threadIdx.x & 31;
     const int2 rg = ranges[tile];
-    const int cnt = gs_load_batch(rg.x + (int)(blockIdx.x - batch_off[tile]) * THREADS, rg.y, list,
-                                  rows, s);
+    if (WALK && rg.x >= rg.y) return;
+    int b0 = rg.x + (WALK ? 0 : (int)(blockIdx.x - batch_off[tile]) * THREADS);
+    do {
+        const int cnt = gs_load_batch(b0, rg.y, list, rows, s);
 #pragma unroll 2
-    for (int k = 0; k < cnt; ++k) {
-        const float4 r = s.row[k][0], u = s.row[k][1];
-        const float dx = fx - r.x, dy = fy - r.y;
-        const float q = r.z * dx * dx + 2.0f * r.w * dx * dy + u.x * dy * dy;
-        const bool hit = inside && q <= 9.0f;
-        if (!__any_sync(0xffffffffu, hit)) continue;
-        // s d (2), s d d^T (3), s, dL/dcolor (3)
-        float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, v8 = 0.0f;
-        if (hit) {
-            const float col[3] = {u.z, u.w, s.row[k][2].x};
-            const float e = expf(-0.5f * q);
-            const float a = u.y * e;
-            const float w = T * a, inv = 1.0f / (1.0f - a);
-            float dA = 0.0f;
+        for (int k = 0; k < cnt; ++k) {
+            const float4 r = s.row[k][0], u = s.row[k][1];
+            const float dx = fx - r.x, dy = fy - r.y;
+            const float q = r.z * dx * dx + 2.0f * r.w * dx * dy + u.x * dy * dy;
+            const bool hit = inside && q <= 9.0f;
+            if (!__any_sync(0xffffffffu, hit)) continue;
+            // s d (2), s d d^T (3), s, dL/dcolor (3)
+            float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, v8 = 0.0f;
+            if (hit) {
+                const float col[3] = {u.z, u.w, s.row[k][2].x};
+                const float e = expf(-0.5f * q);
+                const float a = u.y * e;
+                const float w = T * a, inv = 1.0f / (1.0f - a);
+                float dA = 0.0f;
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                Cl[ch] += w * col[ch];
-                dA += gC[ch] * (T * col[ch] - (Cf[ch] - Cl[ch]) * inv);
+                for (int ch = 0; ch < 3; ++ch) {
+                    Cl[ch] += w * col[ch];
+                    dA += gC[ch] * (T * col[ch] - (Cf[ch] - Cl[ch]) * inv);
+                }
+                v[5] = dA * e;
+                v[0] = v[5] * dx;
+                v[1] = v[5] * dy;
+                v[2] = v[0] * dx;
+                v[3] = v[0] * dy;
+                v[4] = v[1] * dy;
+                v[6] = gC[0] * w;
+                v[7] = gC[1] * w;
+                v8 = gC[2] * w;
+                T *= 1.0f - a;
             }
-            v[5] = dA * e;
-            v[0] = v[5] * dx;
-            v[1] = v[5] * dy;
-            v[2] = v[0] * dx;
-            v[3] = v[0] * dy;
-            v[4] = v[1] * dy;
-            v[6] = gC[0] * w;
-            v[7] = gC[1] * w;
-            v8 = gC[2] * w;
-            T *= 1.0f - a;
+            const float t = warp_sum8(v), t8 = warp_sum(v8);
+            // lane 4 j adds value j, lane 1 value 8
+            const int j = (lane & 3) == 0 ? lane >> 2 : 8;
+            const float mine = j == 8 ? t8 : t;
+            if (((lane & 3) == 0 || lane == 1) && mine != 0.0f)
+                atomicAdd(&g2d[(int64_t)s.id[k] * GS_ROW + j], mine);
         }
-        const float t = warp_sum8(v), t8 = warp_sum(v8);
-        // lane 4 j adds value j, lane 1 value 8
-        const int j = (lane & 3) == 0 ? lane >> 2 : 8;
-        const float mine = j == 8 ? t8 : t;
-        if (((lane & 3) == 0 || lane == 1) && mine != 0.0f)
-            atomicAdd(&g2d[(int64_t)s.id[k] * GS_ROW + j], mine);
-    }
+        if (WALK) __syncthreads();
+        b0 += THREADS;
+    } while (WALK && b0 < rg.y);
 }
 
 // The 2D gradients of each Gaussian (k_gs_render_bwd's sums) -> dL/dx, dL/dF (and the
@@ -1166,6 +1176,38 @@ static SsimWin ssim_window() {
     return k;
 }
 
+// A device buffer of the handle that grows when a call needs it to.
+template <typename T>
+struct GsBuf {
+    T *p = nullptr;
+    int64_t cap = 0;
+
+    void free() {
+        cudaFree(p);
+        p = nullptr;
+        cap = 0;
+    }
+    // At least `need` elements, with half as much again as before when it grows
+    // and that can be had.
+    dw_status grow(int64_t need, const char *what) {
+        if (need <= cap) return DW_OK;
+        const int64_t more = cap / 2 * 3;
+        free();
+        cudaError_t e = cudaErrorMemoryAllocation;
+        for (int64_t want : {std::max(need, more), need}) {
+            e = cudaMalloc((void **)&p, sizeof(T) * (size_t)want);
+            if (e == cudaSuccess) {
+                cap = want;
+                return DW_OK;
+            }
+            cudaGetLastError();
+            p = nullptr;
+            if (e != cudaErrorMemoryAllocation || want == need) break;
+        }
+        return cuda_fail(e, what);
+    }
+};
+
 struct GsHandle {
     int64_t cap = 0;
     int width = 0, height = 0;
@@ -1179,21 +1221,17 @@ struct GsHandle {
     uint32_t *batch_off = nullptr;   // [tiles] first batch of each tile
     uint32_t *big = nullptr;         // [cap + 1] queue of Gaussians meeting many tiles; [cap]: its length
     GsStat *stat = nullptr;
-    // tile list: keys as filled, Gaussians in order
-    int64_t list_cap = 0;
-    unsigned long long *lkey = nullptr;
-    uint32_t *lgid = nullptr;
+    // tile list: keys as filled (the shared-memory sort), Gaussians in order
+    GsBuf<unsigned long long> lkey;
+    GsBuf<uint32_t> lgid;
     // batches of the list: their tiles, and each pixel's colour and
-    // transmittance in front of them
-    int64_t batch_cap = 0;
-    uint32_t *batch_tile = nullptr;
-    float4 *before = nullptr;
+    // transmittance in front of them (empty if there was no memory for it)
+    GsBuf<uint32_t> batch_tile;
+    GsBuf<float4> before;
+    bool kept = false;               // the last gs_render filled `before`
     uint32_t batches = 0;            // of the last gs_render
-    // the radix path's buffers (allocated by the first call that takes it):
-    // depth sort and tile-list sort in turn, `radix_cap` entries
-    int64_t radix_cap = 0;
-    uint32_t *rk[2] = {nullptr, nullptr}, *rv[2] = {nullptr, nullptr}, *rcounts = nullptr;
-    uint32_t *tcnt = nullptr, *toff = nullptr, *bsum = nullptr, *total = nullptr;
+    // the radix path's buffers: depth sort and tile-list sort in turn
+    GsBuf<uint32_t> rk[2], rv[2], rcounts, tcnt, toff, bsum;
     const uint32_t *list = nullptr;  // the sorted Gaussian column of the last gs_render
     int ts = GS_FINE, tiles_x = 0, tiles_y = 0;  // tiles of the last gs_render
     int last_n = -1;  // Gaussians of the last gs_render
@@ -1243,103 +1281,65 @@ static void gs_set_tiles(dw_gs h, int ts) {
     h->tiles_y = ((h->height - 1) >> ts) + 1;
 }
 
-// Grow the tile-list buffers to hold m entries.
-static dw_status gs_list_reserve(dw_gs h, int64_t m) {
-    if (m <= h->list_cap) return DW_OK;
-    const int64_t cap = std::max<int64_t>(m, h->list_cap * 3 / 2);
-    cudaFree(h->lkey);
-    cudaFree(h->lgid);
-    h->lkey = nullptr;
-    h->lgid = nullptr;
-    h->list_cap = 0;
-    cudaError_t e = cudaMalloc((void **)&h->lkey, sizeof(unsigned long long) * (size_t)cap);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->lgid, sizeof(uint32_t) * (size_t)cap);
-    if (e != cudaSuccess) return cuda_fail(e, "gs_render (tile list)");
-    h->list_cap = cap;
-    return DW_OK;
-}
-
-// Grow the batch buffers to hold nb batches of fine tiles (1 KB each; a coarse
-// tile's batch takes four of them).
-static dw_status gs_batch_reserve(dw_gs h, int64_t nb) {
-    if (nb <= h->batch_cap) return DW_OK;
-    const int64_t cap = std::max<int64_t>(nb, h->batch_cap * 3 / 2);
-    cudaFree(h->batch_tile);
-    cudaFree(h->before);
-    h->batch_tile = nullptr;
-    h->before = nullptr;
-    h->batch_cap = 0;
-    cudaError_t e = cudaMalloc((void **)&h->batch_tile, sizeof(uint32_t) * (size_t)cap);
-    if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->before, sizeof(float4) * gs_threads(GS_FINE) * (size_t)cap);
-    if (e != cudaSuccess) return cuda_fail(e, "gs_render (list batches)");
-    h->batch_cap = cap;
-    return DW_OK;
-}
-
-static void gs_radix_free(dw_gs h) {
+static void gs_list_free(dw_gs h) {
+    h->lkey.free();
+    h->lgid.free();
+    h->batch_tile.free();
+    h->before.free();
     for (int k = 0; k < 2; ++k) {
-        cudaFree(h->rk[k]);
-        cudaFree(h->rv[k]);
-        h->rk[k] = h->rv[k] = nullptr;
+        h->rk[k].free();
+        h->rv[k].free();
     }
-    cudaFree(h->rcounts);
-    cudaFree(h->tcnt);
-    cudaFree(h->toff);
-    cudaFree(h->bsum);
-    cudaFree(h->total);
-    h->rcounts = h->tcnt = h->toff = h->bsum = h->total = nullptr;
-    h->radix_cap = 0;
+    h->rcounts.free();
+    h->tcnt.free();
+    h->toff.free();
+    h->bsum.free();
 }
 
-// The radix path's buffers for n Gaussians and m list entries.
-static dw_status gs_radix_reserve(dw_gs h, int64_t n, int64_t m) {
-    const int64_t need = std::max(n, m);
-    if (need <= h->radix_cap) return DW_OK;
-    gs_radix_free(h);
-    const size_t c = (size_t)std::max(need, h->cap), g = (size_t)h->cap;
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 2; ++k) {
-        if (e == cudaSuccess) e = cudaMalloc((void **)&h->rk[k], sizeof(uint32_t) * c);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&h->rv[k], sizeof(uint32_t) * c);
+// Buffers for the counted list: 12 bytes per entry where the tiles are sorted
+// in shared memory, 16 for the radix sorts, and 16 per entry (of full batches)
+// of `before`, which is done without when it cannot be had.
+static dw_status gs_list_reserve(dw_gs h, int64_t n, const GsStat &stat) {
+    const int64_t m = (int64_t)stat.total, batch = stat.batches, both = std::max(n, m);
+    dw_status st = h->lgid.grow(m, "gs_render (tile list)");
+    if (stat.most <= GS_SORT_MAX) {
+        if (st == DW_OK) st = h->lkey.grow(m, "gs_render (tile list)");
+    } else {
+        if (st == DW_OK) st = h->rk[0].grow(both, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->rk[1].grow(both, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->rv[0].grow(both, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->rv[1].grow(n, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->rcounts.grow(256 * ((both - 1) / RS_TILE + 1), "gs_render (radix sort)");
+        if (st == DW_OK) st = h->tcnt.grow(n, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->toff.grow(n, "gs_render (radix sort)");
+        if (st == DW_OK) st = h->bsum.grow((n - 1) / 1024 + 1, "gs_render (radix sort)");
     }
-    if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->rcounts, sizeof(uint32_t) * 256 * ((c + RS_TILE - 1) / RS_TILE));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->tcnt, sizeof(uint32_t) * g);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->toff, sizeof(uint32_t) * g);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->bsum, sizeof(uint32_t) * ((g + 1023) / 1024));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->total, sizeof(uint32_t));
-    if (e != cudaSuccess) {
-        gs_radix_free(h);
-        return cuda_fail(e, "gs_render (radix sort)");
-    }
-    h->radix_cap = (int64_t)c;
-    return DW_OK;
+    if (st == DW_OK) st = h->batch_tile.grow(batch, "gs_render (list batches)");
+    if (st == DW_OK) h->kept = h->before.grow(batch * gs_threads(h->ts), "gs_render (list batches)") == DW_OK;
+    return st;
 }
 
 // The tile lists by two stable sorts: all Gaussians by depth, then the list,
 // filled in that order, by tile.
-static dw_status gs_list_radix(dw_gs h, int n, int64_t m, cudaStream_t s) {
-    dw_status st = gs_radix_reserve(h, n, m);
-    if (st != DW_OK) return st;
-    uint32_t *ka = h->rk[0], *va = h->rv[0], *kb = h->rk[1], *vb = h->rv[1];
+static void gs_list_radix(dw_gs h, int n, int64_t m, cudaStream_t s) {
+    uint32_t *ka = h->rk[0].p, *va = h->rv[0].p, *kb = h->rk[1].p, *vb = h->rv[1].p;
+    uint32_t *tcnt = h->tcnt.p, *toff = h->toff.p, *bsum = h->bsum.p;
     k_gs_order_init<<<grid_for(n, 256), 256, 0, s>>>(h->key, n, ka, va);
-    radix_sort(ka, va, kb, vb, n, 4, h->rcounts, s);  // depth order in va
-    k_gs_tile_count<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, n, h->ts, h->tcnt);
+    radix_sort(ka, va, kb, vb, n, 4, h->rcounts.p, s);  // depth order in va (an even number of passes)
+    k_gs_tile_count<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, n, h->ts, tcnt);
     const int nsb = (n + 1023) / 1024;
-    k_scan1024<<<nsb, 256, 0, s>>>(h->tcnt, n, h->toff, h->bsum);
-    k_rs_scan<<<1, 1024, 0, s>>>(h->bsum, nsb);
-    k_scan_finish<<<grid_for(n, 256), 256, 0, s>>>(h->toff, h->tcnt, n, h->bsum, h->total);
+    k_scan1024<<<nsb, 256, 0, s>>>(tcnt, n, toff, bsum);
+    k_rs_scan<<<1, 1024, 0, s>>>(bsum, nsb);
+    k_scan_finish<<<grid_for(n, 256), 256, 0, s>>>(toff, n, bsum);
     // the list: tile keys to kb, Gaussians to lgid, then both sorted (the depth
     // order in va is read before the sort's second buffers overwrite it)
-    k_gs_duplicate<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, h->toff, n, h->tiles_x, h->ts,
-                                                    kb, h->lgid);
+    k_gs_duplicate<<<grid_for(n, 256), 256, 0, s>>>(va, h->rect, toff, n, h->tiles_x, h->ts, kb,
+                                                    h->lgid.p);
     int bits = 1;
     while ((1ll << bits) < (int64_t)h->tiles_x * h->tiles_y) ++bits;
-    uint32_t *lk = kb, *lv = h->lgid, *lk2 = ka, *lv2 = va;
-    radix_sort(lk, lv, lk2, lv2, (int)m, (bits + 7) / 8, h->rcounts, s);
+    uint32_t *lk = kb, *lv = h->lgid.p, *lk2 = ka, *lv2 = va;
+    radix_sort(lk, lv, lk2, lv2, (int)m, (bits + 7) / 8, h->rcounts.p, s);
     h->list = lv;
-    return DW_OK;
 }
 
 extern "C" dw_status gs_create(int64_t max_gaussians, int32_t width, int32_t height, dw_gs *out) {
@@ -1390,11 +1390,7 @@ extern "C" dw_status gs_destroy(dw_gs h) {
     cudaFree(h->batch_off);
     cudaFree(h->big);
     cudaFree(h->stat);
-    cudaFree(h->lkey);
-    cudaFree(h->lgid);
-    cudaFree(h->batch_tile);
-    cudaFree(h->before);
-    gs_radix_free(h);
+    gs_list_free(h);
     delete h;
     return DW_OK;
 }
@@ -1442,7 +1438,7 @@ static dw_status gs_count(dw_gs h, const GsCam &c, const float *x, const float *
                                                      h->rows, h->rect, h->key, h->tile_count, h->big,
                                                      queued);
     k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, queued, h->rect, h->key, h->tiles_x, h->ts,
-                                                h->tile_count, h->ranges, h->lkey, h->stat);
+                                                h->tile_count, h->ranges, h->lkey.p, h->stat);
     return gs_scan(h, stat, s);
 }
 
@@ -1450,35 +1446,34 @@ static dw_status gs_count(dw_gs h, const GsCam &c, const float *x, const float *
 static dw_status gs_recount(dw_gs h, int n, GsStat &stat, cudaStream_t s) {
     DW_CUDA(cudaMemsetAsync(h->tile_count, 0, sizeof(uint32_t) * (size_t)h->tiles_x * h->tiles_y, s));
     k_gs_list<false><<<grid_for(n, 128), 128, 0, s>>>(h->rect, h->key, n, h->tiles_x, h->ts,
-                                                      h->tile_count, h->ranges, h->lkey);
+                                                      h->tile_count, h->ranges, h->lkey.p);
     k_gs_big<false><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, h->big + h->cap, h->rect, h->key, h->tiles_x,
-                                                h->ts, h->tile_count, h->ranges, h->lkey, h->stat);
+                                                h->ts, h->tile_count, h->ranges, h->lkey.p, h->stat);
     return gs_scan(h, stat, s);
 }
 
 // The counted tiles' lists in order, and their batches.
 static dw_status gs_make_list(dw_gs h, int n, const GsStat &stat, cudaStream_t s) {
     const int ntiles = h->tiles_x * h->tiles_y;
-    dw_status st = gs_list_reserve(h, (int64_t)stat.total);
-    if (st == DW_OK) st = gs_batch_reserve(h, (int64_t)stat.batches << (2 * (h->ts - GS_FINE)));
+    const dw_status st = gs_list_reserve(h, n, stat);
     if (st != DW_OK) return st;
-    h->list = h->lgid;
+    if (stat.most > GS_SORT_MAX) {
+        gs_list_radix(h, n, (int64_t)stat.total, s);
+        k_gs_batches<<<grid_for(ntiles, 256), 256, 0, s>>>(h->tile_count, ntiles, h->ts, h->batch_off,
+                                                           h->ranges, h->batch_tile.p);
+        return DW_OK;
+    }
+    h->list = h->lgid.p;
     k_gs_list<true><<<grid_for(n, 128), 128, 0, s>>>(h->rect, h->key, n, h->tiles_x, h->ts,
-                                                     h->tile_count, h->ranges, h->lkey);
+                                                     h->tile_count, h->ranges, h->lkey.p);
     if (stat.big > 0)
         k_gs_big<true><<<GS_BIG_CTAS, 256, 0, s>>>(h->big, h->big + h->cap, h->rect, h->key, h->tiles_x,
-                                                   h->ts, h->tile_count, h->ranges, h->lkey, h->stat);
-    if (stat.most <= GS_SORT_MAX) {
-        size_t len = 2;
-        while (len < stat.most) len <<= 1;
-        k_gs_tile_sort<<<(unsigned)ntiles, GS_SORT_THREADS, len * sizeof(unsigned long long), s>>>(
-            h->ranges, h->lkey, h->batch_off, h->ts, h->lgid, h->batch_tile);
-    } else {
-        st = gs_list_radix(h, n, (int64_t)stat.total, s);
-        if (st != DW_OK) return st;
-        k_gs_batches<<<grid_for(ntiles, 256), 256, 0, s>>>(h->ranges, ntiles, h->ts, h->batch_off,
-                                                           h->batch_tile);
-    }
+                                                   h->ts, h->tile_count, h->ranges, h->lkey.p, h->stat);
+    size_t len = 2;
+    while (len < stat.most) len <<= 1;
+    auto sort = h->ts == GS_FINE ? k_gs_tile_sort<GS_FINE> : k_gs_tile_sort<GS_COARSE>;
+    sort<<<(unsigned)ntiles, GS_SORT_THREADS, len * sizeof(unsigned long long), s>>>(
+        h->ranges, h->lkey.p, h->batch_off, h->lgid.p, h->batch_tile.p);
     return DW_OK;
 }
 
@@ -1496,27 +1491,30 @@ extern "C" dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, co
     if (nn > 0) {
         GsStat stat;
         st = gs_count(h, c, x, F, sigma0, color, opacity, nn, stat, s);
-        if (st == DW_OK && stat.total > (unsigned long long)GS_LIST_MAX) {
+        bool fits = stat.total <= (unsigned long long)GS_LIST_MAX;
+        if (st == DW_OK && fits && stat.total > 0) st = gs_make_list(h, nn, stat, s);
+        if (st == DW_ERR_OOM || (st == DW_OK && !fits)) {
+            gs_list_free(h);
             gs_set_tiles(h, GS_COARSE);
             st = gs_recount(h, nn, stat, s);
+            if (st != DW_OK) return st;
+            fits = stat.total <= (unsigned long long)GS_LIST_MAX;
+            DW_REQUIRE(fits, "tile list too long (Gaussians x tiles met >= 2^31)");
+            if (stat.total > 0) st = gs_make_list(h, nn, stat, s);
         }
         if (st != DW_OK) return st;
-        DW_REQUIRE(stat.total <= (unsigned long long)GS_LIST_MAX,
-                   "tile list too long (Gaussians x tiles met >= 2^31)");
         h->batches = stat.batches;
-        if (stat.total > 0) {
-            st = gs_make_list(h, nn, stat, s);
-            if (st != DW_OK) return st;
-        }
     } else {
         const size_t ntiles = (size_t)h->tiles_x * h->tiles_y;
         DW_CUDA(cudaMemsetAsync(h->ranges, 0, sizeof(int2) * ntiles, s));
         DW_CUDA(cudaMemsetAsync(h->batch_off, 0, sizeof(uint32_t) * ntiles, s));
         h->batches = 0;
     }
-    auto kern = h->ts == GS_FINE ? k_gs_render_fwd<GS_FINE> : k_gs_render_fwd<GS_COARSE>;
+    auto kern = h->kept ? (h->ts == GS_FINE ? k_gs_render_fwd<GS_FINE, true> : k_gs_render_fwd<GS_COARSE, true>)
+                        : (h->ts == GS_FINE ? k_gs_render_fwd<GS_FINE, false> : k_gs_render_fwd<GS_COARSE, false>);
     kern<<<(unsigned)(h->tiles_x * h->tiles_y), gs_threads(h->ts), 0, s>>>(
-        c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, image, h->image, h->batch_off, h->before);
+        c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, image, h->image, h->batch_off,
+        h->before.p);
     h->last_n = nn;
     const void *in[5] = {x, F, sigma0, color, opacity};
     memcpy(h->last_in, in, sizeof in);
@@ -1542,11 +1540,12 @@ extern "C" dw_status gs_render_backward(dw_gs h, const dw_camera *cam, const flo
     const GsCam c = to_cam(*cam);
     const int nn = (int)n;
     DW_CUDA(cudaMemsetAsync(h->g2d, 0, sizeof(float) * GS_ROW * (size_t)nn, s));
-    auto kern = h->ts == GS_FINE ? k_gs_render_bwd<GS_FINE> : k_gs_render_bwd<GS_COARSE>;
+    auto kern = h->kept ? (h->ts == GS_FINE ? k_gs_render_bwd<GS_FINE, false> : k_gs_render_bwd<GS_COARSE, false>)
+                        : (h->ts == GS_FINE ? k_gs_render_bwd<GS_FINE, true> : k_gs_render_bwd<GS_COARSE, true>);
     if (h->batches > 0)
-        kern<<<h->batches, gs_threads(h->ts), 0, s>>>(c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows,
-                                                      h->batch_tile, h->batch_off, h->before, h->image,
-                                                      g_image, h->g2d);
+        kern<<<h->kept ? h->batches : (unsigned)(h->tiles_x * h->tiles_y), gs_threads(h->ts), 0, s>>>(
+            c, (unsigned)h->tiles_x, h->list, h->ranges, h->rows, h->batch_tile.p, h->batch_off, h->before.p,
+            h->image, g_image, h->g2d);
     k_gs_preprocess_bwd<<<grid_for(nn, 256), 256, 0, s>>>(c, x, F, sigma0, opacity, nn, h->g2d, g_x, g_F,
                                                            g_color, g_opacity);
     DW_LAUNCHED("gs_render_backward");

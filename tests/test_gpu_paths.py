@@ -471,3 +471,43 @@ def test_gaussian_list_on_coarse_tiles(size, n):
         go[order] += (w * (T * c - (C - part) / (1.0 - a))).sum(0) * e
     assert rel_l2(gs[2].cpu().numpy(), gc) <= 1e-4 and rel_l2(gs[3].cpu().numpy(), go) <= 1e-3
     r.close()
+
+
+# Little free memory: room for the list but not for the colours in front of its
+# batches, so the backward walks the tiles; room only for the list on 16 x 16
+# tiles. The same pixels composited in the same order: the same
+# image, gradients up to the order of their sums over pixels, relative L2 1e-5.
+@pytest.mark.parametrize("n", [2000, 4500])  # tiles sorted in shared memory; radix sorts (more per entry)
+def test_gaussian_lists_in_little_memory(n):
+    W = 1024 if n < 4096 else 640
+    f = 0.4 * W
+    cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), f, f, W / 2, W / 2, W, W)
+    d = [to_dev(a) for a in _gaussians(n, 3.0, 7, (0.0005, 0.001))]
+    g_img = torch.randn((3, W, W), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    fine = n * (W // 8) ** 2
+    lists, before = fine * (12 if n < 4096 else 16), ((n + 63) // 64) * 1024 * (W // 8) ** 2
+    got, used = [], []
+    for room in (None, lists + before // 2, int(0.75 * lists)):
+        r = B.GaussianRenderer(n, W, W)
+        img, gs = torch.empty_like(g_img), [torch.zeros_like(d[k]) for k in (0, 1, 3, 4)]
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = []
+        while room is not None and torch.cuda.mem_get_info()[0] - room > 32 << 20:
+            left = torch.cuda.mem_get_info()[0] - room
+            hog.append(torch.empty(min(left, 8 << 30) // (2 << 20) * (2 << 20), dtype=torch.uint8, device="cuda"))
+        free = torch.cuda.mem_get_info()[0]
+        r.render(cam, *d, image=img)
+        r.backward(cam, *d, g_img, *gs)
+        torch.cuda.synchronize()
+        used.append(free - torch.cuda.mem_get_info()[0])
+        got.append((img.cpu(), [a.cpu().numpy() for a in gs]))
+        r.close()
+        hog.clear()
+        torch.cuda.empty_cache()
+    assert used[0] >= lists + before and lists <= used[1] < lists + before and used[2] < lists, (used, lists, before)
+    assert got[0][0].max() > 0.3
+    for img, gs in got[1:]:
+        assert torch.equal(img, got[0][0])
+        for a, b in zip(gs, got[0][1]):
+            assert rel_l2(a, b) <= 1e-5

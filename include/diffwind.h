@@ -123,10 +123,16 @@ enum { DW_NEOHOOKEAN = 0, DW_FIXED_COROTATED = 1 };
 /* P2G accumulation strategies (results agree to float rounding): global float4
  * atomics per particle and node (ATOMIC); per-warp sums of runs of particles
  * that share a cell, one atomic per node and run (WARP); a CTA-wide shared
- * tile (TILE). In mpm_rollout's fused G2P/P2G kernel, AUTO and PAIR run two
- * particles per thread on paired float2 arithmetic with the warp sums; the
- * other strategies run the one-particle-per-thread fused kernel. Outside
- * mpm_rollout PAIR and AUTO use WARP. */
+ * tile (TILE). In the fused G2P/P2G kernel of mpm_rollout and of a segment
+ * adjoint's recompute, PAIR runs two particles per thread on paired float2
+ * arithmetic with the warp sums; the other strategies run the
+ * one-particle-per-thread fused kernel in mpm_rollout and single substeps in the
+ * recompute. Elsewhere PAIR uses WARP. AUTO takes the fastest by the particle
+ * count: kernels that split a particle's work over its stencil's three layers,
+ * for P2G and G2P up to 131,072 particles and for the fused kernel up to 38,912;
+ * above, as PAIR. With AUTO or PAIR a segment adjoint of more than one substep
+ * whose grids fit in the handle's grid tape runs its reverse pass in two
+ * launches per substep (four otherwise). */
 enum { DW_P2G_AUTO = 0, DW_P2G_ATOMIC = 1, DW_P2G_WARP = 2, DW_P2G_TILE = 3, DW_P2G_PAIR = 4 };
 
 typedef struct {

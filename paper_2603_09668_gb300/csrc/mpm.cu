@@ -141,7 +141,7 @@ __global__ void k_g2p(MpmParams P, const float *x, const float *F,
 dw_status launch_g2p(int mode, const MpmParams &P, const float *x, const float *F, const uint8_t *pinned,
                      const float4 *grid_v, const dw_mpm_state &out, int64_t n, int *err,
                      int *reset_count, cudaStream_t s) {
-    if ((mode == DW_P2G_AUTO || mode == DW_P2G_PAIR) && n <= LAYER_MAX_G2P)
+    if (mode == DW_P2G_AUTO && n <= LAYER_MAX_G2P)
         return launch_layer_g2p(P, x, F, pinned, grid_v, out, n, err, reset_count, s);
     DW_CUDA(launch_pdl(k_g2p, grid_for(n, 128), 128, s, P, x, F, pinned, grid_v, out.x, out.v,
                        out.C, out.F, n, err, reset_count));

@@ -137,8 +137,8 @@ dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *
                           int n_substeps, float *g_wind, float *g_E, int *reset_count,
                           cudaStream_t s);
 
-// The layer-split kernels (mpm_layer.cu) and the particle counts up to which
-// they are the faster ones (measured, us): a fused launch with its grid update
+// The layer-split kernels (mpm_layer.cu), which DW_P2G_AUTO takes, and the particle
+// counts up to which they are the faster ones (measured, us): a fused launch with its grid update
 // 7.9 against 11.9 at 5,504 particles, 9.4 / 11.6 at 32,768, 11.5 / 11.7 at
 // 38,912, 12.3 / 11.5 at 40,960, 14.3 / 12.5 at 49,151 of a sheet; 13.7 / 15.6 at
 // 38,912, 15.0 / 15.3 at 40,960, 18.9 / 17.3 at 65,535 of a block. The fused
@@ -146,7 +146,7 @@ dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *
 // SMs) no longer run all at once. The P2G alone takes 5 against 13 at 5,504, a
 // whole substep 26.2 / 26.7 at 100,000 and 41 / 40 at 200,000 of a block.
 constexpr int64_t LAYER_MAX_P2G = 1 << 17, LAYER_MAX_G2P = 1 << 17;
-inline bool layer_fused(int64_t n) { return n <= 32 * 8 * 152; }
+inline bool layer_fused(int mode, int64_t n) { return mode == DW_P2G_AUTO && n <= 32 * 8 * 152; }
 dw_status launch_layer_p2g(const MpmParams &P, const float *x, const float *v, const float *C,
                            const float *F, int64_t n, float4 *grid, int *err,
                            const ActiveBlocks &ab, cudaStream_t st);
@@ -175,9 +175,9 @@ __global__ void k_sort_move(const int *__restrict__ keys, int64_t n, int *__rest
 dw_status exclusive_scan(int *data, int64_t len, int *tmp, int64_t tmp_len, cudaStream_t st);
 
 // host helpers of mpm.cu
-// G2P of n particles (x, F) into `out` (mode DW_P2G_*: AUTO and PAIR take the
-// layer-split kernel where it is the faster one, the others never do); reset_count, when given, is the
-// active-list count to clear.
+// G2P of n particles (x, F) into `out` (mode DW_P2G_*: AUTO takes the layer-split
+// kernel where it is the faster one, the others never do); reset_count, when
+// given, is the active-list count to clear.
 dw_status launch_g2p(int mode, const MpmParams &P, const float *x, const float *F, const uint8_t *pinned,
                      const float4 *grid_v, const dw_mpm_state &out, int64_t n, int *err,
                      int *reset_count, cudaStream_t s);

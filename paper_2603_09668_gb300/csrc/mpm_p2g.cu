@@ -139,7 +139,7 @@ dw_status launch_p2g(int mode, const MpmParams &P, const float *x, const float *
                             const float *C, const float *F, int64_t n, float4 *grid, int *err,
                             const ActiveBlocks &ab, cudaStream_t st) {
     if (n == 0) return DW_OK;
-    if ((mode == DW_P2G_AUTO || mode == DW_P2G_PAIR) && n <= LAYER_MAX_P2G)
+    if (mode == DW_P2G_AUTO && n <= LAYER_MAX_P2G)
         return launch_layer_p2g(P, x, v, C, F, n, grid, err, ab, st);
     if (mode == DW_P2G_ATOMIC) {
         DW_CUDA(launch_pdl(k_p2g_atomic, grid_for(n, 128), 128, st, P, x, v, C, F, n, grid, err, ab));

@@ -158,7 +158,7 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
                          ((reinterpret_cast<uintptr_t>(in.x) | reinterpret_cast<uintptr_t>(in.F) |
                            reinterpret_cast<uintptr_t>(out.x) | reinterpret_cast<uintptr_t>(out.F)) %
                               16 == 0);
-        if (layer_fused(n)) {
+        if (layer_fused(h->desc.p2g_mode, n)) {
             st = launch_layer_g2p2g(h->P, in.x, in.F, pinned, h->grid_v, out, h->grid_mp, n, h->err,
                                     active_blocks(h, 1 - L), h->block_count + L, nullptr, nullptr, s);
             if (st != DW_OK) return st;
@@ -212,7 +212,8 @@ extern "C" dw_status mpm_rollout(dw_mpm h, const dw_mpm_state *state, uint8_t *p
     uint8_t *cur_pin = pinned, *oth_pin = pinned ? h->roll_pinned : nullptr;
     int32_t *cur_ids = ids, *oth_ids = h->roll_ids;
     const unsigned pgrid = grid_for(n, P2G_WARP_THREADS);
-    // the fused kernel: two particles per thread (AUTO, PAIR) or one (the other strategies)
+    // the fused kernel: two particles per thread (PAIR; AUTO above layer_fused's count) or one
+    // (the other strategies)
     const bool pair = h->desc.p2g_mode == DW_P2G_AUTO || h->desc.p2g_mode == DW_P2G_PAIR;
     const unsigned pair_grid = grid_for(n, 64);
     int L = 0;  // active list consumed by the next grid update
@@ -256,7 +257,7 @@ extern "C" dw_status mpm_rollout(dw_mpm h, const dw_mpm_state *state, uint8_t *p
             // multiple of 4, 16-byte aligned arrays)
             const bool pair_vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(cur.x) |
                                                     reinterpret_cast<uintptr_t>(cur.F)) % 16 == 0);
-            if (pair && layer_fused(n)) {
+            if (layer_fused(h->desc.p2g_mode, n)) {
                 const bool keys = sort_every > 0 && (k + 1) % sort_every == 0;
                 const dw_mpm_state out{cur.x, nullptr, nullptr, cur.F, n};  // v and C are not kept
                 st = launch_layer_g2p2g(h->P, cur.x, cur.F, cur_pin, h->grid_v, out, h->grid_mp, n,

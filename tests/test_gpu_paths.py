@@ -511,3 +511,57 @@ def test_gaussian_lists_in_little_memory(n):
         assert torch.equal(img, got[0][0])
         for a, b in zip(gs, got[0][1]):
             assert rel_l2(a, b) <= 1e-5
+
+
+# What each p2g_mode runs, from the kernel names of a captured call: PAIR the
+# paired fused kernel at every size, AUTO the layer kernels up to their counts.
+@pytest.mark.parametrize("mode,n,fused", [("PAIR", 500, "k_g2p2g_pair"), ("PAIR", 38913, "k_g2p2g_pair"),
+                                          ("AUTO", 500, "k_layer_g2p"), ("AUTO", 38913, "k_g2p2g_pair"),
+                                          ("WARP", 500, "k_g2p2g")])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_kernels_of_a_mode(mode, n, fused, tmp_path):
+    pr, st, pin = _mpm_case(n, 24, 0)
+    mpm = B.MPM.from_params(pr, max_particles=n, p2g_mode=getattr(B, "P2G_" + mode))
+    s, pin_d = _dev(st), to_dev(pin)
+    wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
+    mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0)
+    dot = tmp_path / "g.dot"
+    g.debug_dump(str(dot))
+    text = dot.read_text()
+    for name in ("k_g2p2g_pair", "k_layer_g2p", "k_layer_p2g", "k_grid_update_active"):
+        want = (name == fused or name == "k_grid_update_active"
+                or (mode == "AUTO" and name in ("k_layer_g2p", "k_layer_p2g")))  # the rollout's first P2G, last G2P
+        assert (name in text) == want, name
+    assert fused in text
+    mpm.close()
+
+
+# A segment whose recompute runs the paired kernel (P2G_PAIR) on few particles,
+# odd counts and a partly filled last warp, against the one-particle kernels of
+# P2G_WARP: states and gradients, relative L2 1e-4 per block, as the fused reverse
+# pass above. (dL/dE is left out: one number, the sum of n terms of both signs that
+# cancel to 2e-6 here, while every mode is 3e-10 off its float64 value.)
+@pytest.mark.parametrize("n", [33, 130, 1000])
+@pytest.mark.parametrize("material,steps", [(0, 2), (1, 4)])
+def test_paired_recompute_of_a_segment(n, material, steps):
+    pr, st, pin = _mpm_case(n, 24, material, seed=1)
+    wind = B.WindField(to_dev(inputs.fourier_wind(9, 3, seed=4)), 7 * pr["dt"])
+    g = torch.Generator(device="cuda").manual_seed(2)
+    g0 = [torch.randn(a.shape, generator=g, device="cuda") for a in st]
+    got = []
+    for mode in (B.P2G_PAIR, B.P2G_WARP):
+        mpm = B.MPM.from_params(pr, max_particles=n, p2g_mode=mode)
+        gs = B.MpmState(*(a.clone() for a in g0))
+        gw = torch.zeros_like(wind.values)
+        tape = torch.empty((steps - 1) * 24 * n, device="cuda")
+        mpm.segment_adjoint(_dev(st), tape, gs, to_dev(pin), wind, pr["dt"], steps, gw)
+        mpm.device_status()
+        got.append([a.cpu().numpy().astype(np.float64) for a in (tape, *gs, gw)])
+        mpm.close()
+    for k, (a, b) in enumerate(zip(*got)):
+        assert rel_l2(a, b) <= 1e-4, k

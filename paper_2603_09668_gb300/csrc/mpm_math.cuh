@@ -167,28 +167,32 @@ __device__ __forceinline__ bool stress_P(const MpmParams &P, const float F[9], f
 //   Neo-Hookean:      tau = mu F F^T + (lam ln J - mu) I
 //   fixed-corotated:  tau = 2 mu (F - R) F^T + lam (J - 1) J I,
 // which needs no cofactors beyond J's and one product of matrices. Written
-// with explicit fused operations in the order of the paired kernels
-// (affine2), so that a scene's states do not depend on the kernel its size
-// takes it to. Returns false (tau = 0) for det F <= 0.
+// with explicit fused operations in the order of the paired kernels (affine2),
+// so that a particle's stress does not depend on the kernel that its scene's
+// size takes it to. Returns false (tau = 0, whatever F holds) for det F <= 0 or
+// not a number.
 __device__ __forceinline__ bool stress_tau(const MpmParams &P, const float F[9], float tau[9]) {
     const float k0 = __fmaf_rn(-F[5], F[7], __fmul_rn(F[4], F[8])),
                 k1 = __fmaf_rn(-F[3], F[8], __fmul_rn(F[5], F[6])),
                 k2 = __fmaf_rn(-F[4], F[6], __fmul_rn(F[3], F[7]));
     const float J = __fmaf_rn(F[2], k2, __fmaf_rn(F[1], k1, __fmul_rn(F[0], k0)));
-    const bool ok = J > 0.0f;
+    if (!(J > 0.0f)) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) tau[k] = 0.0f;
+        return false;
+    }
     if (P.material == DW_NEOHOOKEAN) {
-        const float mu = ok ? P.mu : 0.0f;
-        const float c = __fmaf_rn(P.lam, ok ? logf(J) : 0.0f, -mu);
+        const float c = __fmaf_rn(P.lam, logf(J), -P.mu);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = i; j < 3; ++j) {
                 const float b = __fmaf_rn(F[3 * i + 2], F[3 * j + 2],
                                           __fmaf_rn(F[3 * i + 1], F[3 * j + 1], __fmul_rn(F[3 * i], F[3 * j])));
-                tau[3 * i + j] = i == j ? __fmaf_rn(mu, b, c) : __fmul_rn(mu, b);
+                tau[3 * i + j] = i == j ? __fmaf_rn(P.mu, b, c) : __fmul_rn(P.mu, b);
                 tau[3 * j + i] = tau[3 * i + j];
             }
-    } else if (ok) {
+    } else {
         float R[9];
         polar_R(F, R);
         const float mu2 = 2.0f * P.mu, c = __fmul_rn(__fmul_rn(P.lam, J - 1.0f), J);
@@ -202,11 +206,8 @@ __device__ __forceinline__ bool stress_tau(const MpmParams &P, const float F[9],
                                           __fmaf_rn(R[3 * i + 1], F[3 * j + 1], __fmul_rn(R[3 * i], F[3 * j])));
                 tau[3 * i + j] = i == j ? __fadd_rn(b, c) : b;
             }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) tau[k] = 0.0f;
     }
-    return ok;
+    return true;
 }
 
 __device__ __forceinline__ void cross3(const float a[3], const float b[3], float c[3]) {

@@ -218,6 +218,11 @@ __device__ __forceinline__ void affine2(const MpmParams &P, const float2 F[9], c
                 const float2 b = fma(R[3 * i + 2], F[3 * j + 2], fma(R[3 * i + 1], F[3 * j + 1], mul(R[3 * i], F[3 * j])));
                 A[3 * i + j] = fma(mk, i == j ? add(b, c) : b, mul(pm, C[3 * i + j]));
             }
+        if (!(ok0 && ok1)) {  // tau = 0 whatever F holds: m C alone
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+                A[k] = make_float2(ok0 ? A[k].x : P.p_mass * C[k].x, ok1 ? A[k].y : P.p_mass * C[k].y);
+        }
     }
 }
 

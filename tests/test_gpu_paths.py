@@ -565,3 +565,38 @@ def test_paired_recompute_of_a_segment(n, material, steps):
         mpm.close()
     for k, (a, b) in enumerate(zip(*got)):
         assert rel_l2(a, b) <= 1e-4, k
+
+
+# A particle whose F is not a number (or has det F = -inf) has no stress: its mass and
+# momentum reach the grid, and the particles around it stay finite; the call
+# reports it. (The paired kernel's Neo-Hookean form never did so.) Against the
+# same call with an inverted F in its place, which adds the same: x, v and F within
+# 1e-6, atomics' order (which C's factor 4 / dx carries beyond that).
+@pytest.mark.parametrize("bad", [float("nan"), float("-inf")])
+@pytest.mark.parametrize("mode,material,steps", [(m, k, s) for m in ("AUTO", "WARP", "ATOMIC", "TILE")
+                                                 for k in (0, 1) for s in (1, 3)]
+                         + [("PAIR", 0, 1), ("PAIR", 1, 3)])
+def test_a_particle_without_a_stress(mode, material, steps, bad):
+    n, p = 200, 70
+    pr, st, pin = _mpm_case(n, 24, material, seed=5)
+    wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
+    out = []
+    for F in (bad, -1.0):
+        st[3][:, p] = np.eye(3).reshape(9) * -1.0
+        st[3][0, p] = F
+        mpm = B.MPM.from_params(pr, max_particles=n, p2g_mode=getattr(B, "P2G_" + mode))
+        s = _dev(st)
+        if steps == 1:
+            mpm.substep(s, s, to_dev(pin), wind, 0.0)
+        else:
+            mpm.rollout(s, to_dev(pin), None, wind, 0.0, steps, 0)
+        with pytest.raises(B.DiffWindError):
+            mpm.device_status()
+        out.append([a.cpu().numpy() for a in s])
+        mpm.close()
+    for k, (a, b) in enumerate(zip(*out)):
+        if k == 3:
+            a, b = np.delete(a, p, 1), np.delete(b, p, 1)
+        assert np.isfinite(a).all(), k
+        if k != 2:
+            assert np.abs(a - b).max() <= 1e-6 * max(1.0, np.abs(b).max()), k

@@ -173,7 +173,11 @@ __device__ __forceinline__ void wind_scatter_block(const MpmParams &P, const Win
                 G.w[a][lt][e] = d == 0 ? 1.0f - tp.fr[a] : (d == 1 ? tp.fr[a] : 0.0f);
             }
     }
-    group_sync(id);
+    // (a cotangent that is not finite must not meet the zero weights of other wind nodes)
+    if (group_any(id, active && !isfinite(g.x + g.y + g.z))) {
+        if (active) wind_sample_adjoint_dev(w, i * P.dx, j * P.dx, k * P.dx, t, g, g_values);
+        return;
+    }
     const int ex = lt & 3, q1 = (lt >> 2) & 3, q2 = lt >> 4;
     float s[3];
 #pragma unroll

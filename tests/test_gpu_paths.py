@@ -600,3 +600,28 @@ def test_a_particle_without_a_stress(mode, material, steps, bad):
         assert np.isfinite(a).all(), k
         if k != 2:
             assert np.abs(a - b).max() <= 1e-6 * max(1.0, np.abs(b).max()), k
+
+
+# Wind cotangents that are not finite reach the wind nodes that their grid nodes
+# sample and no others: the same ones as in the oracle's reverse substep (of a
+# particle whose grid nodes lie between wind nodes, so that no weight is zero).
+@pytest.mark.parametrize("nf,frames", [(6, 2), (5, 3), (9, 2)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_wind_gradient_of_a_bad_cotangent(nf, frames, bad):
+    pr, st, pin = _mpm_case(400, 18, 0, seed=3)
+    wind, t = inputs.fourier_wind(nf, frames, seed=6), 0.3
+    g = [np.random.default_rng(k).standard_normal(a.shape).astype(np.float32) for k, a in enumerate(st)]
+    p = int(np.flatnonzero((pin == 0) & (st[0] * 18 < 7.4).all(0))[3])
+    g[1][0, p] = bad
+    gw = torch.zeros(wind.shape, device="cuda")
+    mpm = B.MPM.from_params(pr, max_particles=400)
+    mpm.substep_adjoint(_dev(st), _dev(g), B.MpmState.empty_like(_dev(st)), to_dev(pin),
+                        B.WindField(to_dev(wind), 1.0), t, gw)
+    ref = oracle.mpm_substep_adjoint(pr, tuple(a.astype(np.float64) for a in st),
+                                     (wind.astype(np.float64), nf, frames, 1.0), t,
+                                     tuple(a.astype(np.float64) for a in g), pinned=pin)[1]
+    got, ref = gw.cpu().numpy().reshape(-1, 3), np.asarray(ref).reshape(-1, 3)
+    assert 0 < np.isfinite(ref).sum() and np.array_equal(np.isfinite(got), np.isfinite(ref))
+    ok = np.isfinite(ref)
+    assert rel_l2(got[ok], ref[ok]) <= 1e-4
+    mpm.close()

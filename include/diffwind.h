@@ -129,7 +129,7 @@ enum { DW_NEOHOOKEAN = 0, DW_FIXED_COROTATED = 1 };
  * one-particle-per-thread fused kernel in mpm_rollout and single substeps in the
  * recompute. Elsewhere PAIR uses WARP. AUTO takes the fastest by the particle
  * count: kernels that split a particle's work over its stencil's three layers,
- * for P2G and G2P up to 131,072 particles and for the fused kernel up to 38,912;
+ * for P2G and the fused kernel up to 38,912 particles and for G2P up to 65,536;
  * above, as PAIR. With AUTO or PAIR a segment adjoint of more than one substep
  * whose grids fit in the handle's grid tape runs its reverse pass in two
  * launches per substep (four otherwise). */

@@ -138,15 +138,25 @@ dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *
                           cudaStream_t s);
 
 // The layer-split kernels (mpm_layer.cu), which DW_P2G_AUTO takes, and the particle
-// counts up to which they are the faster ones (measured, us): a fused launch with its grid update
-// 7.9 against 11.9 at 5,504 particles, 9.4 / 11.6 at 32,768, 11.5 / 11.7 at
-// 38,912, 12.3 / 11.5 at 40,960, 14.3 / 12.5 at 49,151 of a sheet; 13.7 / 15.6 at
-// 38,912, 15.0 / 15.3 at 40,960, 18.9 / 17.3 at 65,535 of a block. The fused
-// line lies where the layer kernel's CTAs (32 particles, eight per SM on 152
-// SMs) no longer run all at once. The P2G alone takes 5 against 13 at 5,504, a
-// whole substep 26.2 / 26.7 at 100,000 and 41 / 40 at 200,000 of a block.
-constexpr int64_t LAYER_MAX_P2G = 1 << 17, LAYER_MAX_G2P = 1 << 17;
-inline bool layer_fused(int mode, int64_t n) { return mode == DW_P2G_AUTO && n <= 32 * 8 * 152; }
+// counts up to which they are the faster ones (measured, us). A fused launch with
+// its grid update: 7.9 against 11.9 at 5,504 particles, 9.4 / 11.6 at 32,768, 11.5 /
+// 11.7 at 38,912, 12.3 / 11.5 at 40,960, 14.3 / 12.5 at 49,151 of a sheet; 13.7 /
+// 15.6 at 38,912, 15.0 / 15.3 at 40,960, 18.9 / 17.3 at 65,535 of a block: the
+// line lies where the layer kernel's CTAs (32 particles, eight per SM on 152 SMs)
+// no longer run all at once.
+// A whole substep, particles in cell order / in random order, of a sheet on 64^3,
+// a sheet on 128^3 and a block on 64^3:
+//   with both layer kernels      with the layer G2P        with neither
+//   5,000:  12.4 12.3 12.3 / 14.4 14.4 14.4;  16.4 18.5 16.5 / 18.0 20.6 18.6;  18.5 20.1 18.5 / 20.4 20.6 20.6
+//   38,912: 14.4 14.4 14.5 / 43.4 29.2 28.7;  18.3 16.5 18.5 / 35.4 24.7 26.7;  18.5 18.1 20.6 / 35.5 26.7 27.2
+//   65,536: 18.5 18.6 20.7 / 69.2 45.2 41.7;  18.4 18.5 20.6 / 50.2 35.7 34.9;  18.6 18.5 20.2 / 49.4 35.2 35.0
+//   131,072: 24.7 25.2 29.1 / 87.8 61.4 56.9 with both,  20.9 22.6 22.7 / 81.9 56.4 53.4 with neither
+// P2G: the line of the fused kernel; above it the layer kernel's gain in cell
+// order (2 us) is gone by 65,536, and in random order, where every particle adds
+// to the grid by itself, it loses a quarter and more. G2P: 65,536, where it has
+// stopped gaining in either order.
+constexpr int64_t LAYER_ROUND = 32 * 8 * 152, LAYER_MAX_P2G = LAYER_ROUND, LAYER_MAX_G2P = 1 << 16;
+inline bool layer_fused(int mode, int64_t n) { return mode == DW_P2G_AUTO && n <= LAYER_ROUND; }
 dw_status launch_layer_p2g(const MpmParams &P, const float *x, const float *v, const float *C,
                            const float *F, int64_t n, float4 *grid, int *err,
                            const ActiveBlocks &ab, cudaStream_t st);

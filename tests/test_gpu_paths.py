@@ -513,6 +513,17 @@ def test_gaussian_lists_in_little_memory(n):
             assert rel_l2(a, b) <= 1e-5
 
 
+def _kernels(call, path):
+    """The kernel names of a call, from its capture (the call has run before)."""
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        call()
+    g.debug_dump(str(path))
+    return path.read_text()
+
+
 # What each p2g_mode runs, from the kernel names of a captured call: PAIR the
 # paired fused kernel at every size, AUTO the layer kernels up to their counts.
 @pytest.mark.parametrize("mode,n,fused", [("PAIR", 500, "k_g2p2g_pair"), ("PAIR", 38913, "k_g2p2g_pair"),
@@ -525,18 +536,12 @@ def test_kernels_of_a_mode(mode, n, fused, tmp_path):
     s, pin_d = _dev(st), to_dev(pin)
     wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
     mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0)
-    torch.cuda.synchronize()
-    g = torch.cuda.CUDAGraph(keep_graph=True)
-    g.enable_debug_mode()
-    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
-        mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0)
-    dot = tmp_path / "g.dot"
-    g.debug_dump(str(dot))
-    text = dot.read_text()
+    text = _kernels(lambda: mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0), tmp_path / "g.dot")
+    layers = ["k_layer_g2p"] if mode == "AUTO" else []  # the last G2P, with the first P2G at fewer particles
+    if layers and n <= 38912:
+        layers.append("k_layer_p2g")
     for name in ("k_g2p2g_pair", "k_layer_g2p", "k_layer_p2g", "k_grid_update_active"):
-        want = (name == fused or name == "k_grid_update_active"
-                or (mode == "AUTO" and name in ("k_layer_g2p", "k_layer_p2g")))  # the rollout's first P2G, last G2P
-        assert (name in text) == want, name
+        assert (name in text) == (name in (fused, "k_grid_update_active", *layers)), name
     assert fused in text
     mpm.close()
 
@@ -624,4 +629,19 @@ def test_wind_gradient_of_a_bad_cotangent(nf, frames, bad):
     assert 0 < np.isfinite(ref).sum() and np.array_equal(np.isfinite(got), np.isfinite(ref))
     ok = np.isfinite(ref)
     assert rel_l2(got[ok], ref[ok]) <= 1e-4
+    mpm.close()
+
+
+# The counts up to which a substep of AUTO runs the layer kernels.
+@pytest.mark.parametrize("n,layers", [(38912, ("p2g", "g2p")), (38913, ("g2p",)), (65536, ("g2p",)), (65537, ())])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_kernels_of_a_substep(n, layers, tmp_path):
+    pr, st, pin = _mpm_case(n, 24, 0)
+    mpm = B.MPM.from_params(pr, max_particles=n)
+    s, pin_d = _dev(st), to_dev(pin)
+    wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
+    mpm.substep(s, s, pin_d, wind, 0.0)
+    text = _kernels(lambda: mpm.substep(s, s, pin_d, wind, 0.0), tmp_path / "g.dot")
+    for k in ("p2g", "g2p"):
+        assert ("k_layer_" + k in text) == (k in layers)
     mpm.close()

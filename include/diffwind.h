@@ -131,8 +131,8 @@ enum { DW_NEOHOOKEAN = 0, DW_FIXED_COROTATED = 1 };
  * count: kernels that split a particle's work over its stencil's three layers,
  * for P2G and the fused kernel up to 38,912 particles and for G2P up to 65,536;
  * above, as PAIR. With AUTO or PAIR a segment adjoint of more than one substep
- * whose grids fit in the handle's grid tape runs its reverse pass in two
- * launches per substep (four otherwise). */
+ * and up to 196,608 particles, whose grids fit in the handle's grid tape, runs
+ * its reverse pass in two launches per substep (four otherwise). */
 enum { DW_P2G_AUTO = 0, DW_P2G_ATOMIC = 1, DW_P2G_WARP = 2, DW_P2G_TILE = 3, DW_P2G_PAIR = 4 };
 
 typedef struct {

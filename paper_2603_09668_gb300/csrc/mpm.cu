@@ -800,9 +800,9 @@ extern "C" dw_status mpm_segment_adjoint(dw_mpm h, const dw_mpm_state *start, fl
     // the recompute keeps each substep's grid when the grid tape fits; for the
     // fused kernels' modes it runs as one fused chain, and with the tape (and
     // more than one substep, so that a single one allocates nothing) so does
-    // the reverse pass
+    // the reverse pass of up to REV_CHAIN_MAX particles
     const bool fused = h->desc.p2g_mode == DW_P2G_AUTO || h->desc.p2g_mode == DW_P2G_PAIR;
-    const bool chain = fused && n > 0 && n_substeps > 1 && ensure_grid_tape(h, n_substeps);
+    const bool chain = fused && n > 0 && n <= REV_CHAIN_MAX && n_substeps > 1 && ensure_grid_tape(h, n_substeps);
     const bool gt = chain || ensure_grid_tape(h, n_substeps - 1);
     if (fused) {
         WindDev wd;

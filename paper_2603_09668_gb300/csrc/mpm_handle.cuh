@@ -131,7 +131,15 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
                             bool keep_grid, bool with_last, int *last_list, cudaStream_t s);
 
 // The reverse pass of a segment whose recompute kept every substep's grid
-// (with_last) and state, fused across substeps (mpm_layer.cu).
+// (with_last) and state, fused across substeps (mpm_layer.cu). Two launches per
+// substep instead of four, which pays up to REV_CHAIN_MAX particles (us per
+// substep of a segment, fused / four launches; a sheet on 64^3, a sheet on 128^3
+// and a block on 64^3, in cell order; in random order):
+//   100,000: 38.4 / 41.5, 43.1 / 46.2, 47.7 / 50.8; 101.1 / 106.8, 93.3 / 94.5, 91.7 / 92.8
+//   140,000: 48.3 / 50.9, 52.0 / 55.2, 56.1 / 58.1; 131.2 / 126.8, 120.6 / 119.3, 122.1 / 120.3
+//   200,000: 62.7 / 63.1, 66.3 / 66.4, 72.9 / 72.8; 197.2 / 188.2, 167.8 / 158.7, 167.1 / 156.7
+//   400,000: 109.0 / 104.9, 114.3 / 110.8, 119.8 / 116.7; 299.8 / 284.1, 286.0 / 264.8, 279.5 / 256.6
+constexpr int64_t REV_CHAIN_MAX = 3 << 16;
 dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *tape,
                           const dw_mpm_state *g, const uint8_t *pinned, const WindDev &wd, float t0,
                           int n_substeps, float *g_wind, float *g_E, int *reset_count,

@@ -645,3 +645,31 @@ def test_kernels_of_a_substep(n, layers, tmp_path):
     for k in ("p2g", "g2p"):
         assert ("k_layer_" + k in text) == (k in layers)
     mpm.close()
+
+
+# The count up to which a segment's reverse pass runs in two launches a substep,
+# and the gradients on both sides of it against P2G_WARP's: relative L2 1e-4 per
+# block (dL/dE left out, as in the paired recompute's test).
+@pytest.mark.parametrize("n,chain", [(196608, True), (196609, False)])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_kernels_of_a_segment(n, chain, tmp_path):
+    pr, st, pin = _mpm_case(n, 64, 0)
+    s, pin_d, steps = _dev(st), to_dev(pin), 3
+    wind = B.WindField(to_dev(inputs.fourier_wind(9, 3, seed=4)), 7 * pr["dt"])
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    g0 = [torch.randn(a.shape, generator=gen, device="cuda") for a in st]
+    got = []
+    for mode in (B.P2G_AUTO, B.P2G_WARP):
+        mpm = B.MPM.from_params(pr, max_particles=n, p2g_mode=mode)
+        gs = B.MpmState(*(a.clone() for a in g0))
+        gw, tape = torch.zeros_like(wind.values), torch.empty((steps - 1) * 24 * n, device="cuda")
+        call = lambda: mpm.segment_adjoint(s, tape, gs, pin_d, wind, 0.0, steps, gw)
+        call()
+        mpm.device_status()
+        got.append([a.cpu().numpy().astype(np.float64) for a in (*gs, gw)])
+        if mode == B.P2G_AUTO:
+            text = _kernels(call, tmp_path / "g.dot")
+            assert ("k_layer_rev" in text) == chain and ("k_rev_g2p" in text) == (not chain)
+        mpm.close()
+    for k, (a, b) in enumerate(zip(*got)):
+        assert rel_l2(a, b) <= 1e-4, k

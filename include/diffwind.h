@@ -129,10 +129,11 @@ enum { DW_NEOHOOKEAN = 0, DW_FIXED_COROTATED = 1 };
  * one-particle-per-thread fused kernel in mpm_rollout and single substeps in the
  * recompute. Elsewhere PAIR uses WARP. AUTO takes the fastest by the particle
  * count: kernels that split a particle's work over its stencil's three layers,
- * for P2G and the fused kernel up to 38,912 particles and for G2P up to 65,536;
- * above, as PAIR. With AUTO or PAIR a segment adjoint of more than one substep
- * and up to 196,608 particles, whose grids fit in the handle's grid tape, runs
- * its reverse pass in two launches per substep (four otherwise). */
+ * for P2G and the fused kernel up to 38,912 particles (the first P2G of a
+ * rollout or segment: 131,072) and for G2P up to 65,536; above, as PAIR. With
+ * AUTO or PAIR a segment adjoint of more than one substep and up to 196,608
+ * particles, whose grids fit in the handle's grid tape, runs its reverse pass in
+ * two launches per substep (four otherwise). */
 enum { DW_P2G_AUTO = 0, DW_P2G_ATOMIC = 1, DW_P2G_WARP = 2, DW_P2G_TILE = 3, DW_P2G_PAIR = 4 };
 
 typedef struct {

@@ -641,7 +641,7 @@ static dw_status substep_impl(dw_mpm h, const dw_mpm_state *in, const dw_mpm_sta
     int64_t n = in->n;
     {
         ProfScope ps(h, DW_K_P2G, s);
-        st = launch_p2g(h->desc.p2g_mode, h->P, in->x, in->v, in->C, in->F, n, h->grid_mp, h->err,
+        st = launch_p2g(h->desc.p2g_mode, LAYER_MAX_P2G, h->P, in->x, in->v, in->C, in->F, n, h->grid_mp, h->err,
                         active_blocks(h), s);
     }
     if (st != DW_OK) return st;
@@ -696,7 +696,7 @@ static dw_status substep_adjoint(dw_mpm h, const dw_mpm_state *in, const float *
     } else {
         {
             ProfScope ps(h, DW_K_P2G, s);
-            st = launch_p2g(h->desc.p2g_mode, h->P, in->x, in->v, in->C, in->F, n, h->grid_mp,
+            st = launch_p2g(h->desc.p2g_mode, LAYER_MAX_P2G, h->P, in->x, in->v, in->C, in->F, n, h->grid_mp,
                             h->err, active_blocks(h), s);
         }
         if (st != DW_OK) return st;
@@ -980,7 +980,7 @@ extern "C" dw_status mpm_substep_noalloc(const dw_mpm_desc *desc, const dw_mpm_s
     DW_CUDA(cudaMemsetAsync(grid_mp, 0, sizeof(float4) * (size_t)nodes, s));
     int64_t n = in->n;
     const ActiveBlocks dense{nullptr, nullptr, nullptr, 0};
-    st = launch_p2g(desc->p2g_mode, P, in->x, in->v, in->C, in->F, n, grid_mp, err, dense, s);
+    st = launch_p2g(desc->p2g_mode, LAYER_MAX_P2G, P, in->x, in->v, in->C, in->F, n, grid_mp, err, dense, s);
     if (st != DW_OK) return st;
     k_grid_update<<<grid_for(nodes, 256), 256, 0, s>>>(P, wd, t, grid_mp, grid_v, 1);
     DW_LAUNCHED("k_grid_update");

@@ -163,7 +163,15 @@ dw_status segment_reverse(MpmHandle *h, const dw_mpm_state *start, const float *
 // order (2 us) is gone by 65,536, and in random order, where every particle adds
 // to the grid by itself, it loses a quarter and more. G2P: 65,536, where it has
 // stopped gaining in either order.
+// The first P2G of a rollout or segment is another matter: the kernels after it
+// keep the split of the SMs' memory that it leaves, and after the layer kernel's
+// (most of it shared memory) they overlap better. A rollout's substep / 20 of them
+// and a segment of 6 (us), block on 64^3 in cell order, layer P2G first against the
+// one-particle one: 40,000: 18.3 / 607, 21.8 / 685; 100,000: 20.5 / 716, 20.9 / 746;
+// 131,072: 27.5 / 772, 28.2 / 779; in random order 30.2 / 953, 41.9 / 1245; 48.7 /
+// 1565, 55.8 / 1765; 57.1 / 1864, 66.2 / 2070 (sheets likewise). Not measured above.
 constexpr int64_t LAYER_ROUND = 32 * 8 * 152, LAYER_MAX_P2G = LAYER_ROUND, LAYER_MAX_G2P = 1 << 16;
+constexpr int64_t LAYER_MAX_CHAIN = 1 << 17;
 inline bool layer_fused(int mode, int64_t n) { return mode == DW_P2G_AUTO && n <= LAYER_ROUND; }
 dw_status launch_layer_p2g(const MpmParams &P, const float *x, const float *v, const float *C,
                            const float *F, int64_t n, float4 *grid, int *err,

@@ -135,11 +135,11 @@ __global__ void __launch_bounds__(P2G_TILE_THREADS) k_p2g_tile(MpmParams P,
     }
 }
 
-dw_status launch_p2g(int mode, const MpmParams &P, const float *x, const float *v,
-                            const float *C, const float *F, int64_t n, float4 *grid, int *err,
+dw_status launch_p2g(int mode, int64_t layer_max, const MpmParams &P, const float *x,
+                            const float *v, const float *C, const float *F, int64_t n, float4 *grid, int *err,
                             const ActiveBlocks &ab, cudaStream_t st) {
     if (n == 0) return DW_OK;
-    if (mode == DW_P2G_AUTO && n <= LAYER_MAX_P2G)
+    if (mode == DW_P2G_AUTO && n <= layer_max)
         return launch_layer_p2g(P, x, v, C, F, n, grid, err, ab, st);
     if (mode == DW_P2G_ATOMIC) {
         DW_CUDA(launch_pdl(k_p2g_atomic, grid_for(n, 128), 128, st, P, x, v, C, F, n, grid, err, ab));

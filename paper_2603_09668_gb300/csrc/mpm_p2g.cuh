@@ -309,7 +309,8 @@ __device__ __forceinline__ void p2g_warp_scatter(const MpmParams &P, P2GParticle
 }
 
 // Launches P2G of n particles into grid (DW_P2G_* strategy); defined in mpm_p2g.cu.
-dw_status launch_p2g(int mode, const MpmParams &P, const float *x, const float *v, const float *C,
+// layer_max: the particle count up to which AUTO takes the layer-split kernel.
+dw_status launch_p2g(int mode, int64_t layer_max, const MpmParams &P, const float *x, const float *v, const float *C,
                      const float *F, int64_t n, float4 *grid, int *err, const ActiveBlocks &ab,
                      cudaStream_t st);
 

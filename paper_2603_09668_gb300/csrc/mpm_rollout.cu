@@ -125,7 +125,7 @@ dw_status segment_recompute(MpmHandle *h, const dw_mpm_state *start, float *tape
     dw_status st;
     {
         ProfScope ps(h, DW_K_P2G, s);
-        st = launch_p2g(h->desc.p2g_mode, h->P, start->x, start->v, start->C, start->F, n,
+        st = launch_p2g(h->desc.p2g_mode, LAYER_MAX_CHAIN, h->P, start->x, start->v, start->C, start->F, n,
                         h->grid_mp, h->err, active_blocks(h, 0), s);
     }
     if (st != DW_OK) return st;
@@ -233,7 +233,7 @@ extern "C" dw_status mpm_rollout(dw_mpm h, const dw_mpm_state *state, uint8_t *p
     }
     {
         ProfScope ps(h, DW_K_P2G, s);
-        st = launch_p2g(h->desc.p2g_mode, h->P, cur.x, cur.v, cur.C, cur.F, n, h->grid_mp, h->err,
+        st = launch_p2g(h->desc.p2g_mode, LAYER_MAX_CHAIN, h->P, cur.x, cur.v, cur.C, cur.F, n, h->grid_mp, h->err,
                         active_blocks(h, L), s);
     }
     if (st != DW_OK) return st;

@@ -537,9 +537,7 @@ def test_kernels_of_a_mode(mode, n, fused, tmp_path):
     wind = B.WindField(to_dev(inputs.constant_wind(2, 1, (1.0, 0.0, 0.0))), 1.0)
     mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0)
     text = _kernels(lambda: mpm.rollout(s, pin_d, None, wind, 0.0, 3, 0), tmp_path / "g.dot")
-    layers = ["k_layer_g2p"] if mode == "AUTO" else []  # the last G2P, with the first P2G at fewer particles
-    if layers and n <= 38912:
-        layers.append("k_layer_p2g")
+    layers = ["k_layer_p2g", "k_layer_g2p"] if mode == "AUTO" else []  # the first P2G, the last G2P
     for name in ("k_g2p2g_pair", "k_layer_g2p", "k_layer_p2g", "k_grid_update_active"):
         assert (name in text) == (name in (fused, "k_grid_update_active", *layers)), name
     assert fused in text

@@ -1330,13 +1330,24 @@ static HomeParams home_params(const dw_lbm_desc &d) {
 // odd count. Up to 2^20 cells the populations (19 floats a cell) stay in L2
 // and the chain always wins (measured, us per call, tile / chain: 32^3 1 step
 // 20.9 / 9.7, 30 steps 517 / 94; 64^3 607 / 213 for 30; 96^3 1 step 47.6 /
-// 38.2). Above, its extra traffic has to pay off over the call: 128^3 2 steps
-// 152 / 166, 3 steps 253 / 222, 4 steps 304 / 285, 30 steps 2281 / 1823;
-// 192^3 4 steps 918 / 930, 10 steps 2295 / 2101.
-static bool home_on_populations(const LbmParams &L, int steps) {
+// 38.2). Above, its extra traffic has to pay off over the call. A step of the chain
+// takes 25 to 27 ps a cell; the tile kernel's falls from 32 at 128^3 to 25 at 200^3
+// and 23 at 256^3, less smoothly the better its tiles fit, and is a quarter more
+// with a mask (the chain's 8% more). Without a mask; with one:
+//   128^3: 2 steps 130 / 137, 171 / 183; 3: 220 / 187, 273 / 239; 4: 258 / 245, 324 / 301; 30: 1922 / 1640, 2305 / 1833
+//   131^3: 3 steps 245 / 231, 303 / 297; 4: 282 / 299, 355 / 369; 10: 704 / 684, 856 / 795; 30: 2106 / 1965, 2527 / 2213
+//   150^3: 3 steps 312 / 313, 390 / 407; 4: 355 / 407, 451 / 508; 10: 884 / 941, 1089 / 1105; 30: 2651 / 2719, 3211 / 3094
+//   160^3: 3 steps 403 / 353, 514 / 453; 4: 469 / 465, 611 / 575; 10: 1170 / 1086, 1478 / 1262; 30: 3505 / 3159, 4383 / 3554
+//   170^3: 3 steps 449 / 461, 572 / 599; 4: 512 / 596, 665 / 745; 10: 1277 / 1382, 1613 / 1626; 30: 3826 / 4003, 4778 / 4564
+//   192^3: 3 steps 639 / 599, 815 / 768; 4: 735 / 785, 961 / 973; 10: 1834 / 1836, 2339 / 2149; 30: 5501 / 5339, 6935 / 6070
+//   203^3: 3 steps 716 / 785, 921 / 1022; 10: 2031 / 2357, 2600 / 2806; 30: 6087 / 6832, 7701 / 7897
+//   256^3: 3 steps 1350 / 1389, 1777 / 1792; 10: 3830 / 4263, 5043 / 5066; 30: 11474 / 12389, 14940 / 14341
+static bool home_on_populations(const LbmParams &L, int steps, bool masked) {
     if (L.ncell <= (1 << 20)) return true;
+    if (L.ncell > (7 << 20)) return false;
     if (steps & 1) return steps >= 3;
-    return steps >= (L.ncell <= (1 << 22) ? 4 : 6);
+    if (L.ncell <= (1 << 21)) return steps >= 4;
+    return steps >= 10 && (masked || L.ncell <= (1 << 22));
 }
 
 // Planes per block: each block also rebuilds the two planes beyond its z
@@ -1391,7 +1402,7 @@ extern "C" dw_status lbm_home_step(dw_lbm h, float *m, const uint8_t *solid, int
     const uint32_t *links = nullptr;
     dw_status st = links_for_call(h, solid, s, &links);
     if (st != DW_OK) return st;
-    if (home_on_populations(L, steps)) {
+    if (home_on_populations(L, steps, links != nullptr)) {
         LbmParams LH = L;  // the inlet populations of this lattice
         for (int i = 0; i < 19; ++i) LH.feq_in[i] = H.g_in[i];
         dim3 rg, rb;

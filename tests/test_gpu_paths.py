@@ -671,3 +671,22 @@ def test_kernels_of_a_segment(n, chain, tmp_path):
         mpm.close()
     for k, (a, b) in enumerate(zip(*got)):
         assert rel_l2(a, b) <= 1e-4, k
+
+
+# HOME-LBM steps on populations or by tiles, by the lattice's cells, the steps of
+# the call and whether there is a mask.
+@pytest.mark.parametrize("shape,steps,masked,chain", [
+    ((128, 128, 64), 1, 0, True), ((128, 128, 65), 1, 0, False), ((128, 128, 65), 3, 0, True),
+    ((128, 128, 128), 4, 0, True), ((128, 128, 129), 8, 1, False), ((128, 128, 129), 10, 0, True),
+    ((256, 128, 129), 10, 0, False), ((256, 128, 129), 10, 1, True), ((256, 128, 224), 3, 0, True),
+    ((256, 128, 225), 3, 0, False), ((256, 128, 225), 30, 1, False)])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_kernels_of_home_steps(shape, steps, masked, chain, tmp_path):
+    lbm = B.LBM(shape, 0.6, u_inlet=(0.05, 0.0, 0.0), bc_x=1)
+    m = lbm.moments()
+    lbm.home_init(m, 1.0, (0.04, 0.0, 0.01))
+    solid = torch.zeros(shape[::-1], dtype=torch.uint8, device="cuda") if masked else None
+    lbm.home_step(m, solid, steps)
+    text = _kernels(lambda: lbm.home_step(m, solid, steps), tmp_path / "g.dot")
+    assert ("k_home_open" in text) == chain and ("k_home_step" in text) == (not chain)
+    lbm.close()

@@ -55,7 +55,7 @@ constexpr int GS_FINE = 3, GS_COARSE = 4;
 __host__ __device__ constexpr int gs_threads(int ts) { return 1 << (2 * ts); }
 constexpr int GS_SORT_MAX = 4096;   // keys of one tile k_gs_tile_sort holds
 constexpr int GS_SORT_THREADS = 128;
-constexpr int GS_BIG_CTAS = 304;    // two per SM
+constexpr int GS_BIG_CTAS = 608;    // four per SM
 constexpr int GS_ROW = 12;          // floats per Gaussian of the packed rows and of the 2D gradients
 constexpr int RS_THREADS = 256;
 constexpr int RS_TILE = RS_THREADS * 16;  // keys per sort block
@@ -495,9 +495,10 @@ __global__ void __launch_bounds__(128) k_gs_list(const int4 *__restrict__ rect,
     });
 }
 
-// The queued Gaussians' tiles, counted or (LIST) listed: 16 warps per Gaussian,
-// so that a few that cover the whole image do not leave a warp each with
-// thousands of tiles.
+// The queued Gaussians' tiles, counted or (LIST) listed: as many warps per
+// Gaussian as there are, up to sixteen, so that a few that cover the whole image
+// do not leave a warp each with thousands of tiles. (Always sixteen: 100,000 of 45
+// tiles each took 478 us to count, most warps without a tile.)
 template <bool LIST>
 __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big,
                                                 const uint32_t *__restrict__ big_count,
@@ -509,15 +510,18 @@ __global__ void __launch_bounds__(256) k_gs_big(const uint32_t *__restrict__ big
                                                 GsStat *__restrict__ stat) {
     const uint32_t queued = *big_count;
     if (!LIST && blockIdx.x == 0 && threadIdx.x == 0) stat->big = queued;
-    // sixteen warps, two blocks, per Gaussian; queued and the step stay far below 2^32
-    static_assert(GS_BIG_CTAS % 2 == 0, "two blocks per Gaussian");
-    const int lane = threadIdx.x & 31, slice = (int)(blockIdx.x % 2) * 8 + (threadIdx.x >> 5);
-    for (uint32_t q = blockIdx.x / 2; q < queued; q += gridDim.x / 2) {
+    if (queued == 0) return;
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * 8, warp = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const uint32_t per = min(16u, max(1u, warps / queued)), groups = warps / per;
+    const int slice = (int)(warp % per), step = 32 * (int)per;
+    if (warp / per >= groups) return;
+    for (uint32_t q = warp / per; q < queued; q += groups) {  // far below 2^32
         const int i = (int)big[q];
         const GsTiles g = gs_tiles(rect[i], true, tiles_x, ts);
         const unsigned long long k = LIST ? gs_key(key, i) : 0ull;
 #pragma unroll 4
-        for (int t = slice * 32 + lane; t < g.count; t += 512) {
+        for (int t = slice * 32 + lane; t < g.count; t += step) {
             const int tile = g.first + t / g.nx * tiles_x + t % g.nx;
             if (LIST)
                 list[atomicAdd(&ranges[tile].y, 1)] = k;

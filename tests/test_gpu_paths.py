@@ -690,3 +690,28 @@ def test_kernels_of_home_steps(shape, steps, masked, chain, tmp_path):
     text = _kernels(lambda: lbm.home_step(m, solid, steps), tmp_path / "g.dot")
     assert ("k_home_open" in text) == chain and ("k_home_step" in text) == (not chain)
     lbm.close()
+
+
+# Queued Gaussians (more than 16 tiles each) in numbers around the queue's warps
+# (4,864: one each, several each, a part each): all are listed in all tiles, each
+# once. Against the image drawn in nine parts of nine tiles each, which queue
+# none: Gaussians on the optical axis, whose pixel offsets are the same floats in
+# the parts, so the same bits.
+@pytest.mark.parametrize("n", [1, 2, 303, 305, 1621, 2433, 4863, 4864, 4865, 9000])
+def test_gaussian_queue_shares(n):
+    W, p = 72, 24
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x, F, s0 = (torch.zeros((k, n), device="cuda") for k in (3, 9, 6))
+    x[2] = torch.linspace(-0.4, 0.4, n, device="cuda")
+    F[::4] = 1.0
+    s0[:3] = 4.0
+    d = (x, F, s0, torch.rand((3, n), generator=g, device="cuda"), torch.full((n,), 0.5 / n ** 0.5, device="cuda"))
+    whole, part = B.GaussianRenderer(n, W, W), B.GaussianRenderer(n, p, p)
+    img = whole.render(B.camera(np.eye(3), (0.0, 0.0, 2.0), 400.0, 400.0, W / 2, W / 2, W, W), *d)
+    assert img.max() > 0.1
+    for y in range(0, W, p):
+        for x0 in range(0, W, p):
+            cam = B.camera(np.eye(3), (0.0, 0.0, 2.0), 400.0, 400.0, W / 2 - x0, W / 2 - y, p, p)
+            assert torch.equal(part.render(cam, *d), img[:, y:y + p, x0:x0 + p]), (x0, y)
+    whole.close()
+    part.close()

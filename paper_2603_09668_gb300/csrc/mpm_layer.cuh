@@ -175,11 +175,10 @@ __device__ __forceinline__ void layer_marks_store(const ActiveBlocks &ab, const 
 __device__ __forceinline__ void layer_p2g(const MpmParams &P, LayerSmem &sm, const Stencil &s,
                                           float A[9], float mv[3], int key, float mass,
                                           float4 *__restrict__ grid, const ActiveBlocks &ab) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5;
     const LayerMarks marks = layer_marks_load(ab, s, key, w);
     const LayerAffine L = layer_affine(P, s, A, mv, w);
     layer_scatter(P, s, L, w, mass, key, sm.rows[w], sm.keys, grid);
-    (void)lane;
     layer_marks_store(ab, marks);
 }
 

@@ -885,7 +885,7 @@ extern "C" dw_status surr_create(int32_t n, dw_surr *out) {
     DW_ALLOC(h->out, sizeof(float) * nv * 16);
     DW_ALLOC(h->out4, sizeof(float) * nv * 4);
     DW_ALLOC(h->g4, sizeof(bf16) * nv * 16);
-    h->part_chunks = std::max(h->nchunks, 2 * h->sms);
+    h->part_chunks = std::max(h->nchunks, h->sms);
     DW_ALLOC(h->part, sizeof(float) * (size_t)h->part_chunks * 27 * 32 * 32);
     DW_ALLOC(h->part_b, sizeof(float) * (size_t)h->part_chunks * 32);
     DW_ALLOC(h->fine, sizeof(float) * 4 * Nc);

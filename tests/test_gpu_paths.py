@@ -715,3 +715,16 @@ def test_gaussian_queue_shares(n):
             assert torch.equal(part.render(cam, *d), img[:, y:y + p, x0:x0 + p]), (x0, y)
     whole.close()
     part.close()
+
+
+# The weight gradient's partial sums are held once per CTA that can run: a
+# 27 x 32 x 32 block of floats each (the mma.sync kernel has fewer chunks at 16^3).
+def test_surrogate_partial_sums_memory():
+    B.Surrogate(16).close()  # the library's own first allocations
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    s = B.Surrogate(16)
+    used = free - torch.cuda.mem_get_info()[0]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert used <= sms * 27 * 32 * 32 * 4 + (10 << 20)
+    s.close()

@@ -361,9 +361,10 @@ __device__ __forceinline__ void tc_layer(TcPipe &pp, uint32_t taddr, const CUten
     if (warp == TC_LOAD_WARP) {
         if (lane == 0) {
             TcSeg c;
-            // A CTA without output slices copies no weights: its MMA thread waits for none,
-            // and nothing else would order a buffer's next copy after the last one.
-            if (tc_segment(n, nxy, 0, c)) {
+            // A CTA without output slices (only where there are fewer slices than CTAs)
+            // copies no weights: its MMA thread waits for none, and nothing else would
+            // order a buffer's next copy after the last one.
+            if (nxy * n >= (int)gridDim.x || tc_segment(n, nxy, 0, c)) {
                 if (own_wt) tc_copy_weights(pp, wb, own_wt, WBYTES);
                 if (next_wt) tc_copy_weights(pp, 1 - wb, next_wt, next_bytes);
             }

@@ -204,25 +204,26 @@ __device__ __forceinline__ void affine2(const MpmParams &P, const float2 F[9], c
                 if (i != j) A[3 * j + i] = fma(mk, tau, mul(pm, C[3 * j + i]));
             }
     } else {
-        float2 R[9];
-        polar_R2(F, ok0, ok1, R);
+        float2 R[9], G[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) G[k] = F[k];
+        if (!(ok0 && ok1)) {  // tau = 0, whatever F holds
+#pragma unroll
+            for (int k = 0; k < 9; ++k) G[k] = make_float2(ok0 ? F[k].x : 0.0f, ok1 ? F[k].y : 0.0f);
+        }
+        polar_R2(G, ok0, ok1, R);
         const float2 mu2 = make_float2(ok0 ? 2.0f * P.mu : 0.0f, ok1 ? 2.0f * P.mu : 0.0f);
         float2 c = mul(mul(s2(P.lam), add(J, s2(-1.0f))), J);
         c = make_float2(ok0 ? c.x : 0.0f, ok1 ? c.y : 0.0f);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) R[k] = mul(mu2, sub(F[k], R[k]));
+        for (int k = 0; k < 9; ++k) R[k] = mul(mu2, sub(G[k], R[k]));
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const float2 b = fma(R[3 * i + 2], F[3 * j + 2], fma(R[3 * i + 1], F[3 * j + 1], mul(R[3 * i], F[3 * j])));
+                const float2 b = fma(R[3 * i + 2], G[3 * j + 2], fma(R[3 * i + 1], G[3 * j + 1], mul(R[3 * i], G[3 * j])));
                 A[3 * i + j] = fma(mk, i == j ? add(b, c) : b, mul(pm, C[3 * i + j]));
             }
-        if (!(ok0 && ok1)) {  // tau = 0 whatever F holds: m C alone
-#pragma unroll
-            for (int k = 0; k < 9; ++k)
-                A[k] = make_float2(ok0 ? A[k].x : P.p_mass * C[k].x, ok1 ? A[k].y : P.p_mass * C[k].y);
-        }
     }
 }
 

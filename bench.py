@@ -335,7 +335,7 @@ ALGO_FLOP_PER_PS = 1991
 # dram__bytes_write.sum of the 41st launch of a 60-substep rollout, re-sorted
 # every 15); valid only for the kernel sources it was taken on (hash of the
 # files below), else reported as null.
-G2P2G_TRAFFIC = {"sha16": "8fe1c5cd625b46ba", "bytes": 20.10e6, "particles": 400040}
+G2P2G_TRAFFIC = {"sha16": "2191357741a775f8", "bytes": 20.09e6, "particles": 400040}
 G2P2G_SOURCES = ("mpm_rollout.cu", "mpm_pair_warp.cuh", "mpm_pair.cuh", "mpm_p2g.cuh",
                  "mpm_math.cuh")
 

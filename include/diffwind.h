@@ -697,9 +697,9 @@ DW_API dw_status lbm_home_init(dw_lbm h, float *m, float rho0, const float u0[3]
 /* Advance m in place by `steps` HOME-LBM steps. The handle's tape is the
  * workspace (max_tape >= 1 suffices): it holds the populations rebuilt from m
  * while the steps of the call run on them in place (the AA pattern of
- * lbm_step), or, for a few steps of a large lattice, a second moment lattice
- * (an odd step count then ends with one device copy back into m). solid as
- * in lbm_step. */
+ * lbm_step), or, for a few steps of a lattice above 2^20 cells and for every
+ * call above 7 x 2^20, a second moment lattice (an odd step count then ends
+ * with one device copy back into m). solid as in lbm_step. */
 DW_API dw_status lbm_home_step(dw_lbm h, float *m, const uint8_t *solid, int32_t steps,
                                dw_stream stream);
 

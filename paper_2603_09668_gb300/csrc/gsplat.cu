@@ -1503,12 +1503,12 @@ extern "C" dw_status gs_render(dw_gs h, const dw_camera *cam, const float *x, co
     h->last_n = -1;  // no picture to differentiate until this call has drawn one
     gs_set_tiles(h, GS_FINE);
     if (nn > 0) {
-        GsStat stat;
+        GsStat stat{};
         st = gs_count(h, c, x, F, sigma0, color, opacity, nn, stat, s);
         bool fits = stat.total <= (unsigned long long)GS_LIST_MAX;
         if (st == DW_OK && fits && stat.total > 0) st = gs_make_list(h, nn, stat, s);
         if (st == DW_ERR_OOM || (st == DW_OK && !fits)) {
-            gs_list_free(h);
+            if (st != DW_OK) gs_list_free(h);
             gs_set_tiles(h, GS_COARSE);
             st = gs_recount(h, nn, stat, s);
             if (st != DW_OK) return st;
